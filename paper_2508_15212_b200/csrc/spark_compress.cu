@@ -25,6 +25,8 @@ window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, floa
                     float* __restrict__ qnorm, const int32_t* __restrict__ seq_lens,
                     int32_t* __restrict__ packed_lens, int max_seq_tokens, int* status)
 {
+    grid_wait();
+    grid_release();
     const int h = blockIdx.x, b = blockIdx.y, j = threadIdx.x;
     const int G = Hq / Hkv;
     // the group's G*W window rows are consecutive in memory, (g outer, w inner)
@@ -357,6 +359,8 @@ struct CompressArgs {
 template <typename E, bool kRank>
 __global__ void __launch_bounds__(256) compress_pages_kernel(CompressArgs A)
 {
+    grid_wait();
+    grid_release();
     extern __shared__ __align__(16) unsigned char image[];
     const int blk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int len = A.lens[b];
@@ -585,6 +589,8 @@ __device__ __forceinline__ void pack_token16(unsigned char* image, int vals_off,
 template <typename E>
 __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 {
+    grid_wait();
+    grid_release();
     extern __shared__ __align__(16) unsigned char image[];
     constexpr bool kBf16 = (sizeof(E) == 2);
     constexpr int kWords = kBf16 ? 8 : 16;                     // 32-bit words of a lane's 16 channels
@@ -675,6 +681,8 @@ struct AppendArgs {
 template <typename E, bool kRank>
 __global__ void __launch_bounds__(32) append_token_kernel(AppendArgs A)
 {
+    grid_wait();
+    grid_release();
     constexpr bool kBf16 = (sizeof(E) == 2);
     const int h = blockIdx.x, b = blockIdx.y, lane = threadIdx.x;
     const PageLayout L = A.L;
@@ -710,6 +718,8 @@ __global__ void __launch_bounds__(32) append_token_kernel(AppendArgs A)
 template <typename E, bool kRank>
 __global__ void __launch_bounds__(1024) append_token_cta_kernel(AppendArgs A)
 {
+    grid_wait();
+    grid_release();
     constexpr bool kBf16 = (sizeof(E) == 2);
     const int b = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const PageLayout L = A.L;
@@ -745,6 +755,8 @@ __global__ void __launch_bounds__(1024) append_token_cta_kernel(AppendArgs A)
 
 __global__ void append_advance_kernel(AppendArgs A)
 {
+    grid_wait();
+    grid_release();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= A.B) return;
     const int t = A.packed_lens[b];
@@ -761,6 +773,8 @@ struct AppendBlockArgs {
 
 __global__ void __launch_bounds__(32) append_block_clear_kernel(AppendBlockArgs B_)
 {
+    grid_wait();
+    grid_release();
     const AppendArgs& A = B_.a;
     const int h = blockIdx.x, b = blockIdx.y, lane = threadIdx.x;
     const int t0 = A.packed_lens[b];
@@ -782,6 +796,8 @@ __global__ void __launch_bounds__(32) append_block_clear_kernel(AppendBlockArgs 
 template <typename E, bool kRank>
 __global__ void __launch_bounds__(32) append_block_token_kernel(AppendBlockArgs B_)
 {
+    grid_wait();
+    grid_release();
     constexpr bool kBf16 = (sizeof(E) == 2);
     const AppendArgs& A = B_.a;
     const int h = blockIdx.x, b = blockIdx.y, tok = blockIdx.z, lane = threadIdx.x;
@@ -811,6 +827,8 @@ __global__ void __launch_bounds__(32) append_block_token_kernel(AppendBlockArgs 
 
 __global__ void append_block_advance_kernel(AppendBlockArgs B_)
 {
+    grid_wait();
+    grid_release();
     const AppendArgs& A = B_.a;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= A.B) return;
@@ -854,24 +872,24 @@ spark_status launch_append(const spark_params& p, const void* k_new, const void*
     if (p.n_kv_heads <= 32) {                                  // one launch: a CTA per sequence, a warp per KV head
         const int threads = p.n_kv_heads * 32;
         if (p.dtype == SPARK_BF16) {
-            if (rank) append_token_cta_kernel<__nv_bfloat16, true><<<p.batch, threads, 0, stream>>>(A);
-            else append_token_cta_kernel<__nv_bfloat16, false><<<p.batch, threads, 0, stream>>>(A);
+            if (rank) launch_kernel(append_token_cta_kernel<__nv_bfloat16, true>, dim3(p.batch), dim3(threads), 0, stream, A);
+            else launch_kernel(append_token_cta_kernel<__nv_bfloat16, false>, dim3(p.batch), dim3(threads), 0, stream, A);
         } else {
-            if (rank) append_token_cta_kernel<float, true><<<p.batch, threads, 0, stream>>>(A);
-            else append_token_cta_kernel<float, false><<<p.batch, threads, 0, stream>>>(A);
+            if (rank) launch_kernel(append_token_cta_kernel<float, true>, dim3(p.batch), dim3(threads), 0, stream, A);
+            else launch_kernel(append_token_cta_kernel<float, false>, dim3(p.batch), dim3(threads), 0, stream, A);
         }
         *launches += 1;
         return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }
     const dim3 grid(p.n_kv_heads, p.batch);
     if (p.dtype == SPARK_BF16) {
-        if (rank) append_token_kernel<__nv_bfloat16, true><<<grid, 32, 0, stream>>>(A);
-        else append_token_kernel<__nv_bfloat16, false><<<grid, 32, 0, stream>>>(A);
+        if (rank) launch_kernel(append_token_kernel<__nv_bfloat16, true>, grid, dim3(32), 0, stream, A);
+        else launch_kernel(append_token_kernel<__nv_bfloat16, false>, grid, dim3(32), 0, stream, A);
     } else {
-        if (rank) append_token_kernel<float, true><<<grid, 32, 0, stream>>>(A);
-        else append_token_kernel<float, false><<<grid, 32, 0, stream>>>(A);
+        if (rank) launch_kernel(append_token_kernel<float, true>, grid, dim3(32), 0, stream, A);
+        else launch_kernel(append_token_kernel<float, false>, grid, dim3(32), 0, stream, A);
     }
-    append_advance_kernel<<<(p.batch + 127) / 128, 128, 0, stream>>>(A);
+    launch_kernel(append_advance_kernel, dim3((p.batch + 127) / 128), dim3(128), 0, stream, A);
     *launches += 2;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }
@@ -891,17 +909,17 @@ spark_status launch_append_block(const spark_params& p, const void* k_new, const
     A.status = static_cast<int*>(workspace);
     Bk.n_new = n_new;
     const int fresh = (n_new + kPageTokens - 1) / kPageTokens + 1;       // pages that can start inside the new tokens
-    append_block_clear_kernel<<<dim3(p.n_kv_heads, p.batch, fresh), 32, 0, stream>>>(Bk);
+    launch_kernel(append_block_clear_kernel, dim3(p.n_kv_heads, p.batch, fresh), dim3(32), 0, stream, Bk);
     const dim3 grid(p.n_kv_heads, p.batch, n_new);
     const bool rank = p.select != SPARK_SELECT_FIXED;
     if (p.dtype == SPARK_BF16) {
-        if (rank) append_block_token_kernel<__nv_bfloat16, true><<<grid, 32, 0, stream>>>(Bk);
-        else append_block_token_kernel<__nv_bfloat16, false><<<grid, 32, 0, stream>>>(Bk);
+        if (rank) launch_kernel(append_block_token_kernel<__nv_bfloat16, true>, grid, dim3(32), 0, stream, Bk);
+        else launch_kernel(append_block_token_kernel<__nv_bfloat16, false>, grid, dim3(32), 0, stream, Bk);
     } else {
-        if (rank) append_block_token_kernel<float, true><<<grid, 32, 0, stream>>>(Bk);
-        else append_block_token_kernel<float, false><<<grid, 32, 0, stream>>>(Bk);
+        if (rank) launch_kernel(append_block_token_kernel<float, true>, grid, dim3(32), 0, stream, Bk);
+        else launch_kernel(append_block_token_kernel<float, false>, grid, dim3(32), 0, stream, Bk);
     }
-    append_block_advance_kernel<<<(p.batch + 127) / 128, 128, 0, stream>>>(Bk);
+    launch_kernel(append_block_advance_kernel, dim3((p.batch + 127) / 128), dim3(128), 0, stream, Bk);
     *launches += 3;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }
@@ -915,6 +933,8 @@ __global__ void __launch_bounds__(128) merge_attn_kernel(int rows, const float* 
                                                          const float* __restrict__ out_b, const float* __restrict__ lse_b,
                                                          float* __restrict__ out, float* __restrict__ lse)
 {
+    grid_wait();
+    grid_release();
     const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (row >= rows) return;
     const float la = lse_a[row], lb = lse_b[row];
@@ -937,7 +957,7 @@ spark_status launch_merge_attn(int rows, const float* out_a, const float* lse_a,
                                float* out, float* lse, cudaStream_t stream)
 {
     if (rows == 0) return SPARK_OK;
-    merge_attn_kernel<<<(rows + 3) / 4, 128, 0, stream>>>(rows, out_a, lse_a, out_b, lse_b, out, lse);
+    launch_kernel(merge_attn_kernel, dim3((rows + 3) / 4), dim3(128), 0, stream, rows, out_a, lse_a, out_b, lse_b, out, lse);
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }
 
@@ -964,6 +984,8 @@ struct UnpackArgs {
 
 __global__ void __launch_bounds__(128) unpack_pages_kernel(UnpackArgs A)
 {
+    grid_wait();
+    grid_release();
     const int blk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const PageLayout L = A.L;
     const int T = L.keep;
@@ -1066,11 +1088,11 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const float eps = p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f;
     const dim3 qgrid(p.n_kv_heads, p.batch);
     if (p.dtype == SPARK_BF16)
-        window_qnorm_kernel<__nv_bfloat16><<<qgrid, kHeadDim, 0, stream>>>(
-            q_win, p.n_q_heads, p.n_kv_heads, p.window, eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
+        launch_kernel(window_qnorm_kernel<__nv_bfloat16>, qgrid, dim3(kHeadDim), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
+                      eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
     else
-        window_qnorm_kernel<float><<<qgrid, kHeadDim, 0, stream>>>(
-            q_win, p.n_q_heads, p.n_kv_heads, p.window, eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
+        launch_kernel(window_qnorm_kernel<float>, qgrid, dim3(kHeadDim), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
+                      eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
 
@@ -1088,11 +1110,11 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const dim3 grid(n_blocks, p.n_kv_heads, p.batch);
     const bool rank = p.select != SPARK_SELECT_FIXED;      // a ratio-free rule: the kernels with the rank sort
     if (p.dtype == SPARK_BF16) {
-        if (rank) compress_pages_kernel<__nv_bfloat16, true><<<grid, 256, A.L.page_bytes, stream>>>(A);
-        else compress_pages4_kernel<__nv_bfloat16><<<grid, 128, A.L.page_bytes, stream>>>(A);
+        if (rank) launch_kernel(compress_pages_kernel<__nv_bfloat16, true>, grid, dim3(256), A.L.page_bytes, stream, A);
+        else launch_kernel(compress_pages4_kernel<__nv_bfloat16>, grid, dim3(128), A.L.page_bytes, stream, A);
     } else {
-        if (rank) compress_pages_kernel<float, true><<<grid, 256, A.L.page_bytes, stream>>>(A);
-        else compress_pages4_kernel<float><<<grid, 128, A.L.page_bytes, stream>>>(A);
+        if (rank) launch_kernel(compress_pages_kernel<float, true>, grid, dim3(256), A.L.page_bytes, stream, A);
+        else launch_kernel(compress_pages4_kernel<float>, grid, dim3(128), A.L.page_bytes, stream, A);
     }
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
@@ -1111,7 +1133,7 @@ spark_status launch_unpack(const spark_params& p, const void* pages, const int32
     A.max_blocks = max_blocks; A.lens = packed_lens; A.max_tokens = max_tokens; A.Hkv = p.n_kv_heads;
     A.n_pool_pages = p.n_pool_pages; A.L = make_layout(p);
     A.mask = mask; A.mu = mu; A.vals = vals; A.v = v; A.vmask = vmask; A.mu_all = mu_all; A.sigma_all = sigma_all;
-    unpack_pages_kernel<<<dim3(n_blocks, p.n_kv_heads, p.batch), 128, 0, stream>>>(A);
+    launch_kernel(unpack_pages_kernel, dim3(n_blocks, p.n_kv_heads, p.batch), dim3(128), 0, stream, A);
     if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
     return SPARK_OK;
 }

@@ -108,7 +108,6 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     const int max_tokens = A.max_blocks * kPageTokens;
 
     prefetch_block_table(A, tid, kDecodeThreads);
-    if (tid == 0) pdl_launch_dependents();
     if (warp == kConsumerWarps) {
         producer_prologue(A, C, lane, kDecodeThreads);
         int p0, p1;
@@ -120,7 +119,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     const int* prefix = C.prefix;
     int c0, c1;
     cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
-    pdl_dependency_wait();                                 // q, qnorm, out and the workspace from here on
+    grid_wait();                                           // q, qnorm, out and the workspace from here on
     write_empty_sequences<kConsumerThreads>(A, prefix, tid);
 
     float* pscr = pscr_all + warp * 32 * GPP;
@@ -392,7 +391,7 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     const size_t smem = A.ring_off + static_cast<size_t>(ns) * A.slot_stride;
     if (!allow_max_smem(decode_scalar_kernel<G, E, R>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
     const int grid = n_sms < kMaxCtas ? n_sms : kMaxCtas;
-    return launch_decode_kernel(decode_scalar_kernel<G, E, R>, grid, kDecodeThreads, smem, stream, A) == cudaSuccess
+    return launch_kernel(decode_scalar_kernel<G, E, R>, dim3(grid), dim3(kDecodeThreads), smem, stream, A) == cudaSuccess
                ? SPARK_OK : SPARK_ERR_CUDA;
 }
 

@@ -42,7 +42,7 @@ struct DecodeArgs {
     int pps;                                 // pages per step (= per ring slot): 1 or 2
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix ((B + 1) ints)
     int ring_off;                            // shared-memory offset of the ring (behind the prefix)
-    int overlap;                             // launched as a programmatic dependent of the preceding kernel
+    int overlap;                             // the page stream need not wait for the kernel before (SPARK_FLAG_OVERLAP_PREVIOUS)
     unsigned seed;                           // sampled recovery: seed of the per-entry draws
     const int* page_rows;                    // ragged pages: slot rows in use per pool page (else null: whole pages)
     int q_by_value;                          // host side only: q is a HOST pointer whose bytes travel as a launch parameter
@@ -161,30 +161,6 @@ __device__ __forceinline__ bool slot_wait(uint64_t* full, volatile int* seq, int
     }
     return mbar_wait(&full[slot], round & 1, abort_flag, status);
 }
-// Programmatic dependent launch (sm_90+).  launch_dependents: the kernel enqueued after this one may be
-// scheduled as CTAs of this grid exit.  dependency_wait: returns once the kernel enqueued before this
-// one has completed and its writes are visible (a no-op for an ordinary launch).
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// Launch helper: ordinary launch, or with the programmatic-stream-serialization attribute.
-template <typename Kernel, typename... More>
-inline cudaError_t launch_decode_kernel(Kernel kernel, int grid, int threads, size_t smem, cudaStream_t stream,
-                                        const DecodeArgs& A, const More&... more)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = A.overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, A, more...);
-}
-
 template <int NT> __device__ __forceinline__ void consumer_sync()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
@@ -274,7 +250,7 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off)
 //
 // All threads first ask the L2 to fetch the block table (when there is one): the producer's page-id
 // loads then find their lines on the way instead of starting a second cold DRAM round trip behind
-// packed_lens.
+// packed_lens.  (A hint: it may run before the kernel ahead has completed.)
 constexpr int kPlanBarrier = 2;
 constexpr int64_t kTablePrefetchMax = 8 << 20;             // bytes of block table asked for at most
 
@@ -292,20 +268,19 @@ __device__ __forceinline__ void prefetch_block_table(const DecodeArgs& A, int ti
 __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads)
 {
     const int max_tokens = A.max_blocks * kPageTokens;
-    // packed_lens first: everything else of the prologue fits under this load's latency
-    int first_len = 0;
-    if (lane < A.B) first_len = A.lens[lane];
     if (lane < A.nslots) { mbar_init(&C.full[lane], 1); mbar_init(&C.empty[lane], 1); }
     C.seq[lane] = 0;
     if (lane == 0) { *C.abort_flag = 0; *C.last_flag = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (!A.overlap) grid_wait();                           // with the flag the page stream does not depend on the kernel before
+    grid_release();
     int running = 0, smin = 0x7fffffff, smax = 0;
     for (int b0 = 0; b0 < A.B; b0 += 32) {
         const int b = b0 + lane;
         int st = 0;
         if (b < A.B) {
-            const int len = b0 == 0 ? first_len : A.lens[b];
+            const int len = A.lens[b];
             if (len < 0 || len > max_tokens) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
             st = steps_of(clamp_len(len, max_tokens), A.pps);
             smin = min(smin, st);

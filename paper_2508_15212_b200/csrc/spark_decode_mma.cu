@@ -240,7 +240,6 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     const int max_tokens = A.max_blocks * kPageTokens;
 
     prefetch_block_table(A, tid, kThreads);
-    if (tid == 0) pdl_launch_dependents();
     if (warp == kNW) {
         producer_prologue(A, C, lane, kThreads);
         int p0, p1;
@@ -252,7 +251,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     const int* prefix = C.prefix;
     int c0, c1;
     cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
-    pdl_dependency_wait();                                 // q, qnorm, out and the workspace from here on
+    grid_wait();                                           // q, qnorm, out and the workspace from here on
     write_empty_sequences<kNT>(A, prefix, tid);
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
@@ -515,7 +514,7 @@ static spark_status launch_bf16_qv(const DecodeArgs& A, int dev, int smem_optin,
     if (!allow_max_smem(decode_bf16_qv_kernel<G, kBytes>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
     QueryBlob<kBytes> blob;                                 // A.q is a host pointer here; the bytes are taken now
     memcpy(&blob, A.q, q_bytes);
-    return launch_decode_kernel(decode_bf16_qv_kernel<G, kBytes>, grid, kThreads, smem, stream, A, blob) == cudaSuccess
+    return launch_kernel(decode_bf16_qv_kernel<G, kBytes>, dim3(grid), dim3(kThreads), smem, stream, A, blob) == cudaSuccess
                ? SPARK_OK : SPARK_ERR_CUDA;
 }
 
@@ -544,7 +543,7 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
         return launch_bf16_qv<G, kBlobLarge>(A, dev, smem_optin, grid, smem, q_bytes, stream);
     }
     if (!allow_max_smem(decode_bf16_kernel<G, kPV>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
-    return launch_decode_kernel(decode_bf16_kernel<G, kPV>, grid, kThreads, smem, stream, A) == cudaSuccess
+    return launch_kernel(decode_bf16_kernel<G, kPV>, dim3(grid), dim3(kThreads), smem, stream, A) == cudaSuccess
                ? SPARK_OK : SPARK_ERR_CUDA;
 }
 

@@ -47,6 +47,8 @@ struct EvictArgs {
 template <typename E, int PASS>
 __global__ void __launch_bounds__(kEvThreads) evict_scores_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     extern __shared__ __align__(16) float ev_smem[];
     float* Ks = ev_smem;                                   // [128][129]
     float* Qs = Ks + kEvTile * kEvStride;                  // [64][129]
@@ -163,6 +165,8 @@ __global__ void __launch_bounds__(kEvThreads) evict_scores_kernel(EvictArgs A)
 
 __global__ void evict_rowstats_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     const int h = blockIdx.x, b = blockIdx.y;
     const int S = min(A.seq_lens[b], A.S_max);
     if (S <= A.budget) return;
@@ -188,6 +192,8 @@ __global__ void evict_rowstats_kernel(EvictArgs A)
 // float's bit pattern: votes are >= 0, so unsigned comparison of the patterns is the order of the values.
 __global__ void __launch_bounds__(256) evict_pool_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     const int h = blockIdx.y, b = blockIdx.z;
     const int S = min(A.seq_lens[b], A.S_max);
     if (S <= A.budget) return;
@@ -255,6 +261,8 @@ __device__ __forceinline__ SelState select_state(const int* hist, int passes, in
 template <int PASS>
 __global__ void __launch_bounds__(kSelThreads) evict_hist_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     __shared__ int sh[256];
     __shared__ SelState st;
     const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
@@ -293,6 +301,8 @@ __global__ void __launch_bounds__(kSelThreads) evict_hist_kernel(EvictArgs A)
 // counts[unit][chunk] = (keys above the threshold, keys equal to it) in the chunk
 __global__ void __launch_bounds__(kSelThreads) evict_count_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     __shared__ SelState st;
     __shared__ int red[2][kSelThreads / 32];
     const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
@@ -330,6 +340,8 @@ __global__ void __launch_bounds__(kSelThreads) evict_count_kernel(EvictArgs A)
 // and handles sequences that are kept whole.
 __global__ void __launch_bounds__(kSelThreads) evict_compact_kernel(EvictArgs A)
 {
+    grid_wait();
+    grid_release();
     __shared__ SelState st;
     __shared__ int s_base_kept, s_base_eq;
     __shared__ int scan_eq[kSelThreads / 32], scan_keep[kSelThreads / 32];
@@ -470,24 +482,24 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
         cudaError_t e2 = bf16 ? cudaFuncSetAttribute(evict_scores_kernel<__nv_bfloat16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
                               : cudaFuncSetAttribute(evict_scores_kernel<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e1 != cudaSuccess || e2 != cudaSuccess) return SPARK_ERR_CUDA;
-        if (bf16) evict_scores_kernel<__nv_bfloat16, 1><<<grid, kEvThreads, smem, stream>>>(A);
-        else evict_scores_kernel<float, 1><<<grid, kEvThreads, smem, stream>>>(A);
-        evict_rowstats_kernel<<<ugrid, 256, 0, stream>>>(A);
-        if (bf16) evict_scores_kernel<__nv_bfloat16, 2><<<grid, kEvThreads, smem, stream>>>(A);
-        else evict_scores_kernel<float, 2><<<grid, kEvThreads, smem, stream>>>(A);
+        if (bf16) launch_kernel(evict_scores_kernel<__nv_bfloat16, 1>, grid, dim3(kEvThreads), smem, stream, A);
+        else launch_kernel(evict_scores_kernel<float, 1>, grid, dim3(kEvThreads), smem, stream, A);
+        launch_kernel(evict_rowstats_kernel, ugrid, dim3(256), 0, stream, A);
+        if (bf16) launch_kernel(evict_scores_kernel<__nv_bfloat16, 2>, grid, dim3(kEvThreads), smem, stream, A);
+        else launch_kernel(evict_scores_kernel<float, 2>, grid, dim3(kEvThreads), smem, stream, A);
         *launches += 3;
     }
     const dim3 sgrid(A.n_chunks, p.n_kv_heads, p.batch);
     if (max_seq_tokens > p.token_budget) {
-        evict_pool_kernel<<<dim3((max_seq_tokens + 255) / 256, p.n_kv_heads, p.batch), 256, 0, stream>>>(A);
-        evict_hist_kernel<0><<<sgrid, kSelThreads, 0, stream>>>(A);
-        evict_hist_kernel<1><<<sgrid, kSelThreads, 0, stream>>>(A);
-        evict_hist_kernel<2><<<sgrid, kSelThreads, 0, stream>>>(A);
-        evict_hist_kernel<3><<<sgrid, kSelThreads, 0, stream>>>(A);
-        evict_count_kernel<<<sgrid, kSelThreads, 0, stream>>>(A);
+        launch_kernel(evict_pool_kernel, dim3((max_seq_tokens + 255) / 256, p.n_kv_heads, p.batch), dim3(256), 0, stream, A);
+        launch_kernel(evict_hist_kernel<0>, sgrid, dim3(kSelThreads), 0, stream, A);
+        launch_kernel(evict_hist_kernel<1>, sgrid, dim3(kSelThreads), 0, stream, A);
+        launch_kernel(evict_hist_kernel<2>, sgrid, dim3(kSelThreads), 0, stream, A);
+        launch_kernel(evict_hist_kernel<3>, sgrid, dim3(kSelThreads), 0, stream, A);
+        launch_kernel(evict_count_kernel, sgrid, dim3(kSelThreads), 0, stream, A);
         *launches += 6;
     }
-    evict_compact_kernel<<<sgrid, kSelThreads, 0, stream>>>(A);
+    launch_kernel(evict_compact_kernel, sgrid, dim3(kSelThreads), 0, stream, A);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }

@@ -137,6 +137,8 @@ __device__ __forceinline__ void tc_stage_rows_async(unsigned dst_u, int rows_all
 template <int PASS>
 __global__ void __launch_bounds__(kTcThreads, 2) evict_scores_tc_kernel(EvictTcArgs A)
 {
+    grid_wait();
+    grid_release();
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     __shared__ __align__(8) uint64_t mma_bar;
     __shared__ unsigned tmem_base_s;
@@ -325,6 +327,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) evict_scores_tc_kernel(EvictTcA
 // merge the per-CTA partials of pass 1 into the rows' softmax normalisers
 __global__ void evict_rowstats_tc_kernel(EvictTcArgs A, float* rowstat)
 {
+    grid_wait();
+    grid_release();
     const int h = blockIdx.x, b = blockIdx.y;
     const int S = min(A.seq_lens[b], A.S_max);
     if (S <= A.budget) return;
@@ -380,9 +384,9 @@ spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, con
         cudaFuncSetAttribute(evict_scores_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return SPARK_ERR_CUDA;
     const dim3 grid(A.parts, p.n_kv_heads, p.batch), ugrid(p.n_kv_heads, p.batch);
-    evict_scores_tc_kernel<1><<<grid, kTcThreads, smem, stream>>>(A);
-    evict_rowstats_tc_kernel<<<ugrid, 256, 0, stream>>>(A, rowstat);
-    evict_scores_tc_kernel<2><<<grid, kTcThreads, smem, stream>>>(A);
+    launch_kernel(evict_scores_tc_kernel<1>, grid, dim3(kTcThreads), smem, stream, A);
+    launch_kernel(evict_rowstats_tc_kernel, ugrid, dim3(256), 0, stream, A, rowstat);
+    launch_kernel(evict_scores_tc_kernel<2>, grid, dim3(kTcThreads), smem, stream, A);
     *launches += 3;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }
