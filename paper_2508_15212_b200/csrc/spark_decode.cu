@@ -77,11 +77,13 @@ template <int G> struct SmemF32 {
     static constexpr int GP = ((G + 1 + 3) / 4) * 4;     // floats per table entry: G scaled queries + 1/a
     static constexpr int GPD = ((G + 1 + 1) / 2) * 2;    // doubles per table entry (degenerate rule: double table)
     static constexpr int GPP = ((G + 3) / 4) * 4;        // floats per probability entry
-    static constexpr int kQtab = kCtrlBytes;
-    static constexpr int kQsum = kQtab + kHeadDim * GPD * 8;     // sized for the double table (>= the float one)
-    static constexpr int kPscr = kQsum + 64;             // Qsum: [8] double
+    static constexpr int kCap = 2;                       // units per epoch (their tables are large)
+    static constexpr int kTabBytes = kHeadDim * GPD * 8; // sized for the double table (>= the float one)
+    static constexpr int kQtab = kCtrlBytes;             // [kCap] tables
+    static constexpr int kQsum = kQtab + kCap * kTabBytes;       // [kCap][8] double
+    static constexpr int kPscr = kQsum + kCap * 64;
     static constexpr int kMerge = kPscr + kConsumerWarps * 32 * GPP * 4;
-    static constexpr int kFixed = (kMerge + merge_bytes(kConsumerWarps, G) + 127) / 128 * 128;   // prefix and ring start here
+    static constexpr int kFixed = (kMerge + merge_bytes(kConsumerWarps, kCap, G) + 127) / 128 * 128;   // prefix and ring start here
 };
 
 template <int G, typename E, int R>
@@ -95,251 +97,267 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     using TabT = typename std::conditional<kDbl, double, float>::type;
     constexpr int GP = kDbl ? S::GPD : S::GP, GPP = S::GPP;
     extern __shared__ __align__(128) unsigned char smem[];
-    const Ctrl C = make_ctrl(smem, A.prefix_off);
-    TabT* qtab = reinterpret_cast<TabT*>(smem + S::kQtab);
-    double* qsum = reinterpret_cast<double*>(smem + S::kQsum);
+    const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
+    double* qsum_all = reinterpret_cast<double*>(smem + S::kQsum);
     float* pscr_all = reinterpret_cast<float*>(smem + S::kPscr);
     float* merge = reinterpret_cast<float*>(smem + S::kMerge);
+    float* unit_ml = merge + merge_state_floats(kConsumerWarps, S::kCap, G);
     unsigned char* ring = smem + A.ring_off;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const PageLayout L = A.L;
     const int NS = A.nslots;
-    const int max_tokens = A.max_blocks * kPageTokens;
 
     prefetch_block_table(A, tid, kDecodeThreads);
     if (warp == kConsumerWarps) {
         producer_prologue(A, C, lane, kDecodeThreads);
         int p0, p1;
         cta_range(*C.plan, static_cast<int>(blockIdx.x), p0, p1);
-        producer_loop(A, C, ring, p0, p1, lane);
+        producer_loop<kConsumerWarps>(A, C, ring, p0, p1, lane);
         return;
     }
     consumer_wait_plan(kDecodeThreads);
-    const int* prefix = C.prefix;
     int c0, c1;
     cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
     grid_wait();                                           // q, qnorm, out and the workspace from here on
-    write_empty_sequences<kConsumerThreads>(A, prefix, tid);
+    write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
 
     float* pscr = pscr_all + warp * 32 * GPP;
-    int base = 0;                                          // ordinal (within this CTA) of the segment's first step
     for (int g = c0; g < c1;) {
-        const Segment sg = locate(prefix, A.B, A.Hkv, g, c1);
-        const int b = sg.b, h = sg.h;
-        const int len = clamp_len(A.lens[b], max_tokens);
+        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, S::kCap, g, c1);
 
         // ---- per-unit table: entry j = { q_0[j]*c, ..., q_{G-1}[j]*c, 1/a[j] },  c = scale*log2(e)
-        for (int idx = tid; idx < kHeadDim * GP; idx += kConsumerThreads) {
-            const int j = idx / GP, e = idx - j * GP;
-            TabT val = 0;
-            if (e < G)
-                val = static_cast<TabT>(load_query<E>(A.q, (static_cast<int64_t>(b) * A.Hq + h * G + e) * kHeadDim + j)) *
-                      static_cast<TabT>(A.scale_log2e);
-            else if (e == G)
-                val = static_cast<TabT>(1) / static_cast<TabT>(A.qnorm[(static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + j]);
-            qtab[idx] = val;
-        }
-        consumer_sync<kConsumerThreads>();
-        if (warp < G) {                                    // Qsum[g] = sum_j q_g[j]*c / a[j]
-            double part = 0.0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const TabT* e = qtab + (lane * 4 + i) * GP;
-                part += static_cast<double>(e[warp]) * static_cast<double>(e[G]);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
-            if (lane == 0) qsum[warp] = part;
-        }
-        consumer_sync<kConsumerThreads>();
-
-        float m_run[G], l_run[G], acc[G][4];
-#pragma unroll
-        for (int gg = 0; gg < G; ++gg) {
-            m_run[gg] = -INFINITY;
-            l_run[gg] = 0.f;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[gg][c] = 0.f;
-        }
-
-        // first ordinal >= base that this warp owns
-        int n = base + ((warp - base) % kConsumerWarps + kConsumerWarps) % kConsumerWarps;
-        for (; n < base + sg.n; n += kConsumerWarps) {
-            const int i = sg.i0 + (n - base);
-            const int slot = n % NS;
-            const bool ok = slot_wait(C.full, C.seq, slot, n / NS, C.abort_flag, A.status);
-            const unsigned char* sbase = ring + static_cast<size_t>(slot) * A.slot_stride;
-            const int n_valid = min(kStepTokens, len - i * kStepTokens);
-            if (ok) {
-                // ---------------- scores: lane = token ----------------
-                float s[G];
-                const bool valid = lane < n_valid;
-                if (valid) {
-                    const unsigned char* page = sbase + (lane >> 4) * L.page_bytes;
-                    const int p = lane & 15;
-                    const uint4 mk = *reinterpret_cast<const uint4*>(page + L.mask_off + p * 16);
-                    const unsigned words[4] = {mk.x, mk.y, mk.z, mk.w};
-                    // kept slot s of token p (see val_offset): fp32 rows hold token p at element p, bf16 rows at
-                    // element (p & 7) * 2 + (p >> 3); rows are 16 elements apart
-                    const unsigned char* vp = page + L.vals_off + (kBf16 ? ((p & 7) * 2 + (p >> 3)) * 2 : p * 4);
-                    constexpr int kRowBytes = kPageTokens * static_cast<int>(sizeof(E));
-                    // sampled rules: fp32 storage sums the score in double as well (bf16 storage: fp32 is ample)
-                    using AccT = typename std::conditional<kBf16, float, double>::type;
-                    AccT a[G];
-#pragma unroll
-                    for (int gg = 0; gg < G; ++gg) a[gg] = 0;
-                    if constexpr (R == 0) {
-                        // fp32 storage is the high-precision configuration: the score of a token is summed in
-                        // double from a double table (products of two fp32 numbers are exact there), so that the
-                        // error of the step is that of the exponentials and of the fp32 value sums alone
-                        const double mu_d = static_cast<double>(*reinterpret_cast<const float*>(page + L.mu_off + p * 4));
-                        double ad[G];
-#pragma unroll
-                        for (int gg = 0; gg < G; ++gg) ad[gg] = 0.0;
-#pragma unroll
-                        for (int wi = 0; wi < 4; ++wi) {
-                            unsigned w = words[wi];
-                            const double* tb = qtab + wi * 32 * GP;
-                            while (w) {
-                                const int bp = __ffs(w) - 1;
-                                w &= w - 1;
-                                const double* e = tb + bp * GP;
-                                const float kv = *reinterpret_cast<const float*>(vp);
-                                vp += kRowBytes;
-                                double tv[GP];
-#pragma unroll
-                                for (int c2 = 0; c2 < GP / 2; ++c2) {
-                                    const double2 f = reinterpret_cast<const double2*>(e)[c2];
-                                    tv[2 * c2] = f.x; tv[2 * c2 + 1] = f.y;
-                                }
-                                const double x = fma(-mu_d, tv[G], static_cast<double>(kv));
-#pragma unroll
-                                for (int gg = 0; gg < G; ++gg) ad[gg] = fma(tv[gg], x, ad[gg]);
-                            }
-                        }
-#pragma unroll
-                        for (int gg = 0; gg < G; ++gg) s[gg] = static_cast<float>(fma(mu_d, qsum[gg], ad[gg]));
-                    } else {
-                        // sampled recovery: every channel contributes, kept ones their stored value, pruned
-                        // ones a draw divided by a[j]
-                        const float mean = *reinterpret_cast<const float*>(page + L.stats_off + p * 4);
-                        const float dev = *reinterpret_cast<const float*>(page + L.stats_off + (kPageTokens + p) * 4);
-                        const unsigned long long unit_t =
-                            (static_cast<unsigned long long>(b * A.Hkv + h) << 40) ^
-                            (static_cast<unsigned long long>(i * kStepTokens + lane) << 8);
+        UnitRef u = ep.first;
 #pragma unroll 1
-                        for (int wi = 0; wi < 4; ++wi) {
-                            const unsigned w = words[wi];
-#pragma unroll 4
-                            for (int bp = 0; bp < 32; ++bp) {
-                                const int j = wi * 32 + bp;
-                                const float* e = qtab + j * GP;
-                                float tv[GP];
+        for (int e = 0; e < ep.n_units; ++e) {
+            if (e) next_unit(C.prefix, A.Hkv, u);
+            TabT* qtab = reinterpret_cast<TabT*>(smem + S::kQtab + e * S::kTabBytes);
+            for (int idx = tid; idx < kHeadDim * GP; idx += kConsumerThreads) {
+                const int j = idx / GP, col = idx - j * GP;
+                TabT val = 0;
+                if (col < G)
+                    val = static_cast<TabT>(load_query<E>(A.q, (static_cast<int64_t>(u.b) * A.Hq + u.h * G + col) * kHeadDim + j)) *
+                          static_cast<TabT>(A.scale_log2e);
+                else if (col == G)
+                    val = static_cast<TabT>(1) / static_cast<TabT>(A.qnorm[(static_cast<int64_t>(u.b) * A.Hkv + u.h) * kHeadDim + j]);
+                qtab[idx] = val;
+            }
+        }
+        consumer_sync<kConsumerThreads>();
+#pragma unroll 1
+        for (int e = 0; e < ep.n_units; ++e)
+            if (warp < G) {                                // Qsum[g] = sum_j q_g[j]*c / a[j]
+                const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kQtab + e * S::kTabBytes);
+                double part = 0.0;
 #pragma unroll
-                                for (int c4 = 0; c4 < GP / 4; ++c4) {
-                                    const float4 f = reinterpret_cast<const float4*>(e)[c4];
-                                    tv[4 * c4] = f.x; tv[4 * c4 + 1] = f.y; tv[4 * c4 + 2] = f.z; tv[4 * c4 + 3] = f.w;
-                                }
-                                AccT x;
-                                if ((w >> bp) & 1u) {
-                                    x = kBf16 ? bf16_bits_to_float(*reinterpret_cast<const unsigned short*>(vp))
-                                              : *reinterpret_cast<const float*>(vp);
+                for (int i = 0; i < 4; ++i) {
+                    const TabT* row = qtab + (lane * 4 + i) * GP;
+                    part += static_cast<double>(row[warp]) * static_cast<double>(row[G]);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+                if (lane == 0) qsum_all[e * 8 + warp] = part;
+            }
+        consumer_sync<kConsumerThreads>();
+
+        // ---- this warp's run of the epoch's steps, unit by unit ----
+        const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kConsumerWarps, run_r = n_ep - run_q * kConsumerWarps;
+        int pos = ep.e0 + warp * run_q + min(warp, run_r); // line position
+        const int pos_end = pos + run_q + (warp < run_r ? 1 : 0);
+        int n = (ep.e0 - c0) + warp;                       // ring step of the warp's next step
+        if (warp == kConsumerWarps - 1) describe_epoch<kConsumerWarps>(A, C, ep, lane);      // for the merge; this warp's run is never the longer
+        u = ep.first;
+        int eu = 0;
+        while (pos < pos_end) {
+            while (pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
+            const int part_end = min(pos_end, u.start + u.steps);
+            const int b = u.b, h = u.h, len = C.lens[u.b];
+            const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kQtab + eu * S::kTabBytes);
+            const double* qsum = qsum_all + eu * 8;
+            float m_run[G], l_run[G], acc[G][4];
+#pragma unroll
+            for (int gg = 0; gg < G; ++gg) {
+                m_run[gg] = -INFINITY;
+                l_run[gg] = 0.f;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[gg][c] = 0.f;
+            }
+
+            for (; pos < part_end; ++pos, n += kConsumerWarps) {
+                const int i = pos - u.start;
+                const int slot = n % NS;
+                const bool ok = slot_wait(C.full, C.seq, slot, n / NS, C.abort_flag, A.status);
+                const unsigned char* sbase = ring + static_cast<size_t>(slot) * A.slot_stride;
+                const int n_valid = min(kStepTokens, len - i * kStepTokens);
+                if (ok) {
+                    // ---------------- scores: lane = token ----------------
+                    float s[G];
+                    const bool valid = lane < n_valid;
+                    if (valid) {
+                        const unsigned char* page = sbase + (lane >> 4) * L.page_bytes;
+                        const int p = lane & 15;
+                        const uint4 mk = *reinterpret_cast<const uint4*>(page + L.mask_off + p * 16);
+                        const unsigned words[4] = {mk.x, mk.y, mk.z, mk.w};
+                        // kept slot s of token p (see val_offset): fp32 rows hold token p at element p, bf16 rows at
+                        // element (p & 7) * 2 + (p >> 3); rows are 16 elements apart
+                        const unsigned char* vp = page + L.vals_off + (kBf16 ? ((p & 7) * 2 + (p >> 3)) * 2 : p * 4);
+                        constexpr int kRowBytes = kPageTokens * static_cast<int>(sizeof(E));
+                        // sampled rules: fp32 storage sums the score in double as well (bf16 storage: fp32 is ample)
+                        using AccT = typename std::conditional<kBf16, float, double>::type;
+                        AccT a[G];
+#pragma unroll
+                        for (int gg = 0; gg < G; ++gg) a[gg] = 0;
+                        if constexpr (R == 0) {
+                            // fp32 storage is the high-precision configuration: the score of a token is summed in
+                            // double from a double table (products of two fp32 numbers are exact there), so that the
+                            // error of the step is that of the exponentials and of the fp32 value sums alone
+                            const double mu_d = static_cast<double>(*reinterpret_cast<const float*>(page + L.mu_off + p * 4));
+                            double ad[G];
+#pragma unroll
+                            for (int gg = 0; gg < G; ++gg) ad[gg] = 0.0;
+#pragma unroll
+                            for (int wi = 0; wi < 4; ++wi) {
+                                unsigned w = words[wi];
+                                const double* tb = qtab + wi * 32 * GP;
+                                while (w) {
+                                    const int bp = __ffs(w) - 1;
+                                    w &= w - 1;
+                                    const double* e = tb + bp * GP;
+                                    const float kv = *reinterpret_cast<const float*>(vp);
                                     vp += kRowBytes;
-                                } else if constexpr (kBf16) {
-                                    x = sample_saliency<R>(A.seed, unit_t, j, mean, dev) * tv[G];
-                                } else {
-                                    x = sample_saliency_f64<R>(A.seed, unit_t, j, mean, dev) * static_cast<double>(tv[G]);
-                                }
+                                    double tv[GP];
 #pragma unroll
-                                for (int gg = 0; gg < G; ++gg)
-                                    a[gg] = fma(static_cast<AccT>(tv[gg]), x, a[gg]);
+                                    for (int c2 = 0; c2 < GP / 2; ++c2) {
+                                        const double2 f = reinterpret_cast<const double2*>(e)[c2];
+                                        tv[2 * c2] = f.x; tv[2 * c2 + 1] = f.y;
+                                    }
+                                    const double x = fma(-mu_d, tv[G], static_cast<double>(kv));
+#pragma unroll
+                                    for (int gg = 0; gg < G; ++gg) ad[gg] = fma(tv[gg], x, ad[gg]);
+                                }
                             }
+#pragma unroll
+                            for (int gg = 0; gg < G; ++gg) s[gg] = static_cast<float>(fma(mu_d, qsum[gg], ad[gg]));
+                        } else {
+                            // sampled recovery: every channel contributes, kept ones their stored value, pruned
+                            // ones a draw divided by a[j]
+                            const float mean = *reinterpret_cast<const float*>(page + L.stats_off + p * 4);
+                            const float dev = *reinterpret_cast<const float*>(page + L.stats_off + (kPageTokens + p) * 4);
+                            const unsigned long long unit_t =
+                                (static_cast<unsigned long long>(b * A.Hkv + h) << 40) ^
+                                (static_cast<unsigned long long>(i * kStepTokens + lane) << 8);
+#pragma unroll 1
+                            for (int wi = 0; wi < 4; ++wi) {
+                                const unsigned w = words[wi];
+#pragma unroll 4
+                                for (int bp = 0; bp < 32; ++bp) {
+                                    const int j = wi * 32 + bp;
+                                    const float* e = qtab + j * GP;
+                                    float tv[GP];
+#pragma unroll
+                                    for (int c4 = 0; c4 < GP / 4; ++c4) {
+                                        const float4 f = reinterpret_cast<const float4*>(e)[c4];
+                                        tv[4 * c4] = f.x; tv[4 * c4 + 1] = f.y; tv[4 * c4 + 2] = f.z; tv[4 * c4 + 3] = f.w;
+                                    }
+                                    AccT x;
+                                    if ((w >> bp) & 1u) {
+                                        x = kBf16 ? bf16_bits_to_float(*reinterpret_cast<const unsigned short*>(vp))
+                                                  : *reinterpret_cast<const float*>(vp);
+                                        vp += kRowBytes;
+                                    } else if constexpr (kBf16) {
+                                        x = sample_saliency<R>(A.seed, unit_t, j, mean, dev) * tv[G];
+                                    } else {
+                                        x = sample_saliency_f64<R>(A.seed, unit_t, j, mean, dev) * static_cast<double>(tv[G]);
+                                    }
+#pragma unroll
+                                    for (int gg = 0; gg < G; ++gg)
+                                        a[gg] = fma(static_cast<AccT>(tv[gg]), x, a[gg]);
+                                }
+                            }
+#pragma unroll
+                            for (int gg = 0; gg < G; ++gg) s[gg] = static_cast<float>(a[gg]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int gg = 0; gg < G; ++gg) s[gg] = -INFINITY;
+                    }
+                    // ---------------- online softmax ----------------
+#pragma unroll
+                    for (int gg = 0; gg < G; ++gg) {
+                        float mt = s[gg];
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, o));
+                        const float m_new = fmaxf(m_run[gg], mt);
+                        const float alpha = exp2f(m_run[gg] - m_new);   // 0 on the first step (m_run = -inf)
+                        const float pg = exp2f(s[gg] - m_new);          // 0 for invalid lanes
+                        l_run[gg] = fmaf(l_run[gg], alpha, pg);
+                        m_run[gg] = m_new;
+                        pscr[lane * GPP + gg] = pg;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) acc[gg][c] *= alpha;
+                    }
+                    __syncwarp();
+                    // ---------------- P.V: lane = channels 4*lane .. 4*lane+3 ----------------
+                    for (int t = 0; t < n_valid; ++t) {
+                        const unsigned char* pg = sbase + (t >> 4) * L.page_bytes;
+                        float vv[4];
+                        if (!kBf16 && L.keep_v < kHeadDim) {   // pruned values (fp32 pages): this lane's nibble of the value mask
+                            const int p = t & 15, wi = lane >> 3, sh = 4 * (lane & 7);
+                            const uint4 vm = *reinterpret_cast<const uint4*>(pg + L.vmask_off + p * 16);
+                            const unsigned word = wi == 0 ? vm.x : (wi == 1 ? vm.y : (wi == 2 ? vm.z : vm.w));
+                            int slot = __popc(word & ((1u << sh) - 1u)) + (wi > 0 ? __popc(vm.x) : 0) +
+                                       (wi > 1 ? __popc(vm.y) : 0) + (wi > 2 ? __popc(vm.z) : 0);
+                            const unsigned nib = (word >> sh) & 0xfu;
+                            const float* vb = reinterpret_cast<const float*>(pg + L.v_off) + p;    // slot s at vb[16 s]
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const bool on = (nib >> c) & 1u;
+                                vv[c] = on ? vb[kPageTokens * slot] : 0.f;
+                                slot += on ? 1 : 0;
+                            }
+                        } else if (kBf16) {                    // 16-byte chunks of a bf16 value row are stored swizzled
+                            const uint2 r = *reinterpret_cast<const uint2*>(
+                                pg + L.v_off + v_chunk_offset(2, t & 15, lane >> 1) + (lane & 1) * 8);
+                            vv[0] = __uint_as_float(r.x << 16); vv[1] = __uint_as_float(r.x & 0xffff0000u);
+                            vv[2] = __uint_as_float(r.y << 16); vv[3] = __uint_as_float(r.y & 0xffff0000u);
+                        } else {
+                            const float4 r = *reinterpret_cast<const float4*>(pg + L.v_off + (t & 15) * (kHeadDim * 4) + lane * 16);
+                            vv[0] = r.x; vv[1] = r.y; vv[2] = r.z; vv[3] = r.w;
+                        }
+                        float pv[GPP];
+#pragma unroll
+                        for (int c4 = 0; c4 < GPP / 4; ++c4) {
+                            const float4 f = reinterpret_cast<const float4*>(pscr + t * GPP)[c4];
+                            pv[4 * c4] = f.x; pv[4 * c4 + 1] = f.y; pv[4 * c4 + 2] = f.z; pv[4 * c4 + 3] = f.w;
                         }
 #pragma unroll
-                        for (int gg = 0; gg < G; ++gg) s[gg] = static_cast<float>(a[gg]);
+                        for (int gg = 0; gg < G; ++gg)
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) acc[gg][c] = fmaf(pv[gg], vv[c], acc[gg][c]);
                     }
-                } else {
-#pragma unroll
-                    for (int gg = 0; gg < G; ++gg) s[gg] = -INFINITY;
-                }
-                // ---------------- online softmax ----------------
-#pragma unroll
-                for (int gg = 0; gg < G; ++gg) {
-                    float mt = s[gg];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, o));
-                    const float m_new = fmaxf(m_run[gg], mt);
-                    const float alpha = exp2f(m_run[gg] - m_new);   // 0 on the first step (m_run = -inf)
-                    const float pg = exp2f(s[gg] - m_new);          // 0 for invalid lanes
-                    l_run[gg] = fmaf(l_run[gg], alpha, pg);
-                    m_run[gg] = m_new;
-                    pscr[lane * GPP + gg] = pg;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[gg][c] *= alpha;
                 }
                 __syncwarp();
-                // ---------------- P.V: lane = channels 4*lane .. 4*lane+3 ----------------
-                for (int t = 0; t < n_valid; ++t) {
-                    const unsigned char* pg = sbase + (t >> 4) * L.page_bytes;
-                    float vv[4];
-                    if (!kBf16 && L.keep_v < kHeadDim) {   // pruned values (fp32 pages): this lane's nibble of the value mask
-                        const int p = t & 15, wi = lane >> 3, sh = 4 * (lane & 7);
-                        const uint4 vm = *reinterpret_cast<const uint4*>(pg + L.vmask_off + p * 16);
-                        const unsigned word = wi == 0 ? vm.x : (wi == 1 ? vm.y : (wi == 2 ? vm.z : vm.w));
-                        int slot = __popc(word & ((1u << sh) - 1u)) + (wi > 0 ? __popc(vm.x) : 0) +
-                                   (wi > 1 ? __popc(vm.y) : 0) + (wi > 2 ? __popc(vm.z) : 0);
-                        const unsigned nib = (word >> sh) & 0xfu;
-                        const float* vb = reinterpret_cast<const float*>(pg + L.v_off) + p;    // slot s at vb[16 s]
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const bool on = (nib >> c) & 1u;
-                            vv[c] = on ? vb[kPageTokens * slot] : 0.f;
-                            slot += on ? 1 : 0;
-                        }
-                    } else if (kBf16) {                    // 16-byte chunks of a bf16 value row are stored swizzled
-                        const uint2 r = *reinterpret_cast<const uint2*>(
-                            pg + L.v_off + v_chunk_offset(2, t & 15, lane >> 1) + (lane & 1) * 8);
-                        vv[0] = __uint_as_float(r.x << 16); vv[1] = __uint_as_float(r.x & 0xffff0000u);
-                        vv[2] = __uint_as_float(r.y << 16); vv[3] = __uint_as_float(r.y & 0xffff0000u);
-                    } else {
-                        const float4 r = *reinterpret_cast<const float4*>(pg + L.v_off + (t & 15) * (kHeadDim * 4) + lane * 16);
-                        vv[0] = r.x; vv[1] = r.y; vv[2] = r.z; vv[3] = r.w;
-                    }
-                    float pv[GPP];
-#pragma unroll
-                    for (int c4 = 0; c4 < GPP / 4; ++c4) {
-                        const float4 f = reinterpret_cast<const float4*>(pscr + t * GPP)[c4];
-                        pv[4 * c4] = f.x; pv[4 * c4 + 1] = f.y; pv[4 * c4 + 2] = f.z; pv[4 * c4 + 3] = f.w;
-                    }
-#pragma unroll
-                    for (int gg = 0; gg < G; ++gg)
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) acc[gg][c] = fmaf(pv[gg], vv[c], acc[gg][c]);
-                }
+                if (lane == 0) mbar_arrive(&C.empty[slot]);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&C.empty[slot]);
-        }
 
-        // ---------------- hand the warp states to the merge ----------------
-        float* mine = merge + warp * G * kRec;
+            // ---------------- the state goes to the merge as record warp + eu ----------------
+            float* mine = merge + (warp + eu) * G * kRec;
 #pragma unroll
-        for (int gg = 0; gg < G; ++gg) {
-            float lsum = l_run[gg];
+            for (int gg = 0; gg < G; ++gg) {
+                float lsum = l_run[gg];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(kFull, lsum, o);
-            *reinterpret_cast<float4*>(mine + gg * kRec + lane * 4) =
-                make_float4(acc[gg][0], acc[gg][1], acc[gg][2], acc[gg][3]);
-            if (lane == 0) {
-                mine[gg * kRec + kHeadDim] = m_run[gg];
-                mine[gg * kRec + kHeadDim + 1] = lsum;
+                for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(kFull, lsum, o);
+                *reinterpret_cast<float4*>(mine + gg * kRec + lane * 4) =
+                    make_float4(acc[gg][0], acc[gg][1], acc[gg][2], acc[gg][3]);
+                if (lane == 0) {
+                    mine[gg * kRec + kHeadDim] = m_run[gg];
+                    mine[gg * kRec + kHeadDim + 1] = lsum;
+                }
             }
         }
         consumer_sync<kConsumerThreads>();
-        merge_and_publish<G, kConsumerWarps>(A, C, merge, sg, tid);
-        g += sg.n;
-        base += sg.n;
+        merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, ep.n_units, tid);
+        g = ep.e1;
     }
 }
 
@@ -382,15 +400,21 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     using S = SmemF32<G>;
     A.pps = 2;
     A.slot_stride = static_cast<int>(align_up(2 * static_cast<size_t>(A.L.page_bytes), 128));
+    A.cap = S::kCap; A.tab_off = S::kQtab;
     A.prefix_off = S::kFixed;
     A.ring_off = S::kFixed + prefix_bytes(A.B);
     int ns = (smem_optin - A.ring_off) / A.slot_stride;
     if (ns > kMaxSlots) ns = kMaxSlots;
     if (ns < 2) return SPARK_ERR_UNSUPPORTED;
+    const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
+    const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    // no more slots than a CTA has steps: a small call then leaves the SM room for the next kernel's CTA, whose
+    // start-up runs under this one's end
+    const int64_t most = max_steps_per_cta(units, A.max_blocks, A.pps, grid);
+    if (ns > most) ns = static_cast<int>(most < 2 ? 2 : most);
     A.nslots = ns;
     const size_t smem = A.ring_off + static_cast<size_t>(ns) * A.slot_stride;
     if (!allow_max_smem(decode_scalar_kernel<G, E, R>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
-    const int grid = n_sms < kMaxCtas ? n_sms : kMaxCtas;
     return launch_kernel(decode_scalar_kernel<G, E, R>, dim3(grid), dim3(kDecodeThreads), smem, stream, A) == cudaSuccess
                ? SPARK_OK : SPARK_ERR_CUDA;
 }
@@ -451,7 +475,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     A.status = reinterpret_cast<int*>(ws);
     A.tickets = reinterpret_cast<int*>(ws + kWorkspaceHeader);
     A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(units * sizeof(int), 256));
-    A.nslots = 0; A.slot_stride = 0; A.pps = 1; A.prefix_off = 0; A.ring_off = 0;
+    A.nslots = 0; A.slot_stride = 0; A.pps = 1; A.cap = 1; A.tab_off = 0; A.prefix_off = 0; A.ring_off = 0;
     A.overlap = (p.flags & SPARK_FLAG_OVERLAP_PREVIOUS) ? 1 : 0;
     A.seed = p.seed;
     A.q_by_value = q_by_value ? 1 : 0;

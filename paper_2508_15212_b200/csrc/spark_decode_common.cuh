@@ -4,9 +4,9 @@
 // Execution shape (both kernels): a persistent grid of one CTA per SM.  Every (sequence, KV head) unit
 // is cut into steps of `pps` pages (16 or 32 tokens); the steps of all units form one line that is
 // divided among the CTAs.  Inside a CTA one producer warp streams pages into a shared-memory ring with
-// bulk asynchronous copies that signal mbarriers; NW consumer warps each take whole steps and keep an
-// online-softmax state (running max m in the log2 domain, running sum l, unnormalised output).  At
-// the end of a unit's run the warps are merged by log-sum-exp; if several CTAs share the unit each
+// bulk asynchronous copies that signal mbarriers; NW consumer warps each take a contiguous run of steps and keep
+// an online-softmax state (running max m in the log2 domain, running sum l, unnormalised output) per unit.
+// At the end of an epoch the warps' states are merged by log-sum-exp; if several CTAs share a unit each
 // writes a partial and the last to arrive (an atomic ticket, no waiting) merges them.
 #pragma once
 
@@ -19,6 +19,7 @@ constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // every device-sid
 constexpr unsigned kClockEvery = 256;                        // polls between two looks at the clock
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRec = kHeadDim + 4;           // floats per head record: 128 outputs, running max, running sum, pad
+constexpr int kMaxCap = 6;                    // units per epoch, at most (see Epoch)
 constexpr float kLn2 = 0.6931471805599453f;
 
 struct DecodeArgs {
@@ -40,7 +41,9 @@ struct DecodeArgs {
     int nslots;
     int slot_stride;
     int pps;                                 // pages per step (= per ring slot): 1 or 2
-    int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix ((B + 1) ints)
+    int cap;                                 // units per epoch
+    int tab_off;                             // shared-memory offset of the epoch's operand tables
+    int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix)
     int overlap;                             // the page stream need not wait for the kernel before (SPARK_FLAG_OVERLAP_PREVIOUS)
     unsigned seed;                           // sampled recovery: seed of the per-entry draws
@@ -52,20 +55,30 @@ struct DecodeArgs {
 constexpr int kMaxQueryByValueBytes = 24 * 1024;
 
 // control block at the start of dynamic shared memory
-constexpr int kCtrlBytes = 1024;                                 // full[32], empty[32], flags, plan
-// the steps-per-sequence prefix sits between a kernel's fixed shared-memory areas and the ring and is as
-// large as the batch needs, so small batches leave its room to the ring
-inline int prefix_bytes(int batch) { return ((batch + 1) * 4 + 127) / 128 * 128; }
+constexpr int kCtrlBytes = 1024;                                 // full[32], empty[32], flags, plan, epoch units
+// the steps-per-sequence prefix and the lengths sit between a kernel's fixed shared-memory areas and the ring and
+// are as large as the batch needs, so small batches leave their room to the ring
+inline int prefix_bytes(int batch) { return ((2 * batch + 1) * 4 + 127) / 128 * 128; }
 
-// Shared merge area for `nw` consumer warps and `g` heads: the warps' states ([warp][head][kRec] floats:
-// 128 outputs, m, l and two spare words that the CTA-wide merge uses for the warp's weight and the head's
-// (M, L)), reused by the final combine for the weights of up to kMaxCtas parts, the heads' (M, L) and one
-// float4 per consumer thread.
-__host__ __device__ constexpr int merge_state_floats(int nw, int g)
+// Shared merge area: `records` states of `g` heads ([record][head][kRec] floats: 128 outputs, m, l, and a spare
+// word for the record's weight), reused by the final combine for the weights of up to kMaxCtas parts, the heads'
+// (M, L) and one float4 per consumer thread; behind it the (M, L) pairs of the epoch's units.
+__host__ __device__ constexpr int merge_state_floats(int nw, int cap, int g)
 {
-    return nw * g * kRec > kMaxCtas * g * 2 + nw * 32 * 4 ? nw * g * kRec : kMaxCtas * g * 2 + nw * 32 * 4;
+    return (nw + cap - 1) * g * kRec > kMaxCtas * g * 2 + nw * 32 * 4 ? (nw + cap - 1) * g * kRec : kMaxCtas * g * 2 + nw * 32 * 4;
 }
-__host__ __device__ constexpr int merge_bytes(int nw, int g) { return merge_state_floats(nw, g) * 4; }
+__host__ __device__ constexpr int merge_bytes(int nw, int cap, int g) { return (merge_state_floats(nw, cap, g) + cap * g * 2) * 4; }
+
+// Units of an epoch that a launch would like: as many as a CTA's run meets when the sequences are equally long, and a
+// few more where a batch of unequal sequences is so short that a CTA may meet many (a unit beyond the cap costs
+// another table build and merge, about 3 us).  A single sequence with several CTAs per unit needs one.
+inline int epoch_cap(int batch, int64_t units, int max_blocks, int grid)
+{
+    if (batch == 1 && 2 * units <= grid) return 1;
+    int64_t c = (units + grid - 1) / grid + 1;
+    if (batch > 1 && units * max_blocks <= static_cast<int64_t>(grid) * 256) c += 3;
+    return c > kMaxCap ? kMaxCap : static_cast<int>(c);
+}
 
 // ---- PTX helpers ----------------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void* p)
@@ -176,30 +189,76 @@ __device__ __forceinline__ int clamp_len(int len, int max_tokens)
     return len < 0 ? 0 : (len > max_tokens ? max_tokens : len);
 }
 
-struct Segment {
-    int b, h, i0, n, steps_b;
-    int unit_start;          // global step index of the unit's first step
+// A (sequence, KV head) unit on the step line.
+struct UnitRef {
+    int b, h;
+    int start;               // line position of its first step
+    int steps;
 };
 
-// Locate global step g (must be < total) and the run of steps it starts inside [g, c1).
-__device__ __forceinline__ Segment locate(const int* prefix, int B, int Hkv, int g, int c1)
+// The unit that holds line position g (must be < total).
+__device__ __forceinline__ UnitRef locate_unit(const int* prefix, int B, int Hkv, int g)
 {
     int lo = 0, hi = B;                                   // first b' in (lo, hi] with Hkv*prefix[b'] > g
+#pragma unroll 1
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (static_cast<int64_t>(Hkv) * prefix[mid] > g) hi = mid; else lo = mid;
     }
-    Segment s;
-    s.b = lo;
-    s.steps_b = prefix[lo + 1] - prefix[lo];
+    UnitRef u;
+    u.b = lo;
+    u.steps = prefix[lo + 1] - prefix[lo];
     const int r = g - Hkv * prefix[lo];
-    s.h = r / s.steps_b;
-    s.i0 = r - s.h * s.steps_b;
-    s.unit_start = Hkv * prefix[lo] + s.h * s.steps_b;
-    const int left = s.steps_b - s.i0;
-    s.n = (c1 - g < left) ? (c1 - g) : left;
-    return s;
+    u.h = r / u.steps;
+    u.start = Hkv * prefix[lo] + u.h * u.steps;
+    return u;
 }
+// The next non-empty unit (the caller knows that there is one).
+__device__ __forceinline__ void next_unit(const int* prefix, int Hkv, UnitRef& u)
+{
+    u.start += u.steps;
+    if (++u.h < Hkv) return;
+    u.h = 0;
+    do { ++u.b; u.steps = prefix[u.b + 1] - prefix[u.b]; } while (u.steps == 0);
+}
+
+// A CTA works through its run of steps in EPOCHS of up to `cap` units.  Inside an epoch of N steps the
+// consumer warps take CONTIGUOUS runs (N / NW steps each, the first N % NW warps one more), so a warp
+// meets a unit boundary only where one falls into its own run: it then writes its state to a record, loads the
+// next unit's operands and goes on, without any CTA-wide barrier.  A run cut by the unit boundaries gives at
+// most NW + cap - 1 records; the part of epoch-unit e that warp w holds is record w + e.  The ring is filled in the
+// order in which the warps consume: ring step n of the epoch is step n / NW of warp n % NW.
+//   Why: with a barrier, a merge and a table build per unit, every unit after a CTA's first cost 3.8 us (as
+//   much as 26 pages at the HBM rate).  Before -> after: append + decode of 8 sequences of 150..4000 tokens
+//   40.9 -> 28.7 us, 32 sequences of 2048 tokens (256 units on 148 SMs) 46.3 -> 44.2 us, 4 of 128K 268 -> 260 us.
+struct Epoch {
+    int e0, e1;              // line positions
+    int n_units;
+    UnitRef first;
+};
+__device__ __forceinline__ Epoch make_epoch(const int* prefix, int B, int Hkv, int cap, int g, int c1)
+{
+    Epoch ep;
+    ep.e0 = g;
+    ep.first = locate_unit(prefix, B, Hkv, g);
+    UnitRef u = ep.first;
+    ep.n_units = 1;
+    int end = u.start + u.steps;
+#pragma unroll 1
+    while (ep.n_units < cap && end < c1) {
+        next_unit(prefix, Hkv, u);
+        end += u.steps;
+        ++ep.n_units;
+    }
+    ep.e1 = min(end, c1);
+    return ep;
+}
+// What the merge needs to know about an epoch's units (kept in shared memory).
+struct EpochUnit {
+    int b, h;
+    int rec0, n_rec;         // its records in the merge area
+    int first_cta, n_parts;  // CTAs that hold a part of the unit
+};
 
 // How the step line is divided among the CTAs.
 //   stream mode : CTA c owns steps [c*chunk, (c+1)*chunk) of the whole line; a CTA may cross unit
@@ -207,38 +266,38 @@ __device__ __forceinline__ Segment locate(const int* prefix, int B, int Hkv, int
 //   aligned mode: all units have the same number of steps and there are several CTAs per unit; unit u
 //                 gets q or q+1 whole CTAs (the first `rem` units get q+1) and is split evenly among
 //                 them, so no CTA crosses a unit boundary and every CTA publishes exactly once.
-//   whole units : all units have the same number of steps and there are more units than CTAs; every CTA
-//                 takes q or q+1 whole units (the first `rem` CTAs take q+1).  No unit is split, so
-//                 there are no partials and no last-arriver merge; used when the uneven deal costs at
-//                 most 25 % over the even split.
 struct Plan {
     int total;        // steps on the line
     int chunk;        // stream mode: steps per CTA
-    int aligned;      // 0: stream, 1: aligned mode, 2: whole units
-    int unit_steps;   // aligned / whole units: steps of every unit
-    int q, rem;       // aligned: CTAs per unit; whole units: units per CTA
+    int aligned;      // 0: stream, 1: aligned mode
+    int unit_steps;   // aligned: steps of every unit
+    int q, rem;       // aligned: CTAs per unit
 };
 
 struct Ctrl {
     uint64_t* full;
     uint64_t* empty;
     volatile int* abort_flag;
-    volatile int* last_flag;
     volatile int* seq;        // [32] revolution + 1 for which each slot was last armed
+    volatile int* last_flag;  // [kMaxCap] this CTA is the last arriver of the epoch's unit
     Plan* plan;
-    int* prefix;
+    EpochUnit* units;         // [kMaxCap]
+    int* prefix;              // [B + 1] steps before each sequence (of one KV head)
+    int* lens;                // [B] clamped lengths
 };
 
-__device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off)
+__device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, int B)
 {
     Ctrl c;
     c.full = reinterpret_cast<uint64_t*>(smem);
     c.empty = c.full + kMaxSlots;
     c.abort_flag = reinterpret_cast<volatile int*>(smem + 512);
-    c.last_flag = reinterpret_cast<volatile int*>(smem + 516);
     c.plan = reinterpret_cast<Plan*>(smem + 528);
+    c.last_flag = reinterpret_cast<volatile int*>(smem + 560);
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
+    c.units = reinterpret_cast<EpochUnit*>(smem + 768);
     c.prefix = reinterpret_cast<int*>(smem + prefix_off);
+    c.lens = c.prefix + B + 1;
     return c;
 }
 
@@ -260,6 +319,7 @@ __device__ __forceinline__ void prefetch_block_table(const DecodeArgs& A, int ti
     int64_t bytes = static_cast<int64_t>(A.B) * A.Hkv * A.max_blocks * 4;
     if (bytes > kTablePrefetchMax) bytes = kTablePrefetchMax;
     const char* base = reinterpret_cast<const char*>(A.block_table);
+#pragma unroll 1
     for (int64_t o = (static_cast<int64_t>(blockIdx.x) * n_threads + tid) * 128; o < bytes;
          o += static_cast<int64_t>(gridDim.x) * n_threads * 128)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + o));
@@ -270,18 +330,20 @@ __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctr
     const int max_tokens = A.max_blocks * kPageTokens;
     if (lane < A.nslots) { mbar_init(&C.full[lane], 1); mbar_init(&C.empty[lane], 1); }
     C.seq[lane] = 0;
-    if (lane == 0) { *C.abort_flag = 0; *C.last_flag = 0; }
+    if (lane == 0) *C.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (!A.overlap) grid_wait();                           // with the flag the page stream does not depend on the kernel before
     grid_release();
     int running = 0, smin = 0x7fffffff, smax = 0;
+#pragma unroll 1
     for (int b0 = 0; b0 < A.B; b0 += 32) {
         const int b = b0 + lane;
         int st = 0;
         if (b < A.B) {
             const int len = A.lens[b];
             if (len < 0 || len > max_tokens) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+            C.lens[b] = clamp_len(len, max_tokens);
             st = steps_of(clamp_len(len, max_tokens), A.pps);
             smin = min(smin, st);
             smax = max(smax, st);
@@ -313,12 +375,6 @@ __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctr
             if (q >= 2 && makespan * 25 <= pl.chunk * 26) {          // within 4 % of the even split
                 pl.aligned = 1; pl.q = q; pl.rem = nct - q * units;
             }
-        } else if (smin == smax && smax > 0) {
-            const int q = units / nct, rem = units - q * nct;
-            const int makespan = (q + (rem ? 1 : 0)) * smax;
-            if (makespan * 4 <= pl.chunk * 5) {                      // within 25 % of the even split
-                pl.aligned = 2; pl.q = q; pl.rem = rem;
-            }
         }
         *C.plan = pl;
     }
@@ -340,12 +396,6 @@ __device__ __forceinline__ void cta_range(const Plan& pl, int cta, int& c0, int&
         c1 = min(pl.total, c0 + pl.chunk);
         return;
     }
-    if (pl.aligned == 2) {                                  // whole units: the first `rem` CTAs take q + 1
-        const int first = cta * pl.q + min(cta, pl.rem);
-        c0 = first * pl.unit_steps;
-        c1 = c0 + (pl.q + (cta < pl.rem ? 1 : 0)) * pl.unit_steps;
-        return;
-    }
     const int big = pl.rem * (pl.q + 1);                   // CTAs that belong to units with q+1 CTAs
     int u, k, n;
     if (cta < big) { u = cta / (pl.q + 1); k = cta - u * (pl.q + 1); n = pl.q + 1; }
@@ -363,12 +413,6 @@ __device__ __forceinline__ void unit_parts(const Plan& pl, int unit_start, int u
         n_parts = (unit_start + unit_steps - 1) / pl.chunk - first_cta + 1;
         return;
     }
-    if (pl.aligned == 2) {
-        const int u2 = unit_start / pl.unit_steps, big = pl.rem * (pl.q + 1);
-        first_cta = u2 < big ? u2 / (pl.q + 1) : pl.rem + (u2 - big) / pl.q;
-        n_parts = 1;
-        return;
-    }
     const int u = unit_start / pl.unit_steps;
     const int n = pl.q + (u < pl.rem ? 1 : 0);
     first_cta = u * pl.q + min(u, pl.rem);
@@ -376,7 +420,7 @@ __device__ __forceinline__ void unit_parts(const Plan& pl, int unit_start, int u
     n_parts = (pl.unit_steps + per - 1) / per;             // trailing CTAs of the unit may be empty
 }
 
-// The producer warp.  Lane i owns ring slot i: it handles this CTA's steps i, i + nslots, i + 2 nslots,
+// The producer warp.  Lane i owns ring slot i: it handles this CTA's ring steps i, i + nslots, i + 2 nslots,
 // ... in order.  Per revolution of the ring every lane looks up the page ids of its step (block-table
 // loads of the next revolution are issued before the current one is polled, so their latency hides
 // behind the wait), then the warp polls: a lane whose slot has been released by the consumers arms
@@ -391,19 +435,17 @@ __device__ __forceinline__ unsigned page_copy_bytes(const DecodeArgs& A, int id)
     return static_cast<unsigned>(A.L.vals_off + rows * kPageTokens * A.L.esize);
 }
 
-__device__ __forceinline__ void producer_page_ids(const DecodeArgs& A, const Ctrl& C, int g, int c1, bool active,
+// page ids of step `i` of unit (b, h)
+__device__ __forceinline__ void producer_page_ids(const DecodeArgs& A, const Ctrl& C, const UnitRef& u, int i,
                                                   int& id0, int& id1, unsigned& n0, unsigned& n1)
 {
-    id0 = -1; id1 = -1; n0 = 0; n1 = 0;
-    if (!active) return;
-    const Segment s = locate(C.prefix, A.B, A.Hkv, g, c1);
-    const int64_t row = (static_cast<int64_t>(s.b) * A.Hkv + s.h) * A.max_blocks;
+    const int64_t row = (static_cast<int64_t>(u.b) * A.Hkv + u.h) * A.max_blocks;
     const int32_t* bt = A.block_table ? A.block_table + row : nullptr;       // no table: pages of a unit are consecutive
-    id0 = bt ? bt[A.pps * s.i0] : static_cast<int>(row + A.pps * s.i0);
+    id1 = -1; n1 = 0;
+    id0 = bt ? bt[A.pps * i] : static_cast<int>(row + A.pps * i);
     if (A.pps == 2) {                                       // second page of the step, if the sequence has one
-        const int len = clamp_len(A.lens[s.b], A.max_blocks * kPageTokens);
-        if (2 * s.i0 + 1 < (len + kPageTokens - 1) / kPageTokens) {
-            id1 = bt ? bt[2 * s.i0 + 1] : static_cast<int>(row + 2 * s.i0 + 1);
+        if (2 * i + 1 < (C.lens[u.b] + kPageTokens - 1) / kPageTokens) {
+            id1 = bt ? bt[2 * i + 1] : static_cast<int>(row + 2 * i + 1);
             if (id1 < 0 || id1 >= A.n_pool_pages) { record_error(A.status, SPARK_ERR_DEVICE_BOUNDS); id1 = 0; }
             n1 = page_copy_bytes(A, id1);
         }
@@ -412,6 +454,7 @@ __device__ __forceinline__ void producer_page_ids(const DecodeArgs& A, const Ctr
     n0 = page_copy_bytes(A, id0);
 }
 
+template <int NW>
 __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C, unsigned char* ring,
                                               int c0, int c1, int lane)
 {
@@ -424,18 +467,36 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
     uint64_t* empty = &C.empty[owner ? lane : 0];
     bool live = true;
     int last_round = -1;                                   // last revolution in which this lane issued
-    int id0, id1;
-    unsigned n0, n1;                                       // bytes to copy of the two pages
-    producer_page_ids(A, C, c0 + lane, c1, owner && lane < n_total, id0, id1, n0, n1);
-    for (int round = 0; round * NS < n_total; ++round) {
-        const int n = round * NS + lane;
-        bool pending = owner && n < n_total;
+    int id0 = -1, id1 = -1;
+    unsigned n0 = 0, n1 = 0;                               // bytes to copy of the two pages
+    Epoch ep;
+    ep.e1 = c0;                                            // no epoch yet
+    // this lane's ring step n -> its step of the line (epoch, warp, place in the warp's run) -> page ids
+    auto lookup = [&](int n) {
+        id0 = id1 = -1; n0 = n1 = 0;
+        if (!owner || n >= n_total) return;
+        while (c0 + n >= ep.e1) ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, ep.e1, c1);
+        const int len = ep.e1 - ep.e0, q = len / NW, r = len - q * NW;
+        const int x = c0 + n - ep.e0, i = x / NW, w = x - i * NW;
+        const int g = ep.e0 + w * q + min(w, r) + i;
+        UnitRef u = ep.first;
+        while (g >= u.start + u.steps) next_unit(C.prefix, A.Hkv, u);
+        producer_page_ids(A, C, u, g - u.start, id0, id1, n0, n1);
+    };
+    // Pass t of the loop looks up ids and then issues copies.  The lookup of revolution r + 1 waits for its block-table
+    // loads, so it runs before revolution r is polled (hidden behind the wait for free slots), except at the start,
+    // where every slot is free and the first copies go out before the second lookup: ids 0 | copies 0 | ids 1 |
+    // ids 2, copies 1 | ids 3, copies 2 ...   (One loop body: this code runs cold, its size is start-up time.)
+    const int n_rounds = (n_total + NS - 1) / NS;
+#pragma unroll 1
+    for (int t = 0; t < n_rounds + 2; ++t) {
+        const int round = t == 1 ? 0 : t - 2;              // revolution whose copies go out in this pass (t = 0, 2: none)
         const int cur0 = id0, cur1 = id1;
         const unsigned b0 = n0, b1 = n1;
-        // next revolution's ids: the lookup waits for its block-table loads, so it runs before the poll
-        // (hidden behind the wait for free slots) except in the first revolution, where every slot is
-        // free and the copies go out first
-        if (round > 0) producer_page_ids(A, C, c0 + n + NS, c1, owner && n + NS < n_total, id0, id1, n0, n1);
+        if (t != 1) lookup((t == 0 ? 0 : t - 1) * NS + lane);
+        if (t == 0 || t == 2) continue;
+        const int n = round * NS + lane;
+        bool pending = owner && n < n_total;
         WaitClock wc;
         while (__any_sync(kFull, pending)) {
             if (pending && (round == 0 || mbar_try_wait(empty, (round - 1) & 1))) {
@@ -450,7 +511,6 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
             if (wc.expired() || *C.abort_flag) { live = false; break; }
         }
         if (!live) break;
-        if (round == 0) producer_page_ids(A, C, c0 + n + NS, c1, owner && n + NS < n_total, id0, id1, n0, n1);
     }
     if (!live) {
         if (lane == 0) { *C.abort_flag = 1; record_error(A.status, SPARK_ERR_DEVICE_TIMEOUT); }
@@ -466,41 +526,67 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
 template <int NT>
 __device__ __forceinline__ void write_empty_sequences(const DecodeArgs& A, const int* prefix, int tid)
 {
+#pragma unroll 1
     for (int b = blockIdx.x; b < A.B; b += gridDim.x)
         if (prefix[b + 1] == prefix[b]) {
+#pragma unroll 1
             for (int i = tid; i < A.Hq * kHeadDim; i += NT)
                 A.out[static_cast<int64_t>(b) * A.Hq * kHeadDim + i] = 0.f;
             if (A.lse)
+#pragma unroll 1
                 for (int i = tid; i < A.Hq; i += NT)
                     A.lse[static_cast<int64_t>(b) * A.Hq + i] = -INFINITY;
         }
 }
 
-// Merge the per-warp states that the NW consumer warps have written to `merge`
-// ([warp][G][kRec]: 128 unnormalised outputs, m, l) and publish the unit's result: directly when this
-// CTA covers the whole unit, else as a partial followed by the last-arriver merge.  Called by all
-// consumer threads after a consumer_sync(); ends with a consumer_sync().
+// The epoch's units as the merge needs them; one warp.  Lane w stands for consumer warp w: a step belongs to the last
+// warp whose run starts at or before it.
+template <int NW>
+__device__ __forceinline__ void describe_epoch(const DecodeArgs& A, const Ctrl& C, const Epoch& ep, int lane)
+{
+    const int n = ep.e1 - ep.e0, q = n / NW, r = n - q * NW;
+    const int run0 = ep.e0 + (lane < NW ? lane * q + min(lane, r) : n);
+    UnitRef u = ep.first;
+#pragma unroll 1
+    for (int e = 0; e < ep.n_units; ++e) {
+        if (e) next_unit(C.prefix, A.Hkv, u);
+        const int w0 = __popc(__ballot_sync(kFull, run0 <= max(u.start, ep.e0))) - 1;
+        const int w1 = __popc(__ballot_sync(kFull, run0 < min(u.start + u.steps, ep.e1))) - 1;
+        if (lane == e) {
+            EpochUnit d;
+            d.b = u.b; d.h = u.h;
+            d.rec0 = w0 + e;
+            d.n_rec = w1 - w0 + 1;
+            unit_parts(*C.plan, u.start, u.steps, d.first_cta, d.n_parts);
+            C.units[e] = d;
+        }
+    }
+}
+
+// Merge the records of an epoch ([record][G][kRec]: 128 unnormalised outputs, m, l) unit by unit and publish
+// the units' results: directly where this CTA holds the whole unit, else as a partial followed by the
+// last-arriver merge (only the first and the last unit of a CTA's run can be split).  Called by all consumer
+// threads after a consumer_sync(); ends with a consumer_sync().
 //
 // Both merges are laid out so that no thread walks a chain of dependent shared-memory loads: the
 // log-sum-exp weights of the parts are computed once, by one warp per head with warp reductions, and the
 // weighted sums then read independent operands.
 template <int G, int NW>
-__device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge,
-                                                  const Segment& sg, int tid)
+__device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge, float* unit_ml,
+                                                  int n_units, int tid)
 {
     constexpr int NT = NW * 32;
-    static_assert(G <= NW && NW <= 32, "one warp per head computes the weights of up to 32 warps");
-    const int b = sg.b, h = sg.h;
+    static_assert(NW <= 32, "one warp computes the weights of up to 32 records");
     const int warp = tid >> 5, lane = tid & 31;
-    int first_cta, n_parts;
-    unit_parts(*C.plan, sg.unit_start, sg.steps_b, first_cta, n_parts);
-    const int unit = b * A.Hkv + h;
-    static_assert(NW >= 2, "the heads' (M, L) live in the spare words of the first two warps' records");
-    constexpr int kWt = kHeadDim + 2, kMl = kHeadDim + 3;     // spare words of a record
-    // ---- weights of the warps: warp g serves head g, lane w holds warp w's (m, l) ----
-    if (warp < G) {
-        const float m = lane < NW ? merge[(lane * G + warp) * kRec + kHeadDim] : -INFINITY;
-        const float l = lane < NW ? merge[(lane * G + warp) * kRec + kHeadDim + 1] : 0.f;
+    constexpr int kWt = kHeadDim + 2;                         // spare word of a record: its weight
+    // ---- weights of the records: a warp serves one head of one unit, lane k holds the unit's record k ----
+#pragma unroll 1
+    for (int pr = warp; pr < n_units * G; pr += NW) {
+        const int e = pr / G, gg = pr - e * G;
+        const int rec0 = C.units[e].rec0, n_rec = C.units[e].n_rec;
+        float* rec = merge + ((rec0 + lane) * G + gg) * kRec;
+        const float m = lane < n_rec ? rec[kHeadDim] : -INFINITY;
+        const float l = lane < n_rec ? rec[kHeadDim + 1] : 0.f;
         float M = m;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
@@ -508,48 +594,68 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
         float Ls = l * wt;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(kFull, Ls, o);
-        if (lane < NW) merge[(lane * G + warp) * kRec + kWt] = wt;
-        if (lane == 0) { merge[warp * kRec + kMl] = M; merge[(G + warp) * kRec + kMl] = Ls; }
+        if (lane < n_rec) rec[kWt] = wt;
+        if (lane == 0) { unit_ml[2 * pr] = M; unit_ml[2 * pr + 1] = Ls; }
     }
     consumer_sync<NT>();
-    // ---- weighted sums: a thread owns two channels of one head ----
-    float* part_out = A.partials + static_cast<int64_t>(blockIdx.x + unit) * G * kRec;
-    for (int idx = tid; idx < G * (kHeadDim / 2); idx += NT) {
-        const int gg = idx / (kHeadDim / 2), c2 = idx - gg * (kHeadDim / 2);
+    // ---- weighted sums: a thread owns two channels of one head of one unit ----
+#pragma unroll 1
+    for (int idx = tid; idx < n_units * G * (kHeadDim / 2); idx += NT) {
+        const int pr = idx / (kHeadDim / 2), c2 = idx - pr * (kHeadDim / 2);
+        const int e = pr / G, gg = pr - e * G;
+        const EpochUnit d = C.units[e];
+        const float* rec = merge + (d.rec0 * G + gg) * kRec;
         float2 v[NW];
+        float f[NW];
 #pragma unroll
-        for (int w = 0; w < NW; ++w) v[w] = *reinterpret_cast<const float2*>(merge + (w * G + gg) * kRec + 2 * c2);
+        for (int k = 0; k < NW; ++k) {                        // every load before the first use
+            v[k] = make_float2(0.f, 0.f);
+            f[k] = 0.f;
+            if (k < d.n_rec) {
+                v[k] = *reinterpret_cast<const float2*>(rec + k * (G * kRec) + 2 * c2);
+                f[k] = rec[k * (G * kRec) + kWt];
+            }
+        }
         float2 O = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const float f = merge[(w * G + gg) * kRec + kWt];
-            O.x = fmaf(v[w].x, f, O.x);
-            O.y = fmaf(v[w].y, f, O.y);
+        for (int k = 0; k < NW; ++k) {
+            O.x = fmaf(v[k].x, f[k], O.x);
+            O.y = fmaf(v[k].y, f[k], O.y);
         }
-        const float M = merge[gg * kRec + kMl], Ls = merge[(G + gg) * kRec + kMl];
-        if (n_parts == 1) {
+        const float M = unit_ml[2 * pr], Ls = unit_ml[2 * pr + 1];
+        const int64_t row = static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg;
+        if (d.n_parts == 1) {
             const float inv = 1.0f / Ls;
-            *reinterpret_cast<float2*>(A.out + (static_cast<int64_t>(b) * A.Hq + h * G + gg) * kHeadDim + 2 * c2) =
-                make_float2(O.x * inv, O.y * inv);
-            if (c2 == 0 && A.lse)
-                A.lse[static_cast<int64_t>(b) * A.Hq + h * G + gg] = (M + log2f(Ls)) * kLn2;
+            *reinterpret_cast<float2*>(A.out + row * kHeadDim + 2 * c2) = make_float2(O.x * inv, O.y * inv);
+            if (c2 == 0 && A.lse) A.lse[row] = (M + log2f(Ls)) * kLn2;
         } else {
+            float* part_out = A.partials + static_cast<int64_t>(blockIdx.x + d.b * A.Hkv + d.h) * G * kRec;
             *reinterpret_cast<float2*>(part_out + gg * kRec + 2 * c2) = O;
             if (c2 == 0) *reinterpret_cast<float2*>(part_out + gg * kRec + kHeadDim) = make_float2(M, Ls);
         }
     }
-    if (n_parts > 1) {
-        // The barrier orders every consumer thread's partial stores before thread 0's gpu-scope
+    bool split = false;
+#pragma unroll 1
+    for (int e = 0; e < n_units; ++e) split = split || C.units[e].n_parts > 1;         // the same in every thread
+    if (split) {
+        // The barrier orders every consumer thread's partial stores before the tickets' gpu-scope
         // release; the last arriver's acquire (same atomic) plus the next barrier orders its reads
         // after all partials.
         consumer_sync<NT>();
-        if (tid == 0) {
-            int old;
-            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(A.tickets + unit) : "memory");
-            *C.last_flag = (old == n_parts - 1) ? 1 : 0;
+        if (tid < n_units) {
+            int last = 0;
+            if (C.units[tid].n_parts > 1) {
+                int old;
+                asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;"
+                             : "=r"(old) : "l"(A.tickets + C.units[tid].b * A.Hkv + C.units[tid].h) : "memory");
+                last = (old == C.units[tid].n_parts - 1) ? 1 : 0;
+            }
+            C.last_flag[tid] = last;
         }
         consumer_sync<NT>();
-        if (*C.last_flag) {
+#pragma unroll 1
+        for (int e = 0; e < n_units; ++e) {
+            if (!C.last_flag[e]) continue;
             // Last CTA of this unit: merge all partials.  Every load is issued before the first use:
             // thread (ph, g, c4) fetches channels 4*c4..4*c4+3 of head g for parts ph, ph+PH, ...;
             // meanwhile warp g turns the (m, l) pairs of head g into weights (lane = part) and the
@@ -557,16 +663,19 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
             // reduced over ph through shared memory.
             constexpr int TPG = G * 32;                  // threads per part group
             constexpr int PH = NT / TPG;                 // part groups
+            static_assert(PH >= 1, "a warp per head");
             constexpr int kBatch = 8;
             constexpr int kMlRegs = kMaxCtas / 32;       // (m, l) pairs a lane may hold
             constexpr int64_t kStride = static_cast<int64_t>(G) * kRec;
+            const int b = C.units[e].b, h = C.units[e].h, n_parts = C.units[e].n_parts, unit = b * A.Hkv + h;
             float* pw = merge;                           // [n_parts][G] weights, n_parts <= kMaxCtas
             float* pML = merge + kMaxCtas * G;           // [G][2]
             float4* red = reinterpret_cast<float4*>(merge + kMaxCtas * G * 2);
-            const float* base = A.partials + static_cast<int64_t>(first_cta + unit) * G * kRec;
+            const float* base = A.partials + static_cast<int64_t>(C.units[e].first_cta + unit) * G * kRec;
             const int ph = tid / TPG, rem = tid - ph * TPG, gg = rem >> 5, c4 = rem & 31;
             const bool worker = ph < PH;
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
             for (int p0 = 0; p0 < n_parts; p0 += kBatch * PH) {
                 float4 o4[kBatch];
 #pragma unroll
@@ -633,9 +742,25 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
                     A.lse[static_cast<int64_t>(b) * A.Hq + h * G + gg] = (M + log2f(Ls)) * kLn2;
             }
             if (tid == 0) A.tickets[unit] = 0;          // ready for the next call
+            consumer_sync<NT>();                        // the merge area is free for the next unit
         }
     }
     consumer_sync<NT>();
+}
+
+// Steps that one CTA of `grid` can own at most (either division of the line), from the cache's capacity alone.
+inline int64_t max_steps_per_cta(int64_t units, int max_blocks, int pps, int grid)
+{
+    const int64_t total = units * ((max_blocks + pps - 1) / pps);
+    const int64_t chunk = (total + grid - 1) / grid;
+    return chunk + chunk / 25 + 1;                          // the aligned division may be 4 % above the even one
+}
+// CTAs of the persistent grid: one per SM, fewer when the cache cannot hold a step for each.
+inline int decode_grid(int n_sms, int64_t units, int max_blocks, int pps)
+{
+    const int64_t total = units * ((max_blocks + pps - 1) / pps);
+    const int64_t g = total < n_sms ? total : n_sms;
+    return g < 1 ? 1 : (g > kMaxCtas ? kMaxCtas : static_cast<int>(g));
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

@@ -33,17 +33,17 @@ namespace spark {
 constexpr int kNW = 15;                       // consumer warps (+ 1 producer warp = 16 warps, 4 per scheduler)
 constexpr int kNT = kNW * 32;
 constexpr int kThreads = kNT + 32;
+constexpr int kMinRing = 20;                  // ring slots that an epoch's units may not take
 constexpr float kSlack = 8.f;                 // log2 units a score may exceed the running reference maximum
 
 constexpr int kVTileBytes = kPageTokens * kHeadDim * 2;                          // dense value rows of one page
 
-// Shared-memory map (fixed part; the steps prefix and the ring follow at offsets chosen by the launcher).
+// Shared-memory map (fixed part; merge area, operand tables, prefix and ring follow at offsets chosen by the launcher).
 template <int G, bool kPV> struct SmemBf16 {
-    static constexpr int kTab = kCtrlBytes;                                      // q, q' high, q' low: 3 x [G][128] bf16
-    static constexpr int kQsum = kTab + 3 * G * kHeadDim * 2;                    // [8] float
-    static constexpr int kMerge = kQsum + 32;
-    static constexpr int kVTile = (kMerge + merge_bytes(kNW, G) + 127) / 128 * 128;   // per-warp tiles (pruned values)
-    static constexpr int kFixed = kVTile + (kPV ? kNW * kVTileBytes : 0);        // prefix and ring start here
+    static constexpr int kQsum = kCtrlBytes;                                     // [kMaxCap][8] float
+    static constexpr int kVTile = (kQsum + kMaxCap * 8 * 4 + 127) / 128 * 128;   // per-warp tiles (pruned values)
+    static constexpr int kMerge = kVTile + (kPV ? kNW * kVTileBytes : 0);
+    static constexpr int kTabBytes = 3 * G * kHeadDim * 2;                       // one unit's q, q' high, q' low: 3 x [G][128] bf16
 };
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
@@ -227,263 +227,275 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     using S = SmemBf16<G, kPV>;
     constexpr bool kShared8 = (G <= 4);        // q' high and low parts share one 8-column operand
     extern __shared__ __align__(128) unsigned char smem[];
-    const Ctrl C = make_ctrl(smem, A.prefix_off);
-    unsigned char* tab = smem + S::kTab;
-    float* qsum_s = reinterpret_cast<float*>(smem + S::kQsum);
+    const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
+    unsigned char* tab_all = smem + A.tab_off;
+    float* qsum_all = reinterpret_cast<float*>(smem + S::kQsum);
     float* merge = reinterpret_cast<float*>(smem + S::kMerge);
+    float* unit_ml = merge + merge_state_floats(kNW, A.cap, G);
     unsigned char* ring = smem + A.ring_off;
     const unsigned ring_u = smem_u32(ring);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const PageLayout L = A.L;
     const int NS = A.nslots;
-    const int max_tokens = A.max_blocks * kPageTokens;
 
     prefetch_block_table(A, tid, kThreads);
     if (warp == kNW) {
         producer_prologue(A, C, lane, kThreads);
         int p0, p1;
         cta_range(*C.plan, static_cast<int>(blockIdx.x), p0, p1);
-        producer_loop(A, C, ring, p0, p1, lane);
+        producer_loop<kNW>(A, C, ring, p0, p1, lane);
         return;
     }
     consumer_wait_plan(kThreads);
-    const int* prefix = C.prefix;
     int c0, c1;
     cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
     grid_wait();                                           // q, qnorm, out and the workspace from here on
-    write_empty_sequences<kNT>(A, prefix, tid);
+    write_empty_sequences<kNT>(A, C.prefix, tid);
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
-    int base = 0;
     for (int g = c0; g < c1;) {
-        const Segment sg = locate(prefix, A.B, A.Hkv, g, c1);
-        const int b = sg.b, h = sg.h;
-        const int len = clamp_len(A.lens[b], max_tokens);
-
-        // ---- per-unit tables, built once per CTA: warp `hd` prepares query head hd ----
-        if (warp < G) {
+        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, g, c1);
+        // ---- the epoch's operand tables: a warp prepares one query head of one unit ----
+#pragma unroll 1
+        for (int pr = warp; pr < ep.n_units * G; pr += kNW) {
+            const int e = pr / G, hd = pr - e * G;
+            UnitRef u = ep.first;
+#pragma unroll 1
+            for (int k = 0; k < e; ++k) next_unit(C.prefix, A.Hkv, u);
             const uint2 qr = *reinterpret_cast<const uint2*>(
                 static_cast<const unsigned short*>(q_src) +
-                (static_cast<int64_t>(b) * A.Hq + h * G + warp) * kHeadDim + 4 * lane);
+                (static_cast<int64_t>(u.b) * A.Hq + u.h * G + hd) * kHeadDim + 4 * lane);
             const float4 a4 = *reinterpret_cast<const float4*>(
-                A.qnorm + (static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + 4 * lane);
-            write_head_tables<G>(tab, qsum_s, warp, lane, qr, a4);
+                A.qnorm + (static_cast<int64_t>(u.b) * A.Hkv + u.h) * kHeadDim + 4 * lane);
+            write_head_tables<G>(tab_all + e * S::kTabBytes, qsum_all + e * 8, hd, lane, qr, a4);
         }
         consumer_sync<kNT>();
-        // second-operand fragments (column r of each operand, channels 32c .. 32c+31):
-        //   Bq[2s], Bq[2s+1] = q[head r][32c+4s .. +3];  Bp / Bpl likewise from the q' parts.
-        unsigned Bq[16], Bp[16], Bpl[kShared8 ? 1 : 16];
-        {
-            const unsigned t0 = smem_u32(tab) + c * 64;
-            const unsigned plane = G * kHeadDim * 2;
-            const int pr = kShared8 ? (r & 3) : r;                     // head of column r in the q' operand
-            const unsigned pofs = kShared8 ? ((r < 4) ? plane : 2 * plane) : plane;
+
+        // ---- this warp's run of the epoch's steps, unit by unit ----
+        const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kNW, run_r = n_ep - run_q * kNW;
+        int pos = ep.e0 + warp * run_q + min(warp, run_r);     // line position
+        const int pos_end = pos + run_q + (warp < run_r ? 1 : 0);
+        int slot = (ep.e0 - c0) + warp, round = slot / NS;     // ring position of the warp's next step, kept incrementally
+        slot -= round * NS;
+        if (warp == kNW - 1) describe_epoch<kNW>(A, C, ep, lane);     // for the merge; this warp's run is never the longer
+        UnitRef u = ep.first;
+        int eu = 0;
+        while (pos < pos_end) {
+            while (pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
+            const int part_end = min(pos_end, u.start + u.steps);
+            int left = C.lens[u.b] - (pos - u.start) * kPageTokens;      // tokens from this step to the unit's end
+            // second-operand fragments (column r of each operand, channels 32c .. 32c+31):
+            //   Bq[2s], Bq[2s+1] = q[head r][32c+4s .. +3];  Bp / Bpl likewise from the q' parts.
+            unsigned Bq[16], Bp[16], Bpl[kShared8 ? 1 : 16];
+            {
+                const unsigned t0 = smem_u32(tab_all + eu * S::kTabBytes) + c * 64;
+                const unsigned plane = G * kHeadDim * 2;
+                const int pr = kShared8 ? (r & 3) : r;                     // head of column r in the q' operand
+                const unsigned pofs = kShared8 ? ((r < 4) ? plane : 2 * plane) : plane;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                uint4 u = make_uint4(0, 0, 0, 0), v = make_uint4(0, 0, 0, 0), x = make_uint4(0, 0, 0, 0);
-                if (r < G) u = lds_u32x4(t0 + r * (kHeadDim * 2) + i * 16);
-                if (pr < G) v = lds_u32x4(t0 + pofs + pr * (kHeadDim * 2) + i * 16);
-                if (!kShared8 && r < G) x = lds_u32x4(t0 + 2 * plane + r * (kHeadDim * 2) + i * 16);
-                Bq[4 * i] = u.x; Bq[4 * i + 1] = u.y; Bq[4 * i + 2] = u.z; Bq[4 * i + 3] = u.w;
-                Bp[4 * i] = v.x; Bp[4 * i + 1] = v.y; Bp[4 * i + 2] = v.z; Bp[4 * i + 3] = v.w;
-                if (!kShared8) { Bpl[4 * i] = x.x; Bpl[4 * i + 1] = x.y; Bpl[4 * i + 2] = x.z; Bpl[4 * i + 3] = x.w; }
+                for (int i = 0; i < 4; ++i) {
+                    uint4 t = make_uint4(0, 0, 0, 0), v = make_uint4(0, 0, 0, 0), x = make_uint4(0, 0, 0, 0);
+                    if (r < G) t = lds_u32x4(t0 + r * (kHeadDim * 2) + i * 16);
+                    if (pr < G) v = lds_u32x4(t0 + pofs + pr * (kHeadDim * 2) + i * 16);
+                    if (!kShared8 && r < G) x = lds_u32x4(t0 + 2 * plane + r * (kHeadDim * 2) + i * 16);
+                    Bq[4 * i] = t.x; Bq[4 * i + 1] = t.y; Bq[4 * i + 2] = t.z; Bq[4 * i + 3] = t.w;
+                    Bp[4 * i] = v.x; Bp[4 * i + 1] = v.y; Bp[4 * i + 2] = v.z; Bp[4 * i + 3] = v.w;
+                    if (!kShared8) { Bpl[4 * i] = x.x; Bpl[4 * i + 1] = x.y; Bpl[4 * i + 2] = x.z; Bpl[4 * i + 3] = x.w; }
+                }
             }
-        }
-        // this thread's two heads in the score layout (columns 2c, 2c+1)
-        bool hv[2];
-        float qsum[2];
+            // this thread's two heads in the score layout (columns 2c, 2c+1)
+            bool hv[2];
+            float qsum[2];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            hv[e] = (2 * c + e < G) && (!kShared8 || c < 2);
-            qsum[e] = hv[e] ? qsum_s[2 * c + e] : 0.f;
-        }
+            for (int e = 0; e < 2; ++e) {
+                hv[e] = (2 * c + e < G) && (!kShared8 || c < 2);
+                qsum[e] = hv[e] ? qsum_all[eu * 8 + 2 * c + e] : 0.f;
+            }
 
-        float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-        float thr[2] = {hv[0] ? -INFINITY : INFINITY, hv[1] ? -INFINITY : INFINITY};
-        float o[8][4];
+            float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+            float thr[2] = {hv[0] ? -INFINITY : INFINITY, hv[1] ? -INFINITY : INFINITY};
+            float o[8][4];
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt) { o[mt][0] = 0.f; o[mt][1] = 0.f; o[mt][2] = 0.f; o[mt][3] = 0.f; }
+            for (int mt = 0; mt < 8; ++mt) { o[mt][0] = 0.f; o[mt][1] = 0.f; o[mt][2] = 0.f; o[mt][3] = 0.f; }
 
-        int n = base + ((warp - base) % kNW + kNW) % kNW;
-        int slot = n % NS, round = n / NS;                 // ring position of step n, kept incrementally
-        for (; n < base + sg.n; n += kNW, slot += kNW) {
-            while (slot >= NS) { slot -= NS; ++round; }
-            const int i = sg.i0 + (n - base);
-            const bool ok = slot_wait(C.full, C.seq, slot, round, C.abort_flag, A.status);
-            const unsigned page = ring_u + static_cast<unsigned>(slot) * A.slot_stride;
-            const int n_valid = min(kPageTokens, len - i * kPageTokens);
-            if (ok) {
-                // ---------------- scores of the page's 16 tokens (rows r and r+8) ----------------
-                float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f}, d3[4] = {0.f, 0.f, 0.f, 0.f};
-                unsigned vaddr[2], vaddr_hi[2], w[2];
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int tok = 8 * j + r;
-                    w[j] = lds_u32(page + L.mask_off + tok * 16 + c * 4);
-                    const int cnt = __popc(w[j]);
-                    int x = cnt;
-                    int t = __shfl_up_sync(kFull, x, 1, 4);
-                    if (c >= 1) x += t;
-                    t = __shfl_up_sync(kFull, x, 2, 4);
-                    if (c >= 2) x += t;
-                    vaddr[j] = page + L.vals_off + (r * 2 + j) * 2 + (x - cnt) * 32;      // see val_offset: token r + 8j
-                    vaddr_hi[j] = vaddr[j] + __popc(w[j] & 0xffffu) * 32;    // upper half of the word walks on its own
-                }
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    unsigned k0[2], k1[2], m0[2], m1[2];
-#pragma unroll
-                    for (int j = 0; j < 2; ++j)
-                        expand_nibble(w[j], 1u << (4 * ks), 2u << (4 * ks), 4u << (4 * ks), 8u << (4 * ks),
-                                      ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j]);
-                    mma_bf16(d1, k0[0], k0[1], k1[0], k1[1], Bq[2 * ks], Bq[2 * ks + 1]);
-                    mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bp[2 * ks], Bp[2 * ks + 1]);
-                    if (!kShared8) mma_bf16(d3, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
-                }
-                // kept q' sums of this thread's heads: high part + low part
-                float rk[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float other = kShared8 ? __shfl_xor_sync(kFull, d2[e], 2) : d3[e];
-                    rk[e] = d2[e] + other;
-                }
-                // ---------------- online softmax over the 16 tokens ----------------
-                // The reference maximum m_run of a head moves only when a score of the page exceeds it
-                // by more than kSlack (log2 units), so most pages skip the warp-wide maximum and the
-                // rescaling; probabilities then lie in (0, 2^kSlack], which fp32 sums and the bf16
-                // high/low split carry without loss.  thr = m_run + kSlack (+inf for unused columns).
-                const float mu[2] = {lds_f32(page + L.mu_off + r * 4), lds_f32(page + L.mu_off + (r + 8) * 4)};
-                float s[2][2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
+            for (; pos < part_end; ++pos, slot += kNW, left -= kPageTokens) {
+                while (slot >= NS) { slot -= NS; ++round; }
+                const bool ok = slot_wait(C.full, C.seq, slot, round, C.abort_flag, A.status);
+                const unsigned page = ring_u + static_cast<unsigned>(slot) * A.slot_stride;
+                const int n_valid = left;                          // >= 16: every row of the page
+                if (ok) {
+                    // ---------------- scores of the page's 16 tokens (rows r and r+8) ----------------
+                    float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f}, d3[4] = {0.f, 0.f, 0.f, 0.f};
+                    unsigned vaddr[2], vaddr_hi[2], w[2];
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const float sv = A.scale_log2e * fmaf(mu[j], qsum[e] - rk[2 * j + e], d1[2 * j + e]);
-                        s[j][e] = (r + 8 * j < n_valid) ? sv : -INFINITY;
-                    }
-                const float over = fmaxf(fmaxf(s[0][0], s[1][0]) - thr[0], fmaxf(s[0][1], s[1][1]) - thr[1]);
-                if (__any_sync(kFull, over > 0.f)) {
-                    float alpha[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        float mt = fmaxf(s[0][e], s[1][e]);
-                        mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 4));
-                        mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 8));
-                        mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 16));
-                        const float m_new = fmaxf(m_run[e], mt);
-                        alpha[e] = hv[e] ? ex2(m_run[e] - m_new) : 1.f;
-                        l_run[e] *= alpha[e];
-                        m_run[e] = m_new;
-                        thr[e] = hv[e] ? m_new + kSlack : INFINITY;
-                    }
-                    float a0 = alpha[0], a1 = alpha[1];      // columns 2c, 2c+1 of every output tile
-                    if (kShared8) {
-                        const float y0 = __shfl_xor_sync(kFull, a0, 2), y1 = __shfl_xor_sync(kFull, a1, 2);
-                        if (c >= 2) { a0 = y0; a1 = y1; }
-                    }
-#pragma unroll
-                    for (int mt = 0; mt < 8; ++mt) {
-                        o[mt][0] *= a0; o[mt][1] *= a1; o[mt][2] *= a0; o[mt][3] *= a1;
-                    }
-                }
-                float ph[2][2], pl[2][2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float p0 = hv[e] ? ex2(s[0][e] - m_run[e]) : 0.f;
-                    const float p1 = hv[e] ? ex2(s[1][e] - m_run[e]) : 0.f;
-                    l_run[e] += p0 + p1;
-                    ph[0][e] = bf16_round(p0); pl[0][e] = p0 - ph[0][e];
-                    ph[1][e] = bf16_round(p1); pl[1][e] = p1 - ph[1][e];
-                }
-                // probabilities: score layout (row = token, cols = heads) -> operand layout (k = token, n = col)
-                unsigned pb0, pb1, pc0 = 0, pc1 = 0;
-                {
-                    const unsigned h0 = pack_bf16(ph[0][0], ph[0][1]), h1 = pack_bf16(ph[1][0], ph[1][1]);
-                    const unsigned l0 = pack_bf16(pl[0][0], pl[0][1]), l1 = pack_bf16(pl[1][0], pl[1][1]);
-                    if (kShared8) {                      // columns 4-7 carry the low parts of heads 0-3
-                        const unsigned x0 = __shfl_xor_sync(kFull, l0, 2), x1 = __shfl_xor_sync(kFull, l1, 2);
-                        pb0 = movmatrix_trans(c < 2 ? h0 : x0);
-                        pb1 = movmatrix_trans(c < 2 ? h1 : x1);
-                    } else {
-                        pb0 = movmatrix_trans(h0); pb1 = movmatrix_trans(h1);
-                        pc0 = movmatrix_trans(l0); pc1 = movmatrix_trans(l1);
-                    }
-                }
-                // ---------------- P.V: out^T[channel][col] += V^T[channel][token] P^T[token][col] ----------------
-                unsigned vbase = page + L.v_off;
-                if (kPV) {
-                    // lane (r, c) expands mask word c of tokens r and r + 8: channels 32c + 8u .. + 7 of a
-                    // token are 16-byte chunk k = 4c + u, stored at chunk index k ^ r ^ ((k >> 3) << 1) of the
-                    // token's row (the extra term keeps the four lanes of a row on different banks)
-                    vbase = smem_u32(smem + S::kVTile) + warp * kVTileBytes;
-                    unsigned vw[2], va[2];
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        vw[j] = lds_u32(page + L.vmask_off + (8 * j + r) * 16 + c * 4);
-                        const int cnt = __popc(vw[j]);
+                        const int tok = 8 * j + r;
+                        w[j] = lds_u32(page + L.mask_off + tok * 16 + c * 4);
+                        const int cnt = __popc(w[j]);
                         int x = cnt;
                         int t = __shfl_up_sync(kFull, x, 1, 4);
                         if (c >= 1) x += t;
                         t = __shfl_up_sync(kFull, x, 2, 4);
                         if (c >= 2) x += t;
-                        va[j] = page + L.v_off + (r * 2 + j) * 2 + (x - cnt) * 32;
+                        vaddr[j] = page + L.vals_off + (r * 2 + j) * 2 + (x - cnt) * 32;      // see val_offset: token r + 8j
+                        vaddr_hi[j] = vaddr[j] + __popc(w[j] & 0xffffu) * 32;    // upper half of the word walks on its own
                     }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                    for (int ks = 0; ks < 8; ++ks) {
+                        unsigned k0[2], k1[2], m0[2], m1[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            expand_nibble(w[j], 1u << (4 * ks), 2u << (4 * ks), 4u << (4 * ks), 8u << (4 * ks),
+                                          ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j]);
+                        mma_bf16(d1, k0[0], k0[1], k1[0], k1[1], Bq[2 * ks], Bq[2 * ks + 1]);
+                        mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bp[2 * ks], Bp[2 * ks + 1]);
+                        if (!kShared8) mma_bf16(d3, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
+                    }
+                    // kept q' sums of this thread's heads: high part + low part
+                    float rk[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float other = kShared8 ? __shfl_xor_sync(kFull, d2[e], 2) : d3[e];
+                        rk[e] = d2[e] + other;
+                    }
+                    // ---------------- online softmax over the 16 tokens ----------------
+                    // The reference maximum m_run of a head moves only when a score of the page exceeds it
+                    // by more than kSlack (log2 units), so most pages skip the warp-wide maximum and the
+                    // rescaling; probabilities then lie in (0, 2^kSlack], which fp32 sums and the bf16
+                    // high/low split carry without loss.  thr = m_run + kSlack (+inf for unused columns).
+                    const float mu[2] = {lds_f32(page + L.mu_off + r * 4), lds_f32(page + L.mu_off + (r + 8) * 4)};
+                    float s[2][2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
-                            unsigned e0, e1, e2, e3;
-                            expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1);
-                            expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3);
-                            sts_u32x4(vbase + (8 * j + r) * (kHeadDim * 2) + (((4 * c + u) ^ r ^ (c & 2)) << 4), e0, e1, e2, e3);
+                            const float sv = A.scale_log2e * fmaf(mu[j], qsum[e] - rk[2 * j + e], d1[2 * j + e]);
+                            s[j][e] = (r + 8 * j < n_valid) ? sv : -INFINITY;
                         }
-                    __syncwarp();
-                }
-                const int mi = lane >> 3, rr = lane & 7;
-                const unsigned vrow = vbase + (((mi >> 1) << 3) + rr) * (kHeadDim * 2);
+                    const float over = fmaxf(fmaxf(s[0][0], s[1][0]) - thr[0], fmaxf(s[0][1], s[1][1]) - thr[1]);
+                    if (__any_sync(kFull, over > 0.f)) {
+                        float alpha[2];
 #pragma unroll
-                for (int mt = 0; mt < 8; ++mt) {
-                    unsigned a0, a1, a2, a3;
-                    ldmatrix_x4_trans(a0, a1, a2, a3, vrow + (((2 * mt + (mi & 1)) ^ rr ^ (kPV ? ((mt >> 2) << 1) : 0)) << 4));
-                    mma_bf16(o[mt], a0, a1, a2, a3, pb0, pb1);
-                    if (!kShared8) mma_bf16(o[mt], a0, a1, a2, a3, pc0, pc1);
+                        for (int e = 0; e < 2; ++e) {
+                            float mt = fmaxf(s[0][e], s[1][e]);
+                            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 4));
+                            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 8));
+                            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 16));
+                            const float m_new = fmaxf(m_run[e], mt);
+                            alpha[e] = hv[e] ? ex2(m_run[e] - m_new) : 1.f;
+                            l_run[e] *= alpha[e];
+                            m_run[e] = m_new;
+                            thr[e] = hv[e] ? m_new + kSlack : INFINITY;
+                        }
+                        float a0 = alpha[0], a1 = alpha[1];      // columns 2c, 2c+1 of every output tile
+                        if (kShared8) {
+                            const float y0 = __shfl_xor_sync(kFull, a0, 2), y1 = __shfl_xor_sync(kFull, a1, 2);
+                            if (c >= 2) { a0 = y0; a1 = y1; }
+                        }
+#pragma unroll
+                        for (int mt = 0; mt < 8; ++mt) {
+                            o[mt][0] *= a0; o[mt][1] *= a1; o[mt][2] *= a0; o[mt][3] *= a1;
+                        }
+                    }
+                    float ph[2][2], pl[2][2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float p0 = hv[e] ? ex2(s[0][e] - m_run[e]) : 0.f;
+                        const float p1 = hv[e] ? ex2(s[1][e] - m_run[e]) : 0.f;
+                        l_run[e] += p0 + p1;
+                        ph[0][e] = bf16_round(p0); pl[0][e] = p0 - ph[0][e];
+                        ph[1][e] = bf16_round(p1); pl[1][e] = p1 - ph[1][e];
+                    }
+                    // probabilities: score layout (row = token, cols = heads) -> operand layout (k = token, n = col)
+                    unsigned pb0, pb1, pc0 = 0, pc1 = 0;
+                    {
+                        const unsigned h0 = pack_bf16(ph[0][0], ph[0][1]), h1 = pack_bf16(ph[1][0], ph[1][1]);
+                        const unsigned l0 = pack_bf16(pl[0][0], pl[0][1]), l1 = pack_bf16(pl[1][0], pl[1][1]);
+                        if (kShared8) {                      // columns 4-7 carry the low parts of heads 0-3
+                            const unsigned x0 = __shfl_xor_sync(kFull, l0, 2), x1 = __shfl_xor_sync(kFull, l1, 2);
+                            pb0 = movmatrix_trans(c < 2 ? h0 : x0);
+                            pb1 = movmatrix_trans(c < 2 ? h1 : x1);
+                        } else {
+                            pb0 = movmatrix_trans(h0); pb1 = movmatrix_trans(h1);
+                            pc0 = movmatrix_trans(l0); pc1 = movmatrix_trans(l1);
+                        }
+                    }
+                    // ---------------- P.V: out^T[channel][col] += V^T[channel][token] P^T[token][col] ----------------
+                    unsigned vbase = page + L.v_off;
+                    if (kPV) {
+                        // lane (r, c) expands mask word c of tokens r and r + 8: channels 32c + 8u .. + 7 of a
+                        // token are 16-byte chunk k = 4c + u, stored at chunk index k ^ r ^ ((k >> 3) << 1) of the
+                        // token's row (the extra term keeps the four lanes of a row on different banks)
+                        vbase = smem_u32(smem + S::kVTile) + warp * kVTileBytes;
+                        unsigned vw[2], va[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            vw[j] = lds_u32(page + L.vmask_off + (8 * j + r) * 16 + c * 4);
+                            const int cnt = __popc(vw[j]);
+                            int x = cnt;
+                            int t = __shfl_up_sync(kFull, x, 1, 4);
+                            if (c >= 1) x += t;
+                            t = __shfl_up_sync(kFull, x, 2, 4);
+                            if (c >= 2) x += t;
+                            va[j] = page + L.v_off + (r * 2 + j) * 2 + (x - cnt) * 32;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                unsigned e0, e1, e2, e3;
+                                expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1);
+                                expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3);
+                                sts_u32x4(vbase + (8 * j + r) * (kHeadDim * 2) + (((4 * c + u) ^ r ^ (c & 2)) << 4), e0, e1, e2, e3);
+                            }
+                        __syncwarp();
+                    }
+                    const int mi = lane >> 3, rr = lane & 7;
+                    const unsigned vrow = vbase + (((mi >> 1) << 3) + rr) * (kHeadDim * 2);
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        unsigned a0, a1, a2, a3;
+                        ldmatrix_x4_trans(a0, a1, a2, a3, vrow + (((2 * mt + (mi & 1)) ^ rr ^ (kPV ? ((mt >> 2) << 1) : 0)) << 4));
+                        mma_bf16(o[mt], a0, a1, a2, a3, pb0, pb1);
+                        if (!kShared8) mma_bf16(o[mt], a0, a1, a2, a3, pc0, pc1);
+                    }
                 }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&C.empty[slot]);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&C.empty[slot]);
-        }
 
-        // ---------------- hand the warp state to the merge ----------------
-        {
-            float lsum[2];
+            // ---------------- the state goes to the merge as record warp + eu ----------------
+            {
+                float* rec = merge + (warp + eu) * G * kRec;
+                float lsum[2];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                lsum[e] = l_run[e];
-                lsum[e] += __shfl_xor_sync(kFull, lsum[e], 4);
-                lsum[e] += __shfl_xor_sync(kFull, lsum[e], 8);
-                lsum[e] += __shfl_xor_sync(kFull, lsum[e], 16);
+                for (int e = 0; e < 2; ++e) {
+                    lsum[e] = l_run[e];
+                    lsum[e] += __shfl_xor_sync(kFull, lsum[e], 4);
+                    lsum[e] += __shfl_xor_sync(kFull, lsum[e], 8);
+                    lsum[e] += __shfl_xor_sync(kFull, lsum[e], 16);
+                }
+#pragma unroll
+                for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        float v = o[mt][q4];
+                        if (kShared8) v += __shfl_xor_sync(kFull, v, 2);       // high-part column + low-part column
+                        const int e = q4 & 1;
+                        if (hv[e]) rec[(2 * c + e) * kRec + 16 * mt + r + ((q4 >> 1) << 3)] = v;
+                    }
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (hv[e] && r == 0) {
+                        rec[(2 * c + e) * kRec + kHeadDim] = m_run[e];
+                        rec[(2 * c + e) * kRec + kHeadDim + 1] = lsum[e];
+                    }
             }
-#pragma unroll
-            for (int mt = 0; mt < 8; ++mt)
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    float v = o[mt][q4];
-                    if (kShared8) v += __shfl_xor_sync(kFull, v, 2);       // high-part column + low-part column
-                    const int e = q4 & 1;
-                    if (hv[e]) merge[(warp * G + 2 * c + e) * kRec + 16 * mt + r + ((q4 >> 1) << 3)] = v;
-                }
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                if (hv[e] && r == 0) {
-                    merge[(warp * G + 2 * c + e) * kRec + kHeadDim] = m_run[e];
-                    merge[(warp * G + 2 * c + e) * kRec + kHeadDim + 1] = lsum[e];
-                }
         }
         consumer_sync<kNT>();
-        merge_and_publish<G, kNW>(A, C, merge, sg, tid);
-        g += sg.n;
-        base += sg.n;
+        merge_and_publish<G, kNW>(A, C, merge, unit_ml, ep.n_units, tid);
+        g = ep.e1;
     }
 }
 
@@ -527,14 +539,28 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
     using S = SmemBf16<G, kPV>;
     A.pps = 1;
     A.slot_stride = static_cast<int>(align_up(static_cast<size_t>(A.L.page_bytes), 128));
-    A.prefix_off = S::kFixed;
-    A.ring_off = S::kFixed + prefix_bytes(A.B);
-    int ns = (smem_optin - A.ring_off) / A.slot_stride;
-    if (ns > kMaxSlots) ns = kMaxSlots;
+    const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
+    const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    A.cap = epoch_cap(A.B, units, A.max_blocks, grid);
+    // An epoch's units take shared memory (operand tables, records) from the ring.  Where a CTA's run is long, a unit
+    // boundary (3 us) is a small part of it and ring slots are worth more: 16 sequences of 8K..128K tokens, seven
+    // heads per group (62 KB of records): 343 us with two units and 24 slots, 338 us with one and 26.  Short runs give
+    // up slots down to kMinRing.
+    const bool long_run = max_steps_per_cta(units, A.max_blocks, A.pps, grid) > 1024;
+    int ns = 0, ns_one = 0;
+    for (int cap = 1; cap <= A.cap; ++cap) {
+        const int tab_off = static_cast<int>(align_up(S::kMerge + merge_bytes(kNW, cap, G), 128));
+        const int prefix_off = tab_off + cap * S::kTabBytes, ring_off = prefix_off + prefix_bytes(A.B);
+        int n = (smem_optin - ring_off) / A.slot_stride;
+        if (n > kMaxSlots) n = kMaxSlots;
+        if (cap == 1) ns_one = n;
+        else if (n < (long_run ? ns_one : (ns_one < kMinRing ? ns_one : kMinRing))) { A.cap = cap - 1; break; }
+        A.tab_off = tab_off; A.prefix_off = prefix_off; A.ring_off = ring_off;
+        ns = n;
+    }
     if (ns < 2) return SPARK_ERR_UNSUPPORTED;
     A.nslots = ns;
     const size_t smem = A.ring_off + static_cast<size_t>(ns) * A.slot_stride;
-    const int grid = n_sms < kMaxCtas ? n_sms : kMaxCtas;
     if (A.q_by_value) {
         const size_t q_bytes = static_cast<size_t>(A.B) * A.Hq * kHeadDim * 2;
         if (kPV || q_bytes > static_cast<size_t>(kBlobLarge)) return SPARK_ERR_UNSUPPORTED;
