@@ -77,7 +77,7 @@ template <int G> struct SmemF32 {
     static constexpr int GP = ((G + 1 + 3) / 4) * 4;     // floats per table entry: G scaled queries + 1/a
     static constexpr int GPD = ((G + 1 + 1) / 2) * 2;    // doubles per table entry (degenerate rule: double table)
     static constexpr int GPP = ((G + 3) / 4) * 4;        // floats per probability entry
-    static constexpr int kCap = 2;                       // units per epoch (their tables are large)
+    static constexpr int kCap = 2;                       // units per epoch at most (their tables are large)
     static constexpr int kTabBytes = kHeadDim * GPD * 8; // sized for the double table (>= the float one)
     static constexpr int kQtab = kCtrlBytes;             // [kCap] tables
     static constexpr int kQsum = kQtab + kCap * kTabBytes;       // [kCap][8] double
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
     float* pscr = pscr_all + warp * 32 * GPP;
     for (int g = c0; g < c1;) {
-        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, S::kCap, g, c1);
+        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, g, c1);
 
         // ---- per-unit table: entry j = { q_0[j]*c, ..., q_{G-1}[j]*c, 1/a[j] },  c = scale*log2(e)
         UnitRef u = ep.first;
@@ -162,14 +162,16 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
         // ---- this warp's run of the epoch's steps, unit by unit ----
         const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kConsumerWarps, run_r = n_ep - run_q * kConsumerWarps;
-        int pos = ep.e0 + warp * run_q + min(warp, run_r); // line position
-        const int pos_end = pos + run_q + (warp < run_r ? 1 : 0);
+        int pos = ep.e0 + (A.cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
+        const int pos_end = A.cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
+        const int stride = A.cap == 1 ? kConsumerWarps : 1;
         int n = (ep.e0 - c0) + warp;                       // ring step of the warp's next step
         if (warp == kConsumerWarps - 1) describe_epoch<kConsumerWarps>(A, C, ep, lane);      // for the merge; this warp's run is never the longer
         u = ep.first;
         int eu = 0;
+        while (pos < pos_end && pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
         while (pos < pos_end) {
-            while (pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
+            u = locate_unit(C.prefix, A.B, A.Hkv, pos);    // (found again for each part: nothing of it stays in registers)
             const int part_end = min(pos_end, u.start + u.steps);
             const int b = u.b, h = u.h, len = C.lens[u.b];
             const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kQtab + eu * S::kTabBytes);
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
                 for (int c = 0; c < 4; ++c) acc[gg][c] = 0.f;
             }
 
-            for (; pos < part_end; ++pos, n += kConsumerWarps) {
+            for (; pos < part_end; pos += stride, n += kConsumerWarps) {
                 const int i = pos - u.start;
                 const int slot = n % NS;
                 const bool ok = slot_wait(C.full, C.seq, slot, n / NS, C.abort_flag, A.status);
@@ -354,10 +356,11 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
                     mine[gg * kRec + kHeadDim + 1] = lsum;
                 }
             }
+            ++eu;
         }
         consumer_sync<kConsumerThreads>();
-        merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, ep.n_units, tid);
-        g = ep.e1;
+        merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, C.epoch[1], tid);
+        g = C.epoch[0];
     }
 }
 
@@ -400,7 +403,7 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     using S = SmemF32<G>;
     A.pps = 2;
     A.slot_stride = static_cast<int>(align_up(2 * static_cast<size_t>(A.L.page_bytes), 128));
-    A.cap = S::kCap; A.tab_off = S::kQtab;
+    A.cap = A.B == 1 && 2 * A.Hkv <= n_sms ? 1 : S::kCap; A.tab_off = S::kQtab;
     A.prefix_off = S::kFixed;
     A.ring_off = S::kFixed + prefix_bytes(A.B);
     int ns = (smem_optin - A.ring_off) / A.slot_stride;

@@ -281,6 +281,7 @@ struct Ctrl {
     volatile int* seq;        // [32] revolution + 1 for which each slot was last armed
     volatile int* last_flag;  // [kMaxCap] this CTA is the last arriver of the epoch's unit
     Plan* plan;
+    volatile int* epoch;      // [2] the epoch's end and its number of units
     EpochUnit* units;         // [kMaxCap]
     int* prefix;              // [B + 1] steps before each sequence (of one KV head)
     int* lens;                // [B] clamped lengths
@@ -294,6 +295,7 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, i
     c.abort_flag = reinterpret_cast<volatile int*>(smem + 512);
     c.plan = reinterpret_cast<Plan*>(smem + 528);
     c.last_flag = reinterpret_cast<volatile int*>(smem + 560);
+    c.epoch = reinterpret_cast<volatile int*>(smem + 592);
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
     c.units = reinterpret_cast<EpochUnit*>(smem + 768);
     c.prefix = reinterpret_cast<int*>(smem + prefix_off);
@@ -476,9 +478,12 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
         id0 = id1 = -1; n0 = n1 = 0;
         if (!owner || n >= n_total) return;
         while (c0 + n >= ep.e1) ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, ep.e1, c1);
-        const int len = ep.e1 - ep.e0, q = len / NW, r = len - q * NW;
-        const int x = c0 + n - ep.e0, i = x / NW, w = x - i * NW;
-        const int g = ep.e0 + w * q + min(w, r) + i;
+        int g = c0 + n;
+        if (A.cap > 1) {
+            const int len = ep.e1 - ep.e0, q = len / NW, r = len - q * NW;
+            const int x = g - ep.e0, i = x / NW, w = x - i * NW;
+            g = ep.e0 + w * q + min(w, r) + i;
+        }
         UnitRef u = ep.first;
         while (g >= u.start + u.steps) next_unit(C.prefix, A.Hkv, u);
         producer_page_ids(A, C, u, g - u.start, id0, id1, n0, n1);
@@ -545,7 +550,19 @@ template <int NW>
 __device__ __forceinline__ void describe_epoch(const DecodeArgs& A, const Ctrl& C, const Epoch& ep, int lane)
 {
     const int n = ep.e1 - ep.e0, q = n / NW, r = n - q * NW;
+    if (lane == 0) { C.epoch[0] = ep.e1; C.epoch[1] = ep.n_units; }
     const int run0 = ep.e0 + (lane < NW ? lane * q + min(lane, r) : n);
+    if (A.cap == 1) {                                      // the warps that have a step hold a record each
+        if (lane == 0) {
+            EpochUnit d;
+            d.b = ep.first.b; d.h = ep.first.h;
+            d.rec0 = 0;
+            d.n_rec = min(NW, n);
+            unit_parts(*C.plan, ep.first.start, ep.first.steps, d.first_cta, d.n_parts);
+            C.units[0] = d;
+        }
+        return;
+    }
     UnitRef u = ep.first;
 #pragma unroll 1
     for (int e = 0; e < ep.n_units; ++e) {

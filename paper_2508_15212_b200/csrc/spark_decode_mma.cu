@@ -274,17 +274,21 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
         // ---- this warp's run of the epoch's steps, unit by unit ----
         const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kNW, run_r = n_ep - run_q * kNW;
-        int pos = ep.e0 + warp * run_q + min(warp, run_r);     // line position
-        const int pos_end = pos + run_q + (warp < run_r ? 1 : 0);
+        int pos = ep.e0 + (A.cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
+        const int pos_end = A.cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
+        const int stride = A.cap == 1 ? kNW : 1;
         int slot = (ep.e0 - c0) + warp, round = slot / NS;     // ring position of the warp's next step, kept incrementally
         slot -= round * NS;
         if (warp == kNW - 1) describe_epoch<kNW>(A, C, ep, lane);     // for the merge; this warp's run is never the longer
         UnitRef u = ep.first;
         int eu = 0;
+        while (pos < pos_end && pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
         while (pos < pos_end) {
-            while (pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
+            u = locate_unit(C.prefix, A.B, A.Hkv, pos);    // (found again for each part: nothing of it stays in registers)
             const int part_end = min(pos_end, u.start + u.steps);
-            int left = C.lens[u.b] - (pos - u.start) * kPageTokens;      // tokens from this step to the unit's end
+            const int cnt = A.cap == 1 ? (part_end - pos + kNW - 1) / kNW : part_end - pos;      // steps of this warp, >= 1
+            pos += cnt * stride;
+            const int tail = C.lens[u.b] - (pos - stride - u.start) * kPageTokens;      // valid rows of the last one (>= 16: all)
             // second-operand fragments (column r of each operand, channels 32c .. 32c+31):
             //   Bq[2s], Bq[2s+1] = q[head r][32c+4s .. +3];  Bp / Bpl likewise from the q' parts.
             unsigned Bq[16], Bp[16], Bpl[kShared8 ? 1 : 16];
@@ -313,20 +317,20 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                 qsum[e] = hv[e] ? qsum_all[eu * 8 + 2 * c + e] : 0.f;
             }
 
-            float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-            float thr[2] = {hv[0] ? -INFINITY : INFINITY, hv[1] ? -INFINITY : INFINITY};
+            // running reference maximum (+inf for an unused column: its probabilities are 0) and sum
+            float m_run[2] = {hv[0] ? -INFINITY : INFINITY, hv[1] ? -INFINITY : INFINITY}, l_run[2] = {0.f, 0.f};
             float o[8][4];
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) { o[mt][0] = 0.f; o[mt][1] = 0.f; o[mt][2] = 0.f; o[mt][3] = 0.f; }
 
-            for (; pos < part_end; ++pos, slot += kNW, left -= kPageTokens) {
+            for (int k = cnt; k > 0; --k, slot += kNW) {
                 while (slot >= NS) { slot -= NS; ++round; }
                 const bool ok = slot_wait(C.full, C.seq, slot, round, C.abort_flag, A.status);
                 const unsigned page = ring_u + static_cast<unsigned>(slot) * A.slot_stride;
-                const int n_valid = left;                          // >= 16: every row of the page
+                const int n_valid = k > 1 ? kPageTokens : tail;
                 if (ok) {
                     // ---------------- scores of the page's 16 tokens (rows r and r+8) ----------------
-                    float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f}, d3[4] = {0.f, 0.f, 0.f, 0.f};
+                    float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f};
                     unsigned vaddr[2], vaddr_hi[2], w[2];
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
@@ -350,20 +354,20 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                                           ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j]);
                         mma_bf16(d1, k0[0], k0[1], k1[0], k1[1], Bq[2 * ks], Bq[2 * ks + 1]);
                         mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bp[2 * ks], Bp[2 * ks + 1]);
-                        if (!kShared8) mma_bf16(d3, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
+                        if (!kShared8) mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
                     }
                     // kept q' sums of this thread's heads: high part + low part
                     float rk[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const float other = kShared8 ? __shfl_xor_sync(kFull, d2[e], 2) : d3[e];
-                        rk[e] = d2[e] + other;
+                        rk[e] = d2[e];
+                        if (kShared8) rk[e] += __shfl_xor_sync(kFull, d2[e], 2);
                     }
                     // ---------------- online softmax over the 16 tokens ----------------
                     // The reference maximum m_run of a head moves only when a score of the page exceeds it
                     // by more than kSlack (log2 units), so most pages skip the warp-wide maximum and the
                     // rescaling; probabilities then lie in (0, 2^kSlack], which fp32 sums and the bf16
-                    // high/low split carry without loss.  thr = m_run + kSlack (+inf for unused columns).
+                    // high/low split carry without loss.
                     const float mu[2] = {lds_f32(page + L.mu_off + r * 4), lds_f32(page + L.mu_off + (r + 8) * 4)};
                     float s[2][2];
 #pragma unroll
@@ -373,8 +377,8 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                             const float sv = A.scale_log2e * fmaf(mu[j], qsum[e] - rk[2 * j + e], d1[2 * j + e]);
                             s[j][e] = (r + 8 * j < n_valid) ? sv : -INFINITY;
                         }
-                    const float over = fmaxf(fmaxf(s[0][0], s[1][0]) - thr[0], fmaxf(s[0][1], s[1][1]) - thr[1]);
-                    if (__any_sync(kFull, over > 0.f)) {
+                    const float over = fmaxf(fmaxf(s[0][0], s[1][0]) - m_run[0], fmaxf(s[0][1], s[1][1]) - m_run[1]);
+                    if (__any_sync(kFull, over > kSlack)) {
                         float alpha[2];
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
@@ -386,7 +390,6 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                             alpha[e] = hv[e] ? ex2(m_run[e] - m_new) : 1.f;
                             l_run[e] *= alpha[e];
                             m_run[e] = m_new;
-                            thr[e] = hv[e] ? m_new + kSlack : INFINITY;
                         }
                         float a0 = alpha[0], a1 = alpha[1];      // columns 2c, 2c+1 of every output tile
                         if (kShared8) {
@@ -401,8 +404,8 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                     float ph[2][2], pl[2][2];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const float p0 = hv[e] ? ex2(s[0][e] - m_run[e]) : 0.f;
-                        const float p1 = hv[e] ? ex2(s[1][e] - m_run[e]) : 0.f;
+                        const float p0 = ex2(s[0][e] - m_run[e]);
+                        const float p1 = ex2(s[1][e] - m_run[e]);
                         l_run[e] += p0 + p1;
                         ph[0][e] = bf16_round(p0); pl[0][e] = p0 - ph[0][e];
                         ph[1][e] = bf16_round(p1); pl[1][e] = p1 - ph[1][e];
@@ -492,10 +495,11 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                         rec[(2 * c + e) * kRec + kHeadDim + 1] = lsum[e];
                     }
             }
+            ++eu;
         }
         consumer_sync<kNT>();
-        merge_and_publish<G, kNW>(A, C, merge, unit_ml, ep.n_units, tid);
-        g = ep.e1;
+        merge_and_publish<G, kNW>(A, C, merge, unit_ml, C.epoch[1], tid);
+        g = C.epoch[0];
     }
 }
 
