@@ -15,37 +15,59 @@ constexpr unsigned kFullMask = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------------
 // a[b][h][j] = max(|mean over the G*W window queries of the group|, eps).
-// One thread per channel; the sum runs in double over (g outer, w inner), so the rounded mean does
-// not depend on launch shape.  Thread 0 of the first head also publishes packed_lens when there is
-// no eviction step.
+// 512 threads: a thread sums 16 bytes' worth of channels over every 32nd (fp32: 16th) row in double, the row groups
+// are then added in a fixed order.  (The sum is exact in double for any order unless its terms differ by more than
+// 2^21.)  The chain that bounds the kernel is a load and a few adds: one thread per channel walking all rows took
+// 8.3 us for 128 rows, this 7.1 (both cold), and the page kernel's first loads now run under it.
+// Thread 0 of the first head also publishes packed_lens when there is no eviction step.
 // ------------------------------------------------------------------------------------------------
+constexpr int kQnThreads = 512;
 template <typename E>
-__global__ void __launch_bounds__(kHeadDim)
+__global__ void __launch_bounds__(kQnThreads)
 window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, float eps,
                     float* __restrict__ qnorm, const int32_t* __restrict__ seq_lens,
                     int32_t* __restrict__ packed_lens, int max_seq_tokens, int* status)
 {
+    constexpr int kVec = 16 / sizeof(E);                       // channels per 16-byte load
+    constexpr int kChunks = kHeadDim / kVec, kGroups = kQnThreads / kChunks;
+    __shared__ double part[kGroups / 2][kHeadDim];
     grid_wait();
     grid_release();
-    const int h = blockIdx.x, b = blockIdx.y, j = threadIdx.x;
-    const int G = Hq / Hkv;
+    const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    const int G = Hq / Hkv, rows = G * W;
+    const int c = tid % kChunks, grp = tid / kChunks;
     // the group's G*W window rows are consecutive in memory, (g outer, w inner)
-    const int64_t base = ((static_cast<int64_t>(b) * Hq + h * G) * W) * kHeadDim + j;
-    const int rows = G * W;
-    double acc = 0.0;
-    int r = 0;
-    for (; r + 32 <= rows; r += 32) {                      // thirty-two loads in flight, summed in order
-        float x[32];
+    const E* src = static_cast<const E*>(q_win) + (static_cast<int64_t>(b) * Hq + h * G) * W * kHeadDim + c * kVec;
+    double acc[kVec];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) x[u] = Elem<E>::load(q_win, base + static_cast<int64_t>(r + u) * kHeadDim);
+    for (int i = 0; i < kVec; ++i) acc[i] = 0.0;
+    const bool aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;
+#pragma unroll 4
+    for (int r = grp; r < rows; r += kGroups) {
+        alignas(16) E x[kVec];
+        const E* row = src + static_cast<int64_t>(r) * kHeadDim;
+        if (aligned) *reinterpret_cast<uint4*>(x) = *reinterpret_cast<const uint4*>(row);
+        else
+            for (int i = 0; i < kVec; ++i) x[i] = row[i];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) acc += static_cast<double>(x[u]);
+        for (int i = 0; i < kVec; ++i) acc[i] += static_cast<double>(static_cast<float>(x[i]));
     }
-    for (; r < rows; ++r)
-        acc += static_cast<double>(Elem<E>::load(q_win, base + static_cast<int64_t>(r) * kHeadDim));
-    const float m = static_cast<float>(acc / static_cast<double>(G * W));
-    qnorm[(static_cast<int64_t>(b) * Hkv + h) * kHeadDim + j] = fmaxf(fabsf(m), eps);
-    if (packed_lens && h == 0 && j == 0) {
+    if (grp >= kGroups / 2)
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) part[grp - kGroups / 2][c * kVec + i] = acc[i];
+    __syncthreads();
+    if (grp < kGroups / 2)
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) part[grp][c * kVec + i] += acc[i];
+    __syncthreads();
+    if (tid < kHeadDim) {
+        double sum = 0.0;
+#pragma unroll
+        for (int g = 0; g < kGroups / 2; ++g) sum += part[g][tid];
+        const float m = static_cast<float>(sum / static_cast<double>(rows));
+        qnorm[(static_cast<int64_t>(b) * Hkv + h) * kHeadDim + tid] = fmaxf(fabsf(m), eps);
+    }
+    if (packed_lens && h == 0 && tid == 0) {
         int len = seq_lens[b];
         if (len < 0 || len > max_seq_tokens) {
             record_error(status, SPARK_ERR_DEVICE_BOUNDS);
@@ -341,6 +363,7 @@ struct CompressArgs {
     const void* v;
     int64_t sb, sh, st;
     const int32_t* lens;          // tokens per sequence AFTER eviction (packed lens)
+    int max_len;                  // upper bound of lens (compress_pages_warp_kernel reads the caller's lengths, unchecked)
     const int32_t* gather;        // optional [B][Hkv][gather_stride] source token positions
     int gather_stride;
     const float* qnorm;
@@ -654,6 +677,284 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
     uint4* dst = reinterpret_cast<uint4*>(A.pages + page_id * L.page_bytes);
     for (int i = threadIdx.x; i < L.page_bytes / 16; i += blockDim.x)
         dst[i] = reinterpret_cast<const uint4*>(image)[i];
+}
+
+// ------------------------------------------------------------------------------------------------
+// Fixed-T pages of bf16 storage, a page per WARP: a token belongs to two lanes (64 channels each), so a step of the
+// selection serves sixteen tokens and needs one shuffle, and a warp owns its page from the loads to the stores
+// without a CTA barrier.
+//   Selection.  Any threshold t with exactly T keys >= t names the kept set, so the search need not descend bit by bit:
+//   it interpolates the count between its two ends (every third step bisects, which bounds it) over the keys' upper
+//   halves, two keys per compare.  Where the boundary falls inside one upper half (a fifth of the tokens), the few
+//   keys that share it are told apart by their full bits, in order of key and then of channel.
+//   What bounds it: issue slots.  183 instructions a token against 308 with eight lanes per token and a bitwise
+//   descent (compress_pages4_kernel, which fp32 storage and sampled recovery keep); 8 heads x 32768 tokens:
+//   104 -> 66 us under the profiler, prefill of 32K tokens 132.4 -> 90.3 us (24 warps a SM; with 16 it took 93.4).
+// ------------------------------------------------------------------------------------------------
+constexpr int kWarpPageWarps = 4;
+constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
+
+__device__ __forceinline__ unsigned bits_max2(unsigned a, unsigned b)          // bf16 pairs; a NaN wins
+{
+    const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const unsigned*>(&r);
+}
+__device__ __forceinline__ unsigned bits_min2(unsigned a, unsigned b)          // bf16 pairs; a NaN loses
+{
+    const __nv_bfloat162 r = __hmin2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const unsigned*>(&r);
+}
+__device__ __forceinline__ unsigned ge_mask_bf16x2(unsigned a, unsigned b)     // 0xFFFF per half where a >= b
+{
+    return __hge2_mask(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+}
+// keys of this lane at or above the threshold (its upper half in both halves of t2)
+__device__ __forceinline__ int count_ge(const unsigned (&hk)[32], unsigned t2)
+{
+    __nv_bfloat162 c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = ge_one_bf16x2(hk[i], t2);
+#pragma unroll
+    for (int j = 4; j < 32; ++j) c[j & 3] = __hadd2(c[j & 3], ge_one_bf16x2(hk[j], t2));   // counts <= 32: exact in bf16
+    const __nv_bfloat162 t = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
+    return static_cast<int>(__low2float(t) + __high2float(t));
+}
+// full key of channel ch (0..63) of this lane's half row
+template <bool kValue>
+__device__ __forceinline__ unsigned full_key(const unsigned char* row, int sw, int half, int ch, const float* a)
+{
+    const int c = 8 * half + (ch >> 3);
+    const unsigned short h = *reinterpret_cast<const unsigned short*>(row + ((c ^ sw) << 4) + (ch & 7) * 2);
+    const float x = fabsf(bf16_bits_to_float(h));
+    return __float_as_uint(kValue ? x : __fmul_rn(a[ch], x));
+}
+
+// One section of a page from the rows in `tile` (16 rows of 256 bytes, 16-byte chunk c of row p at c ^ (p & 7)): kept
+// values in slot order, mask words, and for keys (kValue false) the mean of the pruned saliencies.
+template <bool kValue>
+__device__ __forceinline__ void select_section(const unsigned char* tile, unsigned char* image, int vals_off, int mask_off,
+                                               int mu_off, int T, int n, int lane, const float* a_all, double inv_pruned)
+{
+    const int p = lane & 15, half = lane >> 4, sw = p & 7;
+    const bool live = p < n;
+    const unsigned char* row = tile + p * (kHeadDim * 2);
+    const float* a = a_all + 64 * half;
+    unsigned kept[2] = {live ? 0xffffffffu : 0u, live ? 0xffffffffu : 0u};
+    if (T < kHeadDim) {
+        // upper halves of the keys: word 16 g + j holds channels 32 g + j (low) and 32 g + 16 + j (high)
+        unsigned hk[32];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            unsigned w[16];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + 4 * g + c) ^ sw) << 4));
+                const unsigned x[4] = {v.x, v.y, v.z, v.w};
+                if (kValue) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {               // |V| itself is the key
+                        const unsigned m = x[j] & 0x7fff7fffu;
+                        const int i0 = 8 * c + 2 * j;
+                        if (i0 < 16) { w[i0] = m & 0xffffu; w[i0 + 1] = m >> 16; }
+                        else { w[i0 - 16] |= m << 16; w[i0 - 15] |= m & 0xffff0000u; }
+                    }
+                } else {
+                    const float4 f0 = *reinterpret_cast<const float4*>(a + 32 * g + 8 * c);
+                    const float4 f1 = *reinterpret_cast<const float4*>(a + 32 * g + 8 * c + 4);
+                    const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const unsigned k0 = __float_as_uint(__fmul_rn(f[2 * j], fabsf(__uint_as_float(x[j] << 16))));
+                        const unsigned k1 = __float_as_uint(__fmul_rn(f[2 * j + 1], fabsf(__uint_as_float(x[j] & 0xffff0000u))));
+                        const int i0 = 8 * c + 2 * j;
+                        if (i0 < 16) { w[i0] = k0; w[i0 + 1] = k1; }
+                        else { w[i0 - 16] = __byte_perm(w[i0 - 16], k0, 0x7632); w[i0 - 15] = __byte_perm(w[i0 - 15], k1, 0x7632); }
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) hk[16 * g + j] = w[j];
+        }
+        unsigned mx = hk[0], mn = hk[0];
+#pragma unroll
+        for (int j = 1; j < 32; ++j) { mx = bits_max2(mx, hk[j]); mn = bits_min2(mn, hk[j]); }
+        mx = bits_max2(mx, mx >> 16 | mx << 16); mn = bits_min2(mn, mn >> 16 | mn << 16);
+        mx = bits_max2(mx, __shfl_xor_sync(kFullMask, mx, 16)) & 0xffffu;
+        mn = bits_min2(mn, __shfl_xor_sync(kFullMask, mn, 16)) & 0xffffu;
+        if (__any_sync(kFullMask, mx > 0x7f80u)) {             // NaN saliencies order above infinity, by their bits
+#pragma unroll
+            for (int j = 0; j < 32; ++j) hk[j] = bits_min2(hk[j], 0x7f807f80u);
+            mx = mx > 0x7f80u ? 0x7f80u : mx;
+            mn = mn > 0x7f80u ? 0x7f80u : mn;
+        }
+        int lo = static_cast<int>(mn), hi = static_cast<int>(mx) + 1, c_lo = kHeadDim, c_hi = 0;   // counts at lo (>= T) and hi (< T)
+        bool done = !live || hi - lo == 1;
+        for (int it = 0; !__all_sync(kFullMask, done); ++it) {
+            const int span = hi - lo;
+            int step = span >> 1;
+            if (it % 3 != 2)
+                step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(2 * (c_lo - T) + 1), static_cast<float>(2 * (c_lo - c_hi))));
+            step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
+            const int t = lo + step;
+            int c = count_ge(hk, static_cast<unsigned>(t) * 0x00010001u);
+            c += __shfl_xor_sync(kFullMask, c, 16);
+            if (!done) {
+                if (c >= T) { lo = t; c_lo = c; } else { hi = t; c_hi = c; }
+                done = c == T || hi - lo == 1;
+            }
+        }
+        // keys at or above lo; the kept set when there are exactly T of them
+        const unsigned t2 = static_cast<unsigned>(lo) * 0x00010001u;
+        unsigned ge[2] = {0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 32; ++j) ge[j >> 4] |= ge_mask_bf16x2(hk[j], t2) & (0x00010001u << (j & 15));
+        int need = live && c_lo != T ? T - c_hi : 0;           // keys of upper half `lo` to admit
+        kept[0] &= ge[0]; kept[1] &= ge[1];
+        if (__any_sync(kFullMask, need > 0)) {
+            const unsigned u2 = static_cast<unsigned>(hi) * 0x00010001u;
+            unsigned gt[2] = {0u, 0u};
+            if (hi <= 0x7f80) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) gt[j >> 4] |= ge_mask_bf16x2(hk[j], u2) & (0x00010001u << (j & 15));
+            }
+            unsigned long long cand = 0ull, got = 0ull;
+            if (need > 0) {
+                cand = (static_cast<unsigned long long>(ge[1] & ~gt[1]) << 32) | (ge[0] & ~gt[0]);
+                got = (static_cast<unsigned long long>(gt[1]) << 32) | gt[0];
+            }
+            while (__any_sync(kFullMask, need > 0)) {
+                unsigned best = 0u;                             // largest full key left (keys compare as their bits)
+                unsigned long long eq = 0ull;
+                for (unsigned long long m = need > 0 ? cand : 0ull; m; m &= m - 1) {
+                    const int ch = __ffsll(static_cast<long long>(m)) - 1;
+                    const unsigned k = full_key<kValue>(row, sw, half, ch, a);
+                    if (k > best) { best = k; eq = 0ull; }
+                    if (k == best) eq |= 1ull << ch;
+                }
+                const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
+                if (other > best) eq = 0ull;
+                const int mine = __popcll(eq), theirs = __shfl_xor_sync(kFullMask, mine, 16);
+                int take = half ? need - theirs : need;         // equal keys: lower channels first
+                take = take < 0 ? 0 : (take > mine ? mine : take);
+                unsigned long long rest = eq;
+                for (int k = 0; k < take; ++k) rest &= rest - 1;
+                got |= eq & ~rest;
+                cand &= ~eq;
+                need -= mine + theirs;
+                if (mine + theirs == 0) need = 0;               // (no candidate left)
+            }
+            if (live && c_lo != T) { kept[0] = static_cast<unsigned>(got); kept[1] = static_cast<unsigned>(got >> 32); }
+        }
+    }
+    const int mine = __popc(kept[0]) + __popc(kept[1]);
+    const int theirs = __shfl_xor_sync(kFullMask, mine, 16);
+    unsigned char* dst = image + vals_off + val_offset(2, p, half ? theirs : 0);
+    double pruned = 0.0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const unsigned kb = kept[g];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + 4 * g + c) ^ sw) << 4));
+            const unsigned x[4] = {v.x, v.y, v.z, v.w};
+            float f[8];
+            if (!kValue) {
+                const float4 f0 = *reinterpret_cast<const float4*>(a + 32 * g + 8 * c);
+                const float4 f1 = *reinterpret_cast<const float4*>(a + 32 * g + 8 * c + 4);
+                f[0] = f0.x; f[1] = f0.y; f[2] = f0.z; f[3] = f0.w; f[4] = f1.x; f[5] = f1.y; f[6] = f1.z; f[7] = f1.w;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned h = (i & 1) ? x[i >> 1] >> 16 : x[i >> 1] & 0xffffu;
+                if ((kb >> (8 * c + i)) & 1u) {
+                    *reinterpret_cast<unsigned short*>(dst) = static_cast<unsigned short>(h);
+                    dst += kPageTokens * 2;
+                } else if (!kValue) {
+                    pruned += static_cast<double>(__fmul_rn(f[i], fabsf(__uint_as_float(h << 16))));
+                }
+            }
+        }
+    }
+    *reinterpret_cast<uint2*>(image + mask_off + p * 16 + half * 8) = make_uint2(kept[0], kept[1]);
+    if (!kValue) {
+        pruned += __shfl_xor_sync(kFullMask, pruned, 16);
+        if (half == 0) reinterpret_cast<float*>(image + mu_off)[p] = live ? static_cast<float>(pruned * inv_pruned) : 0.f;
+    }
+}
+
+template <bool kPV>
+__global__ void __launch_bounds__(kWarpPageWarps * 32, kPV ? 5 : 6) compress_pages_warp_kernel(CompressArgs A)
+{
+    extern __shared__ __align__(16) unsigned char page_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blk = blockIdx.x * kWarpPageWarps + warp, h = blockIdx.y, b = blockIdx.z;
+    const PageLayout L = A.L;
+    const int image_bytes = kPV ? L.page_bytes : L.v_off;      // dense value rows go straight to the page
+    float* a_s = reinterpret_cast<float*>(page_smem);
+    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_bytes);
+    unsigned char* image = tile + kTileBytes;
+
+    // Without eviction the kernel before this one is the window norm, and what it waited for is complete (see
+    // grid_release): keys, values and lengths may be read before it ends.
+    if (A.gather) { grid_wait(); grid_release(); }
+    int len = A.lens[b];
+    len = len > A.max_len ? A.max_len : len;
+    const int t0 = blk * kPageTokens;
+    const int n = len - t0 < kPageTokens ? len - t0 : kPageTokens;
+    const int c16 = lane & 15, r2 = lane >> 4;                 // a row per half warp, a 16-byte chunk per lane
+    int64_t src_row = t0 + c16;                                 // lane p (p < 16): the source row of token p
+    if (A.gather && c16 < n) src_row = A.gather[(static_cast<int64_t>(b) * A.Hkv + h) * A.gather_stride + t0 + c16];
+    const int64_t base = static_cast<int64_t>(b) * A.sb + static_cast<int64_t>(h) * A.sh + c16 * 8;
+    uint4 kr[8], vr[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int p = 2 * i + r2;
+        const int64_t row = base + __shfl_sync(kFullMask, src_row, p) * A.st;
+        kr[i] = vr[i] = make_uint4(0, 0, 0, 0);
+        if (p < n) {
+            kr[i] = *reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(A.k) + row);
+            vr[i] = *reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(A.v) + row);
+        }
+    }
+    const int64_t entry = (static_cast<int64_t>(b) * A.Hkv + h) * A.max_blocks + blk;
+    int64_t page_id = 0;
+    if (n > 0) page_id = A.block_table ? A.block_table[entry] : entry;        // no table: contiguous cache
+    const bool page_ok = page_id >= 0 && page_id < A.n_pool_pages;
+    if (!A.gather) { grid_wait(); grid_release(); }
+    a_s[threadIdx.x] = A.qnorm[(static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + threadIdx.x];
+    __syncthreads();
+    if (n <= 0) return;                                        // warp-uniform; no CTA barrier below
+    if (!page_ok) {
+        if (lane == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+        return;
+    }
+    unsigned char* page = A.pages + page_id * L.page_bytes;
+    if (n < kPageTokens)                                       // slots past the end of the sequence are zero
+        for (int i = lane; i < image_bytes / 16; i += 32) reinterpret_cast<uint4*>(image)[i] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int p = 2 * i + r2, off = p * (kHeadDim * 2) + ((c16 ^ (p & 7)) << 4);
+        if (kPV) *reinterpret_cast<uint4*>(tile + off) = vr[i];
+        else {
+            *reinterpret_cast<uint4*>(page + L.v_off + off) = vr[i];
+            *reinterpret_cast<uint4*>(tile + off) = kr[i];
+        }
+    }
+    __syncwarp();
+    if (kPV) {                                                 // value-channel pruning: the same selection on |V|
+        select_section<true>(tile, image, L.v_off, L.vmask_off, 0, L.keep_v, n, lane, a_s, 0.0);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int p = 2 * i + r2;
+            *reinterpret_cast<uint4*>(tile + p * (kHeadDim * 2) + ((c16 ^ (p & 7)) << 4)) = kr[i];
+        }
+        __syncwarp();
+    }
+    select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
+    __syncwarp();
+    for (int i = lane; i < image_bytes / 16; i += 32)
+        reinterpret_cast<uint4*>(page)[i] = reinterpret_cast<const uint4*>(image)[i];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1088,10 +1389,10 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const float eps = p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f;
     const dim3 qgrid(p.n_kv_heads, p.batch);
     if (p.dtype == SPARK_BF16)
-        launch_kernel(window_qnorm_kernel<__nv_bfloat16>, qgrid, dim3(kHeadDim), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
+        launch_kernel(window_qnorm_kernel<__nv_bfloat16>, qgrid, dim3(kQnThreads), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
                       eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
     else
-        launch_kernel(window_qnorm_kernel<float>, qgrid, dim3(kHeadDim), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
+        launch_kernel(window_qnorm_kernel<float>, qgrid, dim3(kQnThreads), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
                       eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
@@ -1107,6 +1408,20 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     A.n_pool_pages = p.n_pool_pages; A.L = make_layout(p); A.status = status;
     A.inv_pruned = p.keep < kHeadDim ? 1.0 / static_cast<double>(kHeadDim - p.keep) : 0.0;
     A.sel = make_select(p);
+    A.max_len = max_packed;
+    if (p.dtype == SPARK_BF16 && p.select == SPARK_SELECT_FIXED && p.recovery == SPARK_RECOVER_DEGENERATE) {
+        if (!evict) A.lens = seq_lens;                         // readable before the window norm has ended
+        const bool pv = A.L.keep_v < kHeadDim;
+        const size_t smem = kHeadDim * 4 + kWarpPageWarps * (kTileBytes + static_cast<size_t>(pv ? A.L.page_bytes : A.L.v_off));
+        if (smem > 48 * 1024 &&                                // capacities near 128 + 128
+            cudaFuncSetAttribute(compress_pages_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+            return SPARK_ERR_CUDA;
+        const dim3 wgrid((n_blocks + kWarpPageWarps - 1) / kWarpPageWarps, p.n_kv_heads, p.batch);
+        const cudaError_t e = pv ? launch_kernel(compress_pages_warp_kernel<true>, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A)
+                                 : launch_kernel(compress_pages_warp_kernel<false>, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A);
+        ++*launches;
+        return e == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
+    }
     const dim3 grid(n_blocks, p.n_kv_heads, p.batch);
     const bool rank = p.select != SPARK_SELECT_FIXED;      // a ratio-free rule: the kernels with the rank sort
     if (p.dtype == SPARK_BF16) {

@@ -77,13 +77,12 @@ template <int G> struct SmemF32 {
     static constexpr int GP = ((G + 1 + 3) / 4) * 4;     // floats per table entry: G scaled queries + 1/a
     static constexpr int GPD = ((G + 1 + 1) / 2) * 2;    // doubles per table entry (degenerate rule: double table)
     static constexpr int GPP = ((G + 3) / 4) * 4;        // floats per probability entry
-    static constexpr int kCap = 2;                       // units per epoch at most (their tables are large)
     static constexpr int kTabBytes = kHeadDim * GPD * 8; // sized for the double table (>= the float one)
-    static constexpr int kQtab = kCtrlBytes;             // [kCap] tables
-    static constexpr int kQsum = kQtab + kCap * kTabBytes;       // [kCap][8] double
-    static constexpr int kPscr = kQsum + kCap * 64;
-    static constexpr int kMerge = kPscr + kConsumerWarps * 32 * GPP * 4;
-    static constexpr int kFixed = (kMerge + merge_bytes(kConsumerWarps, kCap, G) + 127) / 128 * 128;   // prefix and ring start here
+    static constexpr int kQsum = kCtrlBytes;             // [kMaxCap][8] double
+    static constexpr int kPscr = kQsum + kMaxCap * 64;
+    static constexpr int kTab = kPscr + kConsumerWarps * 32 * GPP * 4;       // [cap] tables, then merge area, prefix and ring
+    static constexpr int merge_off(int cap) { return kTab + cap * kTabBytes; }
+    static constexpr int fixed(int cap) { return (merge_off(cap) + merge_bytes(kConsumerWarps, cap, G) + 127) / 128 * 128; }
 };
 
 template <int G, typename E, int R>
@@ -100,8 +99,8 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
     double* qsum_all = reinterpret_cast<double*>(smem + S::kQsum);
     float* pscr_all = reinterpret_cast<float*>(smem + S::kPscr);
-    float* merge = reinterpret_cast<float*>(smem + S::kMerge);
-    float* unit_ml = merge + merge_state_floats(kConsumerWarps, S::kCap, G);
+    float* merge = reinterpret_cast<float*>(smem + S::kTab + A.cap * S::kTabBytes);
+    float* unit_ml = merge + merge_state_floats(kConsumerWarps, A.cap, G);
     unsigned char* ring = smem + A.ring_off;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -131,7 +130,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 #pragma unroll 1
         for (int e = 0; e < ep.n_units; ++e) {
             if (e) next_unit(C.prefix, A.Hkv, u);
-            TabT* qtab = reinterpret_cast<TabT*>(smem + S::kQtab + e * S::kTabBytes);
+            TabT* qtab = reinterpret_cast<TabT*>(smem + S::kTab + e * S::kTabBytes);
             for (int idx = tid; idx < kHeadDim * GP; idx += kConsumerThreads) {
                 const int j = idx / GP, col = idx - j * GP;
                 TabT val = 0;
@@ -147,7 +146,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 #pragma unroll 1
         for (int e = 0; e < ep.n_units; ++e)
             if (warp < G) {                                // Qsum[g] = sum_j q_g[j]*c / a[j]
-                const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kQtab + e * S::kTabBytes);
+                const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kTab + e * S::kTabBytes);
                 double part = 0.0;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -174,7 +173,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
             u = locate_unit(C.prefix, A.B, A.Hkv, pos);    // (found again for each part: nothing of it stays in registers)
             const int part_end = min(pos_end, u.start + u.steps);
             const int b = u.b, h = u.h, len = C.lens[u.b];
-            const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kQtab + eu * S::kTabBytes);
+            const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kTab + eu * S::kTabBytes);
             const double* qsum = qsum_all + eu * 8;
             float m_run[G], l_run[G], acc[G][4];
 #pragma unroll
@@ -403,14 +402,17 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     using S = SmemF32<G>;
     A.pps = 2;
     A.slot_stride = static_cast<int>(align_up(2 * static_cast<size_t>(A.L.page_bytes), 128));
-    A.cap = A.B == 1 && 2 * A.Hkv <= n_sms ? 1 : S::kCap; A.tab_off = S::kQtab;
-    A.prefix_off = S::kFixed;
-    A.ring_off = S::kFixed + prefix_bytes(A.B);
+    const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
+    const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    // Two units per epoch only where CTAs hold several: the second unit's table and records cost a ring slot (of six or
+    // seven: 2 x 7926 tokens, G = 4, T = 89: 43.9 us with six slots, 35.2 us with seven).
+    A.cap = 2 * units <= grid ? 1 : 2;
+    A.tab_off = S::kTab;
+    A.prefix_off = S::fixed(A.cap);
+    A.ring_off = A.prefix_off + prefix_bytes(A.B);
     int ns = (smem_optin - A.ring_off) / A.slot_stride;
     if (ns > kMaxSlots) ns = kMaxSlots;
     if (ns < 2) return SPARK_ERR_UNSUPPORTED;
-    const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
-    const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     // no more slots than a CTA has steps: a small call then leaves the SM room for the next kernel's CTA, whose
     // start-up runs under this one's end
     const int64_t most = max_steps_per_cta(units, A.max_blocks, A.pps, grid);
