@@ -12,10 +12,13 @@
 //   evict_scores_kernel<pass 1>  per 128-token tile and query row: max and sum of exp of the scores
 //   evict_rowstats_kernel        merge the tile partials into the row's softmax normaliser
 //   evict_scores_kernel<pass 2>  recompute the tile's scores, accumulate the column sums = votes
-//   evict_pool_kernel            pooled max of the votes, as order-preserving integer keys
-//   evict_hist_kernel<0..3>      radix select of the k-th largest key, one byte per pass, all SMs
-//   evict_count / compact        ordered compaction of the kept positions into kept_tokens
+//   evict_select_kernel          pooled max of the votes, exact radix select of the k-th largest, ordered compaction
+//                                of the kept positions into kept_tokens: one launch, a cluster per unit
 // Column sums are accumulated inside one CTA in a fixed order, so the votes are reproducible.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "spark_common.cuh"
 
 namespace spark {
@@ -35,10 +38,8 @@ struct EvictArgs {
     float* partial;      // [units][R][n_tiles][2]
     float* rowstat;      // [units][R][2]
     float* votes;        // [units][S_max]
-    unsigned* pooled;    // [units][S_max] pooled votes as order-preserving keys
-    int* hist;           // [units][4][256] radix-select histograms, one per pass
-    int* counts;         // [units][n_chunks][2] keys above / equal to the threshold per 4096-token chunk
-    int n_chunks;
+    unsigned* pooled;    // [units][S_max] pooled votes as order-preserving keys (shares above key_cap only)
+    int key_cap;         // keys a CTA of the select kernel holds in shared memory
     int32_t* kept;       // [units][budget]
     int32_t* packed_lens;
     int* status;
@@ -188,251 +189,238 @@ __global__ void evict_rowstats_kernel(EvictArgs A)
     }
 }
 
-// pooled[t] = max of the votes within (pool-1)/2 positions of t (clamped to the prefix), stored as the
-// float's bit pattern: votes are >= 0, so unsigned comparison of the patterns is the order of the values.
-__global__ void __launch_bounds__(256) evict_pool_kernel(EvictArgs A)
-{
-    grid_wait();
-    grid_release();
-    const int h = blockIdx.y, b = blockIdx.z;
-    const int S = min(A.seq_lens[b], A.S_max);
-    if (S <= A.budget) return;
-    const int P = S - A.W, half = (A.pool - 1) / 2;
-    if (blockIdx.x == 0)                                   // fresh histograms for this call's radix select
-        for (int i = threadIdx.x; i < 1024; i += blockDim.x) A.hist[static_cast<int64_t>(b * A.Hkv + h) * 1024 + i] = 0;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= P) return;
-    const int64_t base = static_cast<int64_t>(b * A.Hkv + h) * A.S_max;
-    float m = A.votes[base + t];
-    for (int u = t - half; u <= t + half; ++u)
-        if (u >= 0 && u < P) m = fmaxf(m, A.votes[base + u]);
-    A.pooled[base + t] = __float_as_uint(m);
-}
-
 // ------------------------------------------------------------------------------------------------
-// Exact top-k of the pooled votes and ordered compaction, spread over the whole GPU.
-//
-// The k-th largest key of a unit is found by a radix select, 8 bits per pass: every CTA histograms its
-// 4096-token chunk into shared memory and adds the non-empty bins to the unit's histogram of that pass
-// (integer atomics: the result does not depend on arrival order).  The choice made by each finished pass
-// (the byte of the threshold, the rank left inside that bin) is recomputed from the stored histograms by
-// whoever needs it, so there is no separate "pick" launch.  After four passes the threshold key and the
-// number of equal keys to admit (lowest positions first) are known; a counting kernel gives every chunk
-// its base position and the compaction kernel writes the kept positions in order.
+// Pooled votes, exact top-k and ordered compaction in ONE launch: a cluster of CTAs per (sequence, KV head), each with
+// an equal share of the prefix.
+//   pooled[t] = max of the votes within (pool-1)/2 positions of t (clamped to the prefix) as the float's bit pattern:
+//   votes are >= 0, so unsigned comparison of the patterns is the order of the values.  The keys stay in the CTA's
+//   shared memory (in the workspace where its share is larger than kKeyCap).
+//   The k-th largest key is found by a radix select of 11 + 10 + 10 bits: every CTA histograms its keys in shared
+//   memory, adds the non-empty bins to the first CTA's over distributed shared memory, and that CTA chooses.  (Every
+//   CTA adding up all the histograms for itself was bound by those reads: 36 us with eight CTAs, 72 us with sixteen.)
+//   Keys above the threshold, and the lowest positions among the equal ones, are written in order; a warp owns a
+//   contiguous piece, and two counts per warp and CTA give it its place.
+// What bounds it: dependent rounds over on-chip memory, a cluster barrier or two each.  As separate launches over all
+// SMs (pool, four 8-bit histograms, count, compact) the 8 x 131072 keys of a prompt took 82 us under the profiler,
+// this 22 us (four CTAs per unit: 30).
 // ------------------------------------------------------------------------------------------------
-constexpr int kSelChunk = 4096;
-constexpr int kSelThreads = 256;
-constexpr int kSelPerThread = kSelChunk / kSelThreads;
+constexpr int kSelThreads = 1024;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelCluster = 8;
+constexpr int kVoteTile = 4 * kSelThreads; // raw votes staged at a time
+constexpr int kVoteHalo = 256;             // widest pooling half that is staged
+constexpr int kKeyCap = 36864;             // keys a CTA keeps in shared memory at most
 
-struct SelState { unsigned prefix, mask; int need; };
+// keys of one CTA for a prefix of P tokens (a multiple of the CTA's threads)
+__host__ __device__ inline int select_share(int P) { return (P + kSelCluster * kSelThreads - 1) / (kSelCluster * kSelThreads) * kSelThreads; }
 
-// Replays the first `passes` picks from the unit's histograms ([4][256]).  One full warp.
-__device__ __forceinline__ SelState select_state(const int* hist, int passes, int k, int lane)
+// The bin (counted from the largest) that holds the need-th largest key, and the rank left inside it: v[] are the
+// cluster's counts of this thread's kPer consecutive bins, largest bin first.
+template <int kPer>
+__device__ __forceinline__ void pick_bin(const int (&v)[kPer], int need, int tid, int* warp_sum, int* out)
 {
-    SelState s;
-    s.prefix = 0u; s.mask = 0u; s.need = k;
-    for (int p = 0; p < passes; ++p) {
-        const int* hp = hist + p * 256;
-        const int shift = 24 - 8 * p;
-        int loc[8], sum = 0;                              // lane l: bins 255 - 8l, 254 - 8l, ... (descending)
+    const int lane = tid & 31, warp = tid >> 5;
+    int sum = 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { loc[i] = hp[255 - 8 * lane - i]; sum += loc[i]; }
-        int inc = sum;
+    for (int i = 0; i < kPer; ++i) sum += v[i];
+    int inc = sum;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int n = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += n; }
-        const unsigned cross = __ballot_sync(0xffffffffu, inc >= s.need);
-        const int src = cross ? __ffs(cross) - 1 : 31;   // lane whose bins contain the need-th largest key
-        int bin = 0, left = 0;
-        if (lane == src) {
-            int need = s.need - (inc - sum), i = 0;
-            for (; i < 7; ++i) { if (loc[i] >= need) break; need -= loc[i]; }
-            bin = 255 - 8 * lane - i;
-            left = need;
-        }
-        bin = __shfl_sync(0xffffffffu, bin, src);
-        left = __shfl_sync(0xffffffffu, left, src);
-        s.need = left;                                    // rank inside the chosen bin
-        s.prefix |= static_cast<unsigned>(bin) << shift;
-        s.mask |= 255u << shift;
-    }
-    return s;
-}
-
-template <int PASS>
-__global__ void __launch_bounds__(kSelThreads) evict_hist_kernel(EvictArgs A)
-{
-    grid_wait();
-    grid_release();
-    __shared__ int sh[256];
-    __shared__ SelState st;
-    const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-    const int S = min(A.seq_lens[b], A.S_max);
-    if (S <= A.budget) return;
-    const int P = S - A.W, k = A.budget - A.W, t0 = chunk * kSelChunk;
-    if (t0 >= P) return;
-    const int unit = b * A.Hkv + h, tid = threadIdx.x, lane = tid & 31;
-    int* hist = A.hist + static_cast<int64_t>(unit) * 1024;
-    sh[tid] = 0;
-    if (tid < 32) {
-        const SelState s = select_state(hist, PASS, k, lane);
-        if (lane == 0) st = s;
-    }
+    for (int o = 1; o < 32; o <<= 1) { const int n = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += n; }
+    if (lane == 31) warp_sum[warp] = inc;
     __syncthreads();
-    const unsigned prefix = st.prefix, mask = st.mask;
-    constexpr int shift = 24 - 8 * PASS;
-    const unsigned* pooled = A.pooled + static_cast<int64_t>(unit) * A.S_max;
-#pragma unroll 4
-    for (int i = 0; i < kSelPerThread; ++i) {              // whole warps iterate together (votes below)
-        const int t = t0 + i * kSelThreads + tid;
-        const unsigned key = t < P ? pooled[t] : 0u;
-        const bool in = t < P && (key & mask) == prefix;
-        const unsigned bin = (key >> shift) & 255u;
-        // lanes that hit the same bin add once: keys of neighbouring tokens mostly share their top bytes
-        const unsigned active = __ballot_sync(0xffffffffu, in);
-        if (in) {
-            const unsigned peers = __match_any_sync(active, bin);
-            if (lane == __ffs(peers) - 1) atomicAdd(&sh[bin], __popc(peers));
-        }
-    }
-    __syncthreads();
-    if (sh[tid]) atomicAdd(&hist[PASS * 256 + tid], sh[tid]);
-}
-
-// counts[unit][chunk] = (keys above the threshold, keys equal to it) in the chunk
-__global__ void __launch_bounds__(kSelThreads) evict_count_kernel(EvictArgs A)
-{
-    grid_wait();
-    grid_release();
-    __shared__ SelState st;
-    __shared__ int red[2][kSelThreads / 32];
-    const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-    const int S = min(A.seq_lens[b], A.S_max);
-    if (S <= A.budget) return;
-    const int P = S - A.W, k = A.budget - A.W, t0 = chunk * kSelChunk;
-    if (t0 >= P) return;
-    const int unit = b * A.Hkv + h, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < 32) {
-        const SelState s = select_state(A.hist + static_cast<int64_t>(unit) * 1024, 4, k, lane);
-        if (lane == 0) st = s;
-    }
-    __syncthreads();
-    const unsigned thr = st.prefix;
-    const unsigned* pooled = A.pooled + static_cast<int64_t>(unit) * A.S_max;
-    int gt = 0, eq = 0;
-#pragma unroll 4
-    for (int i = 0; i < kSelPerThread; ++i) {
-        const int t = t0 + i * kSelThreads + tid;
-        if (t < P) { const unsigned key = pooled[t]; gt += key > thr; eq += key == thr; }
-    }
-    gt = __reduce_add_sync(0xffffffffu, gt);
-    eq = __reduce_add_sync(0xffffffffu, eq);
-    if (lane == 0) { red[0][warp] = gt; red[1][warp] = eq; }
-    __syncthreads();
-    if (tid == 0) {
-        int g = 0, e = 0;
-        for (int w = 0; w < kSelThreads / 32; ++w) { g += red[0][w]; e += red[1][w]; }
-        int* c = A.counts + (static_cast<int64_t>(unit) * A.n_chunks + chunk) * 2;
-        c[0] = g; c[1] = e;
+    int before = __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum[lane] : 0) + inc - sum;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        if (before < need && need <= before + v[i]) { out[0] = kPer * tid + i; out[1] = need - before; }
+        before += v[i];
     }
 }
 
-// Ordered compaction: thread i of the chunk's CTA owns 16 consecutive tokens.  Also publishes packed_lens
-// and handles sequences that are kept whole.
-__global__ void __launch_bounds__(kSelThreads) evict_compact_kernel(EvictArgs A)
+__global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads) evict_select_kernel(EvictArgs A)
 {
-    grid_wait();
-    grid_release();
-    __shared__ SelState st;
-    __shared__ int s_base_kept, s_base_eq;
-    __shared__ int scan_eq[kSelThreads / 32], scan_keep[kSelThreads / 32];
-    const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+    extern __shared__ __align__(16) unsigned key_smem[];
+    __shared__ int hist[2048 + 1024 + 1024], sums[2048 + 1024 + 1024];      // own counts; first CTA: the other CTAs'
+    __shared__ int warp_sum[kSelWarps], warp_gt[kSelWarps], warp_eq[kSelWarps], total[2], pick[2];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = static_cast<int>(cluster.block_rank()), h = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* raw = reinterpret_cast<float*>(key_smem + A.key_cap);              // [kVoteTile + 2 * kVoteHalo]
+    for (int i = tid; i < 4096; i += kSelThreads) hist[i] = sums[i] = 0;
+    grid_wait();
+    grid_release();
     int S = A.seq_lens[b];
     if (S < 0 || S > A.S_max) {
-        if (chunk == 0 && tid == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+        if (rank == 0 && tid == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
         S = S < 0 ? 0 : A.S_max;
     }
     const int unit = b * A.Hkv + h;
     int32_t* kept = A.kept + static_cast<int64_t>(unit) * A.budget;
-    if (chunk == 0 && h == 0 && tid == 0) A.packed_lens[b] = S < A.budget ? S : A.budget;
-    if (S <= A.budget) {                                  // kept whole
-        for (int t = chunk * kSelChunk + tid; t < min(A.budget, (chunk + 1) * kSelChunk); t += kSelThreads)
-            kept[t] = t < S ? t : -1;
-        if (chunk == 0)                                   // budget beyond the chunked range (short max_seq_tokens)
-            for (int t = A.n_chunks * kSelChunk + tid; t < A.budget; t += kSelThreads) kept[t] = t < S ? t : -1;
+    if (rank == 0 && h == 0 && tid == 0) A.packed_lens[b] = S < A.budget ? S : A.budget;
+    if (S <= A.budget) {                                       // kept whole (the same in every CTA of the cluster)
+        for (int t = rank * kSelThreads + tid; t < A.budget; t += kSelCluster * kSelThreads) kept[t] = t < S ? t : -1;
         return;
     }
-    const int P = S - A.W, k = A.budget - A.W, t0 = chunk * kSelChunk;
-    if (chunk == 0)
+    const int P = S - A.W, k = A.budget - A.W, half = (A.pool - 1) / 2;
+    if (rank == 0)
         for (int w = tid; w < A.W; w += kSelThreads) kept[k + w] = P + w;
-    if (t0 >= P) return;
-    if (tid < 32) {
-        const SelState s = select_state(A.hist + static_cast<int64_t>(unit) * 1024, 4, k, lane);
-        if (lane == 0) {
-            st = s;
-            // position of this chunk's first kept token and number of equal keys before the chunk
-            const int* c = A.counts + static_cast<int64_t>(unit) * A.n_chunks * 2;
-            int base_kept = 0, base_eq = 0;
-            for (int cc = 0; cc < chunk; ++cc) {
-                const int take = min(c[2 * cc + 1], max(0, s.need - base_eq));
-                base_kept += c[2 * cc] + take;
-                base_eq += c[2 * cc + 1];
+    if (k == 0) return;                                        // the window alone
+    const int share = select_share(P), c0 = rank * share;
+    const int n = max(0, min(share, P - c0));                  // this CTA's keys: tokens c0 .. c0 + n - 1
+    const int64_t base = static_cast<int64_t>(unit) * A.S_max;
+    unsigned* keys = share <= A.key_cap ? key_smem : A.pooled + base + c0;
+    const float* votes = A.votes + base;
+    cluster.barrier_arrive();                                  // (waited for before the first CTA's sums, zeroed above, are added to)
+    __syncthreads();
+    // The raw votes come through a staging tile (with the pooling halo), the next tile's loads in flight while one is
+    // pooled; very wide pools read the votes from memory.  A thread pools four neighbours; pooled neighbours are
+    // mostly equal, so it counts runs of equal bins and most of the four cost no atomic of their own.
+    const bool staged = half <= kVoteHalo;
+    const int lead = staged ? half : 0;
+    float next[kVoteTile / kSelThreads + 1];
+    auto load_tile = [&](int i0) {
+#pragma unroll
+        for (int u = 0; u <= kVoteTile / kSelThreads; ++u) {
+            const int x = u * kSelThreads + tid, t = c0 + i0 - lead + x;
+            next[u] = (x < kVoteTile + 2 * lead && t >= 0 && t < P) ? votes[t] : 0.f;      // votes are >= 0
+        }
+    };
+    load_tile(0);
+    for (int i0 = 0; i0 < share; i0 += kVoteTile) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u <= kVoteTile / kSelThreads; ++u) {
+            const int x = u * kSelThreads + tid;
+            if (x < kVoteTile + 2 * lead) raw[x] = next[u];
+        }
+        __syncthreads();
+        if (i0 + kVoteTile < share) load_tile(i0 + kVoteTile);
+        const int x = 4 * tid, i = i0 + x;
+        if (i < n) {
+            float m[4];
+            if (half == 3) {
+                const float4 r0 = *reinterpret_cast<const float4*>(raw + x), r1 = *reinterpret_cast<const float4*>(raw + x + 4);
+                const float2 r2 = *reinterpret_cast<const float2*>(raw + x + 8);
+                const float mid = fmaxf(fmaxf(r0.w, r1.x), fmaxf(r1.y, r1.z));           // in all four windows
+                const float yz = fmaxf(r0.y, r0.z), ab = fmaxf(r1.w, r2.x);
+                m[0] = fmaxf(mid, fmaxf(r0.x, yz));
+                m[1] = fmaxf(mid, fmaxf(yz, r1.w));
+                m[2] = fmaxf(mid, fmaxf(r0.z, ab));
+                m[3] = fmaxf(mid, fmaxf(ab, r2.y));
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    m[e] = raw[x + e + lead];
+                    if (staged) {
+                        for (int u = 0; u <= 2 * half; ++u) m[e] = fmaxf(m[e], raw[x + e + u]);
+                    } else {
+                        for (int u = max(0, c0 + i + e - half); u <= min(P - 1, c0 + i + e + half); ++u) m[e] = fmaxf(m[e], votes[u]);
+                    }
+                }
             }
-            s_base_kept = base_kept; s_base_eq = base_eq;
+            int run = 0, bin = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (i + e < n) {
+                    const unsigned key = __float_as_uint(m[e]);
+                    keys[i + e] = key;
+                    const int bn = (key >> 20) & 2047u;
+                    if (run && bn != bin) { atomicAdd(&hist[bin], run); run = 0; }
+                    bin = bn;
+                    ++run;
+                }
+            }
+            atomicAdd(&hist[bin], run);
         }
     }
-    __syncthreads();
-    const unsigned thr = st.prefix;
-    const int need_eq = st.need;
-    const unsigned* pooled = A.pooled + static_cast<int64_t>(unit) * A.S_max;
-    const int tb = t0 + tid * kSelPerThread;
-    unsigned key[kSelPerThread];
-    int eq_cnt = 0;
+    // One pass of the radix select over the bins hp (this CTA) and sum (first CTA): x the chosen bin, y the rank inside it
+    auto choose = [&](int* hp, int* sum, auto per, int want, bool first) {
+        constexpr int kPer = decltype(per)::value, kBins = kPer * kSelThreads;
+        __syncthreads();
+        if (first) cluster.barrier_wait();
+        if (rank > 0) {
+            int* to = cluster.map_shared_rank(sum, 0);
 #pragma unroll
-    for (int i = 0; i < kSelPerThread; ++i) {
-        key[i] = (tb + i < P) ? pooled[tb + i] : 0u;
-        eq_cnt += (tb + i < P && key[i] == thr) ? 1 : 0;
-    }
-    // exclusive scan of eq_cnt over the CTA's threads (threads are in position order)
-    int v = eq_cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const int n = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += n; }
-    if (lane == 31) scan_eq[warp] = v;
-    __syncthreads();
-    int eq_rank = s_base_eq + v - eq_cnt;
-    for (int w = 0; w < warp; ++w) eq_rank += scan_eq[w];
-    unsigned keep_bits = 0u;
-    int keep_cnt = 0;
-#pragma unroll
-    for (int i = 0; i < kSelPerThread; ++i) {
-        const bool live = tb + i < P;
-        const bool eq = live && key[i] == thr;
-        const bool keep = live && (key[i] > thr || (eq && eq_rank < need_eq));
-        eq_rank += eq ? 1 : 0;
-        keep_bits |= keep ? (1u << i) : 0u;
-        keep_cnt += keep ? 1 : 0;
-    }
-    int u = keep_cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const int n = __shfl_up_sync(0xffffffffu, u, o); if (lane >= o) u += n; }
-    if (lane == 31) scan_keep[warp] = u;
-    __syncthreads();
-    int pos = s_base_kept + u - keep_cnt;
-    for (int w = 0; w < warp; ++w) pos += scan_keep[w];
-#pragma unroll
-    for (int i = 0; i < kSelPerThread; ++i)
-        if ((keep_bits >> i) & 1u) {
-            if (pos < k) kept[pos] = tb + i;
-            ++pos;
+            for (int u = 0; u < kPer; ++u) {
+                const int c = hp[u * kSelThreads + tid];
+                if (c) atomicAdd(to + u * kSelThreads + tid, c);
+            }
         }
-    // the thread that owns the last prefix token sees the total
-    if (tb <= P - 1 && P - 1 < tb + kSelPerThread && pos != k) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+        cluster.sync();
+        if (rank == 0) {
+            int v[kPer];
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                const int bin = kBins - 1 - (kPer * tid + u);
+                v[u] = hp[bin] + sum[bin];
+            }
+            pick_bin<kPer>(v, want, tid, warp_sum, pick);
+        }
+        cluster.sync();
+        const int* choice = cluster.map_shared_rank(pick, 0);
+        return make_int2(kBins - 1 - choice[0], choice[1]);
+    };
+    int2 c = choose(hist, sums, std::integral_constant<int, 2>(), k, true);
+    unsigned thr = static_cast<unsigned>(c.x) << 20;
+    int need = c.y;
+#pragma unroll 1
+    for (int pass = 1; pass < 3; ++pass) {
+        const int shift = pass == 1 ? 10 : 0;
+        int* hp = hist + 1024 + 1024 * pass;
+        const unsigned top = thr >> (shift + 10);
+#pragma unroll 4
+        for (int i = tid; i < n; i += kSelThreads) {
+            const unsigned key = keys[i];
+            if ((key >> (shift + 10)) == top) atomicAdd(&hp[(key >> shift) & 1023u], 1);
+        }
+        c = choose(hp, sums + 1024 + 1024 * pass, std::integral_constant<int, 1>(), need, false);
+        thr |= static_cast<unsigned>(c.x) << shift;
+        need = c.y;
+    }
+    // keys above / equal to the threshold, per warp (a contiguous piece each) and per CTA
+    const int seg = share / kSelWarps, s0 = warp * seg;
+    int gt = 0, eq = 0;
+#pragma unroll 4
+    for (int i = s0 + lane; i < s0 + seg; i += 32) {
+        const unsigned key = i < n ? keys[i] : 0u;
+        gt += i < n && key > thr;
+        eq += i < n && key == thr;
+    }
+    gt = __reduce_add_sync(0xffffffffu, gt);
+    eq = __reduce_add_sync(0xffffffffu, eq);
+    if (lane == 0) { warp_gt[warp] = gt; warp_eq[warp] = eq; }
+    __syncthreads();
+    int b_gt = __reduce_add_sync(0xffffffffu, lane < warp ? warp_gt[lane] : 0);        // before this warp's piece
+    int b_eq = __reduce_add_sync(0xffffffffu, lane < warp ? warp_eq[lane] : 0);
+    if (tid == kSelThreads - 1) { total[0] = b_gt + gt; total[1] = b_eq + eq; }
+    cluster.sync();
+    int own_gt = 0;
+    for (int r = 0; r < rank; ++r) {
+        const int* t = cluster.map_shared_rank(total, r);
+        own_gt += t[0]; b_eq += t[1];
+    }
+    if (rank == kSelCluster - 1 && tid == 0 && own_gt + total[0] + need != k) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+    b_gt += own_gt;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int i0 = s0; i0 < s0 + seg && i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const unsigned key = i < n ? keys[i] : 0u;
+        const unsigned mg = __ballot_sync(0xffffffffu, i < n && key > thr), me = __ballot_sync(0xffffffffu, i < n && key == thr);
+        const int eq_rank = b_eq + __popc(me & lt);            // equal keys on lower positions
+        const int pos = b_gt + __popc(mg & lt) + min(eq_rank, need);
+        if (((mg >> lane) & 1u) || (((me >> lane) & 1u) && eq_rank < need)) {
+            if (pos < k) kept[pos] = c0 + i;
+        }
+        b_gt += __popc(mg);
+        b_eq += __popc(me);
+    }
+    cluster.sync();                                            // the others may still be reading this CTA's totals
 }
 
 bool evict_tc_supported(const spark_params& p);
 spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
                                    int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* partial,
-                                   float* rowstat, float* votes, int* status, cudaStream_t stream, int* launches);
+                                   float* votes, int* status, cudaStream_t stream, int* launches);
 
 size_t evict_workspace_bytes(const spark_params& p, int64_t max_seq_tokens)
 {
@@ -443,8 +431,6 @@ size_t evict_workspace_bytes(const spark_params& p, int64_t max_seq_tokens)
     size_t bytes = units * R * tiles * 2 * sizeof(float);
     bytes += units * R * 2 * sizeof(float);
     bytes += 2 * units * static_cast<size_t>(max_seq_tokens) * sizeof(float);      // votes, pooled keys
-    const size_t chunks = (max_seq_tokens + kSelChunk - 1) / kSelChunk;
-    bytes += units * (1024 + 2 * (chunks ? chunks : 1)) * sizeof(int);             // select histograms, chunk counts
     return (bytes + 255) / 256 * 256;
 }
 
@@ -464,17 +450,13 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     A.rowstat = A.partial + units * R * A.n_tiles * 2;
     A.votes = A.rowstat + units * R * 2;
     A.pooled = reinterpret_cast<unsigned*>(A.votes + units * static_cast<size_t>(max_seq_tokens));
-    A.hist = reinterpret_cast<int*>(A.pooled + units * static_cast<size_t>(max_seq_tokens));
-    A.counts = A.hist + units * 1024;
-    A.n_chunks = (max_seq_tokens + kSelChunk - 1) / kSelChunk;
-    if (A.n_chunks < 1) A.n_chunks = 1;
     A.kept = kept_tokens; A.packed_lens = packed_lens;
     const size_t smem = (static_cast<size_t>(kEvTile + kEvRows) * kEvStride + kEvTile) * sizeof(float);
     const dim3 grid(A.n_tiles, p.n_kv_heads, p.batch), ugrid(p.n_kv_heads, p.batch);
     const bool bf16 = p.dtype == SPARK_BF16;
     if (A.n_tiles > 0 && max_seq_tokens > p.token_budget && evict_tc_supported(p)) {
         const spark_status st_tc = launch_evict_votes_tc(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, A.partial,
-                                                         A.rowstat, A.votes, A.status, stream, launches);
+                                                         A.votes, A.status, stream, launches);
         if (st_tc != SPARK_OK) return st_tc;
     } else if (A.n_tiles > 0 && max_seq_tokens > p.token_budget) {
         cudaError_t e1 = bf16 ? cudaFuncSetAttribute(evict_scores_kernel<__nv_bfloat16, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
@@ -489,17 +471,12 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
         else launch_kernel(evict_scores_kernel<float, 2>, grid, dim3(kEvThreads), smem, stream, A);
         *launches += 3;
     }
-    const dim3 sgrid(A.n_chunks, p.n_kv_heads, p.batch);
-    if (max_seq_tokens > p.token_budget) {
-        launch_kernel(evict_pool_kernel, dim3((max_seq_tokens + 255) / 256, p.n_kv_heads, p.batch), dim3(256), 0, stream, A);
-        launch_kernel(evict_hist_kernel<0>, sgrid, dim3(kSelThreads), 0, stream, A);
-        launch_kernel(evict_hist_kernel<1>, sgrid, dim3(kSelThreads), 0, stream, A);
-        launch_kernel(evict_hist_kernel<2>, sgrid, dim3(kSelThreads), 0, stream, A);
-        launch_kernel(evict_hist_kernel<3>, sgrid, dim3(kSelThreads), 0, stream, A);
-        launch_kernel(evict_count_kernel, sgrid, dim3(kSelThreads), 0, stream, A);
-        *launches += 6;
-    }
-    launch_kernel(evict_compact_kernel, sgrid, dim3(kSelThreads), 0, stream, A);
+    const int most = select_share(max_seq_tokens > p.window ? max_seq_tokens - p.window : 1);
+    A.key_cap = most < kKeyCap ? most : kKeyCap;
+    const size_t key_bytes = (static_cast<size_t>(A.key_cap) + kVoteTile + 2 * kVoteHalo) * sizeof(unsigned);
+    if (cudaFuncSetAttribute(evict_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(key_bytes)) != cudaSuccess)
+        return SPARK_ERR_CUDA;
+    launch_kernel(evict_select_kernel, dim3(kSelCluster, p.n_kv_heads, p.batch), dim3(kSelThreads), key_bytes, stream, A);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }
