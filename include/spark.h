@@ -278,6 +278,39 @@ spark_status spark_decode_attn(const spark_params *p, const void *q,
                                void *workspace, size_t workspace_bytes, spark_stream_t stream);
 
 /*
+ * spark_append_dense -- one new token per sequence into a DENSE tail (Sec. "Preliminaries": K <- Cat[K, k], keys as they
+ * are).  The tail is a packed cache of its own with keep = head_dim, dense value rows and the degenerate recovery (anything
+ * else: SPARK_ERR_UNSUPPORTED); its pages receive what spark_append would write, and the token's key and value also go to
+ * row packed_lens[b] of k_tail / v_tail, from where spark_append_block can take them into the pruned prefix and
+ * spark_decode_attn_tail reads them.
+ *   k_tail, v_tail   IN/OUT [B][Hkv][tail_tokens][D], dtype as the cache, 16-byte aligned
+ *   every other argument as for spark_append; a sequence whose tail holds tail_tokens tokens (or has no page left) is left
+ *   unchanged and SPARK_ERR_DEVICE_BOUNDS is recorded
+ */
+spark_status spark_append_dense(const spark_params *p, const void *k_new, const void *v_new,
+                                void *pages, const int32_t *block_table, int32_t max_blocks,
+                                void *k_tail, void *v_tail, int32_t tail_tokens, int32_t *packed_lens,
+                                void *workspace, size_t workspace_bytes, spark_stream_t stream);
+
+/*
+ * spark_decode_attn_tail -- one decode step over a pruned prefix (the packed cache of spark_decode_attn) and a dense tail of
+ * at most 128 tokens: the attention of Sec. "Preliminaries" over the union of the two token sets, merged by their
+ * log-sum-exp inside the prefix's step.
+ *   k_tail, v_tail   [B][Hkv][tail_tokens][D] as written by spark_append_dense; tail_tokens <= 128 (else
+ *                    SPARK_ERR_UNSUPPORTED: decode the tail with spark_decode_attn and use spark_merge_attn)
+ *   tail_lens        [B] int32 tokens in each tail
+ *   tail_out         scratch [B][Hq][D] fp32, 16-byte aligned;  tail_lse  scratch [B][Hq] fp32
+ *   out, lse         the merged result; every other argument as for spark_decode_attn
+ */
+spark_status spark_decode_attn_tail(const spark_params *p, const void *q,
+                                    const void *pages, const int32_t *block_table, int32_t max_blocks,
+                                    const int32_t *packed_lens, const float *qnorm,
+                                    const void *k_tail, const void *v_tail, int32_t tail_tokens,
+                                    const int32_t *tail_lens, float *tail_out, float *tail_lse,
+                                    float *out, float *lse,
+                                    void *workspace, size_t workspace_bytes, spark_stream_t stream);
+
+/*
  * spark_decode_attn_host -- the same decode step for a caller whose query and result live in HOST memory
  * (Sec. "Channel Recovery" / "Preliminaries" as above; only the transport differs).  Enqueues, in this order
  * on `stream`: the copy of q_host to q_dev, spark_decode_attn on q_dev, the copy of out_dev to out_host (and

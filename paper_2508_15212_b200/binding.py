@@ -22,7 +22,8 @@ SPARK_F32, SPARK_BF16 = 0, 1
 _DTYPE_CODE = {torch.float32: SPARK_F32, torch.bfloat16: SPARK_BF16}
 EXPORTS = ["spark_version", "spark_last_launch_count", "spark_keep_count", "spark_page_bytes", "spark_pool_bytes",
            "spark_algorithmic_bytes_per_token", "spark_workspace_bytes", "spark_workspace_init",
-           "spark_compress", "spark_append", "spark_append_block", "spark_merge_attn", "spark_decode_attn", "spark_decode_attn_host", "spark_decode_attn_noalloc", "spark_unpack_pages",
+           "spark_compress", "spark_append", "spark_append_block", "spark_append_dense", "spark_decode_attn_tail", "spark_merge_attn",
+           "spark_decode_attn", "spark_decode_attn_host", "spark_decode_attn_noalloc", "spark_unpack_pages",
            "spark_unpack_value_masks", "spark_unpack_stats", "spark_group_keep", "spark_read_status"]
 
 
@@ -81,6 +82,10 @@ def lib() -> ctypes.CDLL:
         L.spark_append.argtypes = [P, vp, vp, vp, vp, i32, vp, vp, vp, sz, vp]
         L.spark_append_block.restype = i32
         L.spark_append_block.argtypes = [P, vp, vp, i32, vp, vp, i32, vp, vp, vp, sz, vp]
+        L.spark_append_dense.restype = i32
+        L.spark_append_dense.argtypes = [P, vp, vp, vp, vp, i32, vp, vp, i32, vp, vp, sz, vp]
+        L.spark_decode_attn_tail.restype = i32
+        L.spark_decode_attn_tail.argtypes = [P, vp, vp, vp, i32, vp, vp, vp, vp, i32, vp, vp, vp, vp, vp, vp, sz, vp]
         L.spark_merge_attn.restype = i32
         L.spark_merge_attn.argtypes = [i32, i32, i32, vp, vp, vp, vp, vp, vp, vp]
         L.spark_decode_attn.restype = i32
@@ -229,6 +234,35 @@ def spark_decode_attn(p: spark_params, q, pages, block_table, packed_lens, qnorm
                                    _blocks(block_table, max_blocks), _ptr(packed_lens), _ptr(qnorm), _ptr(out), _ptr(lse),
                                    _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
            "spark_decode_attn")
+
+
+def spark_append_dense(p: spark_params, k_new, v_new, pages, block_table, k_tail, v_tail, packed_lens, workspace,
+                       max_blocks=None) -> None:
+    """One new token per sequence into a dense tail: its pages and the rows k_tail, v_tail [B, Hkv, tail_tokens, D]."""
+    assert k_new.is_contiguous() and v_new.is_contiguous()
+    _check(lib().spark_append_dense(ctypes.byref(p), k_new.data_ptr(), v_new.data_ptr(), pages.data_ptr(),
+                                    None if block_table is None else block_table.data_ptr(), _blocks(block_table, max_blocks),
+                                    k_tail.data_ptr(), v_tail.data_ptr(), k_tail.shape[2], packed_lens.data_ptr(),
+                                    workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+                                    torch.cuda.current_stream().cuda_stream),
+           "spark_append_dense")
+
+
+def spark_decode_attn_tail(p: spark_params, q, pages, block_table, packed_lens, qnorm, k_tail, v_tail, tail_lens, tail_out,
+                           tail_lse, out, lse, workspace, max_blocks=None) -> None:
+    """Decode step over a pruned prefix and a dense tail of at most TAIL_MAX tokens."""
+    _check(lib().spark_decode_attn_tail(ctypes.byref(p), q.data_ptr(), pages.data_ptr(),
+                                        None if block_table is None else block_table.data_ptr(),
+                                        _blocks(block_table, max_blocks), packed_lens.data_ptr(), qnorm.data_ptr(),
+                                        k_tail.data_ptr(), v_tail.data_ptr(), k_tail.shape[2], tail_lens.data_ptr(),
+                                        tail_out.data_ptr(), tail_lse.data_ptr(), out.data_ptr(),
+                                        None if lse is None else lse.data_ptr(), workspace.data_ptr(),
+                                        workspace.numel() * workspace.element_size(),
+                                        torch.cuda.current_stream().cuda_stream),
+           "spark_decode_attn_tail")
+
+
+TAIL_MAX = 128              # tokens of a dense tail that spark_decode_attn_tail takes
 
 
 class BoundDecodeHost:

@@ -170,8 +170,8 @@ class DenseTailCache:
     pages keep all 128 channels; every `tail_block` appended tokens the dense copies that this object also keeps
     are handed to the prefix in one spark_append_block call (pruned with the prefill statistics) and the tail
     starts over.  `tail_block=None` never hands them over: the literal "dense appended keys".  A decode step is
-    the prefix step, the tail step and their log-sum-exp merge (spark_merge_attn); all arithmetic is in the
-    library.
+    the tail step and the prefix step, merged by log-sum-exp (spark_decode_attn_tail; spark_merge_attn for tails of more
+    than 128 tokens); all arithmetic is in the library.
     """
 
     def __init__(self, *, batch: int, n_q_heads: int, n_kv_heads: int, window: int, keep: int, dtype: str,
@@ -189,6 +189,7 @@ class DenseTailCache:
         p = self.prefix.params
         self._o = [torch.empty(p.batch, p.n_q_heads, 128, dtype=torch.float32, device=device) for _ in range(2)]
         self._l = [torch.empty(p.batch, p.n_q_heads, dtype=torch.float32, device=device) for _ in range(2)]
+        self._short = cap <= B.TAIL_MAX
 
     def compress(self, q_win, k, v, seq_lens) -> None:
         self.prefix.compress(q_win, k, v, seq_lens)
@@ -198,9 +199,11 @@ class DenseTailCache:
 
     def append(self, k_new, v_new) -> None:
         """One new token per sequence ([B, Hkv, D]); it stays dense until its block is handed to the prefix."""
-        self.tail.append(k_new, v_new)
-        self.k_tail[:, :, self.n_tail].copy_(k_new)
-        self.v_tail[:, :, self.n_tail].copy_(v_new)
+        if self.n_tail >= self.k_tail.shape[2]:
+            raise IndexError(f"the dense tail holds {self.n_tail} tokens and has no room for another")
+        t = self.tail
+        B.spark_append_dense(t.params, k_new, v_new, t.pages, t.block_table, self.k_tail, self.v_tail, t.packed_lens,
+                             t.ws_compress, max_blocks=t.table_blocks)
         self.n_tail += 1
         if self.block and self.n_tail == self.block:
             self.prefix.append_block(self.k_tail, self.v_tail)
@@ -210,6 +213,12 @@ class DenseTailCache:
     def decode(self, q, out: Optional[torch.Tensor] = None, lse: Optional[torch.Tensor] = None):
         if out is None:
             out = torch.empty_like(self._o[0])
+        if self._short:                                    # a short tail: two launches, merged in the prefix's step
+            p = self.prefix
+            B.spark_decode_attn_tail(p.params, q, p.pages, p.block_table, p.packed_lens, p.qnorm, self.k_tail, self.v_tail,
+                                     self.tail.packed_lens, self._o[1], self._l[1], out, lse, p.ws_decode,
+                                     max_blocks=p.table_blocks)
+            return out
         self.prefix.decode(q, out=self._o[0], lse=self._l[0])
         self.tail.decode(q, out=self._o[1], lse=self._l[1])
         B.spark_merge_attn(self._o[0], self._l[0], self._o[1], self._l[1], out, lse)

@@ -201,6 +201,60 @@ spark_status spark_append_block(const spark_params* p, const void* k_new, const 
     return st;
 }
 
+spark_status spark_append_dense(const spark_params* p, const void* k_new, const void* v_new, void* pages,
+                                const int32_t* block_table, int32_t max_blocks, void* k_tail, void* v_tail,
+                                int32_t tail_tokens, int32_t* packed_lens, void* workspace, size_t workspace_bytes,
+                                spark_stream_t stream)
+{
+    spark_status st = check_params(p);
+    if (st != SPARK_OK) return st;
+    if (!k_new || !v_new || !pages || !k_tail || !v_tail || !packed_lens || !workspace) return SPARK_ERR_NULL;
+    if (p->keep != kHeadDim || value_keep(p->keep_v) != kHeadDim || p->select != SPARK_SELECT_FIXED ||
+        p->recovery != SPARK_RECOVER_DEGENERATE)
+        return SPARK_ERR_UNSUPPORTED;
+    if (max_blocks < 1 || max_blocks > kMaxBlocksArg || tail_tokens < 1) return SPARK_ERR_BAD_SHAPE;
+    if (contiguous_pool_too_small(p, block_table, max_blocks)) return SPARK_ERR_BAD_SHAPE;
+    if (misaligned(pages, 16) || misaligned(k_new, 16) || misaligned(v_new, 16) || misaligned(k_tail, 16) || misaligned(v_tail, 16))
+        return SPARK_ERR_BAD_SHAPE;
+    if ((reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < kWorkspaceHeader) return SPARK_ERR_WORKSPACE;
+    int launches = 0;
+    st = launch_append_dense(*p, k_new, v_new, pages, block_table, max_blocks, k_tail, v_tail, tail_tokens, packed_lens, workspace,
+                             static_cast<cudaStream_t>(stream), &launches);
+    if (st == SPARK_OK) g_last_launches = launches;
+    return st;
+}
+
+spark_status spark_decode_attn_tail(const spark_params* p, const void* q, const void* pages, const int32_t* block_table,
+                                    int32_t max_blocks, const int32_t* packed_lens, const float* qnorm, const void* k_tail,
+                                    const void* v_tail, int32_t tail_tokens, const int32_t* tail_lens, float* tail_out,
+                                    float* tail_lse, float* out, float* lse, void* workspace, size_t workspace_bytes,
+                                    spark_stream_t stream)
+{
+    spark_status st = check_params(p);
+    if (st != SPARK_OK) return st;
+    if (!q || !pages || !packed_lens || !qnorm || !k_tail || !v_tail || !tail_lens || !tail_out || !tail_lse || !out || !workspace)
+        return SPARK_ERR_NULL;
+    if (max_blocks < 0 || max_blocks > kMaxBlocksArg || tail_tokens < 1) return SPARK_ERR_BAD_SHAPE;
+    if (tail_tokens > kTailMax) return SPARK_ERR_UNSUPPORTED;
+    if (contiguous_pool_too_small(p, block_table, max_blocks)) return SPARK_ERR_BAD_SHAPE;
+    if (misaligned(pages, 16) || misaligned(q, 16) || misaligned(qnorm, 16) || misaligned(out, 16) || misaligned(lse, 4) ||
+        misaligned(k_tail, 16) || misaligned(v_tail, 16) || misaligned(tail_out, 16) || misaligned(tail_lse, 4))
+        return SPARK_ERR_BAD_SHAPE;
+    if ((reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < decode_workspace_bytes(*p))
+        return SPARK_ERR_WORKSPACE;
+    int launches = 0;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    st = launch_tail_attn(*p, q, k_tail, v_tail, tail_tokens, tail_lens, tail_out, tail_lse, s, &launches);
+    if (st != SPARK_OK) return st;
+    // the step's predecessor is the tail kernel, which writes nothing of the packed cache: its pages may stream meanwhile
+    spark_params over = *p;
+    over.flags |= SPARK_FLAG_OVERLAP_PREVIOUS;
+    st = launch_decode(over, q, pages, block_table, max_blocks, packed_lens, qnorm, out, lse, workspace, workspace_bytes, s,
+                       &launches, false, tail_out, tail_lse);
+    if (st == SPARK_OK) g_last_launches = launches;
+    return st;
+}
+
 spark_status spark_merge_attn(int32_t batch, int32_t n_q_heads, int32_t head_dim, const float* out_a,
                               const float* lse_a, const float* out_b, const float* lse_b, float* out, float* lse,
                               spark_stream_t stream)

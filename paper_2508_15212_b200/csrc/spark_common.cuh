@@ -119,6 +119,15 @@ template <> struct Elem<__nv_bfloat16> {
     }
 };
 
+// four channels of a lane, and the type that sums the scores of a dense tail
+template <int ES> struct LaneVec;
+template <> struct LaneVec<2> { using type = uint2; };
+template <> struct LaneVec<4> { using type = uint4; };
+template <typename E> struct TailAcc;
+template <> struct TailAcc<float> { using type = double; };
+template <> struct TailAcc<__nv_bfloat16> { using type = float; };
+constexpr int kTailMax = 128;         // tokens of a dense tail that tail_attn_kernel takes
+
 // Programmatic dependent launch.  Every kernel of the library is launched so that it may become resident while the
 // kernel before it on the stream drains, and waits at its top, before it reads or writes anything of a caller's
 // (grid_wait: returns once that kernel has completed and its writes are visible; nothing to wait for under an
@@ -169,7 +178,9 @@ int group_keep(int head_dim, int n_groups, const float* prune);
 spark_status launch_decode(const spark_params& p, const void* q, const void* pages,
                            const int32_t* block_table, int32_t max_blocks, const int32_t* packed_lens,
                            const float* qnorm, float* out, float* lse, void* workspace,
-                           size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value = false);
+                           size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value = false,
+                           const float* other_out = nullptr, const float* other_lse = nullptr);
+// other_out / other_lse: attention over further tokens of the same sequences, merged into the result
 // q_by_value: q is a HOST pointer and its bytes travel as a launch parameter (bf16 storage, degenerate recovery,
 // dense value rows, at most query_by_value_limit() bytes; anything else is refused)
 size_t query_by_value_limit();
@@ -181,6 +192,11 @@ spark_status launch_append(const spark_params& p, const void* k_new, const void*
 spark_status launch_append_block(const spark_params& p, const void* k_new, const void* v_new, int32_t n_new,
                                  void* pages, const int32_t* block_table, int32_t max_blocks, const float* qnorm,
                                  int32_t* packed_lens, void* workspace, cudaStream_t stream, int* launches);
+spark_status launch_append_dense(const spark_params& p, const void* k_new, const void* v_new, void* pages,
+                                 const int32_t* block_table, int32_t max_blocks, void* k_tail, void* v_tail, int32_t cap,
+                                 int32_t* packed_lens, void* workspace, cudaStream_t stream, int* launches);
+spark_status launch_tail_attn(const spark_params& p, const void* q, const void* k_tail, const void* v_tail, int32_t cap,
+                              const int32_t* tail_lens, float* out, float* lse, cudaStream_t stream, int* launches);
 spark_status launch_merge_attn(int rows, const float* out_a, const float* lse_a, const float* out_b, const float* lse_b,
                                float* out, float* lse, cudaStream_t stream);
 

@@ -461,7 +461,8 @@ size_t query_by_value_limit() { return kMaxQueryByValueBytes; }
 spark_status launch_decode(const spark_params& p, const void* q, const void* pages,
                            const int32_t* block_table, int32_t max_blocks, const int32_t* packed_lens,
                            const float* qnorm, float* out, float* lse, void* workspace,
-                           size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value)
+                           size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value,
+                           const float* other_out, const float* other_lse)
 {
     (void)workspace_bytes;
     int dev = 0;
@@ -472,6 +473,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     DecodeArgs A;
     A.q = q; A.pages = static_cast<const unsigned char*>(pages); A.block_table = block_table;
     A.max_blocks = max_blocks; A.lens = packed_lens; A.qnorm = qnorm; A.out = out; A.lse = lse;
+    A.other_out = other_out; A.other_lse = other_lse;
     A.B = p.batch; A.Hq = p.n_q_heads; A.Hkv = p.n_kv_heads; A.n_pool_pages = p.n_pool_pages;
     A.L = make_layout(p);
     const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf(static_cast<float>(p.head_dim));

@@ -31,6 +31,8 @@ struct DecodeArgs {
     const float* qnorm;
     float* out;
     float* lse;
+    const float* other_out;                  // attention over further tokens of the same sequences (a dense tail), merged
+    const float* other_lse;                  // into the published result; null: none
     int B, Hq, Hkv;
     int64_t n_pool_pages;
     PageLayout L;
@@ -527,7 +529,7 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
     }
 }
 
-// zero-length sequences: out = 0, lse = -inf (consumer threads)
+// zero-length sequences: out = 0, lse = -inf, or the other token set's result (consumer threads)
 template <int NT>
 __device__ __forceinline__ void write_empty_sequences(const DecodeArgs& A, const int* prefix, int tid)
 {
@@ -536,11 +538,12 @@ __device__ __forceinline__ void write_empty_sequences(const DecodeArgs& A, const
         if (prefix[b + 1] == prefix[b]) {
 #pragma unroll 1
             for (int i = tid; i < A.Hq * kHeadDim; i += NT)
-                A.out[static_cast<int64_t>(b) * A.Hq * kHeadDim + i] = 0.f;
+                A.out[static_cast<int64_t>(b) * A.Hq * kHeadDim + i] =
+                    A.other_out ? A.other_out[static_cast<int64_t>(b) * A.Hq * kHeadDim + i] : 0.f;
             if (A.lse)
 #pragma unroll 1
                 for (int i = tid; i < A.Hq; i += NT)
-                    A.lse[static_cast<int64_t>(b) * A.Hq + i] = -INFINITY;
+                    A.lse[static_cast<int64_t>(b) * A.Hq + i] = A.other_lse ? A.other_lse[static_cast<int64_t>(b) * A.Hq + i] : -INFINITY;
         }
 }
 
@@ -578,6 +581,23 @@ __device__ __forceinline__ void describe_epoch(const DecodeArgs& A, const Ctrl& 
             C.units[e] = d;
         }
     }
+}
+
+// Factors of a row's unnormalised sum (running maximum M, running sum Ls) and of the other token set's output, and the
+// row's log-sum-exp (the identity of merge_attn_kernel).
+struct PublishWeights { float own, other, lse; };
+__device__ __forceinline__ PublishWeights publish_weights(const DecodeArgs& A, int64_t row, float M, float Ls)
+{
+    PublishWeights w;
+    w.own = 1.0f / Ls; w.other = 0.f; w.lse = (M + log2f(Ls)) * kLn2;
+    if (A.other_lse) {
+        const float lb = A.other_lse[row], m = fmaxf(w.lse, lb);
+        const float ea = expf(w.lse - m), eb = expf(lb - m), inv = 1.0f / (ea + eb);
+        w.own *= ea * inv;
+        w.other = eb * inv;
+        w.lse = m + logf(ea + eb);
+    }
+    return w;
 }
 
 // Merge the records of an epoch ([record][G][kRec]: 128 unnormalised outputs, m, l) unit by unit and publish
@@ -642,9 +662,14 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
         const float M = unit_ml[2 * pr], Ls = unit_ml[2 * pr + 1];
         const int64_t row = static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg;
         if (d.n_parts == 1) {
-            const float inv = 1.0f / Ls;
-            *reinterpret_cast<float2*>(A.out + row * kHeadDim + 2 * c2) = make_float2(O.x * inv, O.y * inv);
-            if (c2 == 0 && A.lse) A.lse[row] = (M + log2f(Ls)) * kLn2;
+            const PublishWeights pw = publish_weights(A, row, M, Ls);
+            O.x *= pw.own; O.y *= pw.own;
+            if (A.other_out) {
+                const float2 x = *reinterpret_cast<const float2*>(A.other_out + row * kHeadDim + 2 * c2);
+                O.x = fmaf(pw.other, x.x, O.x); O.y = fmaf(pw.other, x.y, O.y);
+            }
+            *reinterpret_cast<float2*>(A.out + row * kHeadDim + 2 * c2) = O;
+            if (c2 == 0 && A.lse) A.lse[row] = pw.lse;
         } else {
             float* part_out = A.partials + static_cast<int64_t>(blockIdx.x + d.b * A.Hkv + d.h) * G * kRec;
             *reinterpret_cast<float2*>(part_out + gg * kRec + 2 * c2) = O;
@@ -751,12 +776,16 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
                     }
             }
             if (ph == 0) {
-                const float M = pML[2 * gg], Ls = pML[2 * gg + 1];
-                const float inv = 1.0f / Ls;
-                *reinterpret_cast<float4*>(A.out + (static_cast<int64_t>(b) * A.Hq + h * G + gg) * kHeadDim + 4 * c4) =
-                    make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-                if (c4 == 0 && A.lse)
-                    A.lse[static_cast<int64_t>(b) * A.Hq + h * G + gg] = (M + log2f(Ls)) * kLn2;
+                const int64_t row = static_cast<int64_t>(b) * A.Hq + h * G + gg;
+                const PublishWeights w = publish_weights(A, row, pML[2 * gg], pML[2 * gg + 1]);
+                acc.x *= w.own; acc.y *= w.own; acc.z *= w.own; acc.w *= w.own;
+                if (A.other_out) {
+                    const float4 x = *reinterpret_cast<const float4*>(A.other_out + row * kHeadDim + 4 * c4);
+                    acc.x = fmaf(w.other, x.x, acc.x); acc.y = fmaf(w.other, x.y, acc.y);
+                    acc.z = fmaf(w.other, x.z, acc.z); acc.w = fmaf(w.other, x.w, acc.w);
+                }
+                *reinterpret_cast<float4*>(A.out + row * kHeadDim + 4 * c4) = acc;
+                if (c4 == 0 && A.lse) A.lse[row] = w.lse;
             }
             if (tid == 0) A.tickets[unit] = 0;          // ready for the next call
             consumer_sync<NT>();                        // the merge area is free for the next unit

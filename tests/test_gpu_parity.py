@@ -461,6 +461,43 @@ def test_dense_tail_equals_the_oracle_with_appended_keys_left_dense(dtype, block
             assert np.allclose(lse.cpu().numpy(), ref_lse, rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
 
 
+@pytest.mark.parametrize("G", [1, 4, 7, 8])
+@pytest.mark.parametrize("dtype,cap,n_tail", [("bf16", 64, 1), ("bf16", 64, 63), ("bf16", 128, 65), ("bf16", 128, 128), ("bf16", 5, 0),
+                                              ("f32", 128, 127), ("f32", 16, 16)])
+def test_short_dense_tail_equals_the_tail_cache_merged(G, dtype, cap, n_tail):
+    """spark_append_dense + spark_decode_attn_tail at the edges of the tail kernel (no token, one token, around 64, full),
+    with an empty prefix in the batch, against spark_append + two spark_decode_attn + spark_merge_attn.  Both sum the same
+    products in fp32 (scores of fp32 storage in double): they differ by rounding, within the bars to the oracle."""
+    wl = make(dtype, 3, 2 * G, 2, [300, 0, 40], 8, 64, seed=180 + G, sigma=1.0 if dtype == "bf16" else 0.5, gap=False)
+    a = SparkCache(batch=3, n_q_heads=2 * G, n_kv_heads=2, window=8, keep=64, dtype=dtype, max_tokens=300, guard=True)
+    a.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    tails = [SparkCache(batch=3, n_q_heads=2 * G, n_kv_heads=2, window=8, keep=128, dtype=dtype, max_tokens=cap, guard=True) for _ in range(2)]
+    k_tail, v_tail = (torch.zeros(3, 2, cap, 128, dtype=wl.k.dtype, device="cuda") for _ in range(2))
+    for t in tails:
+        t.qnorm.copy_(a.qnorm)
+    for i in range(n_tail):
+        kn, vn = wl.k[:, :, 299 - i].contiguous(), wl.v[:, :, 299 - i].contiguous()
+        tails[0].append(kn, vn)
+        B.spark_append_dense(tails[1].params, kn, vn, tails[1].pages, None, k_tail, v_tail, tails[1].packed_lens,
+                             tails[1].ws_compress, max_blocks=tails[1].table_blocks)
+    assert torch.equal(tails[0].packed_lens, tails[1].packed_lens)
+    assert torch.equal(tails[0].pages, tails[1].pages), "the tail's pages must hold what spark_append writes"
+    o, l = [a.alloc_out(), tails[0].alloc_out()], [a.alloc_lse(), tails[0].alloc_lse()]
+    a.decode(wl.q, out=o[0], lse=l[0])
+    tails[0].decode(wl.q, out=o[1], lse=l[1])
+    ref, ref_lse, out, lse = torch.empty_like(o[0]), torch.empty_like(l[0]), a.alloc_out(), a.alloc_lse()
+    B.spark_merge_attn(o[0], l[0], o[1], l[1], ref, ref_lse)
+    to, tl = tails[1].alloc_out(), tails[1].alloc_lse()
+    B.spark_decode_attn_tail(a.params, wl.q, a.pages, None, a.packed_lens, a.qnorm, k_tail, v_tail, tails[1].packed_lens, to, tl,
+                             out, lse, a.ws_decode, max_blocks=a.table_blocks)
+    assert a.status() == 0 and tails[1].status() == 0
+    assert a.broken_guards() == [] and tails[1].broken_guards() == []
+    assert float((out - ref).abs().max()) <= TOL[dtype]
+    fin = torch.isfinite(ref_lse)
+    assert torch.equal(torch.isneginf(lse), torch.isneginf(ref_lse))
+    assert torch.allclose(lse[fin], ref_lse[fin], rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_host_entry_point_staged_and_mapped_equal_the_device_call(dtype):
     """spark_decode_attn_host: query and result in page-locked host memory, with staging copies or (flag) with the
