@@ -693,6 +693,12 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 // ------------------------------------------------------------------------------------------------
 constexpr int kWarpPageWarps = 4;
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
+// SparK-p: the saliencies of a page (fp32), and over them, once read, mask | mu | slot rows
+__host__ __device__ inline int warp_topp_room(const PageLayout& L)
+{
+    const int image = L.v_off + L.keep * kPageTokens * 2, sal = kPageTokens * kHeadDim * 4;
+    return image > sal ? image : sal;
+}
 
 __device__ __forceinline__ unsigned bits_max2(unsigned a, unsigned b)          // bf16 pairs; a NaN wins
 {
@@ -882,16 +888,221 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
     }
 }
 
-template <bool kPV>
-__global__ void __launch_bounds__(kWarpPageWarps * 32, kPV ? 5 : 6) compress_pages_warp_kernel(CompressArgs A)
+// SparK-p for the same shape of work: the fewest most salient channels whose saliencies (summed in double) reach top_p of
+// the token's total, at least one and at most T.  The token's saliencies sit in `wsm` (fp32, 16 rows of 512 bytes, chunk c of
+// row p at c ^ (p & 7)); `image` (which may lie over `wsm`) receives slots, mask and mean like select_section.  Returns the
+// token's kept count.
+//   A threshold on the keys' upper halves is searched like the fixed rule's, but by the SUM of the keys at or above it, in
+//   fp32 until at most three keys can lie between the ends.  The sum above the upper end is then taken in double and
+//   must be below the goal (else the search is repeated in double), and the keys between are admitted one by one.
+//   About 10000 instructions for sixteen tokens, where a bitonic rank sort per token took 2100 for one: 8 heads x 8192 tokens
+//   172 -> 83 us.
+__device__ __forceinline__ double sum_ge(const unsigned char* wrow, int sw, int half, unsigned lo)        // keys >= lo, in double
+{
+    double s = 0.0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (x[e] >= lo) s += static_cast<double>(__uint_as_float(x[e]));
+    }
+    return s + __shfl_xor_sync(kFullMask, s, 16);
+}
+__device__ __forceinline__ float sum_ge_f32(const unsigned char* wrow, int sw, int half, unsigned lo)
+{
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+        if (v.x >= lo) s[0] += __uint_as_float(v.x);
+        if (v.y >= lo) s[1] += __uint_as_float(v.y);
+        if (v.z >= lo) s[2] += __uint_as_float(v.z);
+        if (v.w >= lo) s[3] += __uint_as_float(v.w);
+    }
+    const float t = (s[0] + s[1]) + (s[2] + s[3]);
+    return t + __shfl_xor_sync(kFullMask, t, 16);
+}
+
+__device__ __forceinline__ int select_section_topp(const unsigned char* tile, unsigned char* wsm, unsigned char* image, int vals_off,
+                                                   int mask_off, int mu_off, int T, float top_p, int n, int lane, const float* a_all)
+{
+    const int p = lane & 15, half = lane >> 4, sw = p & 7;
+    const bool live = p < n;
+    const unsigned char* row = tile + p * (kHeadDim * 2);
+    unsigned char* wrow = wsm + p * (kHeadDim * 4);
+    const float* a = a_all + 64 * half;
+    float top_w = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + c) ^ sw) << 4));
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+        const float4 f0 = *reinterpret_cast<const float4*>(a + 8 * c), f1 = *reinterpret_cast<const float4*>(a + 8 * c + 4);
+        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+        float w[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            w[2 * j] = __fmul_rn(f[2 * j], fabsf(__uint_as_float(x[j] << 16)));
+            w[2 * j + 1] = __fmul_rn(f[2 * j + 1], fabsf(__uint_as_float(x[j] & 0xffff0000u)));
+            top_w = fmaxf(top_w, fmaxf(w[2 * j], w[2 * j + 1]));
+        }
+        *reinterpret_cast<float4*>(wrow + (((16 * half + 2 * c) ^ sw) << 4)) = make_float4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<float4*>(wrow + (((16 * half + 2 * c + 1) ^ sw) << 4)) = make_float4(w[4], w[5], w[6], w[7]);
+    }
+    top_w = fmaxf(top_w, __shfl_xor_sync(kFullMask, top_w, 16));
+    // (a lane reads only what it wrote)
+    const double total = sum_ge(wrow, sw, half, 0u);
+    const double goal = static_cast<double>(top_p) * total;
+    const float goal_f = static_cast<float>(goal);
+    // full-key bounds: the sum of keys >= lo reaches the goal, that of keys >= hi does not
+    unsigned lo = 0u, hi = 0u;
+    double above = 0.0;                                        // sum of the keys >= hi, in double
+    bool exact = false;
+    for (;;) {
+        int l16 = 0, h16 = static_cast<int>(__float_as_uint(top_w) >> 16) + 1;
+        double f_lo = total, f_hi = 0.0;                       // (in the first search fp32 values)
+        bool done = !live;
+        for (int it = 0; !__all_sync(kFullMask, done); ++it) {
+            const int span = h16 - l16;
+            const float vl = __uint_as_float(static_cast<unsigned>(l16) << 16);
+            // every key between the ends is at least vl: fewer than four of them
+            if (span <= 1 || (!exact && vl > 0.f && static_cast<float>(f_lo - f_hi) < 3.9f * vl)) done = true;
+            int step = span >> 1;
+            if (it % 3 != 0)
+                step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(f_lo - goal), static_cast<float>(f_lo - f_hi)));
+            if (it == 0 && span > 0x500) step = span - 0x500;  // first look ten octaves below the largest key
+            step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
+            const int t = l16 + (span > 1 ? step : 0);
+            const unsigned tk = static_cast<unsigned>(t) << 16;
+            const double f = exact ? sum_ge(wrow, sw, half, tk) : static_cast<double>(sum_ge_f32(wrow, sw, half, tk));
+            if (!done) {
+                if (exact ? f >= goal : static_cast<float>(f) >= goal_f) { l16 = t; f_lo = f; } else { h16 = t; f_hi = f; }
+            }
+        }
+        lo = static_cast<unsigned>(l16) << 16;
+        hi = static_cast<unsigned>(h16) << 16;
+        above = sum_ge(wrow, sw, half, hi);
+        const bool bad = live && !exact && above >= goal && goal > 0.0;      // fp32 had put the upper end too low
+        if (!__any_sync(kFullMask, bad)) break;
+        exact = true;                                          // rare: all tokens of the warp again, in double
+    }
+    // kept so far: keys >= hi; candidates: keys in [lo, hi) and, should they not suffice, the ones below
+    unsigned long long got = 0ull;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+        const unsigned nib = (v.x >= hi ? 1u : 0u) | (v.y >= hi ? 2u : 0u) | (v.z >= hi ? 4u : 0u) | (v.w >= hi ? 8u : 0u);
+        got |= static_cast<unsigned long long>(nib) << (4 * c);
+    }
+    if (!live) got = 0ull;
+    int count = __popcll(got);
+    count += __shfl_xor_sync(kFullMask, count, 16);
+    double sum = above;
+    unsigned below = hi;                                       // admitted down to here (exclusive)
+    while (__any_sync(kFullMask, live && count < kHeadDim && (sum < goal || count == 0))) {
+        const bool more = live && count < kHeadDim && (sum < goal || count == 0);
+        unsigned best = 0u;
+        unsigned long long eq = 0ull;
+#pragma unroll 4
+        for (int c = 0; c < 16; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+            const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (x[e] >= below) continue;
+                if (x[e] > best) { best = x[e]; eq = 0ull; }
+                if (x[e] == best) eq |= 1ull << (4 * c + e);
+            }
+        }
+        const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
+        if (other > best) { best = other; eq = 0ull; }
+        const int mine = __popcll(eq), theirs = __shfl_xor_sync(kFullMask, mine, 16);
+        if (more) {
+            const double w = static_cast<double>(__uint_as_float(best));
+            int take = 0;                                      // equal keys: lower channels first, no more than the goal asks for
+            while (take < mine + theirs && (sum < goal || count + take == 0)) { sum += w; ++take; }
+            if (take == 0) take = mine + theirs;               // (not reached: `more` asks for at least one)
+            int own = half ? take - theirs : take;
+            own = own < 0 ? 0 : (own > mine ? mine : own);
+            unsigned long long rest = eq;
+            for (int k = 0; k < own; ++k) rest &= rest - 1;
+            got |= eq & ~rest;
+            count += take;
+            below = best;
+            if (mine + theirs == 0) count = kHeadDim;          // (nothing left)
+        }
+    }
+    count = __popcll(got);
+    count += __shfl_xor_sync(kFullMask, count, 16);
+    if (count > T) {                                           // the page's capacity: the T most salient of them
+        // drop the least salient, higher channels first, until T are left (both lanes of the token take part)
+        for (int drop = count - T; drop > 0; --drop) {
+            unsigned low = 0xffffffffu;
+            int at = -1;
+            for (unsigned long long m = got; m; m &= m - 1) {
+                const int ch = __ffsll(static_cast<long long>(m)) - 1;
+                const unsigned k = *reinterpret_cast<const unsigned*>(wrow + (((16 * half + (ch >> 2)) ^ sw) << 4) + (ch & 3) * 4);
+                if (k <= low) { low = k; at = ch; }
+            }
+            const unsigned pair_mask = 0x00010001u << p;
+            const unsigned other = __shfl_xor_sync(pair_mask, low, 16);
+            const bool mine = half ? low <= other : low < other;
+            if (mine && at >= 0) got &= ~(1ull << at);
+        }
+        count = T;
+    }
+    __syncwarp();
+    double pruned = 0.0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (!((got >> (4 * c + e)) & 1ull)) pruned += static_cast<double>(__uint_as_float(x[e]));
+    }
+    pruned += __shfl_xor_sync(kFullMask, pruned, 16);
+    __syncwarp();                                              // every row of `wsm` has been read: the image may go over it
+    for (int i = lane; i < T * 2; i += 32) reinterpret_cast<uint4*>(image + vals_off)[i] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    const unsigned kept[2] = {static_cast<unsigned>(got), static_cast<unsigned>(got >> 32)};
+    const int mine = __popcll(got);
+    const int theirs = __shfl_xor_sync(kFullMask, mine, 16);
+    unsigned char* dst = image + vals_off + val_offset(2, p, half ? theirs : 0);
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + 4 * g + c) ^ sw) << 4));
+            const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if ((kept[g] >> (8 * c + i)) & 1u) {
+                    *reinterpret_cast<unsigned short*>(dst) = static_cast<unsigned short>((i & 1) ? x[i >> 1] >> 16 : x[i >> 1] & 0xffffu);
+                    dst += kPageTokens * 2;
+                }
+        }
+    *reinterpret_cast<uint2*>(image + mask_off + p * 16 + half * 8) = make_uint2(kept[0], kept[1]);
+    if (half == 0)
+        reinterpret_cast<float*>(image + mu_off)[p] =
+            live && count < kHeadDim ? static_cast<float>(pruned / static_cast<double>(kHeadDim - count)) : 0.f;
+    return live ? count : 0;
+}
+
+template <bool kPV, bool kTopP>
+__global__ void __launch_bounds__(kWarpPageWarps * 32, kTopP ? 4 : (kPV ? 5 : 6)) compress_pages_warp_kernel(CompressArgs A)
 {
     extern __shared__ __align__(16) unsigned char page_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int blk = blockIdx.x * kWarpPageWarps + warp, h = blockIdx.y, b = blockIdx.z;
     const PageLayout L = A.L;
-    const int image_bytes = kPV ? L.page_bytes : L.v_off;      // dense value rows go straight to the page
+    // dense value rows go straight to the page; SparK-p pages carry the slot rows behind them, and in shared memory those
+    // (and the head of the page) come to lie over the saliencies
+    const int image_bytes = kPV ? L.page_bytes : L.v_off;
+    const int image_room = kTopP ? warp_topp_room(L) : image_bytes;
     float* a_s = reinterpret_cast<float*>(page_smem);
-    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_bytes);
+    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_room);
     unsigned char* image = tile + kTileBytes;
 
     // Without eviction the kernel before this one is the window norm, and what it waited for is complete (see
@@ -929,7 +1140,7 @@ __global__ void __launch_bounds__(kWarpPageWarps * 32, kPV ? 5 : 6) compress_pag
         return;
     }
     unsigned char* page = A.pages + page_id * L.page_bytes;
-    if (n < kPageTokens)                                       // slots past the end of the sequence are zero
+    if (!kTopP && n < kPageTokens)                             // slots past the end of the sequence are zero
         for (int i = lane; i < image_bytes / 16; i += 32) reinterpret_cast<uint4*>(image)[i] = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -951,7 +1162,16 @@ __global__ void __launch_bounds__(kWarpPageWarps * 32, kPV ? 5 : 6) compress_pag
         }
         __syncwarp();
     }
-    select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
+    if (kTopP) {
+        const int n_kept = select_section_topp(tile, image, image, L.v_off, L.mask_off, L.mu_off, L.keep, A.sel.top_p, n, lane, a_s);
+        const int rows = __reduce_max_sync(kFullMask, n_kept);
+        __syncwarp();
+        for (int i = lane; i < L.keep * 2; i += 32)
+            reinterpret_cast<uint4*>(page + L.vals_off)[i] = reinterpret_cast<const uint4*>(image + L.v_off)[i];
+        if (lane == 0) reinterpret_cast<int*>(A.pages + rows_offset(A.n_pool_pages, L.page_bytes))[page_id] = rows;
+    } else {
+        select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
+    }
     __syncwarp();
     for (int i = lane; i < image_bytes / 16; i += 32)
         reinterpret_cast<uint4*>(page)[i] = reinterpret_cast<const uint4*>(image)[i];
@@ -1432,16 +1652,15 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     A.inv_pruned = p.keep < kHeadDim ? 1.0 / static_cast<double>(kHeadDim - p.keep) : 0.0;
     A.sel = make_select(p);
     A.max_len = max_packed;
-    if (p.dtype == SPARK_BF16 && p.select == SPARK_SELECT_FIXED && p.recovery == SPARK_RECOVER_DEGENERATE) {
+    const bool pv = A.L.keep_v < kHeadDim, topp = p.select == SPARK_SELECT_TOP_P;
+    if (p.dtype == SPARK_BF16 && p.recovery == SPARK_RECOVER_DEGENERATE && (p.select == SPARK_SELECT_FIXED || (topp && !pv))) {
         if (!evict) A.lens = seq_lens;                         // readable before the window norm has ended
-        const bool pv = A.L.keep_v < kHeadDim;
-        const size_t smem = kHeadDim * 4 + kWarpPageWarps * (kTileBytes + static_cast<size_t>(pv ? A.L.page_bytes : A.L.v_off));
-        if (smem > 48 * 1024 &&                                // capacities near 128 + 128
-            cudaFuncSetAttribute(compress_pages_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+        const size_t smem = kHeadDim * 4 + kWarpPageWarps * (kTileBytes + static_cast<size_t>(topp ? warp_topp_room(A.L) : (pv ? A.L.page_bytes : A.L.v_off)));
+        auto kernel = topp ? compress_pages_warp_kernel<false, true> : (pv ? compress_pages_warp_kernel<true, false> : compress_pages_warp_kernel<false, false>);
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
             return SPARK_ERR_CUDA;
         const dim3 wgrid((n_blocks + kWarpPageWarps - 1) / kWarpPageWarps, p.n_kv_heads, p.batch);
-        const cudaError_t e = pv ? launch_kernel(compress_pages_warp_kernel<true>, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A)
-                                 : launch_kernel(compress_pages_warp_kernel<false>, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A);
+        const cudaError_t e = launch_kernel(kernel, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A);
         ++*launches;
         return e == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }
