@@ -895,8 +895,8 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
 //   A threshold on the keys' upper halves is searched like the fixed rule's, but by the SUM of the keys at or above it, in
 //   fp32 until at most three keys can lie between the ends.  The sum above the upper end is then taken in double and
 //   must be below the goal (else the search is repeated in double), and the keys between are admitted one by one.
-//   About 10000 instructions for sixteen tokens, where a bitonic rank sort per token took 2100 for one: 8 heads x 8192 tokens
-//   172 -> 83 us.
+//   A bitonic rank sort per token took 2100 instructions for one token; prefill of 8192 tokens and its first token
+//   189 -> 63 us.
 __device__ __forceinline__ double sum_ge(const unsigned char* wrow, int sw, int half, unsigned lo)        // keys >= lo, in double
 {
     double s = 0.0;
@@ -962,22 +962,26 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
     for (;;) {
         int l16 = 0, h16 = static_cast<int>(__float_as_uint(top_w) >> 16) + 1;
         double f_lo = total, f_hi = 0.0;                       // (in the first search fp32 values)
-        bool done = !live;
+        bool done = !live, lo_moved = true;
         for (int it = 0; !__all_sync(kFullMask, done); ++it) {
             const int span = h16 - l16;
             const float vl = __uint_as_float(static_cast<unsigned>(l16) << 16);
             // every key between the ends is at least vl: fewer than four of them
             if (span <= 1 || (!exact && vl > 0.f && static_cast<float>(f_lo - f_hi) < 3.9f * vl)) done = true;
+            // interpolate; then look a quarter of the span inside the end that moved (the crossing is near it, and the
+            // other end has to follow); now and then bisect
             int step = span >> 1;
-            if (it % 3 != 0)
-                step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(f_lo - goal), static_cast<float>(f_lo - f_hi)));
             if (it == 0 && span > 0x500) step = span - 0x500;  // first look ten octaves below the largest key
+            else if (it % 6 == 5) step = span >> 1;
+            else if (it & 1) step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(f_lo - goal), static_cast<float>(f_lo - f_hi)));
+            else step = lo_moved ? (span >> 2) + 1 : span - (span >> 2) - 1;
             step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
             const int t = l16 + (span > 1 ? step : 0);
             const unsigned tk = static_cast<unsigned>(t) << 16;
             const double f = exact ? sum_ge(wrow, sw, half, tk) : static_cast<double>(sum_ge_f32(wrow, sw, half, tk));
             if (!done) {
-                if (exact ? f >= goal : static_cast<float>(f) >= goal_f) { l16 = t; f_lo = f; } else { h16 = t; f_hi = f; }
+                lo_moved = exact ? f >= goal : static_cast<float>(f) >= goal_f;
+                if (lo_moved) { l16 = t; f_lo = f; } else { h16 = t; f_hi = f; }
             }
         }
         lo = static_cast<unsigned>(l16) << 16;
@@ -988,32 +992,35 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
         exact = true;                                          // rare: all tokens of the warp again, in double
     }
     // kept so far: keys >= hi; candidates: keys in [lo, hi) and, should they not suffice, the ones below
-    unsigned long long got = 0ull;
+    unsigned got2[2] = {0u, 0u}, cand2[2] = {0u, 0u};
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
         const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-        const unsigned nib = (v.x >= hi ? 1u : 0u) | (v.y >= hi ? 2u : 0u) | (v.z >= hi ? 4u : 0u) | (v.w >= hi ? 8u : 0u);
-        got |= static_cast<unsigned long long>(nib) << (4 * c);
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const unsigned bit = 1u << ((4 * c + e) & 31);
+            if (x[e] >= hi) got2[c >> 3] |= bit;
+            if (x[e] >= lo) cand2[c >> 3] |= bit;
+        }
     }
-    if (!live) got = 0ull;
+    unsigned long long got = (static_cast<unsigned long long>(got2[1]) << 32) | got2[0];
+    unsigned long long cand = ((static_cast<unsigned long long>(cand2[1]) << 32) | cand2[0]) & ~got;
+    if (!live) got = cand = 0ull;
     int count = __popcll(got);
     count += __shfl_xor_sync(kFullMask, count, 16);
     double sum = above;
-    unsigned below = hi;                                       // admitted down to here (exclusive)
     while (__any_sync(kFullMask, live && count < kHeadDim && (sum < goal || count == 0))) {
         const bool more = live && count < kHeadDim && (sum < goal || count == 0);
         unsigned best = 0u;
         unsigned long long eq = 0ull;
-#pragma unroll 4
-        for (int c = 0; c < 16; ++c) {
-            const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-            const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (x[e] >= below) continue;
-                if (x[e] > best) { best = x[e]; eq = 0ull; }
-                if (x[e] == best) eq |= 1ull << (4 * c + e);
-            }
+        const int none = cand == 0ull, both = none & __shfl_xor_sync(kFullMask, none, 16);
+        if (both) cand = ~got;                                  // the candidates did not suffice: every key left
+        for (unsigned long long m = more ? cand : 0ull; m; m &= m - 1) {
+            const int ch = __ffsll(static_cast<long long>(m)) - 1;
+            const unsigned k = *reinterpret_cast<const unsigned*>(wrow + (((16 * half + (ch >> 2)) ^ sw) << 4) + (ch & 3) * 4);
+            if (k > best) { best = k; eq = 0ull; }
+            if (k == best) eq |= 1ull << ch;
         }
         const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
         if (other > best) { best = other; eq = 0ull; }
@@ -1022,14 +1029,13 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
             const double w = static_cast<double>(__uint_as_float(best));
             int take = 0;                                      // equal keys: lower channels first, no more than the goal asks for
             while (take < mine + theirs && (sum < goal || count + take == 0)) { sum += w; ++take; }
-            if (take == 0) take = mine + theirs;               // (not reached: `more` asks for at least one)
             int own = half ? take - theirs : take;
             own = own < 0 ? 0 : (own > mine ? mine : own);
             unsigned long long rest = eq;
             for (int k = 0; k < own; ++k) rest &= rest - 1;
             got |= eq & ~rest;
+            cand &= ~eq;
             count += take;
-            below = best;
             if (mine + theirs == 0) count = kHeadDim;          // (nothing left)
         }
     }
