@@ -111,13 +111,13 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     if (warp == kConsumerWarps) {
         producer_prologue(A, C, lane, kDecodeThreads);
         int p0, p1;
-        cta_range(*C.plan, static_cast<int>(blockIdx.x), p0, p1);
+        cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), p0, p1);
         producer_loop<kConsumerWarps>(A, C, ring, p0, p1, lane);
         return;
     }
     consumer_wait_plan(kDecodeThreads);
     int c0, c1;
-    cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
+    cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
     grid_wait();                                           // q, qnorm, out and the workspace from here on
     write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
 
@@ -406,6 +406,7 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     // Two units per epoch only where CTAs hold several: the second unit's table and records cost a ring slot (of six or
     // seven: 2 x 7926 tokens, G = 4, T = 89: 43.9 us with six slots, 35.2 us with seven).
+    A.whole_steps = 0;                                     // (a step is 32 tokens of double sums: splitting pays)
     A.cap = 2 * units <= grid ? 1 : 2;
     A.tab_off = S::kTab;
     A.prefix_off = S::fixed(A.cap);

@@ -19,7 +19,7 @@ constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // every device-sid
 constexpr unsigned kClockEvery = 256;                        // polls between two looks at the clock
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRec = kHeadDim + 4;           // floats per head record: 128 outputs, running max, running sum, pad
-constexpr int kMaxCap = 6;                    // units per epoch, at most (see Epoch)
+constexpr int kMaxCap = 8;                    // units per epoch, at most (see Epoch)
 constexpr float kLn2 = 0.6931471805599453f;
 
 struct DecodeArgs {
@@ -44,6 +44,7 @@ struct DecodeArgs {
     int slot_stride;
     int pps;                                 // pages per step (= per ring slot): 1 or 2
     int cap;                                 // units per epoch
+    int whole_steps;                         // a step per consumer warp; units up to this are not split (see Plan)
     int tab_off;                             // shared-memory offset of the epoch's operand tables
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix)
@@ -71,14 +72,16 @@ __host__ __device__ constexpr int merge_state_floats(int nw, int cap, int g)
 }
 __host__ __device__ constexpr int merge_bytes(int nw, int cap, int g) { return (merge_state_floats(nw, cap, g) + cap * g * 2) * 4; }
 
-// Units of an epoch that a launch would like: as many as a CTA's run meets when the sequences are equally long, and a
-// few more where a batch of unequal sequences is so short that a CTA may meet many (a unit beyond the cap costs
-// another table build and merge, about 3 us).  A single sequence with several CTAs per unit needs one.
+// Units of an epoch that a launch would like: as many as a CTA's run meets when the sequences are equally long, and the
+// most where a batch of unequal sequences is so short that a CTA may meet many (a unit beyond the cap costs a second
+// epoch: 8 sequences of 150..4000 tokens, whose CTAs meet up to seven units, took 23.9 us with five and 20.9 with
+// eight).  A single sequence with several CTAs per unit needs one.
 inline int epoch_cap(int batch, int64_t units, int max_blocks, int grid)
 {
     if (batch == 1 && 2 * units <= grid) return 1;
     int64_t c = (units + grid - 1) / grid + 1;
-    if (batch > 1 && units * max_blocks <= static_cast<int64_t>(grid) * 256) c += 3;
+    const int64_t run = units * max_blocks / grid;                            // a CTA's steps in a full cache
+    if (batch > 1 && run <= 256) c = run <= 160 ? kMaxCap : c + 3;
     return c > kMaxCap ? kMaxCap : static_cast<int>(c);
 }
 
@@ -268,10 +271,14 @@ struct EpochUnit {
 //   aligned mode: all units have the same number of steps and there are several CTAs per unit; unit u
 //                 gets q or q+1 whole CTAs (the first `rem` units get q+1) and is split evenly among
 //                 them, so no CTA crosses a unit boundary and every CTA publishes exactly once.
+//   whole units : CTA u owns unit u.  For units of at most a step per warp, where a split saves nothing and adds a
+//                 partial, a ticket and the last arriver's merge (240 tokens: 8.4 us against 9.1; with two steps per warp
+//                 9.7 against 9.2), and for units of up to three steps per warp where they fill most of the grid anyway
+//                 (16 sequences of 60..700 tokens, 128 units: 12.7 us against 18.7).
 struct Plan {
     int total;        // steps on the line
     int chunk;        // stream mode: steps per CTA
-    int aligned;      // 0: stream, 1: aligned mode
+    int aligned;      // 0: stream, 1: aligned mode, 2: whole units
     int unit_steps;   // aligned: steps of every unit
     int q, rem;       // aligned: CTAs per unit
 };
@@ -297,7 +304,7 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, i
     c.abort_flag = reinterpret_cast<volatile int*>(smem + 512);
     c.plan = reinterpret_cast<Plan*>(smem + 528);
     c.last_flag = reinterpret_cast<volatile int*>(smem + 560);
-    c.epoch = reinterpret_cast<volatile int*>(smem + 592);
+    c.epoch = reinterpret_cast<volatile int*>(smem + 600);
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
     c.units = reinterpret_cast<EpochUnit*>(smem + 768);
     c.prefix = reinterpret_cast<int*>(smem + prefix_off);
@@ -361,11 +368,8 @@ __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctr
         if (b < A.B) C.prefix[b + 1] = running + inc;
         running += __shfl_sync(kFull, inc, 31);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        smin = min(smin, __shfl_xor_sync(kFull, smin, o));
-        smax = max(smax, __shfl_xor_sync(kFull, smax, o));
-    }
+    smin = __reduce_min_sync(kFull, smin);
+    smax = __reduce_max_sync(kFull, smax);
     if (lane == 0) {
         C.prefix[0] = 0;
         Plan pl;
@@ -373,7 +377,9 @@ __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctr
         pl.total = A.Hkv * running;
         pl.chunk = (pl.total + nct - 1) / nct;
         pl.aligned = 0; pl.unit_steps = smax; pl.q = 0; pl.rem = 0;
-        if (smin == smax && smax > 0 && units <= nct) {
+        if (units <= nct && (smax <= A.whole_steps || (2 * units > nct && smax <= 3 * A.whole_steps))) {
+            pl.aligned = 2;
+        } else if (smin == smax && smax > 0 && units <= nct) {
             const int q = nct / units;
             const int makespan = (smax + q - 1) / q;
             if (q >= 2 && makespan * 25 <= pl.chunk * 26) {          // within 4 % of the even split
@@ -393,8 +399,15 @@ __device__ __forceinline__ void consumer_wait_plan(int n_threads)
 }
 
 // This CTA's run of steps [c0, c1) on the line.
-__device__ __forceinline__ void cta_range(const Plan& pl, int cta, int& c0, int& c1)
+__device__ __forceinline__ void cta_range(const Plan& pl, const int* prefix, int B, int Hkv, int cta, int& c0, int& c1)
 {
+    if (pl.aligned == 2) {
+        const int b = cta / Hkv, h = cta - b * Hkv;
+        const int steps = b < B ? prefix[b + 1] - prefix[b] : 0;
+        c0 = b < B ? Hkv * prefix[b] + h * steps : 0;
+        c1 = c0 + steps;
+        return;
+    }
     if (!pl.aligned) {
         c0 = min(pl.total, cta * pl.chunk);
         c1 = min(pl.total, c0 + pl.chunk);
@@ -412,6 +425,7 @@ __device__ __forceinline__ void cta_range(const Plan& pl, int cta, int& c0, int&
 // The CTAs that hold a part of the unit starting at step `unit_start` with `unit_steps` steps.
 __device__ __forceinline__ void unit_parts(const Plan& pl, int unit_start, int unit_steps, int& first_cta, int& n_parts)
 {
+    if (pl.aligned == 2) { first_cta = 0; n_parts = 1; return; }
     if (!pl.aligned) {
         first_cta = unit_start / pl.chunk;
         n_parts = (unit_start + unit_steps - 1) / pl.chunk - first_cta + 1;

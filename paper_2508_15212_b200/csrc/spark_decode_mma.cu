@@ -243,32 +243,43 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     if (warp == kNW) {
         producer_prologue(A, C, lane, kThreads);
         int p0, p1;
-        cta_range(*C.plan, static_cast<int>(blockIdx.x), p0, p1);
+        cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), p0, p1);
         producer_loop<kNW>(A, C, ring, p0, p1, lane);
         return;
     }
     consumer_wait_plan(kThreads);
     int c0, c1;
-    cta_range(*C.plan, static_cast<int>(blockIdx.x), c0, c1);
+    cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
     grid_wait();                                           // q, qnorm, out and the workspace from here on
     write_empty_sequences<kNT>(A, C.prefix, tid);
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
     for (int g = c0; g < c1;) {
         const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, g, c1);
-        // ---- the epoch's operand tables: a warp prepares one query head of one unit ----
+        // ---- the epoch's operand tables: a warp prepares one query head of one unit at a time, the next one's loads
+        //      in flight meanwhile (first pass: only loads) ----
+        {
+            uint2 qr = make_uint2(0, 0);
+            float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int n_heads = ep.n_units * G;
 #pragma unroll 1
-        for (int pr = warp; pr < ep.n_units * G; pr += kNW) {
-            const int e = pr / G, hd = pr - e * G;
-            UnitRef u = ep.first;
+            for (int pr = warp - kNW; pr < n_heads; pr += kNW) {
+                const uint2 q_now = qr;
+                const float4 a_now = a4;
+                const int next = pr + kNW, e = next / G;
+                if (next < n_heads) {
+                    UnitRef u = ep.first;
 #pragma unroll 1
-            for (int k = 0; k < e; ++k) next_unit(C.prefix, A.Hkv, u);
-            const uint2 qr = *reinterpret_cast<const uint2*>(
-                static_cast<const unsigned short*>(q_src) +
-                (static_cast<int64_t>(u.b) * A.Hq + u.h * G + hd) * kHeadDim + 4 * lane);
-            const float4 a4 = *reinterpret_cast<const float4*>(
-                A.qnorm + (static_cast<int64_t>(u.b) * A.Hkv + u.h) * kHeadDim + 4 * lane);
-            write_head_tables<G>(tab_all + e * S::kTabBytes, qsum_all + e * 8, hd, lane, qr, a4);
+                    for (int k = 0; k < e; ++k) next_unit(C.prefix, A.Hkv, u);
+                    qr = *reinterpret_cast<const uint2*>(
+                        static_cast<const unsigned short*>(q_src) +
+                        (static_cast<int64_t>(u.b) * A.Hq + u.h * G + next - e * G) * kHeadDim + 4 * lane);
+                    a4 = *reinterpret_cast<const float4*>(
+                        A.qnorm + (static_cast<int64_t>(u.b) * A.Hkv + u.h) * kHeadDim + 4 * lane);
+                }
+                if (pr >= 0)
+                    write_head_tables<G>(tab_all + (pr / G) * S::kTabBytes, qsum_all + (pr / G) * 8, pr % G, lane, q_now, a_now);
+            }
         }
         consumer_sync<kNT>();
 
@@ -545,6 +556,7 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
     A.slot_stride = static_cast<int>(align_up(static_cast<size_t>(A.L.page_bytes), 128));
     const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    A.whole_steps = kNW;
     A.cap = epoch_cap(A.B, units, A.max_blocks, grid);
     // An epoch's units take shared memory (operand tables, records) from the ring.  Where a CTA's run is long, a unit
     // boundary (3 us) is a small part of it and ring slots are worth more: 16 sequences of 8K..128K tokens, seven
