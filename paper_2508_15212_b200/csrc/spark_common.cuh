@@ -180,7 +180,8 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
                            const float* qnorm, float* out, float* lse, void* workspace,
                            size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value = false,
                            const float* other_out = nullptr, const float* other_lse = nullptr);
-// other_out / other_lse: attention over further tokens of the same sequences, merged into the result
+// other_out / other_lse: attention over further tokens of the same sequences, merged into the result.  The kernel that writes
+// them must be the one enqueued just before, and must write nothing else that this step uses: it is waited for only there.
 // q_by_value: q is a HOST pointer and its bytes travel as a launch parameter (bf16 storage, degenerate recovery,
 // dense value rows, at most query_by_value_limit() bytes; anything else is refused)
 size_t query_by_value_limit();

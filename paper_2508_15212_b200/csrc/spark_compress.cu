@@ -1250,6 +1250,13 @@ __global__ void __launch_bounds__(1024) append_token_cta_kernel(AppendArgs A)
     constexpr bool kBf16 = (sizeof(E) == 2);
     const int b = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const PageLayout L = A.L;
+    // ask for the head's rows before the length is known: one round trip less in the chain
+    {
+        const int64_t unit = static_cast<int64_t>(b) * A.Hkv + h, row = unit * kHeadDim + lane * 4;
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(static_cast<const E*>(A.k_new) + row));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(static_cast<const E*>(A.v_new) + row));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(A.qnorm + row));
+    }
     const int t = A.packed_lens[b];
     __syncthreads();
     const int blk = t / kPageTokens, p = t - blk * kPageTokens;

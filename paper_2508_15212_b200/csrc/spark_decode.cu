@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     consumer_wait_plan(kDecodeThreads);
     int c0, c1;
     cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
-    grid_wait();                                           // q, qnorm, out and the workspace from here on
-    write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
+    if (!A.late_wait) {
+        grid_wait();                                       // q, qnorm, out and the workspace from here on
+        write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
+    }
 
     float* pscr = pscr_all + warp * 32 * GPP;
     for (int g = c0; g < c1;) {
@@ -361,6 +363,10 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
         merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, C.epoch[1], tid);
         g = C.epoch[0];
     }
+    if (A.late_wait) {
+        grid_wait();
+        write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -475,6 +481,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     A.q = q; A.pages = static_cast<const unsigned char*>(pages); A.block_table = block_table;
     A.max_blocks = max_blocks; A.lens = packed_lens; A.qnorm = qnorm; A.out = out; A.lse = lse;
     A.other_out = other_out; A.other_lse = other_lse;
+    A.late_wait = other_lse ? 1 : 0;
     A.B = p.batch; A.Hq = p.n_q_heads; A.Hkv = p.n_kv_heads; A.n_pool_pages = p.n_pool_pages;
     A.L = make_layout(p);
     const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf(static_cast<float>(p.head_dim));

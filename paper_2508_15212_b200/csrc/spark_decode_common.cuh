@@ -48,6 +48,7 @@ struct DecodeArgs {
     int tab_off;                             // shared-memory offset of the epoch's operand tables
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix)
+    int late_wait;                           // the kernel before writes only other_out / other_lse: wait where they are read
     int overlap;                             // the page stream need not wait for the kernel before (SPARK_FLAG_OVERLAP_PREVIOUS)
     unsigned seed;                           // sampled recovery: seed of the per-entry draws
     const int* page_rows;                    // ragged pages: slot rows in use per pool page (else null: whole pages)
@@ -676,6 +677,7 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
         const float M = unit_ml[2 * pr], Ls = unit_ml[2 * pr + 1];
         const int64_t row = static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg;
         if (d.n_parts == 1) {
+            if (A.late_wait) grid_wait();
             const PublishWeights pw = publish_weights(A, row, M, Ls);
             O.x *= pw.own; O.y *= pw.own;
             if (A.other_out) {
@@ -790,6 +792,7 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
                     }
             }
             if (ph == 0) {
+                if (A.late_wait) grid_wait();
                 const int64_t row = static_cast<int64_t>(b) * A.Hq + h * G + gg;
                 const PublishWeights w = publish_weights(A, row, pML[2 * gg], pML[2 * gg + 1]);
                 acc.x *= w.own; acc.y *= w.own; acc.z *= w.own; acc.w *= w.own;

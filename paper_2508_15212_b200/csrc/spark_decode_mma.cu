@@ -250,8 +250,10 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     consumer_wait_plan(kThreads);
     int c0, c1;
     cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
-    grid_wait();                                           // q, qnorm, out and the workspace from here on
-    write_empty_sequences<kNT>(A, C.prefix, tid);
+    if (!A.late_wait) {
+        grid_wait();                                       // q, qnorm, out and the workspace from here on
+        write_empty_sequences<kNT>(A, C.prefix, tid);
+    }
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
     for (int g = c0; g < c1;) {
@@ -511,6 +513,10 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
         consumer_sync<kNT>();
         merge_and_publish<G, kNW>(A, C, merge, unit_ml, C.epoch[1], tid);
         g = C.epoch[0];
+    }
+    if (A.late_wait) {
+        grid_wait();
+        write_empty_sequences<kNT>(A, C.prefix, tid);
     }
 }
 

@@ -36,6 +36,13 @@ __global__ void __launch_bounds__(1024) append_dense_kernel(AppendDenseArgs A)
     grid_release();
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const PageLayout L = A.L;
+    // the first head's row before the length: one round trip less in the chain
+    Vec k_first, v_first;
+    if (warp < A.Hkv) {
+        const int64_t first = (static_cast<int64_t>(b) * A.Hkv + warp) * 32 + lane;
+        k_first = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.k_new) + first * kLaneBytes);
+        v_first = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.v_new) + first * kLaneBytes);
+    }
     const int t = A.lens[b];
     __syncthreads();
     const int blk = t / kPageTokens, p = t - blk * kPageTokens;
@@ -49,8 +56,11 @@ __global__ void __launch_bounds__(1024) append_dense_kernel(AppendDenseArgs A)
             if (lane == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
             continue;
         }
-        const Vec k = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.k_new) + (unit * 32 + lane) * kLaneBytes);
-        const Vec v = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.v_new) + (unit * 32 + lane) * kLaneBytes);
+        Vec k = k_first, v = v_first;
+        if (h != warp) {
+            k = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.k_new) + (unit * 32 + lane) * kLaneBytes);
+            v = *reinterpret_cast<const Vec*>(static_cast<const unsigned char*>(A.v_new) + (unit * 32 + lane) * kLaneBytes);
+        }
         const int64_t row = unit * A.cap + t;
         *reinterpret_cast<Vec*>(static_cast<unsigned char*>(A.k_tail) + (row * 32 + lane) * kLaneBytes) = k;
         *reinterpret_cast<Vec*>(static_cast<unsigned char*>(A.v_tail) + (row * 32 + lane) * kLaneBytes) = v;
@@ -80,6 +90,10 @@ __global__ void __launch_bounds__(1024) append_dense_kernel(AppendDenseArgs A)
 // ------------------------------------------------------------------------------------------------
 constexpr int kTailThreads = 256;
 
+template <int ES> struct TailPair;
+template <> struct TailPair<2> { using type = unsigned; };
+template <> struct TailPair<4> { using type = uint2; };
+
 struct TailArgs {
     const void* q;
     const void* k;
@@ -102,18 +116,23 @@ __global__ void __launch_bounds__(kTailThreads) tail_attn_kernel(TailArgs A)
     grid_wait();
     grid_release();
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int n = A.lens[b];
-    n = n < 0 ? 0 : (n > A.cap ? A.cap : n);
+    // rows of the first 64 tokens before the length is known (they exist up to cap; what is past the length is not used)
     const int64_t unit = static_cast<int64_t>(b) * A.Hkv + h, row0 = static_cast<int64_t>(b) * A.Hq + h * G;
     const E* k = static_cast<const E*>(A.k) + unit * A.cap * kHeadDim;
     const E* v = static_cast<const E*>(A.v) + unit * A.cap * kHeadDim;
-    // keys of this thread's tokens (32 channels of tokens t and t + 64) and the query
     constexpr int kVecs = 32 * sizeof(E) / 16;
-    const int t0 = tid >> 2, c = tid & 3;
+    using Pair = typename TailPair<sizeof(E)>::type;
+    const int t0 = tid >> 2, c = tid & 3, grp = tid >> 6, c2 = tid & 63;
     uint4 kr[kVecs];
-    if (t0 < n)
+    Pair vr[16];
+    if (t0 < A.cap)
 #pragma unroll
         for (int i = 0; i < kVecs; ++i) kr[i] = reinterpret_cast<const uint4*>(k + static_cast<int64_t>(t0) * kHeadDim + 32 * c)[i];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+        if (grp + 4 * i < A.cap) vr[i] = *reinterpret_cast<const Pair*>(v + static_cast<int64_t>(grp + 4 * i) * kHeadDim + 2 * c2);
+    int n = A.lens[b];
+    n = n < 0 ? 0 : (n > A.cap ? A.cap : n);
     for (int i = tid; i < G * kHeadDim; i += kTailThreads) q_s[i / kHeadDim][i % kHeadDim] = Elem<E>::load(A.q, row0 * kHeadDim + i);
     __syncthreads();
     for (int t = t0; t < ((n + 63) & ~63); t += 64) {          // whole warps iterate together
@@ -174,12 +193,24 @@ __global__ void __launch_bounds__(kTailThreads) tail_attn_kernel(TailArgs A)
         }
     }
     __syncthreads();
-    const int grp = tid >> 6, c2 = tid & 63;                   // tokens grp, grp + 4, ...; channels 2*c2, 2*c2 + 1
+    // weighted sum: tokens grp, grp + 4, ...; channels 2*c2, 2*c2 + 1
     float2 acc[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) acc[g] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int t = grp + 4 * i;
+        if (t >= n) break;
+        const E* x = reinterpret_cast<const E*>(&vr[i]);
+        const float v0 = static_cast<float>(x[0]), v1 = static_cast<float>(x[1]);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            acc[g].x = fmaf(prob[g][t], v0, acc[g].x);
+            acc[g].y = fmaf(prob[g][t], v1, acc[g].y);
+        }
+    }
 #pragma unroll 8
-    for (int t = grp; t < n; t += 4) {
+    for (int t = 64 + grp; t < n; t += 4) {
         const E* x = v + static_cast<int64_t>(t) * kHeadDim + 2 * c2;
         const float v0 = static_cast<float>(x[0]), v1 = static_cast<float>(x[1]);
 #pragma unroll
