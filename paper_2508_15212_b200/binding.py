@@ -6,6 +6,7 @@ stream.  There is no fallback: if the library is missing the import of a functio
 from __future__ import annotations
 
 import ctypes
+import operator
 import os
 from typing import Optional
 
@@ -125,8 +126,9 @@ def _blocks(block_table, max_blocks) -> int:
     return int(max_blocks)
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """The current stream's handle.  (torch.cuda.current_stream() builds a Stream object: 2 us of a 7 us call.)"""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def make_params(*, batch, n_q_heads, n_kv_heads, window, keep, dtype, n_pool_pages, head_dim=128,
@@ -244,7 +246,7 @@ def spark_append_dense(p: spark_params, k_new, v_new, pages, block_table, k_tail
                                     None if block_table is None else block_table.data_ptr(), _blocks(block_table, max_blocks),
                                     k_tail.data_ptr(), v_tail.data_ptr(), k_tail.shape[2], packed_lens.data_ptr(),
                                     workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                    torch.cuda.current_stream().cuda_stream),
+                                    _stream()),
            "spark_append_dense")
 
 
@@ -258,8 +260,47 @@ def spark_decode_attn_tail(p: spark_params, q, pages, block_table, packed_lens, 
                                         tail_out.data_ptr(), tail_lse.data_ptr(), out.data_ptr(),
                                         None if lse is None else lse.data_ptr(), workspace.data_ptr(),
                                         workspace.numel() * workspace.element_size(),
-                                        torch.cuda.current_stream().cuda_stream),
+                                        _stream()),
            "spark_decode_attn_tail")
+
+
+class BoundTail:
+    """spark_append_dense and spark_decode_attn_tail on the buffers of one prefix + tail pair, marshalled once: a call
+    converts only what changes from token to token (the new rows, the query, the result and the stream)."""
+
+    def __init__(self, prefix, tail, k_tail, v_tail, tail_out, tail_lse):
+        self.buffers = self.current(prefix, tail, k_tail, v_tail)
+        self._alive = (prefix.params, tail.params, tail_out, tail_lse)
+        cap = int(k_tail.shape[2])
+        self._append_fn, self._decode_fn = lib().spark_append_dense, lib().spark_decode_attn_tail
+        self._p_tail, self._p_prefix = ctypes.byref(tail.params), ctypes.byref(prefix.params)
+        self._append_args = (_ptr(tail.pages), _ptr(tail.block_table), tail.table_blocks, _ptr(k_tail), _ptr(v_tail), cap,
+                             _ptr(tail.packed_lens), _ptr(tail.ws_compress), tail.ws_compress.numel())
+        self._decode_args = (_ptr(prefix.pages), _ptr(prefix.block_table), prefix.table_blocks, _ptr(prefix.packed_lens),
+                             _ptr(prefix.qnorm), _ptr(k_tail), _ptr(v_tail), cap, _ptr(tail.packed_lens), _ptr(tail_out),
+                             _ptr(tail_lse))
+        self._ws = (_ptr(prefix.ws_decode), prefix.ws_decode.numel())
+
+    @staticmethod
+    def current(prefix, tail, k_tail, v_tail):
+        return (prefix.pages, prefix.block_table, prefix.packed_lens, prefix.qnorm, prefix.ws_decode, prefix.params, tail.pages,
+                tail.block_table, tail.packed_lens, tail.ws_compress, tail.params, k_tail, v_tail)
+
+    def matches(self, prefix, tail, k_tail, v_tail) -> bool:
+        """Whether the pair still has the buffers that were marshalled."""
+        return all(map(operator.is_, self.buffers, self.current(prefix, tail, k_tail, v_tail)))
+
+    def append(self, k_new, v_new) -> None:
+        assert k_new.is_contiguous() and v_new.is_contiguous()
+        code = self._append_fn(self._p_tail, k_new.data_ptr(), v_new.data_ptr(), *self._append_args, _stream())
+        if code != SPARK_OK:
+            raise SparkError(code, "spark_append_dense")
+
+    def decode(self, q, out, lse) -> None:
+        code = self._decode_fn(self._p_prefix, q.data_ptr(), *self._decode_args, out.data_ptr(),
+                               None if lse is None else lse.data_ptr(), *self._ws, _stream())
+        if code != SPARK_OK:
+            raise SparkError(code, "spark_decode_attn_tail")
 
 
 TAIL_MAX = 128              # tokens of a dense tail that spark_decode_attn_tail takes
@@ -278,7 +319,7 @@ class BoundDecodeHost:
         self._args = (ctypes.byref(p), _ptr(q_host), _ptr(q_dev), _ptr(pages), _ptr(block_table),
                       _blocks(block_table, max_blocks), _ptr(packed_lens), _ptr(qnorm), _ptr(out_dev), _ptr(out_host),
                       None, None, _ptr(workspace), workspace.numel() * workspace.element_size())
-        self._stream = None if stream is None else ctypes.c_void_p(stream)
+        self._stream = stream
         self.out_host = out_host
 
     def __call__(self) -> None:
@@ -302,7 +343,7 @@ class BoundDecode:
         self._args = (ctypes.byref(p), _ptr(q), _ptr(pages), _ptr(block_table), _blocks(block_table, max_blocks),
                       _ptr(packed_lens), _ptr(qnorm), _ptr(out), _ptr(lse), _ptr(workspace),
                       workspace.numel() * workspace.element_size())
-        self._stream = None if stream is None else ctypes.c_void_p(stream)
+        self._stream = stream
         self.out = out
 
     def __call__(self) -> None:

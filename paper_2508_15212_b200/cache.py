@@ -190,6 +190,7 @@ class DenseTailCache:
         self._o = [torch.empty(p.batch, p.n_q_heads, 128, dtype=torch.float32, device=device) for _ in range(2)]
         self._l = [torch.empty(p.batch, p.n_q_heads, dtype=torch.float32, device=device) for _ in range(2)]
         self._short = cap <= B.TAIL_MAX
+        self._bound = None
 
     def compress(self, q_win, k, v, seq_lens) -> None:
         self.prefix.compress(q_win, k, v, seq_lens)
@@ -197,13 +198,18 @@ class DenseTailCache:
         self.tail.packed_lens.zero_()
         self.n_tail = 0
 
+    def _calls(self) -> "B.BoundTail":
+        """The calls on this pair's buffers, marshalled once (and again should a buffer have been replaced)."""
+        b = self._bound
+        if b is None or not b.matches(self.prefix, self.tail, self.k_tail, self.v_tail):
+            b = self._bound = B.BoundTail(self.prefix, self.tail, self.k_tail, self.v_tail, self._o[1], self._l[1])
+        return b
+
     def append(self, k_new, v_new) -> None:
         """One new token per sequence ([B, Hkv, D]); it stays dense until its block is handed to the prefix."""
         if self.n_tail >= self.k_tail.shape[2]:
             raise IndexError(f"the dense tail holds {self.n_tail} tokens and has no room for another")
-        t = self.tail
-        B.spark_append_dense(t.params, k_new, v_new, t.pages, t.block_table, self.k_tail, self.v_tail, t.packed_lens,
-                             t.ws_compress, max_blocks=t.table_blocks)
+        self._calls().append(k_new, v_new)
         self.n_tail += 1
         if self.block and self.n_tail == self.block:
             self.prefix.append_block(self.k_tail, self.v_tail)
@@ -214,10 +220,7 @@ class DenseTailCache:
         if out is None:
             out = torch.empty_like(self._o[0])
         if self._short:                                    # a short tail: two launches, merged in the prefix's step
-            p = self.prefix
-            B.spark_decode_attn_tail(p.params, q, p.pages, p.block_table, p.packed_lens, p.qnorm, self.k_tail, self.v_tail,
-                                     self.tail.packed_lens, self._o[1], self._l[1], out, lse, p.ws_decode,
-                                     max_blocks=p.table_blocks)
+            self._calls().decode(q, out, lse)
             return out
         self.prefix.decode(q, out=self._o[0], lse=self._l[0])
         self.tail.decode(q, out=self._o[1], lse=self._l[1])
