@@ -684,14 +684,15 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 // selection serves sixteen tokens and needs one shuffle, and a warp owns its page from the loads to the stores
 // without a CTA barrier.
 //   Selection.  Any threshold t with exactly T keys >= t names the kept set, so the search need not descend bit by bit:
-//   it interpolates the count between its two ends (every third step bisects, which bounds it) over the keys' upper
-//   halves, two keys per compare.  Where the boundary falls inside one upper half (a fifth of the tokens), the few
-//   keys that share it are told apart by their full bits, in order of key and then of channel.
+//   it interpolates the count between its two ends (every sixth step bisects, which bounds it) over the keys' upper
+//   halves, two keys per compare, until T is hit or at most two keys lie between the ends; those (and any that share an
+//   upper half) are told apart by their full bits, in order of key and then of channel.
 //   What bounds it: issue slots.  183 instructions a token against 308 with eight lanes per token and a bitwise
 //   descent (compress_pages4_kernel, which fp32 storage and sampled recovery keep); 8 heads x 32768 tokens:
-//   104 -> 66 us under the profiler, prefill of 32K tokens 132.4 -> 90.3 us (24 warps a SM; with 16 it took 93.4).
+//   104 -> 62 us; prefill of 32K tokens 132.4 -> 88 us (24 warps a SM; with 16 3 us more).
 // ------------------------------------------------------------------------------------------------
 constexpr int kWarpPageWarps = 4;
+constexpr int kFewKeys = 2;            // keys left between the ends that are told apart by their full bits
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
 // SparK-p: the saliencies of a page (fp32), and over them, once read, mask | mu | slot rows
 __host__ __device__ inline int warp_topp_room(const PageLayout& L)
@@ -794,19 +795,32 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
             mn = mn > 0x7f80u ? 0x7f80u : mn;
         }
         int lo = static_cast<int>(mn), hi = static_cast<int>(mx) + 1, c_lo = kHeadDim, c_hi = 0;   // counts at lo (>= T) and hi (< T)
+        // weights of the two ends (distances of their counts from T; an end that stays while the other moves twice counts half:
+        // the "Illinois" false position), every sixth step bisects
+        float w_lo = static_cast<float>(kHeadDim - T) + 0.5f, w_hi = static_cast<float>(T) - 0.5f;
+        int side = 0;
         bool done = !live || hi - lo == 1;
         for (int it = 0; !__all_sync(kFullMask, done); ++it) {
             const int span = hi - lo;
             int step = span >> 1;
-            if (it % 3 != 2)
-                step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(2 * (c_lo - T) + 1), static_cast<float>(2 * (c_lo - c_hi))));
+            if (it % 6 != 5) step = static_cast<int>(static_cast<float>(span) * __fdividef(w_lo, w_lo + w_hi));
             step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
             const int t = lo + step;
             int c = count_ge(hk, static_cast<unsigned>(t) * 0x00010001u);
             c += __shfl_xor_sync(kFullMask, c, 16);
             if (!done) {
-                if (c >= T) { lo = t; c_lo = c; } else { hi = t; c_hi = c; }
-                done = c == T || hi - lo == 1;
+                if (c >= T) {
+                    lo = t; c_lo = c;
+                    w_lo = static_cast<float>(c - T) + 0.5f;
+                    if (side > 0) w_hi *= 0.5f;
+                    side = 1;
+                } else {
+                    hi = t; c_hi = c;
+                    w_hi = static_cast<float>(T - c) - 0.5f;
+                    if (side < 0) w_lo *= 0.5f;
+                    side = -1;
+                }
+                done = c == T || hi - lo == 1 || c_lo - c_hi <= kFewKeys;
             }
         }
         // keys at or above lo; the kept set when there are exactly T of them
@@ -814,7 +828,7 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
         unsigned ge[2] = {0u, 0u};
 #pragma unroll
         for (int j = 0; j < 32; ++j) ge[j >> 4] |= ge_mask_bf16x2(hk[j], t2) & (0x00010001u << (j & 15));
-        int need = live && c_lo != T ? T - c_hi : 0;           // keys of upper half `lo` to admit
+        int need = live && c_lo != T ? T - c_hi : 0;           // keys between the ends to admit
         kept[0] &= ge[0]; kept[1] &= ge[1];
         if (__any_sync(kFullMask, need > 0)) {
             const unsigned u2 = static_cast<unsigned>(hi) * 0x00010001u;
