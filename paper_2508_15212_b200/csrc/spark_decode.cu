@@ -109,15 +109,12 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
     prefetch_block_table(A, tid, kDecodeThreads);
     if (warp == kConsumerWarps) {
-        producer_prologue(A, C, lane, kDecodeThreads);
-        int p0, p1;
-        cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), p0, p1);
-        producer_loop<kConsumerWarps>(A, C, ring, p0, p1, lane);
+        const CtaRun run = producer_prologue(A, C, lane, kDecodeThreads);
+        producer_loop<kConsumerWarps>(A, C, ring, run, lane);
         return;
     }
     consumer_wait_plan(kDecodeThreads);
-    int c0, c1;
-    cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
+    const int c0 = C.run->c0, c1 = C.run->c1;
     if (!A.late_wait) {
         grid_wait();                                       // q, qnorm, out and the workspace from here on
         write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
@@ -125,7 +122,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
     float* pscr = pscr_all + warp * 32 * GPP;
     for (int g = c0; g < c1;) {
-        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, g, c1);
+        const Epoch ep = make_epoch(C.prefix, A.Hkv, A.cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
 
         // ---- per-unit table: entry j = { q_0[j]*c, ..., q_{G-1}[j]*c, 1/a[j] },  c = scale*log2(e)
         UnitRef u = ep.first;
@@ -172,7 +169,6 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
         int eu = 0;
         while (pos < pos_end && pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
         while (pos < pos_end) {
-            u = locate_unit(C.prefix, A.B, A.Hkv, pos);    // (found again for each part: nothing of it stays in registers)
             const int part_end = min(pos_end, u.start + u.steps);
             const int b = u.b, h = u.h, len = C.lens[u.b];
             const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kTab + eu * S::kTabBytes);
@@ -358,6 +354,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
                 }
             }
             ++eu;
+            if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kConsumerThreads>();
         merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, C.epoch[1], tid);
@@ -410,6 +407,7 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     A.slot_stride = static_cast<int>(align_up(2 * static_cast<size_t>(A.L.page_bytes), 128));
     const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    set_divisors(A, units, grid);
     // Two units per epoch only where CTAs hold several: the second unit's table and records cost a ring slot (of six or
     // seven: 2 x 7926 tokens, G = 4, T = 89: 43.9 us with six slots, 35.2 us with seven).
     A.whole_steps = 0;                                     // (a step is 32 tokens of double sums: splitting pays)

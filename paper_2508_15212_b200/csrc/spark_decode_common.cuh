@@ -22,6 +22,19 @@ constexpr int kRec = kHeadDim + 4;           // floats per head record: 128 outp
 constexpr int kMaxCap = 8;                    // units per epoch, at most (see Epoch)
 constexpr float kLn2 = 0.6931471805599453f;
 
+// Division of 0 <= x < 2^32 by a divisor the host knows: a multiply and a correction (an integer division is some
+// 130 cycles, and seven of them stood in a row between the plan and a CTA's first page copy).
+struct FastDiv {
+    unsigned d, m;
+    static FastDiv of(unsigned d) { FastDiv f; f.d = d; f.m = d > 1 ? static_cast<unsigned>((1ull << 32) / d) : 0xffffffffu; return f; }
+    __device__ __forceinline__ int div(int x) const
+    {
+        unsigned q = __umulhi(static_cast<unsigned>(x), m);          // the quotient or one less
+        if (static_cast<unsigned>(x) - q * d >= d) ++q;
+        return static_cast<int>(q);
+    }
+};
+
 struct DecodeArgs {
     const void* q;
     const unsigned char* pages;
@@ -43,6 +56,9 @@ struct DecodeArgs {
     int nslots;
     int slot_stride;
     int pps;                                 // pages per step (= per ring slot): 1 or 2
+    FastDiv by_grid, by_hkv;                 // CTAs of the grid; KV heads
+    int per_unit, extra;                     // aligned mode (see Plan): CTAs per unit; units with one more
+    FastDiv by_q, by_q1;                     // per_unit and per_unit + 1
     int cap;                                 // units per epoch
     int whole_steps;                         // a step per consumer warp; units up to this are not split (see Plan)
     int tab_off;                             // shared-memory offset of the epoch's operand tables
@@ -242,12 +258,12 @@ struct Epoch {
     int n_units;
     UnitRef first;
 };
-__device__ __forceinline__ Epoch make_epoch(const int* prefix, int B, int Hkv, int cap, int g, int c1)
+__device__ __forceinline__ Epoch make_epoch(const int* prefix, int Hkv, int cap, const UnitRef& first, int g, int c1)
 {
     Epoch ep;
     ep.e0 = g;
-    ep.first = locate_unit(prefix, B, Hkv, g);
-    UnitRef u = ep.first;
+    ep.first = first;
+    UnitRef u = first;
     ep.n_units = 1;
     int end = u.start + u.steps;
 #pragma unroll 1
@@ -284,6 +300,12 @@ struct Plan {
     int q, rem;       // aligned: CTAs per unit
 };
 
+// A CTA's run of steps [c0, c1) on the line and the unit of its first step.
+struct CtaRun {
+    int c0, c1;
+    UnitRef first;           // meaningful when c0 < c1
+};
+
 struct Ctrl {
     uint64_t* full;
     uint64_t* empty;
@@ -293,6 +315,7 @@ struct Ctrl {
     Plan* plan;
     volatile int* epoch;      // [2] the epoch's end and its number of units
     EpochUnit* units;         // [kMaxCap]
+    CtaRun* run;
     int* prefix;              // [B + 1] steps before each sequence (of one KV head)
     int* lens;                // [B] clamped lengths
 };
@@ -308,6 +331,8 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, i
     c.epoch = reinterpret_cast<volatile int*>(smem + 600);
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
     c.units = reinterpret_cast<EpochUnit*>(smem + 768);
+    c.run = reinterpret_cast<CtaRun*>(smem + 960);
+    static_assert(768 + kMaxCap * sizeof(EpochUnit) <= 960 && 960 + sizeof(CtaRun) <= kCtrlBytes, "control block");
     c.prefix = reinterpret_cast<int*>(smem + prefix_off);
     c.lens = c.prefix + B + 1;
     return c;
@@ -337,14 +362,25 @@ __device__ __forceinline__ void prefetch_block_table(const DecodeArgs& A, int ti
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + o));
 }
 
-__device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads)
+__device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads)
 {
     const int max_tokens = A.max_blocks * kPageTokens;
     if (lane < A.nslots) { mbar_init(&C.full[lane], 1); mbar_init(&C.empty[lane], 1); }
     C.seq[lane] = 0;
-    if (lane == 0) *C.abort_flag = 0;
+    if (lane == 0) { *C.abort_flag = 0; C.prefix[0] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // what does not depend on the lengths, before the wait: this CTA's unit in whole-unit mode (wb, wh), and its unit, its
+    // place k among the unit's n CTAs in aligned mode
+    const int cta = static_cast<int>(blockIdx.x), nct = static_cast<int>(gridDim.x), units = A.B * A.Hkv;
+    const int wb = A.by_hkv.div(cta), wh = cta - wb * A.Hkv;
+    int u = 0, k = 0, n = 1, ub = 0;
+    if (A.per_unit > 0) {
+        const int big = A.extra * (A.per_unit + 1);                 // CTAs that belong to units with q + 1 CTAs
+        if (cta < big) { u = A.by_q1.div(cta); k = cta - u * (A.per_unit + 1); n = A.per_unit + 1; }
+        else { const int v = A.by_q.div(cta - big); u = A.extra + v; k = cta - big - v * A.per_unit; n = A.per_unit; }
+        ub = A.by_hkv.div(u);
+    }
     if (!A.overlap) grid_wait();                           // with the flag the page stream does not depend on the kernel before
     grid_release();
     int running = 0, smin = 0x7fffffff, smax = 0;
@@ -361,66 +397,52 @@ __device__ __forceinline__ void producer_prologue(const DecodeArgs& A, const Ctr
             smax = max(smax, st);
         }
         int inc = st;
+        if (A.B > 1)
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int n = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += n;
-        }
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += x;
+            }
         if (b < A.B) C.prefix[b + 1] = running + inc;
-        running += __shfl_sync(kFull, inc, 31);
+        running += __shfl_sync(kFull, inc, A.B > 1 ? 31 : 0);
     }
     smin = __reduce_min_sync(kFull, smin);
     smax = __reduce_max_sync(kFull, smax);
-    if (lane == 0) {
-        C.prefix[0] = 0;
-        Plan pl;
-        const int nct = static_cast<int>(gridDim.x), units = A.B * A.Hkv;
-        pl.total = A.Hkv * running;
-        pl.chunk = (pl.total + nct - 1) / nct;
-        pl.aligned = 0; pl.unit_steps = smax; pl.q = 0; pl.rem = 0;
-        if (units <= nct && (smax <= A.whole_steps || (2 * units > nct && smax <= 3 * A.whole_steps))) {
-            pl.aligned = 2;
-        } else if (smin == smax && smax > 0 && units <= nct) {
-            const int q = nct / units;
-            const int makespan = (smax + q - 1) / q;
-            if (q >= 2 && makespan * 25 <= pl.chunk * 26) {          // within 4 % of the even split
-                pl.aligned = 1; pl.q = q; pl.rem = nct - q * units;
-            }
-        }
-        *C.plan = pl;
+    __syncwarp();                                          // the prefix is written
+    Plan pl;                                               // (the same in every lane)
+    pl.total = A.Hkv * running;
+    pl.chunk = A.by_grid.div(pl.total + nct - 1);
+    pl.aligned = 0; pl.unit_steps = smax; pl.q = A.per_unit; pl.rem = A.extra;
+    CtaRun run;
+    run.first.b = run.first.h = run.first.start = run.first.steps = 0;
+    if (units <= nct && (smax <= A.whole_steps || (2 * units > nct && smax <= 3 * A.whole_steps))) {
+        pl.aligned = 2;
+        run.first.b = wb; run.first.h = wh;
+        run.first.steps = wb < A.B ? C.prefix[wb + 1] - C.prefix[wb] : 0;
+        run.first.start = wb < A.B ? A.Hkv * C.prefix[wb] + wh * run.first.steps : 0;
+        run.c0 = run.first.start;
+        run.c1 = run.c0 + run.first.steps;
+    } else if (smin == smax && smax > 0 && A.per_unit >= 2 && A.by_q.div(smax + A.per_unit - 1) * 25 <= pl.chunk * 26) {
+        pl.aligned = 1;                                    // the longest share is within 4 % of the even split
+        const int per = (n == A.per_unit ? A.by_q : A.by_q1).div(smax + n - 1);
+        run.first.b = ub; run.first.h = u - ub * A.Hkv; run.first.steps = smax; run.first.start = u * smax;
+        run.c0 = run.first.start + min(smax, k * per);
+        run.c1 = run.first.start + min(smax, (k + 1) * per);
+    } else {
+        run.c0 = min(pl.total, cta * pl.chunk);
+        run.c1 = min(pl.total, run.c0 + pl.chunk);
+        if (run.c0 < run.c1) run.first = locate_unit(C.prefix, A.B, A.Hkv, run.c0);
     }
+    if (lane == 0) { *C.plan = pl; *C.run = run; }
     __syncwarp();
     asm volatile("bar.arrive %0, %1;" ::"n"(kPlanBarrier), "r"(n_threads) : "memory");
+    return run;
 }
 
 // consumer side of the prologue: returns once the plan, the prefix and the ring barriers are in place
 __device__ __forceinline__ void consumer_wait_plan(int n_threads)
 {
     asm volatile("bar.sync %0, %1;" ::"n"(kPlanBarrier), "r"(n_threads) : "memory");
-}
-
-// This CTA's run of steps [c0, c1) on the line.
-__device__ __forceinline__ void cta_range(const Plan& pl, const int* prefix, int B, int Hkv, int cta, int& c0, int& c1)
-{
-    if (pl.aligned == 2) {
-        const int b = cta / Hkv, h = cta - b * Hkv;
-        const int steps = b < B ? prefix[b + 1] - prefix[b] : 0;
-        c0 = b < B ? Hkv * prefix[b] + h * steps : 0;
-        c1 = c0 + steps;
-        return;
-    }
-    if (!pl.aligned) {
-        c0 = min(pl.total, cta * pl.chunk);
-        c1 = min(pl.total, c0 + pl.chunk);
-        return;
-    }
-    const int big = pl.rem * (pl.q + 1);                   // CTAs that belong to units with q+1 CTAs
-    int u, k, n;
-    if (cta < big) { u = cta / (pl.q + 1); k = cta - u * (pl.q + 1); n = pl.q + 1; }
-    else { u = pl.rem + (cta - big) / pl.q; k = (cta - big) - (u - pl.rem) * pl.q; n = pl.q; }
-    const int per = (pl.unit_steps + n - 1) / n;
-    c0 = u * pl.unit_steps + min(pl.unit_steps, k * per);
-    c1 = u * pl.unit_steps + min(pl.unit_steps, (k + 1) * per);
 }
 
 // The CTAs that hold a part of the unit starting at step `unit_start` with `unit_steps` steps.
@@ -475,10 +497,10 @@ __device__ __forceinline__ void producer_page_ids(const DecodeArgs& A, const Ctr
 
 template <int NW>
 __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C, unsigned char* ring,
-                                              int c0, int c1, int lane)
+                                              const CtaRun& run, int lane)
 {
     const PageLayout L = A.L;
-    const int NS = A.nslots, n_total = c1 - c0;
+    const int c0 = run.c0, c1 = run.c1, NS = A.nslots, n_total = c1 - c0;
     const uint64_t policy = policy_evict_first();
     const bool owner = lane < NS;
     unsigned char* dst = ring + static_cast<size_t>(lane) * A.slot_stride;
@@ -489,12 +511,14 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
     int id0 = -1, id1 = -1;
     unsigned n0 = 0, n1 = 0;                               // bytes to copy of the two pages
     Epoch ep;
-    ep.e1 = c0;                                            // no epoch yet
+    ep.e1 = c0;                                            // (a CTA without steps has no first unit)
+    if (n_total > 0) ep = make_epoch(C.prefix, A.Hkv, A.cap, run.first, c0, c1);
     // this lane's ring step n -> its step of the line (epoch, warp, place in the warp's run) -> page ids
     auto lookup = [&](int n) {
         id0 = id1 = -1; n0 = n1 = 0;
         if (!owner || n >= n_total) return;
-        while (c0 + n >= ep.e1) ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, ep.e1, c1);
+        while (c0 + n >= ep.e1)
+            ep = make_epoch(C.prefix, A.Hkv, A.cap, locate_unit(C.prefix, A.B, A.Hkv, ep.e1), ep.e1, c1);
         int g = c0 + n;
         if (A.cap > 1) {
             const int len = ep.e1 - ep.e0, q = len / NW, r = len - q * NW;
@@ -509,9 +533,8 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
     // loads, so it runs before revolution r is polled (hidden behind the wait for free slots), except at the start,
     // where every slot is free and the first copies go out before the second lookup: ids 0 | copies 0 | ids 1 |
     // ids 2, copies 1 | ids 3, copies 2 ...   (One loop body: this code runs cold, its size is start-up time.)
-    const int n_rounds = (n_total + NS - 1) / NS;
 #pragma unroll 1
-    for (int t = 0; t < n_rounds + 2; ++t) {
+    for (int t = 0; t < 2 || (t - 2) * NS < n_total; ++t) {
         const int round = t == 1 ? 0 : t - 2;              // revolution whose copies go out in this pass (t = 0, 2: none)
         const int cur0 = id0, cur1 = id1;
         const unsigned b0 = n0, b1 = n1;
@@ -824,6 +847,16 @@ inline int decode_grid(int n_sms, int64_t units, int max_blocks, int pps)
     const int64_t total = units * ((max_blocks + pps - 1) / pps);
     const int64_t g = total < n_sms ? total : n_sms;
     return g < 1 ? 1 : (g > kMaxCtas ? kMaxCtas : static_cast<int>(g));
+}
+
+inline void set_divisors(DecodeArgs& A, int64_t units, int grid)
+{
+    A.by_grid = FastDiv::of(grid);
+    A.by_hkv = FastDiv::of(A.Hkv);
+    A.per_unit = static_cast<int>(grid / units);
+    A.extra = A.per_unit > 0 ? static_cast<int>(grid - A.per_unit * units) : 0;
+    A.by_q = FastDiv::of(A.per_unit > 0 ? A.per_unit : 1);
+    A.by_q1 = FastDiv::of(A.per_unit + 1);
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

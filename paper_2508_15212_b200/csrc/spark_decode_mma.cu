@@ -241,15 +241,12 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
     prefetch_block_table(A, tid, kThreads);
     if (warp == kNW) {
-        producer_prologue(A, C, lane, kThreads);
-        int p0, p1;
-        cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), p0, p1);
-        producer_loop<kNW>(A, C, ring, p0, p1, lane);
+        const CtaRun run = producer_prologue(A, C, lane, kThreads);
+        producer_loop<kNW>(A, C, ring, run, lane);
         return;
     }
     consumer_wait_plan(kThreads);
-    int c0, c1;
-    cta_range(*C.plan, C.prefix, A.B, A.Hkv, static_cast<int>(blockIdx.x), c0, c1);
+    const int c0 = C.run->c0, c1 = C.run->c1;
     if (!A.late_wait) {
         grid_wait();                                       // q, qnorm, out and the workspace from here on
         write_empty_sequences<kNT>(A, C.prefix, tid);
@@ -257,7 +254,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
     for (int g = c0; g < c1;) {
-        const Epoch ep = make_epoch(C.prefix, A.B, A.Hkv, A.cap, g, c1);
+        const Epoch ep = make_epoch(C.prefix, A.Hkv, A.cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
         // ---- the epoch's operand tables: a warp prepares one query head of one unit at a time, the next one's loads
         //      in flight meanwhile (first pass: only loads) ----
         {
@@ -290,14 +287,13 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
         int pos = ep.e0 + (A.cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
         const int pos_end = A.cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
         const int stride = A.cap == 1 ? kNW : 1;
-        int slot = (ep.e0 - c0) + warp, round = slot / NS;     // ring position of the warp's next step, kept incrementally
+        int slot = (ep.e0 - c0) + warp, round = slot < NS ? 0 : slot / NS;     // ring position of the warp's next step, kept incrementally
         slot -= round * NS;
         if (warp == kNW - 1) describe_epoch<kNW>(A, C, ep, lane);     // for the merge; this warp's run is never the longer
         UnitRef u = ep.first;
         int eu = 0;
         while (pos < pos_end && pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
         while (pos < pos_end) {
-            u = locate_unit(C.prefix, A.B, A.Hkv, pos);    // (found again for each part: nothing of it stays in registers)
             const int part_end = min(pos_end, u.start + u.steps);
             const int cnt = A.cap == 1 ? (part_end - pos + kNW - 1) / kNW : part_end - pos;      // steps of this warp, >= 1
             pos += cnt * stride;
@@ -509,6 +505,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
                     }
             }
             ++eu;
+            if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kNT>();
         merge_and_publish<G, kNW>(A, C, merge, unit_ml, C.epoch[1], tid);
@@ -562,6 +559,7 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
     A.slot_stride = static_cast<int>(align_up(static_cast<size_t>(A.L.page_bytes), 128));
     const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
+    set_divisors(A, units, grid);
     A.whole_steps = kNW;
     A.cap = epoch_cap(A.B, units, A.max_blocks, grid);
     // An epoch's units take shared memory (operand tables, records) from the ring.  Where a CTA's run is long, a unit
