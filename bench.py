@@ -9,9 +9,10 @@ outside the timed region (prefill side); its time is reported under "compress". 
 copies of the packed cache so that each launch reads cold data (copies * bytes >= 4 * L2).
 
 Timing.  The steps are captured in CUDA graphs and timed with CUDA events on the launching stream:
-  value          exactly K steps in one region bracketed by barrier + synchronize, ORDINARY launches;
+  value          exactly K steps in one region bracketed by barrier + synchronize; every step
+                 waits for the one before it to complete;
   replays        the same graph replayed >= 50 times, each replay timed on its own: median and minimum;
-  value_pdl      the same K steps launched with SPARK_FLAG_OVERLAP_PREVIOUS (programmatic dependent launch:
+  value_pdl      the same K steps launched with SPARK_FLAG_OVERLAP_PREVIOUS (no wait for the step before:
                  step i+1 may start its page stream while step i drains), a pipelined-throughput figure that
                  holds only when the kernel enqueued before the step does not write the cache.
 With the default workload (the 32K headline configuration) the run also times the 4x128K, the evicted
@@ -607,12 +608,12 @@ def main():
             "warmup": max(args.warmup, 3), "ms_per_step": us_step / 1e3, "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "storage_dtype": cfg["dtype"], "data": "synthetic",
             "config": dict(workload_desc(cfg, keep, work.copies, keep_v),
-                           launch="ordinary launches, K steps replayed from CUDA graphs",
+                           launch="each step waits for the one before, K steps replayed from CUDA graphs",
                            **({"variant": {k_: v_ for k_, v_ in variant.items() if v_}} if variant else {})),
             "replays": {"n": t_plain["replays"], "steps_per_replay": t_plain["steps_per_replay"],
                         "median_us_per_step": t_plain["median_us"], "min_us_per_step": t_plain["min_us"]},
             "value_pdl": t_pdl["us_step"],
-            "value_pdl_note": ("same steps with SPARK_FLAG_OVERLAP_PREVIOUS (programmatic dependent launch): step i+1 "
+            "value_pdl_note": ("same steps with SPARK_FLAG_OVERLAP_PREVIOUS (no wait for the step before): step i+1 "
                                "starts its page stream while step i drains; valid only when the kernel enqueued before "
                                "the step does not write the cache, so it is not the headline"),
             "hbm_gbs": gbs, "hbm_gbs_all_gpus": dist_utils.aggregate_throughput(work.alg_bytes / 1e9, world, us_step * 1e-6),

@@ -379,7 +379,7 @@ struct CompressArgs {
     int* status;
 };
 
-template <typename E, bool kRank>
+template <typename E>
 __global__ void __launch_bounds__(256) compress_pages_kernel(CompressArgs A)
 {
     grid_wait();
@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(256) compress_pages_kernel(CompressArgs A)
             ? A.gather[(static_cast<int64_t>(b) * A.Hkv + h) * A.gather_stride + t] : t;
         const int64_t row = static_cast<int64_t>(b) * A.sb + static_cast<int64_t>(h) * A.sh +
                             static_cast<int64_t>(src_t) * A.st + lane * 4;
-        const int n_kept = pack_token_kv<kBf16, kRank>(image, L, p, lane, a, A.k, A.v, row, A.inv_pruned, A.sel);
-        if (kRank && L.ragged && lane == 0) atomicMax(&rows_used, n_kept);
+        const int n_kept = pack_token_kv<kBf16, true>(image, L, p, lane, a, A.k, A.v, row, A.inv_pruned, A.sel);
+        if (L.ragged && lane == 0) atomicMax(&rows_used, n_kept);
     }
     __syncthreads();
 
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(256) compress_pages_kernel(CompressArgs A)
     uint4* dst = reinterpret_cast<uint4*>(A.pages + page_id * L.page_bytes);
     for (int i = threadIdx.x; i < L.page_bytes / 16; i += blockDim.x)
         dst[i] = reinterpret_cast<const uint4*>(image)[i];
-    if (kRank && L.ragged && threadIdx.x == 0)
+    if (L.ragged && threadIdx.x == 0)
         reinterpret_cast<int*>(A.pages + rows_offset(A.n_pool_pages, L.page_bytes))[page_id] = rows_used;
 }
 
@@ -1694,10 +1694,10 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const dim3 grid(n_blocks, p.n_kv_heads, p.batch);
     const bool rank = p.select != SPARK_SELECT_FIXED;      // a ratio-free rule: the kernels with the rank sort
     if (p.dtype == SPARK_BF16) {
-        if (rank) launch_kernel(compress_pages_kernel<__nv_bfloat16, true>, grid, dim3(256), A.L.page_bytes, stream, A);
+        if (rank) launch_kernel(compress_pages_kernel<__nv_bfloat16>, grid, dim3(256), A.L.page_bytes, stream, A);
         else launch_kernel(compress_pages4_kernel<__nv_bfloat16>, grid, dim3(128), A.L.page_bytes, stream, A);
     } else {
-        if (rank) launch_kernel(compress_pages_kernel<float, true>, grid, dim3(256), A.L.page_bytes, stream, A);
+        if (rank) launch_kernel(compress_pages_kernel<float>, grid, dim3(256), A.L.page_bytes, stream, A);
         else launch_kernel(compress_pages4_kernel<float>, grid, dim3(128), A.L.page_bytes, stream, A);
     }
     ++*launches;

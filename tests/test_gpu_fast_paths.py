@@ -1,0 +1,75 @@
+"""The selection searches, the division of a decode step among CTAs and the eviction's select kernel at the sizes where
+they change branch, against the oracle with the bars of test_gpu_parity.py."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2508_15212_b200.cache import SparkCache
+from test_gpu_parity import built, check_case, check_eviction_case, make, to_np  # noqa: F401  (built: module fixture)
+
+pytestmark = pytest.mark.gpu
+
+LENS = [1, 15, 16, 17, 63]
+
+
+def tied_workload(kind, seed):
+    """Saliencies with many exact ties ("equal"), or distinct ones that share their upper 16 bits ("near")."""
+    wl = make("bf16", len(LENS), 8, 2, LENS, 8, 64, seed=seed, gap=False)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    sign = torch.where(torch.rand(wl.k.shape, generator=g, device="cuda") < 0.5, -1.0, 1.0)
+    if kind == "equal":
+        wl.q_win = torch.full_like(wl.q_win, 2.0)
+        wl.q_win[..., ::3] = 1.0
+        wl.k = (sign * 2.0 ** torch.randint(-1, 2, wl.k.shape, generator=g, device="cuda")).to(wl.k.dtype)
+        wl.k[2] = 0.0                                            # a sequence of all-zero keys
+    else:
+        wl.q_win = (1.0 + 2.0 ** -7 * torch.randint(0, 3, wl.q_win.shape, generator=g, device="cuda")).to(wl.q_win.dtype)
+        wl.k = sign.to(wl.k.dtype)
+    wl.v = (torch.randint(-2, 3, wl.v.shape, generator=g, device="cuda")).to(wl.v.dtype)
+    return wl
+
+
+@pytest.mark.parametrize("kind", ["equal", "near"])
+@pytest.mark.parametrize("keep,keep_v", [(1, 0), (25, 127), (64, 64), (127, 1), (128, 100)])
+def test_fixed_selection_with_ties(kind, keep, keep_v):
+    check_case(tied_workload(kind, 200 + keep), keep, keep_v=keep_v)
+
+
+@pytest.mark.parametrize("kind", ["equal", "near"])
+@pytest.mark.parametrize("p,cap", [(0.01, 128), (0.5, 128), (0.95, 128), (1.0, 128), (0.95, 40)])
+def test_top_p_selection_with_ties(kind, p, cap):
+    """Exact sums (few distinct powers of two) or sums far from the goal: the kept sets must be the oracle's."""
+    wl = tied_workload(kind, 300)
+    wl_cpu = wl.to("cpu")
+    _, a = oracle.window_mean(wl_cpu.q_win, 2)
+    ref = oracle.select_variant(wl_cpu.k, wl_cpu.seq_lens, a, top_p=p, cap=cap)
+    cache = SparkCache(batch=len(LENS), n_q_heads=8, n_kv_heads=2, window=8, keep=cap, dtype="bf16", max_tokens=max(LENS), top_p=p,
+                       guard=True)
+    cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    u = cache.unpack(want_v=False)
+    assert cache.status() == 0 and cache.broken_guards() == []
+    assert np.array_equal(u["mask"].cpu().numpy().view(np.uint32), ref["mask"])
+    assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("name,Hq,Hkv,lens", [
+    ("units of at most a step per warp", 8, 4, [240, 1, 0, 17]),
+    ("units up to three steps per warp that fill the grid", 16, 8, [60 + 42 * i for i in range(16)]),
+    ("one step more than that", 16, 8, [721] + [60 + 42 * i for i in range(15)]),
+    ("short ragged units, several per CTA", 8, 4, [4000, 150, 700, 1300, 16, 0, 2900, 333]),
+    ("more tiny units than an epoch holds", 16, 8, [1 + (7 * i) % 40 for i in range(60)]),
+    ("seven heads per group", 28, 4, [100 + 97 * i for i in range(20)]),
+])
+def test_division_of_the_step(name, Hq, Hkv, lens):
+    check_case(make("bf16", len(lens), Hq, Hkv, lens, 8, 64, seed=400 + len(lens), gap=False), 64, check_vals=False)
+
+
+@pytest.mark.parametrize("lens,W,budget,G,pool", [
+    ([1500, 900], 8, 8, 4, 7),              # the window alone
+    ([5000, 4100], 16, 600, 2, 601),        # pooling wider than the staging tile's halo
+    ([9000], 4, 1025, 1, 1),                # no pooling, a share that is not full
+    ([300001], 4, 64, 1, 7),                # a share beyond shared memory
+])
+def test_eviction_select_edges(lens, W, budget, G, pool):
+    check_eviction_case("bf16", lens, W, budget, G, Hkv=1 if lens[0] > 100000 else 2, pool=pool, seed=500)
