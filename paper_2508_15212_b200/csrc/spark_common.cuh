@@ -129,13 +129,21 @@ template <> struct TailAcc<__nv_bfloat16> { using type = float; };
 constexpr int kTailMax = 128;         // tokens of a dense tail that tail_attn_kernel takes
 
 // Programmatic dependent launch.  Every kernel of the library is launched so that it may become resident while the
-// kernel before it on the stream drains, and waits at its top, before it reads or writes anything of a caller's
-// (grid_wait: returns once that kernel has completed and its writes are visible; nothing to wait for under an
-// ordinary predecessor).  So the order of a stream is unchanged and the launch latency and a kernel's own set-up
-// (barrier initialisation) run under the predecessor's last CTAs: back-to-back decode steps on one stream went
+// kernel before it on the stream drains (grid_release lets the next kernel become resident; grid_wait returns once the
+// kernel before has completed and its writes are visible, at once under an ordinary predecessor), so that the launch
+// latency and a kernel's own set-up run under the predecessor's last CTAs: back-to-back decode steps on one stream went
 // from 27.0 to 25.4 us (1 x 32K tokens), from 14.35 to 12.7 us (fp32, 1024 tokens); append + decode 44.5 to 40.9 us.
-// grid_release lets the next kernel become resident; it comes AFTER the wait, so a kernel whose predecessor has
-// released it may rely on everything enqueued before that predecessor.
+//   Rule: a kernel releases only behind its own wait.  So a kernel that has started may rely on everything enqueued
+// before its predecessor, and the order of a stream is unchanged for every kernel that waits at its top, before it
+// touches anything of a caller's.  All do, with these exceptions, each of which reads early only what its predecessor
+// cannot write:
+//   - compress_pages_warp_kernel without eviction: keys, values, lengths and block table; behind the window norm;
+//   - evict_scores_tc_kernel<2>: queries, keys and lengths; behind pass 1 of the same call;
+//   - a decode step with SPARK_FLAG_OVERLAP_PREVIOUS: lengths, block table and pages; the caller vouches for the
+//     predecessor.  Its consumers wait and release, not its producer (consumer_wait_previous);
+//   - a decode step merged with a dense tail (late_wait): everything but the tail's result; behind tail_attn_kernel, which
+//     writes nothing else.  The one kernel that releases before it waits: its successor may rely on everything enqueued
+//     before the tail kernel, and not on the tail's result, which only this step reads.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

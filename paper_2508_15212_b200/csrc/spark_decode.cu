@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     consumer_wait_plan(kDecodeThreads);
     const int c0 = C.run->c0, c1 = C.run->c1;
     if (!A.late_wait) {
-        grid_wait();                                       // q, qnorm, out and the workspace from here on
+        consumer_wait_previous(A);                         // q, qnorm, out and the workspace from here on
         write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
     }
 

@@ -64,7 +64,8 @@ struct DecodeArgs {
     int tab_off;                             // shared-memory offset of the epoch's operand tables
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix)
-    int late_wait;                           // the kernel before writes only other_out / other_lse: wait where they are read
+    int late_wait;                           // the kernel before waited at its top, released after that and writes only other_out /
+                                             // other_lse: wait where they are read (a successor may be released before that)
     int overlap;                             // the page stream need not wait for the kernel before (SPARK_FLAG_OVERLAP_PREVIOUS)
     unsigned seed;                           // sampled recovery: seed of the per-entry draws
     const int* page_rows;                    // ragged pages: slot rows in use per pool page (else null: whole pages)
@@ -382,7 +383,7 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
         ub = A.by_hkv.div(u);
     }
     if (!A.overlap) grid_wait();                           // with the flag the page stream does not depend on the kernel before
-    grid_release();
+    if (!A.overlap || A.late_wait) grid_release();         // (otherwise the consumers release, see consumer_wait_previous)
     int running = 0, smin = 0x7fffffff, smax = 0;
 #pragma unroll 1
     for (int b0 = 0; b0 < A.B; b0 += 32) {
@@ -443,6 +444,16 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
 __device__ __forceinline__ void consumer_wait_plan(int n_threads)
 {
     asm volatile("bar.sync %0, %1;" ::"n"(kPlanBarrier), "r"(n_threads) : "memory");
+}
+
+// Consumers of a step without a late wait: what the kernel before writes is complete from here on.  A step whose page
+// stream started early (SPARK_FLAG_OVERLAP_PREVIOUS) releases its successor only here: released at its top, the successor
+// could start, and with the flag read its own cache, while a kernel two places ahead of it (an append to that cache, itself
+// released early) was still writing; the flag only promises something of the kernel just before.
+__device__ __forceinline__ void consumer_wait_previous(const DecodeArgs& A)
+{
+    grid_wait();
+    if (A.overlap) grid_release();
 }
 
 // The CTAs that hold a part of the unit starting at step `unit_start` with `unit_steps` steps.

@@ -248,7 +248,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     consumer_wait_plan(kThreads);
     const int c0 = C.run->c0, c1 = C.run->c1;
     if (!A.late_wait) {
-        grid_wait();                                       // q, qnorm, out and the workspace from here on
+        consumer_wait_previous(A);                         // q, qnorm, out and the workspace from here on
         write_empty_sequences<kNT>(A, C.prefix, tid);
     }
 

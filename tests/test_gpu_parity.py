@@ -349,6 +349,38 @@ def test_overlap_flag_gives_identical_results_back_to_back():
         SparkCache(batch=1, n_q_heads=4, n_kv_heads=1, window=4, keep=64, dtype="bf16", max_tokens=64, flags=6)
 
 
+@pytest.mark.parametrize("writer", ["append", "append_block", "compress"])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_overlap_flag_with_a_writer_two_calls_ahead(dtype, writer):
+    """A call that writes cache A, a flagged step of another cache, a flagged step of A: both steps keep the flag's
+    condition (the kernel just before writes no page of theirs), so every output is that of the calls without it."""
+    wl = make(dtype, 2, 8, 2, [200, 120], 8, 64, seed=141, gap=False)
+    other = make(dtype, 1, 8, 2, [40], 8, 64, seed=142, gap=False)
+    blocks = [(wl.k[:, :, 8 * i:8 * i + 8].contiguous(), wl.v[:, :, 8 * i:8 * i + 8].contiguous()) for i in range(15)]
+    prompts = [torch.roll(wl.k, 3 * i, 2).contiguous() for i in range(15)]
+    outs = []
+    for flags in (0, B.SPARK_FLAG_OVERLAP_PREVIOUS):
+        kw = dict(n_q_heads=8, n_kv_heads=2, window=8, keep=64, dtype=dtype, flags=flags)
+        a, b = SparkCache(batch=2, max_tokens=400, **kw), SparkCache(batch=1, max_tokens=40, **kw)
+        a.max_src_tokens = 200
+        a.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+        b.compress(other.q_win, other.k, other.v, other.seq_lens)
+        got = [torch.empty(2, 8, 128, device="cuda") for _ in range(15)]
+        torch.cuda.synchronize()
+        for i, (kb, vb) in enumerate(blocks):                  # enqueued without a wait of the host
+            if writer == "append":
+                a.append(kb[:, :, 0].contiguous(), vb[:, :, 0].contiguous())
+            elif writer == "append_block":
+                a.append_block(kb, vb)
+            else:
+                a.compress(wl.q_win, prompts[i], wl.v, wl.seq_lens)
+            b.decode(other.q)
+            a.decode(wl.q, out=got[i])
+        assert a.status() == 0 and b.status() == 0
+        outs.append(torch.stack(got))
+    assert torch.equal(outs[0], outs[1])
+
+
 @pytest.mark.parametrize("dtype,keep", [("bf16", 64), ("bf16", 25), ("f32", 38)])
 def test_append_tokens_equals_compressing_the_longer_sequence(dtype, keep):
     """Prefill S0 tokens, append n more one at a time: the cache must equal what pruning all S0 + n
