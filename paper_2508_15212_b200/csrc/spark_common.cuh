@@ -163,6 +163,32 @@ inline cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 bloc
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
+// Device properties the launchers need, looked up once per device and then served from a table
+// (spark_decode.cu); `dev` is the current device.
+constexpr int kMaxDevices = 64;
+struct DeviceInfo { int n_sms; int smem_optin; };
+bool device_info(int* dev, DeviceInfo* info);
+
+// Raises a kernel's dynamic shared-memory limit to all that the device gives beside its static part, once per device and
+// kernel.  (Setting it to what a launch needs, launch by launch, lets one thread lower it between another's call and launch.)
+template <typename Kernel> inline bool allow_max_smem(Kernel kernel, int dev, int smem_optin, unsigned char (&done)[kMaxDevices])
+{
+    if (dev < 0 || dev >= kMaxDevices) return false;
+    if (done[dev]) return true;                           // a racing first call only repeats the same setting
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, kernel) != cudaSuccess) return false;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - static_cast<int>(at.sharedSizeBytes)) != cudaSuccess)
+        return false;
+    done[dev] = 1;
+    return true;
+}
+template <typename Kernel> inline bool allow_max_smem(Kernel kernel, unsigned char (&done)[kMaxDevices])
+{
+    int dev = 0;
+    DeviceInfo info;
+    return device_info(&dev, &info) && allow_max_smem(kernel, dev, info.smem_optin, done);
+}
+
 // host-side validation of a parameter block (spark_api.cu)
 spark_status check_params(const spark_params* p);
 

@@ -1684,8 +1684,8 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
         if (!evict) A.lens = seq_lens;                         // readable before the window norm has ended
         const size_t smem = kHeadDim * 4 + kWarpPageWarps * (kTileBytes + static_cast<size_t>(topp ? warp_topp_room(A.L) : (pv ? A.L.page_bytes : A.L.v_off)));
         auto kernel = topp ? compress_pages_warp_kernel<false, true> : (pv ? compress_pages_warp_kernel<true, false> : compress_pages_warp_kernel<false, false>);
-        if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-            return SPARK_ERR_CUDA;
+        static unsigned char smem_raised[3][kMaxDevices] = {};
+        if (smem > 48 * 1024 && !allow_max_smem(kernel, smem_raised[topp ? 2 : (pv ? 1 : 0)])) return SPARK_ERR_CUDA;
         const dim3 wgrid((n_blocks + kWarpPageWarps - 1) / kWarpPageWarps, p.n_kv_heads, p.batch);
         const cudaError_t e = launch_kernel(kernel, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A);
         ++*launches;

@@ -872,22 +872,6 @@ inline void set_divisors(DecodeArgs& A, int64_t units, int grid)
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Device properties the launchers need, looked up once per device and then served from a table
-// (spark_decode.cu); `dev` is the current device.
-struct DeviceInfo { int n_sms; int smem_optin; };
-bool device_info(int* dev, DeviceInfo* info);
-
-// Raises a kernel's dynamic shared-memory limit to the device maximum, once per device and kernel.
-constexpr int kMaxDevices = 64;
-template <typename Kernel> inline bool allow_max_smem(Kernel kernel, int dev, int smem_optin, unsigned char (&done)[kMaxDevices])
-{
-    if (dev < 0 || dev >= kMaxDevices) return false;
-    if (done[dev]) return true;                           // a racing first call only repeats the same setting
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin) != cudaSuccess) return false;
-    done[dev] = 1;
-    return true;
-}
-
 // per-dtype launchers (spark_decode.cu: fp32 storage, spark_decode_mma.cu: bf16 storage)
 spark_status launch_decode_f32(int G, const DecodeArgs& A, int dev, const DeviceInfo& info, cudaStream_t stream);
 spark_status launch_decode_bf16(int G, const DecodeArgs& A, int dev, const DeviceInfo& info, cudaStream_t stream);

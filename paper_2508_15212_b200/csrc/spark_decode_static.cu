@@ -23,7 +23,6 @@ constexpr size_t kNoAllocScratchBytes =
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
-constexpr int kMaxDevices = 64;
 static std::mutex g_setup_mutex;
 static void* g_scratch_addr[kMaxDevices] = {};
 

@@ -459,11 +459,10 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
                                                          A.votes, A.status, stream, launches);
         if (st_tc != SPARK_OK) return st_tc;
     } else if (A.n_tiles > 0 && max_seq_tokens > p.token_budget) {
-        cudaError_t e1 = bf16 ? cudaFuncSetAttribute(evict_scores_kernel<__nv_bfloat16, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
-                              : cudaFuncSetAttribute(evict_scores_kernel<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        cudaError_t e2 = bf16 ? cudaFuncSetAttribute(evict_scores_kernel<__nv_bfloat16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
-                              : cudaFuncSetAttribute(evict_scores_kernel<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e1 != cudaSuccess || e2 != cudaSuccess) return SPARK_ERR_CUDA;
+        static unsigned char smem_raised[4][kMaxDevices] = {};
+        if (!(bf16 ? allow_max_smem(evict_scores_kernel<__nv_bfloat16, 1>, smem_raised[0]) && allow_max_smem(evict_scores_kernel<__nv_bfloat16, 2>, smem_raised[1])
+                   : allow_max_smem(evict_scores_kernel<float, 1>, smem_raised[2]) && allow_max_smem(evict_scores_kernel<float, 2>, smem_raised[3])))
+            return SPARK_ERR_CUDA;
         if (bf16) launch_kernel(evict_scores_kernel<__nv_bfloat16, 1>, grid, dim3(kEvThreads), smem, stream, A);
         else launch_kernel(evict_scores_kernel<float, 1>, grid, dim3(kEvThreads), smem, stream, A);
         launch_kernel(evict_rowstats_kernel, ugrid, dim3(256), 0, stream, A);
@@ -474,8 +473,8 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     const int most = select_share(max_seq_tokens > p.window ? max_seq_tokens - p.window : 1);
     A.key_cap = most < kKeyCap ? most : kKeyCap;
     const size_t key_bytes = (static_cast<size_t>(A.key_cap) + kVoteTile + 2 * kVoteHalo) * sizeof(unsigned);
-    if (cudaFuncSetAttribute(evict_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(key_bytes)) != cudaSuccess)
-        return SPARK_ERR_CUDA;
+    static unsigned char select_raised[kMaxDevices] = {};
+    if (!allow_max_smem(evict_select_kernel, select_raised)) return SPARK_ERR_CUDA;
     launch_kernel(evict_select_kernel, dim3(kSelCluster, p.n_kv_heads, p.batch), dim3(kSelThreads), key_bytes, stream, A);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;

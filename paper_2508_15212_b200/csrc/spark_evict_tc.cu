@@ -448,11 +448,11 @@ spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, con
     const int n_tiles = (max_seq_tokens + kTcTile - 1) / kTcTile;
     // Two CTAs are resident per SM; a CTA pays a fixed start-up (tensor-memory allocation, the query
     // block, the first key tile), so the tiles are cut into about one wave of CTAs, at least 8 tiles each.
-    int dev = 0, n_sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SPARK_ERR_CUDA;
+    int dev = 0;
+    DeviceInfo info;
+    if (!device_info(&dev, &info)) return SPARK_ERR_CUDA;
     const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
-    const int64_t wave = 2 * static_cast<int64_t>(n_sms);
+    const int64_t wave = 2 * static_cast<int64_t>(info.n_sms);
     int64_t per = (static_cast<int64_t>(n_tiles) * units + wave - 1) / wave;
     if (per < 8) per = 8;
     if (per > n_tiles) per = n_tiles > 0 ? n_tiles : 1;
@@ -460,8 +460,9 @@ spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, con
     A.parts = (n_tiles + A.tiles_per_cta - 1) / A.tiles_per_cta;
     A.partial = partial; A.votes = votes; A.status = status;
     const size_t smem = static_cast<size_t>(Rpad) * 256 + 2 * kTcTile * 256 + 1024;     // queries, two key buffers, alignment slack
-    if (cudaFuncSetAttribute(evict_scores_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess ||
-        cudaFuncSetAttribute(evict_scores_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    static unsigned char smem_raised[2][kMaxDevices] = {};
+    if (!allow_max_smem(evict_scores_tc_kernel<1>, dev, info.smem_optin, smem_raised[0]) ||
+        !allow_max_smem(evict_scores_tc_kernel<2>, dev, info.smem_optin, smem_raised[1]))
         return SPARK_ERR_CUDA;
     const dim3 grid(A.parts, p.n_kv_heads, p.batch);
     launch_kernel(evict_scores_tc_kernel<1>, grid, dim3(kTcThreads), smem, stream, A);

@@ -1,10 +1,14 @@
 """The selection searches, the division of a decode step among CTAs and the eviction's select kernel at the sizes where
 they change branch, against the oracle with the bars of test_gpu_parity.py."""
+import ctypes
+import threading
+
 import numpy as np
 import pytest
 import torch
 
 import oracle
+from paper_2508_15212_b200 import binding as B
 from paper_2508_15212_b200.cache import SparkCache
 from test_gpu_parity import built, check_case, check_eviction_case, make, to_np  # noqa: F401  (built: module fixture)
 
@@ -73,3 +77,33 @@ def test_division_of_the_step(name, Hq, Hkv, lens):
 ])
 def test_eviction_select_edges(lens, W, budget, G, pool):
     check_eviction_case("bf16", lens, W, budget, G, Hkv=1 if lens[0] > 100000 else 2, pool=pool, seed=500)
+
+
+def test_threads_with_different_shared_memory_needs():
+    """Prompts of two sizes evicted and pruned by three threads on their own streams: the launches of the larger size must
+    not depend on what another thread last asked the driver for (set launch by launch, some six calls in 8000 were refused)."""
+    made = []
+    for n in (200, 200, 20000):
+        wl = make("bf16", 1, 1, 1, [n], 4, 64, seed=600, gap=False)
+        cache = SparkCache(batch=1, n_q_heads=1, n_kv_heads=1, window=4, keep=64, dtype="bf16", max_tokens=n, token_budget=64)
+        cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+        made.append((wl, cache, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    refused, start = [0] * len(made), threading.Barrier(len(made))
+
+    def work(i):
+        wl, c, stream = made[i]
+        p = [ctypes.c_void_p(t.data_ptr()) for t in (wl.q_win, wl.k, wl.v, wl.seq_lens, c.pages, c.qnorm, c.packed_lens, c.kept_tokens, c.ws_compress)]
+        args = (ctypes.byref(c.params), p[0], p[1], p[2], *wl.k.stride()[:3], p[3], wl.k.shape[2], p[4], None, c.table_blocks,
+                *p[5:], c.ws_compress.numel(), ctypes.c_void_p(stream.cuda_stream))
+        start.wait()
+        refused[i] = sum(B.lib().spark_compress(*args) != 0 for _ in range(8000))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(made))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert refused == [0] * len(made)
+    assert all(cache.status() == 0 for _, cache, _ in made)
