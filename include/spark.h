@@ -298,7 +298,7 @@ spark_status spark_append_dense(const spark_params *p, const void *k_new, const 
  * log-sum-exp inside the prefix's step.
  *   k_tail, v_tail   [B][Hkv][tail_tokens][D] as written by spark_append_dense; tail_tokens <= 128 (else
  *                    SPARK_ERR_UNSUPPORTED: decode the tail with spark_decode_attn and use spark_merge_attn)
- *   tail_lens        [B] int32 tokens in each tail
+ *   tail_lens        [B] int32 tokens in each tail; one outside 0 .. tail_tokens is clamped and SPARK_ERR_DEVICE_BOUNDS recorded
  *   tail_out         scratch [B][Hq][D] fp32, 16-byte aligned;  tail_lse  scratch [B][Hq] fp32
  *   out, lse         the merged result; every other argument as for spark_decode_attn
  */

@@ -244,9 +244,9 @@ spark_status spark_decode_attn_tail(const spark_params* p, const void* q, const 
         return SPARK_ERR_WORKSPACE;
     int launches = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    st = launch_tail_attn(*p, q, k_tail, v_tail, tail_tokens, tail_lens, tail_out, tail_lse, s, &launches);
+    st = launch_tail_attn(*p, q, k_tail, v_tail, tail_tokens, tail_lens, tail_out, tail_lse, workspace, s, &launches);
     if (st != SPARK_OK) return st;
-    // the step's predecessor is the tail kernel, which writes tail_out and tail_lse alone: the step runs beside it and waits
+    // the step's predecessor is the tail kernel, which writes tail_out, tail_lse and the status word alone: the step runs beside it and waits
     // where it merges the two (waiting at its top: 25.4 us a token, append included; this: 23.5)
     spark_params over = *p;
     over.flags |= SPARK_FLAG_OVERLAP_PREVIOUS;

@@ -215,7 +215,8 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
                            size_t workspace_bytes, cudaStream_t stream, int* launches, bool q_by_value = false,
                            const float* other_out = nullptr, const float* other_lse = nullptr);
 // other_out / other_lse: attention over further tokens of the same sequences, merged into the result.  The kernel that writes
-// them must be the one enqueued just before, and must write nothing else that this step uses: it is waited for only there.
+// them must be the one enqueued just before, and must write nothing else that this step uses (the status word, which both
+// only set by compare-and-swap, excepted): it is waited for only there.
 // q_by_value: q is a HOST pointer and its bytes travel as a launch parameter (bf16 storage, degenerate recovery,
 // dense value rows, at most query_by_value_limit() bytes; anything else is refused)
 size_t query_by_value_limit();
@@ -231,7 +232,7 @@ spark_status launch_append_dense(const spark_params& p, const void* k_new, const
                                  const int32_t* block_table, int32_t max_blocks, void* k_tail, void* v_tail, int32_t cap,
                                  int32_t* packed_lens, void* workspace, cudaStream_t stream, int* launches);
 spark_status launch_tail_attn(const spark_params& p, const void* q, const void* k_tail, const void* v_tail, int32_t cap,
-                              const int32_t* tail_lens, float* out, float* lse, cudaStream_t stream, int* launches);
+                              const int32_t* tail_lens, float* out, float* lse, void* workspace, cudaStream_t stream, int* launches);
 spark_status launch_merge_attn(int rows, const float* out_a, const float* lse_a, const float* out_b, const float* lse_b,
                                float* out, float* lse, cudaStream_t stream);
 

@@ -103,6 +103,7 @@ struct TailArgs {
     float scale_log2e;
     float* out;
     float* lse;
+    int* status;
 };
 
 template <int G, typename E>
@@ -132,7 +133,10 @@ __global__ void __launch_bounds__(kTailThreads) tail_attn_kernel(TailArgs A)
     for (int i = 0; i < 16; ++i)
         if (grp + 4 * i < A.cap) vr[i] = *reinterpret_cast<const Pair*>(v + static_cast<int64_t>(grp + 4 * i) * kHeadDim + 2 * c2);
     int n = A.lens[b];
-    n = n < 0 ? 0 : (n > A.cap ? A.cap : n);
+    if (n < 0 || n > A.cap) {
+        if (tid == 0 && h == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+        n = n < 0 ? 0 : A.cap;
+    }
     for (int i = tid; i < G * kHeadDim; i += kTailThreads) q_s[i / kHeadDim][i % kHeadDim] = Elem<E>::load(A.q, row0 * kHeadDim + i);
     __syncthreads();
     for (int t = t0; t < ((n + 63) & ~63); t += 64) {          // whole warps iterate together
@@ -252,13 +256,13 @@ template <int G> static cudaError_t launch_tail_g(const spark_params& p, const T
 }
 
 spark_status launch_tail_attn(const spark_params& p, const void* q, const void* k_tail, const void* v_tail, int32_t cap,
-                              const int32_t* tail_lens, float* out, float* lse, cudaStream_t stream, int* launches)
+                              const int32_t* tail_lens, float* out, float* lse, void* workspace, cudaStream_t stream, int* launches)
 {
     TailArgs A;
     A.q = q; A.k = k_tail; A.v = v_tail; A.lens = tail_lens; A.Hq = p.n_q_heads; A.Hkv = p.n_kv_heads; A.cap = cap;
     const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf(static_cast<float>(p.head_dim));
     A.scale_log2e = scale * 1.4426950408889634f;
-    A.out = out; A.lse = lse;
+    A.out = out; A.lse = lse; A.status = static_cast<int*>(workspace);
     cudaError_t e = cudaErrorInvalidValue;
     switch (p.n_q_heads / p.n_kv_heads) {
         case 1: e = launch_tail_g<1>(p, A, stream); break;

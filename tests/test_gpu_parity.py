@@ -530,6 +530,25 @@ def test_short_dense_tail_equals_the_tail_cache_merged(G, dtype, cap, n_tail):
     assert torch.allclose(lse[fin], ref_lse[fin], rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
 
 
+@pytest.mark.parametrize("bad", [-1, 65])
+def test_tail_length_out_of_range_is_recorded(bad):
+    """A tail length outside 0 .. capacity is recorded and clamped, as a length of the pruned prefix is."""
+    wl = make("bf16", 2, 8, 2, [100, 80], 8, 64, seed=185, gap=False)
+    a = SparkCache(batch=2, n_q_heads=8, n_kv_heads=2, window=8, keep=64, dtype="bf16", max_tokens=100)
+    a.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    k_tail, v_tail = (x[:, :, :64].contiguous() for x in (wl.k, wl.v))
+    outs = []
+    for n in (bad, min(max(bad, 0), 64)):
+        lens = torch.tensor([3, n], dtype=torch.int32, device="cuda")
+        to, tl, out, lse = a.alloc_out(), a.alloc_lse(), a.alloc_out(), a.alloc_lse()
+        B.spark_decode_attn_tail(a.params, wl.q, a.pages, None, a.packed_lens, a.qnorm, k_tail, v_tail, lens, to, tl, out, lse,
+                                 a.ws_decode, max_blocks=a.table_blocks)
+        assert a.status() == (6 if n == bad else 0)
+        B.spark_workspace_init(a.ws_decode)
+        outs.append((out, lse))
+    assert all(torch.equal(x, y) for x, y in zip(*outs))
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_host_entry_point_staged_and_mapped_equal_the_device_call(dtype):
     """spark_decode_attn_host: query and result in page-locked host memory, with staging copies or (flag) with the
