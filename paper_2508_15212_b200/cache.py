@@ -185,6 +185,7 @@ class DenseTailCache:
         tdt = _TDT[dtype]
         self.k_tail = torch.zeros(batch, n_kv_heads, cap, 128, dtype=tdt, device=device)
         self.v_tail = torch.zeros(batch, n_kv_heads, cap, 128, dtype=tdt, device=device)
+        self._row, self._row_dtype = torch.Size((batch, n_kv_heads, 128)), tdt       # a token's rows
         self.n_tail = 0
         p = self.prefix.params
         self._o = [torch.empty(p.batch, p.n_q_heads, 128, dtype=torch.float32, device=device) for _ in range(2)]
@@ -205,10 +206,19 @@ class DenseTailCache:
             b = self._bound = B.BoundTail(self.prefix, self.tail, self.k_tail, self.v_tail, self._o[1], self._l[1])
         return b
 
+    def _check_row(self, x) -> None:
+        if x.dtype != self._row_dtype or x.device != self.k_tail.device:
+            raise RuntimeError(f"the tail holds {self._row_dtype} on {self.k_tail.device}, got {x.dtype} on {x.device}")
+        if x.shape != self._row[max(0, len(self._row) - x.dim()):] or x.numel() != self._row.numel():    # (leading ones may be left out)
+            raise RuntimeError(f"a token's rows have the shape {tuple(self._row)}, got {tuple(x.shape)}")
+
     def append(self, k_new, v_new) -> None:
         """One new token per sequence ([B, Hkv, D]); it stays dense until its block is handed to the prefix."""
         if self.n_tail >= self.k_tail.shape[2]:
             raise IndexError(f"the dense tail holds {self.n_tail} tokens and has no room for another")
+        for x in (k_new, v_new):                           # the library takes pointers: nothing behind them checks this
+            if x.shape != self._row or x.dtype != self._row_dtype or x.device != self.k_tail.device:
+                self._check_row(x)
         self._calls().append(k_new, v_new)
         self.n_tail += 1
         if self.block and self.n_tail == self.block:
