@@ -6,7 +6,6 @@ stream.  There is no fallback: if the library is missing the import of a functio
 from __future__ import annotations
 
 import ctypes
-import operator
 import os
 from typing import Optional
 
@@ -238,69 +237,32 @@ def spark_decode_attn(p: spark_params, q, pages, block_table, packed_lens, qnorm
            "spark_decode_attn")
 
 
+# The two calls of a dense tail come once per token and layer: their pointers are read with data_ptr() and handed over as
+# plain integers (as cheap as arguments converted once and kept, and nothing has to watch whether a buffer has moved).
 def spark_append_dense(p: spark_params, k_new, v_new, pages, block_table, k_tail, v_tail, packed_lens, workspace,
                        max_blocks=None) -> None:
     """One new token per sequence into a dense tail: its pages and the rows k_tail, v_tail [B, Hkv, tail_tokens, D]."""
     assert k_new.is_contiguous() and v_new.is_contiguous()
-    _check(lib().spark_append_dense(ctypes.byref(p), k_new.data_ptr(), v_new.data_ptr(), pages.data_ptr(),
+    code = lib().spark_append_dense(ctypes.byref(p), k_new.data_ptr(), v_new.data_ptr(), pages.data_ptr(),
                                     None if block_table is None else block_table.data_ptr(), _blocks(block_table, max_blocks),
                                     k_tail.data_ptr(), v_tail.data_ptr(), k_tail.shape[2], packed_lens.data_ptr(),
-                                    workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                    _stream()),
-           "spark_append_dense")
+                                    workspace.data_ptr(), workspace.nbytes, _stream())
+    if code != SPARK_OK:
+        raise SparkError(code, "spark_append_dense")
 
 
 def spark_decode_attn_tail(p: spark_params, q, pages, block_table, packed_lens, qnorm, k_tail, v_tail, tail_lens, tail_out,
                            tail_lse, out, lse, workspace, max_blocks=None) -> None:
     """Decode step over a pruned prefix and a dense tail of at most TAIL_MAX tokens."""
-    _check(lib().spark_decode_attn_tail(ctypes.byref(p), q.data_ptr(), pages.data_ptr(),
+    code = lib().spark_decode_attn_tail(ctypes.byref(p), q.data_ptr(), pages.data_ptr(),
                                         None if block_table is None else block_table.data_ptr(),
                                         _blocks(block_table, max_blocks), packed_lens.data_ptr(), qnorm.data_ptr(),
                                         k_tail.data_ptr(), v_tail.data_ptr(), k_tail.shape[2], tail_lens.data_ptr(),
                                         tail_out.data_ptr(), tail_lse.data_ptr(), out.data_ptr(),
-                                        None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                        workspace.numel() * workspace.element_size(),
-                                        _stream()),
-           "spark_decode_attn_tail")
-
-
-class BoundTail:
-    """spark_append_dense and spark_decode_attn_tail on the buffers of one prefix + tail pair, marshalled once: a call
-    converts only what changes from token to token (the new rows, the query, the result and the stream)."""
-
-    def __init__(self, prefix, tail, k_tail, v_tail, tail_out, tail_lse):
-        self.buffers = self.current(prefix, tail, k_tail, v_tail)
-        self._alive = (prefix.params, tail.params, tail_out, tail_lse)
-        cap = int(k_tail.shape[2])
-        self._append_fn, self._decode_fn = lib().spark_append_dense, lib().spark_decode_attn_tail
-        self._p_tail, self._p_prefix = ctypes.byref(tail.params), ctypes.byref(prefix.params)
-        self._append_args = (_ptr(tail.pages), _ptr(tail.block_table), tail.table_blocks, _ptr(k_tail), _ptr(v_tail), cap,
-                             _ptr(tail.packed_lens), _ptr(tail.ws_compress), tail.ws_compress.numel())
-        self._decode_args = (_ptr(prefix.pages), _ptr(prefix.block_table), prefix.table_blocks, _ptr(prefix.packed_lens),
-                             _ptr(prefix.qnorm), _ptr(k_tail), _ptr(v_tail), cap, _ptr(tail.packed_lens), _ptr(tail_out),
-                             _ptr(tail_lse))
-        self._ws = (_ptr(prefix.ws_decode), prefix.ws_decode.numel())
-
-    @staticmethod
-    def current(prefix, tail, k_tail, v_tail):
-        return (prefix.pages, prefix.block_table, prefix.packed_lens, prefix.qnorm, prefix.ws_decode, prefix.params, tail.pages,
-                tail.block_table, tail.packed_lens, tail.ws_compress, tail.params, k_tail, v_tail)
-
-    def matches(self, prefix, tail, k_tail, v_tail) -> bool:
-        """Whether the pair still has the buffers that were marshalled."""
-        return all(map(operator.is_, self.buffers, self.current(prefix, tail, k_tail, v_tail)))
-
-    def append(self, k_new, v_new) -> None:
-        assert k_new.is_contiguous() and v_new.is_contiguous()
-        code = self._append_fn(self._p_tail, k_new.data_ptr(), v_new.data_ptr(), *self._append_args, _stream())
-        if code != SPARK_OK:
-            raise SparkError(code, "spark_append_dense")
-
-    def decode(self, q, out, lse) -> None:
-        code = self._decode_fn(self._p_prefix, q.data_ptr(), *self._decode_args, out.data_ptr(),
-                               None if lse is None else lse.data_ptr(), *self._ws, _stream())
-        if code != SPARK_OK:
-            raise SparkError(code, "spark_decode_attn_tail")
+                                        None if lse is None else lse.data_ptr(), workspace.data_ptr(), workspace.nbytes,
+                                        _stream())
+    if code != SPARK_OK:
+        raise SparkError(code, "spark_decode_attn_tail")
 
 
 TAIL_MAX = 128              # tokens of a dense tail that spark_decode_attn_tail takes

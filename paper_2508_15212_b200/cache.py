@@ -191,20 +191,12 @@ class DenseTailCache:
         self._o = [torch.empty(p.batch, p.n_q_heads, 128, dtype=torch.float32, device=device) for _ in range(2)]
         self._l = [torch.empty(p.batch, p.n_q_heads, dtype=torch.float32, device=device) for _ in range(2)]
         self._short = cap <= B.TAIL_MAX
-        self._bound = None
 
     def compress(self, q_win, k, v, seq_lens) -> None:
         self.prefix.compress(q_win, k, v, seq_lens)
         self.tail.qnorm.copy_(self.prefix.qnorm)           # the tail is dense: qnorm only has to be a valid divisor
         self.tail.packed_lens.zero_()
         self.n_tail = 0
-
-    def _calls(self) -> "B.BoundTail":
-        """The calls on this pair's buffers, marshalled once (and again should a buffer have been replaced)."""
-        b = self._bound
-        if b is None or not b.matches(self.prefix, self.tail, self.k_tail, self.v_tail):
-            b = self._bound = B.BoundTail(self.prefix, self.tail, self.k_tail, self.v_tail, self._o[1], self._l[1])
-        return b
 
     def _check_row(self, x) -> None:
         if x.dtype != self._row_dtype or x.device != self.k_tail.device:
@@ -219,7 +211,9 @@ class DenseTailCache:
         for x in (k_new, v_new):                           # the library takes pointers: nothing behind them checks this
             if x.shape != self._row or x.dtype != self._row_dtype or x.device != self.k_tail.device:
                 self._check_row(x)
-        self._calls().append(k_new, v_new)
+        t = self.tail
+        B.spark_append_dense(t.params, k_new, v_new, t.pages, t.block_table, self.k_tail, self.v_tail, t.packed_lens, t.ws_compress,
+                             max_blocks=t.table_blocks)
         self.n_tail += 1
         if self.block and self.n_tail == self.block:
             self.prefix.append_block(self.k_tail, self.v_tail)
@@ -230,7 +224,9 @@ class DenseTailCache:
         if out is None:
             out = torch.empty_like(self._o[0])
         if self._short:                                    # a short tail: two launches, merged in the prefix's step
-            self._calls().decode(q, out, lse)
+            p = self.prefix
+            B.spark_decode_attn_tail(p.params, q, p.pages, p.block_table, p.packed_lens, p.qnorm, self.k_tail, self.v_tail,
+                                     self.tail.packed_lens, self._o[1], self._l[1], out, lse, p.ws_decode, max_blocks=p.table_blocks)
             return out
         self.prefix.decode(q, out=self._o[0], lse=self._l[0])
         self.tail.decode(q, out=self._o[1], lse=self._l[1])
