@@ -181,7 +181,7 @@ class DenseTailCache:
         self.prefix = SparkCache(batch=batch, n_q_heads=n_q_heads, n_kv_heads=n_kv_heads, window=window, keep=keep,
                                  dtype=dtype, max_tokens=max_tokens, device=device, **prefix_kw)
         self.tail = SparkCache(batch=batch, n_q_heads=n_q_heads, n_kv_heads=n_kv_heads, window=window, keep=128,
-                               dtype=dtype, max_tokens=cap, device=device)
+                               dtype=dtype, max_tokens=cap, device=device, softmax_scale=prefix_kw.get("softmax_scale", 0.0))
         tdt = _TDT[dtype]
         self.k_tail = torch.zeros(batch, n_kv_heads, cap, 128, dtype=tdt, device=device)
         self.v_tail = torch.zeros(batch, n_kv_heads, cap, 128, dtype=tdt, device=device)

@@ -493,6 +493,35 @@ def test_dense_tail_equals_the_oracle_with_appended_keys_left_dense(dtype, block
             assert np.allclose(lse.cpu().numpy(), ref_lse, rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("max_tail", [64, 200])
+def test_dense_tail_uses_the_prefix_softmax_scale(dtype, max_tail):
+    """A scale of the caller's holds for the appended tokens as for the pruned ones, whichever kernel serves the tail."""
+    from paper_2508_15212_b200.cache import DenseTailCache
+    keep, lens0, n_app, scale = 38, [50, 90], 20, 0.04
+    full = make(dtype, 2, 8, 2, [l + n_app for l in lens0], 8, keep, seed=161, sigma=1.0 if dtype == "bf16" else 0.5)
+    cache = DenseTailCache(batch=2, n_q_heads=8, n_kv_heads=2, window=8, keep=keep, dtype=dtype, max_tokens=max(lens0),
+                           tail_block=None, max_tail=max_tail, softmax_scale=scale)
+    lens0_t = torch.tensor(lens0, dtype=torch.int32, device="cuda")
+    cache.compress(full.q_win, full.k[:, :, :max(lens0)].contiguous(), full.v[:, :, :max(lens0)].contiguous(), lens0_t)
+    for i in range(n_app):
+        idx = (lens0_t.long() + i).view(2, 1, 1, 1).expand(2, 2, 1, 128)
+        cache.append(full.k.gather(2, idx).squeeze(2).contiguous(), full.v.gather(2, idx).squeeze(2).contiguous())
+    wl_cpu = full.to("cpu")
+    _, a = oracle.window_mean(wl_cpu.q_win, 2)
+    c = oracle.compress(wl_cpu.k, wl_cpu.seq_lens, keep, a)
+    mask, mu, lens = c["mask"].copy(), c["mu"].copy(), [l + n_app for l in lens0]
+    for b, l in enumerate(lens0):
+        mask[b, :, l:l + n_app] = 0xFFFFFFFF
+        mu[b, :, l:l + n_app] = 0.0
+    ref, ref_lse = oracle.decode_attn(wl_cpu.q, wl_cpu.k, wl_cpu.v, lens, mask, mu, a, scale=scale)
+    lse = torch.empty(2, 8, dtype=torch.float32, device="cuda")
+    out = cache.decode(full.q, lse=lse)
+    assert cache.status() == 0
+    assert float(np.abs(out.cpu().numpy() - ref).max()) <= TOL[dtype]
+    assert np.allclose(lse.cpu().numpy(), ref_lse, rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
+
+
 @pytest.mark.parametrize("G", [1, 4, 7, 8])
 @pytest.mark.parametrize("dtype,cap,n_tail", [("bf16", 64, 1), ("bf16", 64, 63), ("bf16", 128, 65), ("bf16", 128, 128), ("bf16", 5, 0),
                                               ("f32", 128, 127), ("f32", 16, 16)])
