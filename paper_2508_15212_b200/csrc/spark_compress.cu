@@ -910,7 +910,8 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
 //   fp32 until at most three keys can lie between the ends.  The sum above the upper end is then taken in double and
 //   must be below the goal (else the search is repeated in double), and the keys between are admitted one by one.
 //   A bitonic rank sort per token took 2100 instructions for one token; prefill of 8192 tokens and its first token
-//   189 -> 63 us.
+//   189 -> 63 us.  The sort still decides (rank_mask) where sums in another order could decide otherwise: a total that is not
+//   finite, or a sum within rounding of the goal whose terms do not add up exactly.
 __device__ __forceinline__ double sum_ge(const unsigned char* wrow, int sw, int half, unsigned lo)        // keys >= lo, in double
 {
     double s = 0.0;
@@ -937,6 +938,29 @@ __device__ __forceinline__ float sum_ge_f32(const unsigned char* wrow, int sw, i
     }
     const float t = (s[0] + s[1]) + (s[2] + s[3]);
     return t + __shfl_xor_sync(kFullMask, t, 16);
+}
+
+// Mask words of one token by the rank sort that the append kernels use (called by the whole warp; a page rarely needs it, so
+// it stays out of line and costs the loop above no registers).
+__device__ __noinline__ uint4 rank_mask(const unsigned char* wrow, int sw, int lane, float top_p, int cap)
+{
+    const uint4 v = *reinterpret_cast<const uint4*>(wrow + ((lane ^ sw) << 4));
+    const unsigned key[4] = {v.x, v.y, v.z, v.w};
+    SelectArgs sel;
+    sel.select = SPARK_SELECT_TOP_P; sel.top_p = top_p; sel.recovery = SPARK_RECOVER_DEGENERATE;
+    sel.rank_keep[0] = sel.rank_keep[1] = sel.rank_keep[2] = sel.rank_keep[3] = 0u;
+    bool kept[4];
+    select_by_rank(key, lane, sel, cap, kept);
+    unsigned nib = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) nib |= kept[i] ? (1u << i) : 0u;
+    const unsigned w = nib << (4 * (lane & 7));
+    uint4 m;
+    m.x = __reduce_or_sync(kFullMask, lane < 8 ? w : 0u);
+    m.y = __reduce_or_sync(kFullMask, (lane >> 3) == 1 ? w : 0u);
+    m.z = __reduce_or_sync(kFullMask, (lane >> 3) == 2 ? w : 0u);
+    m.w = __reduce_or_sync(kFullMask, lane >= 24 ? w : 0u);
+    return m;
 }
 
 __device__ __forceinline__ int select_section_topp(const unsigned char* tile, unsigned char* wsm, unsigned char* image, int vals_off,
@@ -969,6 +993,8 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
     const double total = sum_ge(wrow, sw, half, 0u);
     const double goal = static_cast<double>(top_p) * total;
     const float goal_f = static_cast<float>(goal);
+    const bool finite = total < static_cast<double>(INFINITY);                  // (false for NaN)
+    const bool search = live && finite;
     // full-key bounds: the sum of keys >= lo reaches the goal, that of keys >= hi does not
     unsigned lo = 0u, hi = 0u;
     double above = 0.0;                                        // sum of the keys >= hi, in double
@@ -976,7 +1002,7 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
     for (;;) {
         int l16 = 0, h16 = static_cast<int>(__float_as_uint(top_w) >> 16) + 1;
         double f_lo = total, f_hi = 0.0;                       // (in the first search fp32 values)
-        bool done = !live, lo_moved = true;
+        bool done = !search, lo_moved = true;
         for (int it = 0; !__all_sync(kFullMask, done); ++it) {
             const int span = h16 - l16;
             const float vl = __uint_as_float(static_cast<unsigned>(l16) << 16);
@@ -1001,7 +1027,7 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
         lo = static_cast<unsigned>(l16) << 16;
         hi = static_cast<unsigned>(h16) << 16;
         above = sum_ge(wrow, sw, half, hi);
-        const bool bad = live && !exact && above >= goal && goal > 0.0;      // fp32 had put the upper end too low
+        const bool bad = search && !exact && above >= goal && goal > 0.0;      // fp32 had put the upper end too low
         if (!__any_sync(kFullMask, bad)) break;
         exact = true;                                          // rare: all tokens of the warp again, in double
     }
@@ -1020,12 +1046,12 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
     }
     unsigned long long got = (static_cast<unsigned long long>(got2[1]) << 32) | got2[0];
     unsigned long long cand = ((static_cast<unsigned long long>(cand2[1]) << 32) | cand2[0]) & ~got;
-    if (!live) got = cand = 0ull;
+    if (!search) got = cand = 0ull;
     int count = __popcll(got);
     count += __shfl_xor_sync(kFullMask, count, 16);
-    double sum = above;
-    while (__any_sync(kFullMask, live && count < kHeadDim && (sum < goal || count == 0))) {
-        const bool more = live && count < kHeadDim && (sum < goal || count == 0);
+    double sum = above, before = -1.0;                         // before the last key admitted here
+    while (__any_sync(kFullMask, search && count < kHeadDim && (sum < goal || count == 0))) {
+        const bool more = search && count < kHeadDim && (sum < goal || count == 0);
         unsigned best = 0u;
         unsigned long long eq = 0ull;
         const int none = cand == 0ull, both = none & __shfl_xor_sync(kFullMask, none, 16);
@@ -1042,7 +1068,7 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
         if (more) {
             const double w = static_cast<double>(__uint_as_float(best));
             int take = 0;                                      // equal keys: lower channels first, no more than the goal asks for
-            while (take < mine + theirs && (sum < goal || count + take == 0)) { sum += w; ++take; }
+            while (take < mine + theirs && (sum < goal || count + take == 0)) { before = sum; sum += w; ++take; }
             int own = half ? take - theirs : take;
             own = own < 0 ? 0 : (own > mine ? mine : own);
             unsigned long long rest = eq;
@@ -1051,6 +1077,26 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
             cand &= ~eq;
             count += take;
             if (mine + theirs == 0) count = kHeadDim;          // (nothing left)
+        }
+    }
+    const double slack = total * 0x1p-44;                      // more than 128 roundings
+    const bool close = live && (!finite || fabs(sum - goal) <= slack || fabs(before - goal) <= slack);
+    if (__any_sync(kFullMask, close)) {
+        // 128 terms add up exactly in double, in any order, when their exponents span at most 22
+        unsigned least = 0x7f800000u;
+#pragma unroll 1
+        for (int c = 0; c < 16; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
+            const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) least = x[e] ? min(least, x[e]) : least;
+        }
+        least = min(least, __shfl_xor_sync(kFullMask, least, 16));
+        const bool rank = close && (!finite || static_cast<int>(__float_as_uint(top_w) >> 23) - static_cast<int>(least >> 23) > 22);
+        for (unsigned todo = __ballot_sync(kFullMask, rank) & 0xffffu; todo; todo &= todo - 1) {
+            const int tok = __ffs(todo) - 1;
+            const uint4 m = rank_mask(wsm + tok * (kHeadDim * 4), tok & 7, lane, top_p, T);
+            if (p == tok) got = half ? (static_cast<unsigned long long>(m.w) << 32) | m.z : (static_cast<unsigned long long>(m.y) << 32) | m.x;
         }
     }
     count = __popcll(got);

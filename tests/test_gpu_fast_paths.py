@@ -57,6 +57,43 @@ def test_top_p_selection_with_ties(kind, p, cap):
     assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("p,cap", [(0.5, 128), (0.95, 128), (1.0, 128), (1.0, 40), (0.95, 40)])
+def test_top_p_of_odd_values_equals_appending_them(p, cap):
+    """Infinities, NaN, all-zero rows, saliencies over more than 22 octaves (their sums round, and p = 1 asks for all of
+    them) and subnormal ones: the prefill keeps what the append kernels, which sort every token's channels, keep."""
+    n = 100
+    wl = make("bf16", 1, 8, 2, [n], 8, 64, seed=310, gap=False)
+    g = torch.Generator(device="cuda").manual_seed(310)
+    k = wl.k.float()
+
+    def anywhere(tokens, value, how_many):
+        for t in tokens:
+            at = torch.randperm(128, generator=g, device="cuda")[:how_many]
+            k[:, :, t, at] = value
+
+    anywhere(range(0, 10), float("nan"), 1)
+    anywhere(range(5, 12), float("inf"), 2)
+    anywhere(range(12, 16), float("nan"), 60)
+    k[:, :, 16] = float("nan")
+    k[:, :, 17] = float("-inf")
+    k[:, :, 18] = 0.0
+    for t in range(20, 60):                                      # 40 to 60 octaves, rounded sums
+        k[:, :, t] *= 2.0 ** torch.randint(-30, 31, k[:, :, t].shape, generator=g, device="cuda")
+    for t in range(60, 80):
+        k[:, :, t] *= 2.0 ** -126
+    anywhere(range(70, 90), 0.0, 100)
+    wl.k = k.to(torch.bfloat16)
+    kw = dict(batch=1, n_q_heads=8, n_kv_heads=2, window=8, keep=cap, dtype="bf16", max_tokens=n, top_p=p)
+    whole, grown = SparkCache(**kw), SparkCache(**kw)
+    whole.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    grown.compress(wl.q_win, wl.k, wl.v, torch.zeros_like(wl.seq_lens))
+    grown.append_block(wl.k, wl.v)
+    assert whole.status() == 0 and grown.status() == 0
+    a, b = whole.unpack(), grown.unpack()
+    assert torch.equal(a["mask"], b["mask"]) and torch.equal(a["vals"].view(torch.int16), b["vals"].view(torch.int16))
+    assert torch.allclose(a["mu"], b["mu"], rtol=1e-6, atol=0, equal_nan=True)
+
+
 @pytest.mark.parametrize("name,Hq,Hkv,lens", [
     ("units of at most a step per warp", 8, 4, [240, 1, 0, 17]),
     ("units up to three steps per warp that fill the grid", 16, 8, [60 + 42 * i for i in range(16)]),
