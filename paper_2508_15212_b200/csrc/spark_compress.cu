@@ -1359,21 +1359,23 @@ __global__ void append_advance_kernel(AppendArgs A)
 
 // Block append: n_new tokens per sequence at once (the keys a caller has kept dense for a while and now hands
 // over for pruning).  Three launches: fresh pages are zeroed, every (sequence, head, new token) gets a warp that
-// prunes it exactly like append_token_kernel, packed_lens advances by the tokens that found room.
+// prunes it exactly like append_token_kernel, packed_lens advances by the tokens that found room.  Up to eight warps a
+// CTA: with one, 128 sequences x 8 heads x 64 tokens (65536 CTAs) were bound by starting CTAs, 78 us a call against 53.
 struct AppendBlockArgs {
     AppendArgs a;
-    int n_new;
+    int n_new, n_fresh;           // new tokens; pages that can start inside them
 };
+constexpr int kBlockWarps = 8;
 
-__global__ void __launch_bounds__(32) append_block_clear_kernel(AppendBlockArgs B_)
+__global__ void __launch_bounds__(kBlockWarps * 32) append_block_clear_kernel(AppendBlockArgs B_)
 {
     grid_wait();
     grid_release();
     const AppendArgs& A = B_.a;
-    const int h = blockIdx.x, b = blockIdx.y, lane = threadIdx.x;
+    const int h = blockIdx.x, b = blockIdx.y, lane = threadIdx.x & 31, fresh = (blockIdx.z * blockDim.x + threadIdx.x) >> 5;
     const int t0 = A.packed_lens[b];
-    if (t0 < 0) return;
-    const int blk = (t0 + kPageTokens - 1) / kPageTokens + static_cast<int>(blockIdx.z);   // pages that start at or after t0
+    if (t0 < 0 || fresh >= B_.n_fresh) return;
+    const int blk = (t0 + kPageTokens - 1) / kPageTokens + fresh;          // pages that start at or after t0
     if (static_cast<int64_t>(blk) * kPageTokens >= static_cast<int64_t>(t0) + B_.n_new || blk >= A.max_blocks) return;
     const int64_t entry = (static_cast<int64_t>(b) * A.Hkv + h) * A.max_blocks + blk;
     const int64_t page_id = A.block_table ? A.block_table[entry] : entry;
@@ -1388,13 +1390,14 @@ __global__ void __launch_bounds__(32) append_block_clear_kernel(AppendBlockArgs 
 }
 
 template <typename E, bool kRank>
-__global__ void __launch_bounds__(32) append_block_token_kernel(AppendBlockArgs B_)
+__global__ void __launch_bounds__(kBlockWarps * 32) append_block_token_kernel(AppendBlockArgs B_)
 {
     grid_wait();
     grid_release();
     constexpr bool kBf16 = (sizeof(E) == 2);
     const AppendArgs& A = B_.a;
-    const int h = blockIdx.x, b = blockIdx.y, tok = blockIdx.z, lane = threadIdx.x;
+    const int h = blockIdx.x, b = blockIdx.y, tok = (blockIdx.z * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (tok >= B_.n_new) return;
     const PageLayout L = A.L;
     const int t0 = A.packed_lens[b];
     const int64_t t = static_cast<int64_t>(t0) + tok;
@@ -1502,16 +1505,17 @@ spark_status launch_append_block(const spark_params& p, const void* k_new, const
     A.sel = make_select(p);
     A.status = static_cast<int*>(workspace);
     Bk.n_new = n_new;
-    const int fresh = (n_new + kPageTokens - 1) / kPageTokens + 1;       // pages that can start inside the new tokens
-    launch_kernel(append_block_clear_kernel, dim3(p.n_kv_heads, p.batch, fresh), dim3(32), 0, stream, Bk);
-    const dim3 grid(p.n_kv_heads, p.batch, n_new);
+    Bk.n_fresh = (n_new + kPageTokens - 1) / kPageTokens + 1;
+    const int clear_warps = Bk.n_fresh < kBlockWarps ? Bk.n_fresh : kBlockWarps, warps = n_new < kBlockWarps ? n_new : kBlockWarps;
+    launch_kernel(append_block_clear_kernel, dim3(p.n_kv_heads, p.batch, (Bk.n_fresh + clear_warps - 1) / clear_warps), dim3(32 * clear_warps), 0, stream, Bk);
+    const dim3 grid(p.n_kv_heads, p.batch, (n_new + warps - 1) / warps), block(32 * warps);
     const bool rank = p.select != SPARK_SELECT_FIXED;
     if (p.dtype == SPARK_BF16) {
-        if (rank) launch_kernel(append_block_token_kernel<__nv_bfloat16, true>, grid, dim3(32), 0, stream, Bk);
-        else launch_kernel(append_block_token_kernel<__nv_bfloat16, false>, grid, dim3(32), 0, stream, Bk);
+        if (rank) launch_kernel(append_block_token_kernel<__nv_bfloat16, true>, grid, block, 0, stream, Bk);
+        else launch_kernel(append_block_token_kernel<__nv_bfloat16, false>, grid, block, 0, stream, Bk);
     } else {
-        if (rank) launch_kernel(append_block_token_kernel<float, true>, grid, dim3(32), 0, stream, Bk);
-        else launch_kernel(append_block_token_kernel<float, false>, grid, dim3(32), 0, stream, Bk);
+        if (rank) launch_kernel(append_block_token_kernel<float, true>, grid, block, 0, stream, Bk);
+        else launch_kernel(append_block_token_kernel<float, false>, grid, block, 0, stream, Bk);
     }
     launch_kernel(append_block_advance_kernel, dim3((p.batch + 127) / 128), dim3(128), 0, stream, Bk);
     *launches += 3;

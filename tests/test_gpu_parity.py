@@ -433,8 +433,9 @@ def test_append_with_more_than_32_kv_heads():
     assert float(np.abs(cache.decode(full.q).cpu().numpy() - o_ref).max()) <= TOL["bf16"]
 
 
-def test_block_append_equals_appending_one_token_at_a_time():
-    lens0, n = [37, 530, 16], 45
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 45, 129])               # (a CTA takes eight new tokens, or eight fresh pages)
+def test_block_append_equals_appending_one_token_at_a_time(n):
+    lens0 = [37, 530, 16]
     full = make("bf16", 3, 8, 2, [l + n for l in lens0], 8, 38, seed=152)
     S = max(lens0) + n
     lens0_t = torch.tensor(lens0, dtype=torch.int32, device="cuda")
