@@ -202,17 +202,19 @@ __global__ void evict_rowstats_kernel(EvictArgs A)
 //   contiguous piece, and two counts per warp and CTA give it its place.
 // What bounds it: dependent rounds over on-chip memory, a cluster barrier or two each.  As separate launches over all
 // SMs (pool, four 8-bit histograms, count, compact) the 8 x 131072 keys of a prompt took 82 us under the profiler,
-// this 22 us (four CTAs per unit: 30).
+// this 22 us (four CTAs per unit: 30).  Keys in the workspace (1M tokens, two units) are asked for eight at a time: 393 us a
+// prefill with one or four at a time, 336 so.
 // ------------------------------------------------------------------------------------------------
 constexpr int kSelThreads = 1024;
 constexpr int kSelWarps = kSelThreads / 32;
-constexpr int kSelCluster = 8;
+constexpr int kSelCluster = 8;             // CTAs per unit, at most (see select_cluster)
+constexpr int kSelBatch = 8;               // keys a thread asks for at once where it has that many
 constexpr int kVoteTile = 4 * kSelThreads; // raw votes staged at a time
 constexpr int kVoteHalo = 256;             // widest pooling half that is staged
 constexpr int kKeyCap = 36864;             // keys a CTA keeps in shared memory at most
 
 // keys of one CTA for a prefix of P tokens (a multiple of the CTA's threads)
-__host__ __device__ inline int select_share(int P) { return (P + kSelCluster * kSelThreads - 1) / (kSelCluster * kSelThreads) * kSelThreads; }
+__host__ __device__ inline int select_share(int P, int ctas) { return (P + ctas * kSelThreads - 1) / (ctas * kSelThreads) * kSelThreads; }
 
 // The bin (counted from the largest) that holds the need-th largest key, and the rank left inside it: v[] are the
 // cluster's counts of this thread's kPer consecutive bins, largest bin first.
@@ -236,14 +238,14 @@ __device__ __forceinline__ void pick_bin(const int (&v)[kPer], int need, int tid
     }
 }
 
-__global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads) evict_select_kernel(EvictArgs A)
+__global__ void __launch_bounds__(kSelThreads) evict_select_kernel(EvictArgs A)
 {
     extern __shared__ __align__(16) unsigned key_smem[];
     __shared__ int hist[2048 + 1024 + 1024], sums[2048 + 1024 + 1024];      // own counts; first CTA: the other CTAs'
     __shared__ int warp_sum[kSelWarps], warp_gt[kSelWarps], warp_eq[kSelWarps], total[2], pick[2];
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = static_cast<int>(cluster.block_rank()), h = blockIdx.y, b = blockIdx.z;
+    const int rank = static_cast<int>(cluster.block_rank()), ctas = gridDim.x, h = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float* raw = reinterpret_cast<float*>(key_smem + A.key_cap);              // [kVoteTile + 2 * kVoteHalo]
     for (int i = tid; i < 4096; i += kSelThreads) hist[i] = sums[i] = 0;
@@ -258,14 +260,14 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
     int32_t* kept = A.kept + static_cast<int64_t>(unit) * A.budget;
     if (rank == 0 && h == 0 && tid == 0) A.packed_lens[b] = S < A.budget ? S : A.budget;
     if (S <= A.budget) {                                       // kept whole (the same in every CTA of the cluster)
-        for (int t = rank * kSelThreads + tid; t < A.budget; t += kSelCluster * kSelThreads) kept[t] = t < S ? t : -1;
+        for (int t = rank * kSelThreads + tid; t < A.budget; t += ctas * kSelThreads) kept[t] = t < S ? t : -1;
         return;
     }
     const int P = S - A.W, k = A.budget - A.W, half = (A.pool - 1) / 2;
     if (rank == 0)
         for (int w = tid; w < A.W; w += kSelThreads) kept[k + w] = P + w;
     if (k == 0) return;                                        // the window alone
-    const int share = select_share(P), c0 = rank * share;
+    const int share = select_share(P, ctas), c0 = rank * share;
     const int n = max(0, min(share, P - c0));                  // this CTA's keys: tokens c0 .. c0 + n - 1
     const int64_t base = static_cast<int64_t>(unit) * A.S_max;
     unsigned* keys = share <= A.key_cap ? key_smem : A.pooled + base + c0;
@@ -368,11 +370,16 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
         const int shift = pass == 1 ? 10 : 0;
         int* hp = hist + 1024 + 1024 * pass;
         const unsigned top = thr >> (shift + 10);
-#pragma unroll 4
-        for (int i = tid; i < n; i += kSelThreads) {
-            const unsigned key = keys[i];
-            if ((key >> (shift + 10)) == top) atomicAdd(&hp[(key >> shift) & 1023u], 1);
+        auto count = [&](unsigned key) { if ((key >> (shift + 10)) == top) atomicAdd(&hp[(key >> shift) & 1023u], 1); };
+        int i = tid;
+        for (; i + (kSelBatch - 1) * kSelThreads < n; i += kSelBatch * kSelThreads) {
+            unsigned key[kSelBatch];
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u) key[u] = keys[i + u * kSelThreads];
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u) count(key[u]);
         }
+        for (; i < n; i += kSelThreads) count(keys[i]);
         c = choose(hp, sums + 1024 + 1024 * pass, std::integral_constant<int, 1>(), need, false);
         thr |= static_cast<unsigned>(c.x) << shift;
         need = c.y;
@@ -380,11 +387,18 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
     // keys above / equal to the threshold, per warp (a contiguous piece each) and per CTA
     const int seg = share / kSelWarps, s0 = warp * seg;
     int gt = 0, eq = 0;
-#pragma unroll 4
-    for (int i = s0 + lane; i < s0 + seg; i += 32) {
-        const unsigned key = i < n ? keys[i] : 0u;
-        gt += i < n && key > thr;
-        eq += i < n && key == thr;
+    const int s1 = min(n, s0 + seg);                           // (the same in every lane)
+    auto above = [&](unsigned key) { gt += key > thr; eq += key == thr; };
+    {
+        int i = s0 + lane;
+        for (; i - lane + 32 * kSelBatch <= s1; i += 32 * kSelBatch) {
+            unsigned key[kSelBatch];
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u) key[u] = keys[i + 32 * u];
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u) above(key[u]);
+        }
+        for (; i < s1; i += 32) above(keys[i]);
     }
     gt = __reduce_add_sync(0xffffffffu, gt);
     eq = __reduce_add_sync(0xffffffffu, eq);
@@ -399,13 +413,11 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
         const int* t = cluster.map_shared_rank(total, r);
         own_gt += t[0]; b_eq += t[1];
     }
-    if (rank == kSelCluster - 1 && tid == 0 && own_gt + total[0] + need != k) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+    if (rank == ctas - 1 && tid == 0 && own_gt + total[0] + need != k) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
     b_gt += own_gt;
     const unsigned lt = (1u << lane) - 1u;
-    for (int i0 = s0; i0 < s0 + seg && i0 < n; i0 += 32) {
-        const int i = i0 + lane;
-        const unsigned key = i < n ? keys[i] : 0u;
-        const unsigned mg = __ballot_sync(0xffffffffu, i < n && key > thr), me = __ballot_sync(0xffffffffu, i < n && key == thr);
+    auto place = [&](int i, bool on, unsigned key) {           // the warp's keys at i - lane .. i - lane + 31
+        const unsigned mg = __ballot_sync(0xffffffffu, on && key > thr), me = __ballot_sync(0xffffffffu, on && key == thr);
         const int eq_rank = b_eq + __popc(me & lt);            // equal keys on lower positions
         const int pos = b_gt + __popc(mg & lt) + min(eq_rank, need);
         if (((mg >> lane) & 1u) || (((me >> lane) & 1u) && eq_rank < need)) {
@@ -413,8 +425,30 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
         }
         b_gt += __popc(mg);
         b_eq += __popc(me);
+    };
+    int i0 = s0;
+    for (; i0 + 32 * kSelBatch <= s1; i0 += 32 * kSelBatch) {
+        unsigned key[kSelBatch];
+#pragma unroll
+        for (int u = 0; u < kSelBatch; ++u) key[u] = keys[i0 + 32 * u + lane];
+#pragma unroll
+        for (int u = 0; u < kSelBatch; ++u) place(i0 + 32 * u + lane, true, key[u]);
     }
+    for (; i0 < s1; i0 += 32) place(i0 + lane, i0 + lane < s1, i0 + lane < s1 ? keys[i0 + lane] : 0u);
     cluster.sync();                                            // the others may still be reading this CTA's totals
+}
+
+// CTAs per unit (a power of two).  A barrier of the cluster costs more than the keys it spares a CTA below some 8000, and a
+// cluster of 1024-thread CTAs that does not fit beside the others waits for a whole second round: 64 x 1500 tokens with 8 KV
+// heads (512 units) took 559 us an evicting prefill with eight CTAs per unit and takes 268 with one, 4 x 8000 85.5 and 66;
+// with 16 units of 60000 four are better than eight (156 against 164), with four units of 32768 or 131072 eight (67.5, 188)
+// than four (69.5, 199).  Very wide pools are bound by their pooling, which wants every SM.
+inline int select_cluster(int64_t units, int prefix, int pool)
+{
+    if (pool > 64) return kSelCluster;
+    int c = prefix <= 8192 ? 1 : (units <= 12 ? 8 : (units <= 32 ? 4 : (units <= 64 ? 2 : 1)));
+    while (c < kSelCluster && select_share(prefix, c) > kKeyCap) c *= 2;  // the keys stay on chip if they can
+    return c;
 }
 
 bool evict_tc_supported(const spark_params& p);
@@ -470,12 +504,17 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
         else launch_kernel(evict_scores_kernel<float, 2>, grid, dim3(kEvThreads), smem, stream, A);
         *launches += 3;
     }
-    const int most = select_share(max_seq_tokens > p.window ? max_seq_tokens - p.window : 1);
+    DeviceInfo info;
+    int dev = 0;
+    if (!device_info(&dev, &info)) return SPARK_ERR_CUDA;
+    const int prefix = max_seq_tokens > p.window ? max_seq_tokens - p.window : 1;
+    const int ctas = select_cluster(static_cast<int64_t>(units), prefix, p.pool_kernel);
+    const int most = select_share(prefix, ctas);
     A.key_cap = most < kKeyCap ? most : kKeyCap;
     const size_t key_bytes = (static_cast<size_t>(A.key_cap) + kVoteTile + 2 * kVoteHalo) * sizeof(unsigned);
     static unsigned char select_raised[kMaxDevices] = {};
-    if (!allow_max_smem(evict_select_kernel, select_raised)) return SPARK_ERR_CUDA;
-    launch_kernel(evict_select_kernel, dim3(kSelCluster, p.n_kv_heads, p.batch), dim3(kSelThreads), key_bytes, stream, A);
+    if (!allow_max_smem(evict_select_kernel, dev, info.smem_optin, select_raised)) return SPARK_ERR_CUDA;
+    launch_cluster(evict_select_kernel, ctas, dim3(ctas, p.n_kv_heads, p.batch), dim3(kSelThreads), key_bytes, stream, A);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
 }

@@ -57,6 +57,13 @@ def test_top_p_selection_with_ties(kind, p, cap):
     assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("n_seq,longest", [(1, 8200), (2, 8200), (4, 9000), (8, 8500), (9, 8300), (20, 700)])
+def test_eviction_select_clusters(n_seq, longest):
+    """Eight, four, two and one CTA per (sequence, KV head), by the number of units and the longest prefix."""
+    lens = [max(40, longest - 977 * (i % 8)) for i in range(n_seq)]
+    check_eviction_case("bf16", lens, 4, 300, 1, Hkv=8, pool=7, seed=501)
+
+
 @pytest.mark.parametrize("p,cap", [(0.5, 128), (0.95, 128), (1.0, 128), (1.0, 40), (0.95, 40)])
 def test_top_p_of_odd_values_equals_appending_them(p, cap):
     """Infinities, NaN, all-zero rows, saliencies over more than 22 octaves (their sums round, and p = 1 asks for all of
