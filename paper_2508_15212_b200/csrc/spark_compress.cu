@@ -7,6 +7,8 @@
 // token (App. "Caching Pruned Channel Statistics").  With value-channel pruning (App. "Pruning Value
 // Cache Channels") the same per-token selection runs on |V[t][j]| and the page stores the kept values and a
 // second mask instead of the dense value row.
+#include <type_traits>
+
 #include "spark_common.cuh"
 
 namespace spark {
@@ -15,24 +17,23 @@ constexpr unsigned kFullMask = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------------
 // a[b][h][j] = max(|mean over the G*W window queries of the group|, eps).
-// 512 threads: a thread sums 16 bytes' worth of channels over every 32nd (fp32: 16th) row in double, the row groups
-// are then added in a fixed order.  (The sum is exact in double for any order unless its terms differ by more than
+// 128 to 512 threads (qnorm_threads): a thread sums 16 bytes' worth of channels over every 32nd (fp32: 16th) row of 512
+// threads in double, the row groups are then added in a fixed order.  (The sum is exact in double for any order unless its terms differ by more than
 // 2^21.)  The chain that bounds the kernel is a load and a few adds: one thread per channel walking all rows took
 // 8.3 us for 128 rows, this 7.1 (both cold), and the page kernel's first loads now run under it.
 // Thread 0 of the first head also publishes packed_lens when there is no eviction step.
 // ------------------------------------------------------------------------------------------------
-constexpr int kQnThreads = 512;
-template <typename E>
-__global__ void __launch_bounds__(kQnThreads)
+template <typename E, int kThreads, bool kReleaseEarly>
+__global__ void __launch_bounds__(kThreads)
 window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, float eps,
                     float* __restrict__ qnorm, const int32_t* __restrict__ seq_lens,
                     int32_t* __restrict__ packed_lens, int max_seq_tokens, int* status)
 {
     constexpr int kVec = 16 / sizeof(E);                       // channels per 16-byte load
-    constexpr int kChunks = kHeadDim / kVec, kGroups = kQnThreads / kChunks;
+    constexpr int kChunks = kHeadDim / kVec, kGroups = kThreads / kChunks;
     __shared__ double part[kGroups / 2][kHeadDim];
     grid_wait();
-    grid_release();
+    if (kReleaseEarly) grid_release();
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     const int G = Hq / Hkv, rows = G * W;
     const int c = tid % kChunks, grp = tid / kChunks;
@@ -59,6 +60,7 @@ window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, floa
     if (grp < kGroups / 2)
 #pragma unroll
         for (int i = 0; i < kVec; ++i) part[grp][c * kVec + i] += acc[i];
+    if (!kReleaseEarly) grid_release();
     __syncthreads();
     if (tid < kHeadDim) {
         double sum = 0.0;
@@ -691,7 +693,7 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 //   descent (compress_pages4_kernel, which fp32 storage and sampled recovery keep); 8 heads x 32768 tokens:
 //   104 -> 62 us; prefill of 32K tokens 132.4 -> 88 us (24 warps a SM; with 16 3 us more).
 // ------------------------------------------------------------------------------------------------
-constexpr int kWarpPageWarps = 4;
+constexpr int kWarpPageWarps = 4;      // pages (warps) of a CTA; one where no sequence has more (1000 x 16 tokens: 84 us with four, 57 with one)
 constexpr int kFewKeys = 2;            // keys left between the ends that are told apart by their full bits
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
 // SparK-p: the saliencies of a page (fp32), and over them, once read, mask | mu | slot rows
@@ -1156,12 +1158,12 @@ __device__ __forceinline__ int select_section_topp(const unsigned char* tile, un
     return live ? count : 0;
 }
 
-template <bool kPV, bool kTopP>
-__global__ void __launch_bounds__(kWarpPageWarps * 32, kTopP ? 4 : (kPV ? 5 : 6)) compress_pages_warp_kernel(CompressArgs A)
+template <bool kPV, bool kTopP, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kTopP ? 4 : (kPV ? 5 : 6))) compress_pages_warp_kernel(CompressArgs A)
 {
     extern __shared__ __align__(16) unsigned char page_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int blk = blockIdx.x * kWarpPageWarps + warp, h = blockIdx.y, b = blockIdx.z;
+    const int blk = blockIdx.x * kWarps + warp, h = blockIdx.y, b = blockIdx.z;
     const PageLayout L = A.L;
     // dense value rows go straight to the page; SparK-p pages carry the slot rows behind them, and in shared memory those
     // (and the head of the page) come to lie over the saliencies
@@ -1198,7 +1200,9 @@ __global__ void __launch_bounds__(kWarpPageWarps * 32, kTopP ? 4 : (kPV ? 5 : 6)
     if (n > 0) page_id = A.block_table ? A.block_table[entry] : entry;        // no table: contiguous cache
     const bool page_ok = page_id >= 0 && page_id < A.n_pool_pages;
     if (!A.gather) { grid_wait(); grid_release(); }
-    a_s[threadIdx.x] = A.qnorm[(static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < kHeadDim / (32 * kWarps); ++i)
+        a_s[i * (32 * kWarps) + threadIdx.x] = A.qnorm[(static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + i * (32 * kWarps) + threadIdx.x];
     __syncthreads();
     if (n <= 0) return;                                        // warp-uniform; no CTA barrier below
     if (!page_ok) {
@@ -1687,6 +1691,28 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_pages_kernel(UnpackArgs
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
+// Threads of the window norm per (sequence, KV head) with `rows` window rows.  Few units: as many as shorten the chain of
+// loads (the page kernel of 1 x 32768 tokens waits for it: 65.7, 63.5, 61.3 us a prefill with 128, 256, 512).  Many units:
+// as many as keep them resident together (us per prefill of one-token prompts with 128, 256, 512 threads: 512 units x 64
+// rows 12.4, 12.4, 15.8; 1024 x 128 18.5, 19.4, 27.4; 512 x 512 34.7, 22.6, 22.7; 4096 x 16 39, 49, 74).  fp32 rows take
+// twice the threads (512 x 64: 15.2, 14.8, 13.3; 1024 x 64: 16.7, 16.1, 17.8; 4096 x 16: 38, 43, 51).
+inline int qnorm_threads(int64_t units, int rows, bool bf16)
+{
+    if (!bf16) return units <= 512 ? 512 : 128;
+    return units <= 256 ? 512 : (rows > 128 ? 256 : 128);
+}
+
+// Released at its top, the window norm lets the page kernel become resident beside it and load keys and values meanwhile.
+// With a CTA of the norm on half the SMs or more, a small page kernel's CTAs crowd onto the SMs that are left, so it is let in
+// at the end (16 x 60 tokens with 8 KV heads: 18.7 us a prefill released at the top, 11.9 at the end; 16 x 200 18.8 and 17.3).
+// A page kernel that fills every SM anyway, or a long norm, is better let in early (16 x 400: 20.9 and 21.8; 32 x 100 with
+// 512 window rows: 23.0 and 25.3).
+inline bool qnorm_release_early(int64_t units, int rows, int n_blocks)
+{
+    const int64_t page_ctas = units * ((n_blocks + kWarpPageWarps - 1) / kWarpPageWarps);
+    return units <= 64 || rows > 256 || page_ctas > 740;
+}
+
 size_t compress_workspace_bytes(const spark_params& p, int64_t max_seq_tokens)
 {
     return kWorkspaceHeader + evict_workspace_bytes(p, max_seq_tokens);
@@ -1706,19 +1732,31 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
                                                kept_tokens, workspace, stream, launches);
         if (st_e != SPARK_OK) return st_e;
     }
-    const float eps = p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f;
-    const dim3 qgrid(p.n_kv_heads, p.batch);
-    if (p.dtype == SPARK_BF16)
-        launch_kernel(window_qnorm_kernel<__nv_bfloat16>, qgrid, dim3(kQnThreads), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
-                      eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
-    else
-        launch_kernel(window_qnorm_kernel<float>, qgrid, dim3(kQnThreads), 0, stream, q_win, p.n_q_heads, p.n_kv_heads, p.window,
-                      eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
-    ++*launches;
-    if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
-
     const int max_packed = (evict && p.token_budget < max_seq_tokens) ? p.token_budget : max_seq_tokens;
     const int n_blocks = (max_packed + kPageTokens - 1) / kPageTokens;
+    const float eps = p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f;
+    const dim3 qgrid(p.n_kv_heads, p.batch);
+    const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
+    const int rows = p.n_q_heads / p.n_kv_heads * p.window;
+    auto window_norm = [&](auto elem, auto threads, auto early) {
+        constexpr int kThreads = decltype(threads)::value;
+        launch_kernel(window_qnorm_kernel<decltype(elem), kThreads, decltype(early)::value>, qgrid, dim3(kThreads), 0, stream, q_win, p.n_q_heads,
+                      p.n_kv_heads, p.window, eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
+    };
+    auto by_threads = [&](auto elem, auto early) {
+        const int n = qnorm_threads(units, rows, p.dtype == SPARK_BF16);
+        if (n == 128) window_norm(elem, std::integral_constant<int, 128>(), early);
+        else if (n == 256) window_norm(elem, std::integral_constant<int, 256>(), early);
+        else window_norm(elem, std::integral_constant<int, 512>(), early);
+    };
+    auto by_release = [&](auto elem) {
+        if (qnorm_release_early(units, rows, n_blocks)) by_threads(elem, std::true_type());
+        else by_threads(elem, std::false_type());
+    };
+    if (p.dtype == SPARK_BF16) by_release(__nv_bfloat16());
+    else by_release(0.f);
+    ++*launches;
+    if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
     if (n_blocks == 0) return SPARK_OK;
     CompressArgs A;
     A.k = k; A.v = v; A.sb = sb; A.sh = sh; A.st = st;
@@ -1732,12 +1770,17 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const bool pv = A.L.keep_v < kHeadDim, topp = p.select == SPARK_SELECT_TOP_P;
     if (p.dtype == SPARK_BF16 && p.recovery == SPARK_RECOVER_DEGENERATE && (p.select == SPARK_SELECT_FIXED || (topp && !pv))) {
         if (!evict) A.lens = seq_lens;                         // readable before the window norm has ended
-        const size_t smem = kHeadDim * 4 + kWarpPageWarps * (kTileBytes + static_cast<size_t>(topp ? warp_topp_room(A.L) : (pv ? A.L.page_bytes : A.L.v_off)));
-        auto kernel = topp ? compress_pages_warp_kernel<false, true> : (pv ? compress_pages_warp_kernel<true, false> : compress_pages_warp_kernel<false, false>);
-        static unsigned char smem_raised[3][kMaxDevices] = {};
+        const int warps = n_blocks == 1 ? 1 : kWarpPageWarps;
+        const size_t smem = kHeadDim * 4 + warps * (kTileBytes + static_cast<size_t>(topp ? warp_topp_room(A.L) : (pv ? A.L.page_bytes : A.L.v_off)));
+        auto pick = [&](auto w) {
+            constexpr int kWarps = decltype(w)::value;
+            return topp ? compress_pages_warp_kernel<false, true, kWarps> : (pv ? compress_pages_warp_kernel<true, false, kWarps> : compress_pages_warp_kernel<false, false, kWarps>);
+        };
+        auto kernel = warps == 1 ? pick(std::integral_constant<int, 1>()) : pick(std::integral_constant<int, kWarpPageWarps>());
+        static unsigned char smem_raised[3][kMaxDevices] = {};                // (a single warp needs less than the limit)
         if (smem > 48 * 1024 && !allow_max_smem(kernel, smem_raised[topp ? 2 : (pv ? 1 : 0)])) return SPARK_ERR_CUDA;
-        const dim3 wgrid((n_blocks + kWarpPageWarps - 1) / kWarpPageWarps, p.n_kv_heads, p.batch);
-        const cudaError_t e = launch_kernel(kernel, wgrid, dim3(kWarpPageWarps * 32), smem, stream, A);
+        const dim3 wgrid((n_blocks + warps - 1) / warps, p.n_kv_heads, p.batch);
+        const cudaError_t e = launch_kernel(kernel, wgrid, dim3(warps * 32), smem, stream, A);
         ++*launches;
         return e == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }
