@@ -446,14 +446,17 @@ spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, con
     A.q_win = q_win; A.k = k; A.sb = sb; A.sh = sh; A.st = st; A.seq_lens = seq_lens;
     A.Hq = p.n_q_heads; A.Hkv = p.n_kv_heads; A.W = p.window; A.budget = p.token_budget; A.S_max = max_seq_tokens;
     const int n_tiles = (max_seq_tokens + kTcTile - 1) / kTcTile;
-    // Two CTAs are resident per SM; a CTA pays a fixed start-up (tensor-memory allocation, the query
-    // block, the first key tile), so the tiles are cut into about one wave of CTAs, at least 8 tiles each.
+    // A CTA pays a fixed start-up (tensor-memory allocation, the query block, the first key tile), so the tiles are cut into
+    // one wave of CTAs, at least 8 tiles each.  Up to 128 query rows two CTAs are resident per SM; above that one takes 129 KB
+    // of shared memory and all 512 tensor-memory columns.  (us per evicting prefill with 129 to 256 rows, cut for two CTAs per
+    // SM -> for one: 1 x 131072 with 28 / 4 heads 188 -> 169, with 64 / 8 heads 308 -> 296, 2 x 20000 102 -> 72.)
     int dev = 0;
     DeviceInfo info;
     if (!device_info(&dev, &info)) return SPARK_ERR_CUDA;
     const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
-    const int64_t wave = 2 * static_cast<int64_t>(info.n_sms);
-    int64_t per = (static_cast<int64_t>(n_tiles) * units + wave - 1) / wave;
+    const int64_t wave = (Rpad <= 128 ? 2 : 1) * static_cast<int64_t>(info.n_sms);
+    const int64_t parts = units < wave ? wave / units : 1;
+    int64_t per = (n_tiles + parts - 1) / parts;
     if (per < 8) per = 8;
     if (per > n_tiles) per = n_tiles > 0 ? n_tiles : 1;
     A.tiles_per_cta = static_cast<int>(per);
