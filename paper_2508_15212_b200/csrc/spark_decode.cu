@@ -80,9 +80,8 @@ template <int G> struct SmemF32 {
     static constexpr int kTabBytes = kHeadDim * GPD * 8; // sized for the double table (>= the float one)
     static constexpr int kQsum = kCtrlBytes;             // [kMaxCap][8] double
     static constexpr int kPscr = kQsum + kMaxCap * 64;
-    static constexpr int kTab = kPscr + kConsumerWarps * 32 * GPP * 4;       // [cap] tables, then merge area, prefix and ring
-    static constexpr int merge_off(int cap) { return kTab + cap * kTabBytes; }
-    static constexpr int fixed(int cap) { return (merge_off(cap) + merge_bytes(kConsumerWarps, cap, G) + 127) / 128 * 128; }
+    static constexpr int kMl = kPscr + kConsumerWarps * 32 * GPP * 4;        // [kMaxCap][G] (M, L) of the epoch's units
+    static constexpr int kEnd = (kMl + kMaxCap * G * 8 + 127) / 128 * 128;   // then prefix, ring, records, tables
 };
 
 template <int G, typename E, int R>
@@ -99,22 +98,23 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
     double* qsum_all = reinterpret_cast<double*>(smem + S::kQsum);
     float* pscr_all = reinterpret_cast<float*>(smem + S::kPscr);
-    float* merge = reinterpret_cast<float*>(smem + S::kTab + A.cap * S::kTabBytes);
-    float* unit_ml = merge + merge_state_floats(kConsumerWarps, A.cap, G);
+    float* unit_ml = reinterpret_cast<float*>(smem + S::kMl);
     unsigned char* ring = smem + A.ring_off;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const PageLayout L = A.L;
-    const int NS = A.nslots;
 
     prefetch_block_table(A, tid, kDecodeThreads);
     if (warp == kConsumerWarps) {
-        const CtaRun run = producer_prologue(A, C, lane, kDecodeThreads);
-        producer_loop<kConsumerWarps>(A, C, ring, run, lane);
+        Plan pl;
+        const CtaRun run = producer_prologue(A, C, lane, kDecodeThreads, pl);
+        producer_loop<kConsumerWarps>(A, C, ring, run, pl, lane);
         return;
     }
     consumer_wait_plan(kDecodeThreads);
-    const int c0 = C.run->c0, c1 = C.run->c1;
+    const int c0 = C.run->c0, c1 = C.run->c1, NS = C.plan->nslots, cap = C.plan->cap;
+    float* merge = reinterpret_cast<float*>(smem + C.plan->merge_off);
+    unsigned char* tabs = smem + C.plan->tab_off;
     if (!A.late_wait) {
         consumer_wait_previous(A);                         // q, qnorm, out and the workspace from here on
         write_empty_sequences<kConsumerThreads>(A, C.prefix, tid);
@@ -122,14 +122,14 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
     float* pscr = pscr_all + warp * 32 * GPP;
     for (int g = c0; g < c1;) {
-        const Epoch ep = make_epoch(C.prefix, A.Hkv, A.cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
+        const Epoch ep = make_epoch(C.prefix, A.Hkv, cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
 
         // ---- per-unit table: entry j = { q_0[j]*c, ..., q_{G-1}[j]*c, 1/a[j] },  c = scale*log2(e)
         UnitRef u = ep.first;
 #pragma unroll 1
         for (int e = 0; e < ep.n_units; ++e) {
             if (e) next_unit(C.prefix, A.Hkv, u);
-            TabT* qtab = reinterpret_cast<TabT*>(smem + S::kTab + e * S::kTabBytes);
+            TabT* qtab = reinterpret_cast<TabT*>(tabs + e * S::kTabBytes);
             for (int idx = tid; idx < kHeadDim * GP; idx += kConsumerThreads) {
                 const int j = idx / GP, col = idx - j * GP;
                 TabT val = 0;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 #pragma unroll 1
         for (int e = 0; e < ep.n_units; ++e)
             if (warp < G) {                                // Qsum[g] = sum_j q_g[j]*c / a[j]
-                const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kTab + e * S::kTabBytes);
+                const TabT* qtab = reinterpret_cast<const TabT*>(tabs + e * S::kTabBytes);
                 double part = 0.0;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -160,9 +160,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
 
         // ---- this warp's run of the epoch's steps, unit by unit ----
         const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kConsumerWarps, run_r = n_ep - run_q * kConsumerWarps;
-        int pos = ep.e0 + (A.cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
-        const int pos_end = A.cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
-        const int stride = A.cap == 1 ? kConsumerWarps : 1;
+        int pos = ep.e0 + (cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
+        const int pos_end = cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
+        const int stride = cap == 1 ? kConsumerWarps : 1;
         int n = (ep.e0 - c0) + warp;                       // ring step of the warp's next step
         if (warp == kConsumerWarps - 1) describe_epoch<kConsumerWarps>(A, C, ep, lane);      // for the merge; this warp's run is never the longer
         u = ep.first;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
         while (pos < pos_end) {
             const int part_end = min(pos_end, u.start + u.steps);
             const int b = u.b, h = u.h, len = C.lens[u.b];
-            const TabT* qtab = reinterpret_cast<const TabT*>(smem + S::kTab + eu * S::kTabBytes);
+            const TabT* qtab = reinterpret_cast<const TabT*>(tabs + eu * S::kTabBytes);
             const double* qsum = qsum_all + eu * 8;
             float m_run[G], l_run[G], acc[G][4];
 #pragma unroll
@@ -408,22 +408,24 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     set_divisors(A, units, grid);
-    // Two units per epoch only where CTAs hold several: the second unit's table and records cost a ring slot (of six or
-    // seven: 2 x 7926 tokens, G = 4, T = 89: 43.9 us with six slots, 35.2 us with seven).
     A.whole_steps = 0;                                     // (a step is 32 tokens of double sums: splitting pays)
-    A.cap = 2 * units <= grid ? 1 : 2;
-    A.tab_off = S::kTab;
-    A.prefix_off = S::fixed(A.cap);
+    A.prefix_off = S::kEnd;
     A.ring_off = A.prefix_off + prefix_bytes(A.B);
-    int ns = (smem_optin - A.ring_off) / A.slot_stride;
-    if (ns > kMaxSlots) ns = kMaxSlots;
-    if (ns < 2) return SPARK_ERR_UNSUPPORTED;
     // no more slots than a CTA has steps: a small call then leaves the SM room for the next kernel's CTA, whose
     // start-up runs under this one's end
-    const int64_t most = max_steps_per_cta(units, A.max_blocks, A.pps, grid);
-    if (ns > most) ns = static_cast<int>(most < 2 ? 2 : most);
-    A.nslots = ns;
-    const size_t smem = A.ring_off + static_cast<size_t>(ns) * A.slot_stride;
+    const int64_t steps = max_steps_per_cta(units, A.max_blocks, A.pps, grid);
+    const EpochRoom room = epoch_room(A, kConsumerWarps, G, S::kTabBytes, smem_optin, steps < 2 ? 2 : (steps > kMaxSlots ? kMaxSlots : static_cast<int>(steps)));
+    const int one = room.ns[0];
+    if (one < 2) return SPARK_ERR_UNSUPPORTED;
+    A.caps.by_units = 1;
+    A.caps.shortest = A.caps.even = 1;
+    if (A.B > 1 || 2 * units > grid) {                     // (see choose_cap: a slot per warp, and one of them to spare)
+        const int enough = one < kConsumerWarps ? one : kConsumerWarps;
+        A.caps.even = room.with(enough) < 2 ? 1 : 2;
+        A.caps.shortest = room.with(enough > 2 ? enough - 1 : 2);
+    }
+    A.caps.middle = A.caps.longest = A.caps.even;
+    const size_t smem = room.bytes(A.caps.shortest);
     if (!allow_max_smem(decode_scalar_kernel<G, E, R>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
     return launch_kernel(decode_scalar_kernel<G, E, R>, dim3(grid), dim3(kDecodeThreads), smem, stream, A) == cudaSuccess
                ? SPARK_OK : SPARK_ERR_CUDA;
@@ -488,7 +490,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     A.status = reinterpret_cast<int*>(ws);
     A.tickets = reinterpret_cast<int*>(ws + kWorkspaceHeader);
     A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(units * sizeof(int), 256));
-    A.nslots = 0; A.slot_stride = 0; A.pps = 1; A.cap = 1; A.tab_off = 0; A.prefix_off = 0; A.ring_off = 0;
+    A.slot_stride = 0; A.pps = 1; A.caps = EpochCaps{}; A.prefix_off = 0; A.ring_off = 0;
     A.overlap = (p.flags & SPARK_FLAG_OVERLAP_PREVIOUS) ? 1 : 0;
     A.seed = p.seed;
     A.q_by_value = q_by_value ? 1 : 0;

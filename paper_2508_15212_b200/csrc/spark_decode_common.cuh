@@ -35,6 +35,19 @@ struct FastDiv {
     }
 };
 
+// Units per epoch that a launch may use, and what each number leaves for the ring.  An epoch's units take shared memory
+// (operand tables, records) from the ring, so the number is chosen with the plan, from the lengths: few where CTAs' runs are
+// long and a unit boundary (3 us) is a small part of them, many where a CTA meets many units, one where it meets one.
+// (Chosen from the cache's capacity instead, eight sequences of 150..4000 tokens took 19.6 us in a cache for 4016 tokens,
+// 27.0 in one for 16 K and 35.6 in one for 128 K; 32 x 2048 41.6 and, in a cache for 32 K, 49.3.)
+struct EpochCaps {
+    unsigned long long slots;                // ring slots with 1 .. kMaxCap units (a byte each)
+    int tail_base, tail_step;                // bytes of the record area with one unit, and more for each further one
+    int shortest, middle, even, longest;     // units for runs of up to kRunShort, kRunMiddle, kRunLong steps and above
+    int by_units;                            // CUDA-core kernel: by the units that a CTA may meet (see choose_cap)
+};
+constexpr int kRunShort = 160, kRunMiddle = 512, kRunLong = 1024;
+
 struct DecodeArgs {
     const void* q;
     const unsigned char* pages;
@@ -53,17 +66,15 @@ struct DecodeArgs {
     int* status;
     int* tickets;
     float* partials;
-    int nslots;
     int slot_stride;
     int pps;                                 // pages per step (= per ring slot): 1 or 2
     FastDiv by_grid, by_hkv;                 // CTAs of the grid; KV heads
     int per_unit, extra;                     // aligned mode (see Plan): CTAs per unit; units with one more
     FastDiv by_q, by_q1;                     // per_unit and per_unit + 1
-    int cap;                                 // units per epoch
+    EpochCaps caps;                          // units per epoch, chosen with the plan
     int whole_steps;                         // a step per consumer warp; units up to this are not split (see Plan)
-    int tab_off;                             // shared-memory offset of the epoch's operand tables
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
-    int ring_off;                            // shared-memory offset of the ring (behind the prefix)
+    int ring_off;                            // shared-memory offset of the ring (behind the prefix); records and tables follow it
     int late_wait;                           // the kernel before waited at its top, released after that and writes only other_out /
                                              // other_lse: wait where they are read (a successor may be released before that)
     int overlap;                             // the page stream need not wait for the kernel before (SPARK_FLAG_OVERLAP_PREVIOUS)
@@ -81,26 +92,13 @@ constexpr int kCtrlBytes = 1024;                                 // full[32], em
 // are as large as the batch needs, so small batches leave their room to the ring
 inline int prefix_bytes(int batch) { return ((2 * batch + 1) * 4 + 127) / 128 * 128; }
 
-// Shared merge area: `records` states of `g` heads ([record][head][kRec] floats: 128 outputs, m, l, and a spare
+// Shared merge area: `nw + cap - 1` states of `g` heads ([record][head][kRec] floats: 128 outputs, m, l, and a spare
 // word for the record's weight), reused by the final combine for the weights of up to kMaxCtas parts, the heads'
-// (M, L) and one float4 per consumer thread; behind it the (M, L) pairs of the epoch's units.
-__host__ __device__ constexpr int merge_state_floats(int nw, int cap, int g)
+// (M, L) and one float4 per consumer thread.
+__host__ __device__ constexpr int merge_step(int g) { return (g * kRec * 4 + 127) / 128 * 128; }
+__host__ __device__ constexpr int merge_base(int nw, int g)
 {
-    return (nw + cap - 1) * g * kRec > kMaxCtas * g * 2 + nw * 32 * 4 ? (nw + cap - 1) * g * kRec : kMaxCtas * g * 2 + nw * 32 * 4;
-}
-__host__ __device__ constexpr int merge_bytes(int nw, int cap, int g) { return (merge_state_floats(nw, cap, g) + cap * g * 2) * 4; }
-
-// Units of an epoch that a launch would like: as many as a CTA's run meets when the sequences are equally long, and the
-// most where a batch of unequal sequences is so short that a CTA may meet many (a unit beyond the cap costs a second
-// epoch: 8 sequences of 150..4000 tokens, whose CTAs meet up to seven units, took 23.9 us with five and 20.9 with
-// eight).  A single sequence with several CTAs per unit needs one.
-inline int epoch_cap(int batch, int64_t units, int max_blocks, int grid)
-{
-    if (batch == 1 && 2 * units <= grid) return 1;
-    int64_t c = (units + grid - 1) / grid + 1;
-    const int64_t run = units * max_blocks / grid;                            // a CTA's steps in a full cache
-    if (batch > 1 && run <= 256) c = run <= 160 ? kMaxCap : c + 3;
-    return c > kMaxCap ? kMaxCap : static_cast<int>(c);
+    return ((nw * g * kRec > kMaxCtas * g * 2 + nw * 32 * 4 ? nw * g * kRec : kMaxCtas * g * 2 + nw * 32 * 4) * 4 + 127) / 128 * 128;
 }
 
 // ---- PTX helpers ----------------------------------------------------------------------------------
@@ -299,6 +297,8 @@ struct Plan {
     int aligned;      // 0: stream, 1: aligned mode, 2: whole units
     int unit_steps;   // aligned: steps of every unit
     int q, rem;       // aligned: CTAs per unit
+    int cap, nslots;  // units per epoch and the ring slots that they leave
+    int merge_off, tab_off;      // shared-memory offsets of the records and of the operand tables (behind the ring)
 };
 
 // A CTA's run of steps [c0, c1) on the line and the unit of its first step.
@@ -328,8 +328,9 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, i
     c.empty = c.full + kMaxSlots;
     c.abort_flag = reinterpret_cast<volatile int*>(smem + 512);
     c.plan = reinterpret_cast<Plan*>(smem + 528);
-    c.last_flag = reinterpret_cast<volatile int*>(smem + 560);
-    c.epoch = reinterpret_cast<volatile int*>(smem + 600);
+    c.last_flag = reinterpret_cast<volatile int*>(smem + 576);
+    c.epoch = reinterpret_cast<volatile int*>(smem + 608);
+    static_assert(528 + sizeof(Plan) <= 576 && 576 + kMaxCap * 4 <= 608, "control block");
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
     c.units = reinterpret_cast<EpochUnit*>(smem + 768);
     c.run = reinterpret_cast<CtaRun*>(smem + 960);
@@ -363,10 +364,28 @@ __device__ __forceinline__ void prefetch_block_table(const DecodeArgs& A, int ti
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + o));
 }
 
-__device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads)
+// Units per epoch for this plan, never more than a CTA can meet.  `least` = steps of the shortest non-empty sequence.
+//   Tensor-core kernel: by the length of a CTA's run.  us with 1, 2, 3, 5, 6, 8 units: runs of 100 steps (8 x 150..4000
+//   tokens) 35, 27, 22.5, 22.6, 19.6, 19.6; 221 (32 x 2048, three met) 49.3, 45.3, 41.0; 344 (12 x 1000..16000) 77, 66, 64, 64,
+//   62, 63; 459 (32 x 1000..16000, 28 / 4 heads, T = 38) 100, 90, 85, 83, 84, 90; 919 (32 x 1000..16000) 171, 157, 151, 151, 148,
+//   151; 1900 steps (16 x 8K..128K, seven heads per group) 338 with one and 26 slots, 343 with two and 24.
+//   CUDA-core kernel: it is bound by its warps, and a warp needs a slot: eight at most, of which the tables of a second unit
+//   take one.  So a CTA that meets two units keeps one per epoch where slots are short (16 x 2000 tokens, fp32, T = 89: 112 us
+//   with seven slots, 121 with six), and one that may meet more takes them together (8 x 150..4000 tokens: 79 us with one, 66
+//   with three to six).
+__device__ __forceinline__ int choose_cap(const EpochCaps& E, const Plan& pl, int least)
+{
+    if (pl.aligned) return 1;
+    const int meets = static_cast<int>(__fdividef(static_cast<float>(pl.chunk), static_cast<float>(least))) + 2;       // at most
+    if (E.by_units) return meets <= 2 ? E.even : min(meets, E.shortest);
+    return min(meets, pl.chunk <= kRunShort ? E.shortest : (pl.chunk <= kRunMiddle ? E.middle : (pl.chunk <= kRunLong ? E.even : E.longest)));
+}
+
+__device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads, Plan& pl)
 {
     const int max_tokens = A.max_blocks * kPageTokens;
-    if (lane < A.nslots) { mbar_init(&C.full[lane], 1); mbar_init(&C.empty[lane], 1); }
+    mbar_init(&C.full[lane], 1);                           // (all kMaxSlots = 32; the plan says how many are used)
+    mbar_init(&C.empty[lane], 1);
     C.seq[lane] = 0;
     if (lane == 0) { *C.abort_flag = 0; C.prefix[0] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -384,7 +403,7 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
     }
     if (!A.overlap) grid_wait();                           // with the flag the page stream does not depend on the kernel before
     if (!A.overlap || A.late_wait) grid_release();         // (otherwise the consumers release, see consumer_wait_previous)
-    int running = 0, smin = 0x7fffffff, smax = 0;
+    int running = 0, smin = 0x7fffffff, smax = 0, least = 0x7fffffff;
 #pragma unroll 1
     for (int b0 = 0; b0 < A.B; b0 += 32) {
         const int b = b0 + lane;
@@ -396,6 +415,7 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
             st = steps_of(clamp_len(len, max_tokens), A.pps);
             smin = min(smin, st);
             smax = max(smax, st);
+            if (st > 0) least = min(least, st);
         }
         int inc = st;
         if (A.B > 1)
@@ -409,8 +429,8 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
     }
     smin = __reduce_min_sync(kFull, smin);
     smax = __reduce_max_sync(kFull, smax);
+    least = __reduce_min_sync(kFull, least);
     __syncwarp();                                          // the prefix is written
-    Plan pl;                                               // (the same in every lane)
     pl.total = A.Hkv * running;
     pl.chunk = A.by_grid.div(pl.total + nct - 1);
     pl.aligned = 0; pl.unit_steps = smax; pl.q = A.per_unit; pl.rem = A.extra;
@@ -434,6 +454,10 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
         run.c1 = min(pl.total, run.c0 + pl.chunk);
         if (run.c0 < run.c1) run.first = locate_unit(C.prefix, A.B, A.Hkv, run.c0);
     }
+    pl.cap = choose_cap(A.caps, pl, least);
+    pl.nslots = static_cast<int>(A.caps.slots >> (8 * (pl.cap - 1))) & 255;
+    pl.merge_off = A.ring_off + pl.nslots * A.slot_stride;
+    pl.tab_off = pl.merge_off + A.caps.tail_base + (pl.cap - 1) * A.caps.tail_step;
     if (lane == 0) { *C.plan = pl; *C.run = run; }
     __syncwarp();
     asm volatile("bar.arrive %0, %1;" ::"n"(kPlanBarrier), "r"(n_threads) : "memory");
@@ -508,10 +532,10 @@ __device__ __forceinline__ void producer_page_ids(const DecodeArgs& A, const Ctr
 
 template <int NW>
 __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C, unsigned char* ring,
-                                              const CtaRun& run, int lane)
+                                              const CtaRun& run, const Plan& pl, int lane)
 {
     const PageLayout L = A.L;
-    const int c0 = run.c0, c1 = run.c1, NS = A.nslots, n_total = c1 - c0;
+    const int c0 = run.c0, c1 = run.c1, NS = pl.nslots, n_total = c1 - c0;
     const uint64_t policy = policy_evict_first();
     const bool owner = lane < NS;
     unsigned char* dst = ring + static_cast<size_t>(lane) * A.slot_stride;
@@ -523,15 +547,15 @@ __device__ __forceinline__ void producer_loop(const DecodeArgs& A, const Ctrl& C
     unsigned n0 = 0, n1 = 0;                               // bytes to copy of the two pages
     Epoch ep;
     ep.e1 = c0;                                            // (a CTA without steps has no first unit)
-    if (n_total > 0) ep = make_epoch(C.prefix, A.Hkv, A.cap, run.first, c0, c1);
+    if (n_total > 0) ep = make_epoch(C.prefix, A.Hkv, pl.cap, run.first, c0, c1);
     // this lane's ring step n -> its step of the line (epoch, warp, place in the warp's run) -> page ids
     auto lookup = [&](int n) {
         id0 = id1 = -1; n0 = n1 = 0;
         if (!owner || n >= n_total) return;
         while (c0 + n >= ep.e1)
-            ep = make_epoch(C.prefix, A.Hkv, A.cap, locate_unit(C.prefix, A.B, A.Hkv, ep.e1), ep.e1, c1);
+            ep = make_epoch(C.prefix, A.Hkv, pl.cap, locate_unit(C.prefix, A.B, A.Hkv, ep.e1), ep.e1, c1);
         int g = c0 + n;
-        if (A.cap > 1) {
+        if (pl.cap > 1) {
             const int len = ep.e1 - ep.e0, q = len / NW, r = len - q * NW;
             const int x = g - ep.e0, i = x / NW, w = x - i * NW;
             g = ep.e0 + w * q + min(w, r) + i;
@@ -604,7 +628,7 @@ __device__ __forceinline__ void describe_epoch(const DecodeArgs& A, const Ctrl& 
     const int n = ep.e1 - ep.e0, q = n / NW, r = n - q * NW;
     if (lane == 0) { C.epoch[0] = ep.e1; C.epoch[1] = ep.n_units; }
     const int run0 = ep.e0 + (lane < NW ? lane * q + min(lane, r) : n);
-    if (A.cap == 1) {                                      // the warps that have a step hold a record each
+    if (C.plan->cap == 1) {                                // the warps that have a step hold a record each
         if (lane == 0) {
             EpochUnit d;
             d.b = ep.first.b; d.h = ep.first.h;
@@ -858,6 +882,31 @@ inline int decode_grid(int n_sms, int64_t units, int max_blocks, int pps)
     const int64_t total = units * ((max_blocks + pps - 1) / pps);
     const int64_t g = total < n_sms ? total : n_sms;
     return g < 1 ? 1 : (g > kMaxCtas ? kMaxCtas : static_cast<int>(g));
+}
+
+// Ring slots for every number of units per epoch (at most `most` slots): with(n) = the largest number of units that leaves
+// at least n of them, bytes(c) = the shared memory of a launch that may choose up to c units.
+struct EpochRoom {
+    int ns[kMaxCap];
+    size_t used[kMaxCap];
+    int with(int slots) const { int c = 1; while (c < kMaxCap && ns[c] >= slots) ++c; return c; }
+    size_t bytes(int cap) const { size_t b = used[0]; for (int c = 1; c < cap; ++c) b = used[c] > b ? used[c] : b; return b; }
+};
+inline EpochRoom epoch_room(DecodeArgs& A, int nw, int g, int tab_bytes, int smem_optin, int most)
+{
+    EpochRoom r;
+    A.caps.tail_base = merge_base(nw, g);
+    A.caps.tail_step = merge_step(g);
+    A.caps.slots = 0;
+    for (int cap = 1; cap <= kMaxCap; ++cap) {
+        const int tail = A.caps.tail_base + (cap - 1) * A.caps.tail_step + cap * tab_bytes, room = smem_optin - A.ring_off - tail;
+        int n = room > 0 ? room / A.slot_stride : 0;
+        n = n > kMaxSlots ? kMaxSlots : (n > most ? most : n);
+        r.ns[cap - 1] = n;
+        r.used[cap - 1] = A.ring_off + static_cast<size_t>(n) * A.slot_stride + tail;
+        A.caps.slots |= static_cast<unsigned long long>(n) << (8 * (cap - 1));
+    }
+    return r;
 }
 
 inline void set_divisors(DecodeArgs& A, int64_t units, int grid)

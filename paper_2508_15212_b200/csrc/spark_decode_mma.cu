@@ -38,11 +38,13 @@ constexpr float kSlack = 8.f;                 // log2 units a score may exceed t
 
 constexpr int kVTileBytes = kPageTokens * kHeadDim * 2;                          // dense value rows of one page
 
-// Shared-memory map (fixed part; merge area, operand tables, prefix and ring follow at offsets chosen by the launcher).
+// Shared-memory map (fixed part; prefix and ring follow at offsets chosen by the launcher, records and operand tables at
+// offsets chosen with the plan).
 template <int G, bool kPV> struct SmemBf16 {
     static constexpr int kQsum = kCtrlBytes;                                     // [kMaxCap][8] float
     static constexpr int kVTile = (kQsum + kMaxCap * 8 * 4 + 127) / 128 * 128;   // per-warp tiles (pruned values)
-    static constexpr int kMerge = kVTile + (kPV ? kNW * kVTileBytes : 0);
+    static constexpr int kMl = kVTile + (kPV ? kNW * kVTileBytes : 0);           // [kMaxCap][G] (M, L) of the epoch's units
+    static constexpr int kEnd = (kMl + kMaxCap * G * 8 + 127) / 128 * 128;
     static constexpr int kTabBytes = 3 * G * kHeadDim * 2;                       // one unit's q, q' high, q' low: 3 x [G][128] bf16
 };
 
@@ -228,25 +230,25 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     constexpr bool kShared8 = (G <= 4);        // q' high and low parts share one 8-column operand
     extern __shared__ __align__(128) unsigned char smem[];
     const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
-    unsigned char* tab_all = smem + A.tab_off;
     float* qsum_all = reinterpret_cast<float*>(smem + S::kQsum);
-    float* merge = reinterpret_cast<float*>(smem + S::kMerge);
-    float* unit_ml = merge + merge_state_floats(kNW, A.cap, G);
+    float* unit_ml = reinterpret_cast<float*>(smem + S::kMl);
     unsigned char* ring = smem + A.ring_off;
     const unsigned ring_u = smem_u32(ring);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const PageLayout L = A.L;
-    const int NS = A.nslots;
 
     prefetch_block_table(A, tid, kThreads);
     if (warp == kNW) {
-        const CtaRun run = producer_prologue(A, C, lane, kThreads);
-        producer_loop<kNW>(A, C, ring, run, lane);
+        Plan pl;
+        const CtaRun run = producer_prologue(A, C, lane, kThreads, pl);
+        producer_loop<kNW>(A, C, ring, run, pl, lane);
         return;
     }
     consumer_wait_plan(kThreads);
-    const int c0 = C.run->c0, c1 = C.run->c1;
+    const int c0 = C.run->c0, c1 = C.run->c1, NS = C.plan->nslots, cap = C.plan->cap;
+    float* merge = reinterpret_cast<float*>(smem + C.plan->merge_off);
+    unsigned char* tab_all = smem + C.plan->tab_off;
     if (!A.late_wait) {
         consumer_wait_previous(A);                         // q, qnorm, out and the workspace from here on
         write_empty_sequences<kNT>(A, C.prefix, tid);
@@ -254,7 +256,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
     for (int g = c0; g < c1;) {
-        const Epoch ep = make_epoch(C.prefix, A.Hkv, A.cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
+        const Epoch ep = make_epoch(C.prefix, A.Hkv, cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
         // ---- the epoch's operand tables: a warp prepares one query head of one unit at a time, the next one's loads
         //      in flight meanwhile (first pass: only loads) ----
         {
@@ -284,9 +286,9 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
         // ---- this warp's run of the epoch's steps, unit by unit ----
         const int n_ep = ep.e1 - ep.e0, run_q = n_ep / kNW, run_r = n_ep - run_q * kNW;
-        int pos = ep.e0 + (A.cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
-        const int pos_end = A.cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
-        const int stride = A.cap == 1 ? kNW : 1;
+        int pos = ep.e0 + (cap == 1 ? warp : warp * run_q + min(warp, run_r));     // line position
+        const int pos_end = cap == 1 ? ep.e1 : pos + run_q + (warp < run_r ? 1 : 0);
+        const int stride = cap == 1 ? kNW : 1;
         int slot = (ep.e0 - c0) + warp, round = slot < NS ? 0 : slot / NS;     // ring position of the warp's next step, kept incrementally
         slot -= round * NS;
         if (warp == kNW - 1) describe_epoch<kNW>(A, C, ep, lane);     // for the merge; this warp's run is never the longer
@@ -295,7 +297,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
         while (pos < pos_end && pos >= u.start + u.steps) { next_unit(C.prefix, A.Hkv, u); ++eu; }
         while (pos < pos_end) {
             const int part_end = min(pos_end, u.start + u.steps);
-            const int cnt = A.cap == 1 ? (part_end - pos + kNW - 1) / kNW : part_end - pos;      // steps of this warp, >= 1
+            const int cnt = cap == 1 ? (part_end - pos + kNW - 1) / kNW : part_end - pos;      // steps of this warp, >= 1
             pos += cnt * stride;
             const int tail = C.lens[u.b] - (pos - stride - u.start) * kPageTokens;      // valid rows of the last one (>= 16: all)
             // second-operand fragments (column r of each operand, channels 32c .. 32c+31):
@@ -561,26 +563,24 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     set_divisors(A, units, grid);
     A.whole_steps = kNW;
-    A.cap = epoch_cap(A.B, units, A.max_blocks, grid);
-    // An epoch's units take shared memory (operand tables, records) from the ring.  Where a CTA's run is long, a unit
-    // boundary (3 us) is a small part of it and ring slots are worth more: 16 sequences of 8K..128K tokens, seven
-    // heads per group (62 KB of records): 343 us with two units and 24 slots, 338 us with one and 26.  Short runs give
-    // up slots down to kMinRing.
-    const bool long_run = max_steps_per_cta(units, A.max_blocks, A.pps, grid) > 1024;
-    int ns = 0, ns_one = 0;
-    for (int cap = 1; cap <= A.cap; ++cap) {
-        const int tab_off = static_cast<int>(align_up(S::kMerge + merge_bytes(kNW, cap, G), 128));
-        const int prefix_off = tab_off + cap * S::kTabBytes, ring_off = prefix_off + prefix_bytes(A.B);
-        int n = (smem_optin - ring_off) / A.slot_stride;
-        if (n > kMaxSlots) n = kMaxSlots;
-        if (cap == 1) ns_one = n;
-        else if (n < (long_run ? ns_one : (ns_one < kMinRing ? ns_one : kMinRing))) { A.cap = cap - 1; break; }
-        A.tab_off = tab_off; A.prefix_off = prefix_off; A.ring_off = ring_off;
-        ns = n;
+    A.prefix_off = S::kEnd;
+    A.ring_off = A.prefix_off + prefix_bytes(A.B);
+    const EpochRoom room = epoch_room(A, kNW, G, S::kTabBytes, smem_optin, kMaxSlots);
+    const int one = room.ns[0];
+    if (one < 2) return SPARK_ERR_UNSUPPORTED;
+    // Equally long sequences: a CTA's run meets `meets` units.  Unequal ones: more, the shorter the run (see EpochCaps).
+    const int ring = room.with(one < kMinRing ? one : kMinRing), free = room.with(one);
+    const int meets = static_cast<int>((units + grid - 1) / grid) + 1;
+    auto up_to = [](int c, int most) { return c < most ? c : most; };
+    A.caps.by_units = 0;
+    A.caps.shortest = A.caps.middle = A.caps.even = A.caps.longest = 1;
+    if (A.B > 1 || 2 * units > grid) {
+        A.caps.shortest = up_to(A.B > 1 ? kMaxCap : meets, ring);
+        A.caps.middle = up_to(A.B > 1 ? meets + 3 : meets, ring);
+        A.caps.even = up_to(meets, ring);
+        A.caps.longest = up_to(meets, free);               // no slot lost
     }
-    if (ns < 2) return SPARK_ERR_UNSUPPORTED;
-    A.nslots = ns;
-    const size_t smem = A.ring_off + static_cast<size_t>(ns) * A.slot_stride;
+    const size_t smem = room.bytes(A.caps.shortest);
     if (A.q_by_value) {
         const size_t q_bytes = static_cast<size_t>(A.B) * A.Hq * kHeadDim * 2;
         if (kPV || q_bytes > static_cast<size_t>(kBlobLarge)) return SPARK_ERR_UNSUPPORTED;

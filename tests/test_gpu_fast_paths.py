@@ -113,6 +113,28 @@ def test_division_of_the_step(name, Hq, Hkv, lens):
     check_case(make("bf16", len(lens), Hq, Hkv, lens, 8, 64, seed=400 + len(lens), gap=False), 64, check_vals=False)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("Hq,Hkv,lens", [
+    (8, 4, [4000, 150, 700, 1300, 16, 0, 2900, 333]),
+    (8, 8, [1000] * 20),
+    (28, 4, [100 + 97 * i for i in range(20)]),
+    (16, 2, [5000, 1, 5000, 40, 3000, 900]),
+])
+def test_division_of_the_step_with_head_room(dtype, Hq, Hkv, lens):
+    """Units per epoch and ring slots follow the lengths: a cache with room for sixteen times the longest sequence gives what
+    one without gives, bit for bit (the grid, which follows the capacity too, is full in both)."""
+    wl = make(dtype, len(lens), Hq, Hkv, lens, 8, 64, seed=450 + len(lens), sigma=1.0 if dtype == "bf16" else 0.5, gap=False)
+    check_case(wl, 64, check_vals=False)
+    outs = []
+    for room in (1, 16):
+        cache = SparkCache(batch=len(lens), n_q_heads=Hq, n_kv_heads=Hkv, window=8, keep=64, dtype=dtype, max_tokens=room * max(lens))
+        cache.max_src_tokens = max(lens)
+        cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+        outs.append(cache.decode(wl.q))
+        assert cache.status() == 0
+    assert torch.equal(*outs)
+
+
 @pytest.mark.parametrize("lens,W,budget,G,pool", [
     ([1500, 900], 8, 8, 4, 7),              # the window alone
     ([5000, 4100], 16, 600, 2, 601),        # pooling wider than the staging tile's halo
