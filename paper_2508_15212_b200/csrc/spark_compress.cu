@@ -695,6 +695,7 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 // ------------------------------------------------------------------------------------------------
 constexpr int kWarpPageWarps = 4;      // pages (warps) of a CTA; one where no sequence has more (1000 x 16 tokens: 84 us with four, 57 with one)
 constexpr int kFewKeys = 2;            // keys left between the ends that are told apart by their full bits
+constexpr int kAdmitPasses = 4;        // values of the boundary's upper half admitted one by one; more go to the bitwise descent
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
 // SparK-p: the saliencies of a page (fp32), and over them, once read, mask | mu | slot rows
 __host__ __device__ inline int warp_topp_room(const PageLayout& L)
@@ -736,6 +737,36 @@ __device__ __forceinline__ unsigned full_key(const unsigned char* row, int sw, i
     const unsigned short h = *reinterpret_cast<const unsigned short*>(row + ((c ^ sw) << 4) + (ch & 7) * 2);
     const float x = fabsf(bf16_bits_to_float(h));
     return __float_as_uint(kValue ? x : __fmul_rn(a[ch], x));
+}
+
+// Mask words of a token from its kept channels 4 * lane .. 4 * lane + 3 (whole warp).
+__device__ __forceinline__ uint4 mask_words(const bool (&kept)[4], int lane)
+{
+    unsigned nib = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) nib |= kept[i] ? (1u << i) : 0u;
+    const unsigned w = nib << (4 * (lane & 7));
+    uint4 m;
+    m.x = __reduce_or_sync(kFullMask, lane < 8 ? w : 0u);
+    m.y = __reduce_or_sync(kFullMask, (lane >> 3) == 1 ? w : 0u);
+    m.z = __reduce_or_sync(kFullMask, (lane >> 3) == 2 ? w : 0u);
+    m.w = __reduce_or_sync(kFullMask, lane >= 24 ? w : 0u);
+    return m;
+}
+// Mask words of one token by the bitwise descent (called by the whole warp, rarely, so out of line).  Keys that nearly all
+// share their upper half (constant keys under window means within 1 % of each other) are its case: admitted value by value
+// 8192 such tokens took 328 us a prefill (the descent for every token 39), this takes 67.
+template <bool kValue>
+__device__ __noinline__ uint4 descent_mask(const unsigned char* row, int sw, int lane, int T, const float* a)
+{
+    const uint2 v = *reinterpret_cast<const uint2*>(row + (((lane >> 1) ^ sw) << 4) + (lane & 1) * 8);
+    const float f[4] = {__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u)};
+    unsigned key[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) key[i] = __float_as_uint(kValue ? fabsf(f[i]) : __fmul_rn(a[4 * lane + i], fabsf(f[i])));
+    bool kept[4];
+    select_top_t(key, T, lane, kept);
+    return mask_words(kept, lane);
 }
 
 // One section of a page from the rows in `tile` (16 rows of 256 bytes, 16-byte chunk c of row p at c ^ (p & 7)): kept
@@ -844,7 +875,15 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
                 cand = (static_cast<unsigned long long>(ge[1] & ~gt[1]) << 32) | (ge[0] & ~gt[0]);
                 got = (static_cast<unsigned long long>(gt[1]) << 32) | gt[0];
             }
-            while (__any_sync(kFullMask, need > 0)) {
+            for (int pass = 0; __any_sync(kFullMask, need > 0); ++pass) {
+                if (pass == kAdmitPasses || (pass == 1 && __any_sync(kFullMask, need > 0 && __popcll(cand) > 8))) {   // many distinct keys in one upper half
+                    for (unsigned todo = __ballot_sync(kFullMask, need > 0) & 0xffffu; todo; todo &= todo - 1) {
+                        const int tok = __ffs(todo) - 1;
+                        const uint4 m = descent_mask<kValue>(tile + tok * (kHeadDim * 2), tok & 7, lane, T, a_all);
+                        if (p == tok) got = half ? (static_cast<unsigned long long>(m.w) << 32) | m.z : (static_cast<unsigned long long>(m.y) << 32) | m.x;
+                    }
+                    break;
+                }
                 unsigned best = 0u;                             // largest full key left (keys compare as their bits)
                 unsigned long long eq = 0ull;
                 for (unsigned long long m = need > 0 ? cand : 0ull; m; m &= m - 1) {
@@ -953,16 +992,7 @@ __device__ __noinline__ uint4 rank_mask(const unsigned char* wrow, int sw, int l
     sel.rank_keep[0] = sel.rank_keep[1] = sel.rank_keep[2] = sel.rank_keep[3] = 0u;
     bool kept[4];
     select_by_rank(key, lane, sel, cap, kept);
-    unsigned nib = 0u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) nib |= kept[i] ? (1u << i) : 0u;
-    const unsigned w = nib << (4 * (lane & 7));
-    uint4 m;
-    m.x = __reduce_or_sync(kFullMask, lane < 8 ? w : 0u);
-    m.y = __reduce_or_sync(kFullMask, (lane >> 3) == 1 ? w : 0u);
-    m.z = __reduce_or_sync(kFullMask, (lane >> 3) == 2 ? w : 0u);
-    m.w = __reduce_or_sync(kFullMask, lane >= 24 ? w : 0u);
-    return m;
+    return mask_words(kept, lane);
 }
 
 __device__ __forceinline__ int select_section_topp(const unsigned char* tile, unsigned char* wsm, unsigned char* image, int vals_off,
