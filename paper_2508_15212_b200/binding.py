@@ -126,8 +126,12 @@ def _blocks(block_table, max_blocks) -> int:
 
 
 def _stream() -> int:
-    """The current stream's handle.  (torch.cuda.current_stream() builds a Stream object: 2 us of a 7 us call.)"""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    """The current stream's handle.  (torch.cuda.current_stream() builds a Stream object: 2 us of a 7 us call; the functions
+    that give the bare handle are private to torch, so a version without them takes the public way.)"""
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def make_params(*, batch, n_q_heads, n_kv_heads, window, keep, dtype, n_pool_pages, head_dim=128,

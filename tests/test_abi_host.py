@@ -133,3 +133,18 @@ def test_misaligned_pointers_and_oversized_tables_are_refused_on_the_host(lib):
     assert rc == 2
     rc = lib.spark_append(ctypes.byref(p), one, one, one, one, 4, off8, one, ws, 1 << 20, null)
     assert rc == 2
+
+
+@pytest.mark.parametrize("gone", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_stream_handle_without_torchs_private_functions(monkeypatch, gone):
+    """Every call looks the current stream up; a torch without the private functions takes the public one."""
+    import types
+
+    import torch
+    have = {"_cuda_getCurrentRawStream": lambda device: 40 + device, "_cuda_getDevice": lambda: 2}
+    monkeypatch.setattr(torch, "_C", types.SimpleNamespace(**have))
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=7))
+    assert B._stream() == 42
+    del have[gone]
+    monkeypatch.setattr(torch, "_C", types.SimpleNamespace(**have))
+    assert B._stream() == 7
