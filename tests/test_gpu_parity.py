@@ -560,6 +560,55 @@ def test_short_dense_tail_equals_the_tail_cache_merged(G, dtype, cap, n_tail):
     assert torch.allclose(lse[fin], ref_lse[fin], rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
 
 
+@pytest.mark.parametrize("name,dtype,G,lens,prefix_kw", [
+    ("pages in a pool", "bf16", 4, [3000, 0, 700], dict(paged=True)),
+    ("pruned values", "bf16", 4, [3000, 0, 700], dict(keep_v=64)),
+    ("adaptive rule, pages in a pool", "bf16", 7, [900, 33, 2100], dict(top_p=0.95, keep=128, paged=True)),
+    ("sampled recovery", "bf16", 2, [400, 0, 130], dict(recovery=1, seed=7)),
+    ("sampled recovery, fp32", "f32", 4, [400, 20, 130], dict(recovery=2, seed=9)),
+    ("one long sequence", "bf16", 4, [20000], dict()),
+    ("one long sequence, fp32", "f32", 2, [6000], dict()),
+    ("equal lengths", "bf16", 8, [2048] * 6, dict()),
+    ("many short ones", "bf16", 1, [1 + 37 * i % 300 for i in range(40)], dict()),
+])
+def test_tail_steps_back_to_back_over_every_kind_of_prefix(name, dtype, G, lens, prefix_kw):
+    """spark_append_dense + spark_decode_attn_tail, twelve times without a wait of the host (each prefix step starts beside its
+    tail kernel, and tail_out, the partial results and the tickets are used again by the next): every result against two
+    ordinary steps and spark_merge_attn.  Same products, summed in another order: the bars to the oracle."""
+    n, Bn, kw = 12, len(lens), dict(prefix_kw)
+    keep = kw.pop("keep", 64)
+    if kw.pop("paged", False):
+        kw["block_table"], kw["n_pool_pages"] = permuted_block_table(Bn, 2, lens, "cuda", seed=5, spare=3)
+    wl = make(dtype, Bn, 2 * G, 2, lens, 8, 64, seed=190, sigma=1.0 if dtype == "bf16" else 0.5, gap=False)
+    a = SparkCache(batch=Bn, n_q_heads=2 * G, n_kv_heads=2, window=8, keep=keep, dtype=dtype, max_tokens=max(lens), guard=True, **kw)
+    a.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    tails = [SparkCache(batch=Bn, n_q_heads=2 * G, n_kv_heads=2, window=8, keep=128, dtype=dtype, max_tokens=64, guard=True) for _ in range(2)]
+    k_tail, v_tail = (torch.zeros(Bn, 2, 64, 128, dtype=wl.k.dtype, device="cuda") for _ in range(2))
+    for t in tails:
+        t.qnorm.copy_(a.qnorm)
+    rows = [(wl.k[:, :, -1 - i].contiguous(), wl.v[:, :, -1 - i].contiguous()) for i in range(n)]
+    qs = [(wl.q * (1.0 + 0.125 * (i % 3))).contiguous() for i in range(n)]
+    to, tl = tails[1].alloc_out(), tails[1].alloc_lse()
+    got = [(torch.empty(Bn, 2 * G, 128, device="cuda"), torch.empty(Bn, 2 * G, device="cuda")) for _ in range(n)]
+    torch.cuda.synchronize()
+    for (kn, vn), q, (out, lse) in zip(rows, qs, got):
+        B.spark_append_dense(tails[1].params, kn, vn, tails[1].pages, None, k_tail, v_tail, tails[1].packed_lens, tails[1].ws_compress,
+                             max_blocks=tails[1].table_blocks)
+        B.spark_decode_attn_tail(a.params, q, a.pages, a.block_table, a.packed_lens, a.qnorm, k_tail, v_tail, tails[1].packed_lens,
+                                 to, tl, out, lse, a.ws_decode, max_blocks=a.table_blocks)
+    assert a.status() == 0 and tails[1].status() == 0
+    o, l = [a.alloc_out(), tails[0].alloc_out()], [a.alloc_lse(), tails[0].alloc_lse()]
+    ref, ref_lse = torch.empty_like(o[0]), torch.empty_like(l[0])
+    for (kn, vn), q, (out, lse) in zip(rows, qs, got):
+        tails[0].append(kn, vn)
+        a.decode(q, out=o[0], lse=l[0])
+        tails[0].decode(q, out=o[1], lse=l[1])
+        B.spark_merge_attn(o[0], l[0], o[1], l[1], ref, ref_lse)
+        assert float((out - ref).abs().max()) <= TOL[dtype]
+        assert torch.allclose(lse, ref_lse, rtol=0, atol=1e-3 if dtype == "bf16" else 2e-5)
+    assert a.status() == 0 and a.broken_guards() == [] and tails[1].broken_guards() == []
+
+
 @pytest.mark.parametrize("bad", [-1, 65])
 def test_tail_length_out_of_range_is_recorded(bad):
     """A tail length outside 0 .. capacity is recorded and clamped, as a length of the pruned prefix is."""
