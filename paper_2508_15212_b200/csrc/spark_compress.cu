@@ -353,12 +353,9 @@ __device__ __forceinline__ int pack_token_kv(unsigned char* image, const PageLay
 }
 
 // ------------------------------------------------------------------------------------------------
-// One CTA builds one page (16 tokens of one KV head) in shared memory and writes it out with
-// coalesced 16-byte stores.  One warp per token, two rounds; a lane owns channels 4*lane .. 4*lane+3.
-//
-// Selection is exact: the saliency is one __fmul_rn, its bit pattern (non-negative float) is an
-// order-preserving 31-bit key, the T-th largest key is found by a bitwise radix descent with warp
-// ballots, and keys equal to it are admitted in ascending channel order until T channels are kept.
+// The ratio-free rules that sort (SparK-g; SparK-p on fp32 storage, with pruned values or sampled recovery): one CTA builds
+// one page (16 tokens of one KV head) in shared memory and writes it out with coalesced 16-byte stores.  One warp per token,
+// two rounds; a lane owns channels 4*lane .. 4*lane+3; keys are chosen by select_by_rank, pruned values by select_top_t.
 // ------------------------------------------------------------------------------------------------
 struct CompressArgs {
     const void* k;
@@ -429,14 +426,13 @@ __global__ void __launch_bounds__(256) compress_pages_kernel(CompressArgs A)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Fixed-T pages, four tokens per warp.  Most of what the selection costs per token is warp-wide
+// Fixed-T pages of fp32 storage and of sampled recovery, four tokens per warp.  Most of what the selection costs per token is warp-wide
 // bookkeeping (reductions, votes, loop control) that serves one token when a warp owns one token.  Here a
 // token belongs to EIGHT lanes (16 channels per lane), a warp carries four tokens through the same
 // instructions, and the radix descent compares two keys per instruction while it works on the keys' upper
-// 16 bits (the bf16 image of a non-negative float orders like the float): `set.ge.u32.bf16x2` yields a
-// 0xFFFF / 0 half-word mask per key, eight such masks are folded into one word with one logic op each and
-// counted with one population count.  Below bit 16 the descent continues on the full keys.  The result is
-// the same exact top-T set, with ties to the lower channel, as select_top_t.
+// 16 bits (the bf16 image of a non-negative float orders like the float): a compare yields 1.0 or
+// 0 per key, and the ones are added in half precision (at most 8 a half: exact).  Below bit 16 the descent continues on the
+// full keys.  The result is the same exact top-T set, with ties to the lower channel, as select_top_t.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ int group8_sum(int v)              // (a masked hardware reduction measured slower)
 {

@@ -22,7 +22,7 @@ constexpr int kRec = kHeadDim + 4;           // floats per head record: 128 outp
 constexpr int kMaxCap = 8;                    // units per epoch, at most (see Epoch)
 constexpr float kLn2 = 0.6931471805599453f;
 
-// Division of 0 <= x < 2^32 by a divisor the host knows: a multiply and a correction (an integer division is some
+// Division of 0 <= x < 2^31 by a divisor the host knows: a multiply and a correction (an integer division is some
 // 130 cycles, and seven of them stood in a row between the plan and a CTA's first page copy).
 struct FastDiv {
     unsigned d, m;
@@ -251,7 +251,7 @@ __device__ __forceinline__ void next_unit(const int* prefix, int Hkv, UnitRef& u
 // order in which the warps consume: ring step n of the epoch is step n / NW of warp n % NW.
 //   Why: with a barrier, a merge and a table build per unit, every unit after a CTA's first cost 3.8 us (as
 //   much as 26 pages at the HBM rate).  Before -> after: append + decode of 8 sequences of 150..4000 tokens
-//   40.9 -> 28.7 us, 32 sequences of 2048 tokens (256 units on 148 SMs) 46.3 -> 44.2 us, 4 of 128K 268 -> 260 us.
+//   40.9 -> 30.1 us, 32 sequences of 2048 tokens (256 units on 148 SMs) 46.1 -> 44.1 us, 4 of 128K 265 -> 258 us.
 struct Epoch {
     int e0, e1;              // line positions
     int n_units;

@@ -435,7 +435,7 @@ bool evict_tc_supported(const spark_params& p)
     return p.dtype == SPARK_BF16 && R <= 256;
 }
 
-// Tensor-core votes: same workspace regions as the CUDA-core path (partial, rowstat, votes).
+// Tensor-core votes: the workspace regions `partial` and `votes` of the CUDA-core path (row statistics stay on chip).
 spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
                                    int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* partial,
                                    float* votes, int* status, cudaStream_t stream, int* launches)
