@@ -33,7 +33,10 @@ namespace spark {
 constexpr int kNW = 15;                       // consumer warps (+ 1 producer warp = 16 warps, 4 per scheduler)
 constexpr int kNT = kNW * 32;
 constexpr int kThreads = kNT + 32;
-constexpr int kMinRing = 20;                  // ring slots that an epoch's units may not take
+// Ring slots that an epoch's units may not take: matters with six or more heads per group, whose records are large.  us with
+// 12, 16, 20, 23: 16 x 300..5000 tokens, 64 / 8 heads 46.8, 48.9, 49.6, 55.4; 8 x 300..4000 24.0, 24.0, 25.8, 28.2;
+// 12 x 1000..16000, 28 / 4 heads, T = 89 41.3, 41.3, 40.6, 46.6, at T = 64 39.3, 39.3, 39.2, 38.3.
+constexpr int kMinRing = 20;
 constexpr float kSlack = 8.f;                 // log2 units a score may exceed the running reference maximum
 
 constexpr int kVTileBytes = kPageTokens * kHeadDim * 2;                          // dense value rows of one page
