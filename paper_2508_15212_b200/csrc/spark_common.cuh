@@ -137,7 +137,7 @@ constexpr int kTailMax = 128;         // tokens of a dense tail that tail_attn_k
 // before its predecessor, and the order of a stream is unchanged for every kernel that waits at its top, before it
 // touches anything of a caller's.  All do, with these exceptions, each of which reads early only what its predecessor
 // cannot write:
-//   - compress_pages_warp_kernel without eviction: keys, values, lengths and block table; behind the window norm;
+//   - compress_pages_warp_kernel and compress_topp_kernel without eviction: keys, values, lengths and block table; behind the window norm;
 //   - evict_scores_tc_kernel<2>: queries, keys and lengths; behind pass 1 of the same call;
 //   - a decode step with SPARK_FLAG_OVERLAP_PREVIOUS: lengths, block table and pages; the caller vouches for the
 //     predecessor.  Its consumers wait and release, not its producer (consumer_wait_previous);

@@ -693,12 +693,6 @@ constexpr int kWarpPageWarps = 4;      // pages (warps) of a CTA; one where no s
 constexpr int kFewKeys = 2;            // keys left between the ends that are told apart by their full bits
 constexpr int kAdmitPasses = 4;        // values of the boundary's upper half admitted one by one; more go to the bitwise descent
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
-// SparK-p: the saliencies of a page (fp32), and over them, once read, mask | mu | slot rows
-__host__ __device__ inline int warp_topp_room(const PageLayout& L)
-{
-    const int image = L.v_off + L.keep * kPageTokens * 2, sal = kPageTokens * kHeadDim * 4;
-    return image > sal ? image : sal;
-}
 
 __device__ __forceinline__ unsigned bits_max2(unsigned a, unsigned b)          // bf16 pairs; a NaN wins
 {
@@ -939,269 +933,16 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
     }
 }
 
-// SparK-p for the same shape of work: the fewest most salient channels whose saliencies (summed in double) reach top_p of
-// the token's total, at least one and at most T.  The token's saliencies sit in `wsm` (fp32, 16 rows of 512 bytes, chunk c of
-// row p at c ^ (p & 7)); `image` (which may lie over `wsm`) receives slots, mask and mean like select_section.  Returns the
-// token's kept count.
-//   A threshold on the keys' upper halves is searched like the fixed rule's, but by the SUM of the keys at or above it, in
-//   fp32 until at most three keys can lie between the ends.  The sum above the upper end is then taken in double and
-//   must be below the goal (else the search is repeated in double), and the keys between are admitted one by one.
-//   A bitonic rank sort per token took 2100 instructions for one token; prefill of 8192 tokens and its first token
-//   189 -> 63 us.  The sort still decides (rank_mask) where sums in another order could decide otherwise: a total that is not
-//   finite, or a sum within rounding of the goal whose terms do not add up exactly.
-__device__ __forceinline__ double sum_ge(const unsigned char* wrow, int sw, int half, unsigned lo)        // keys >= lo, in double
-{
-    double s = 0.0;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-        const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (x[e] >= lo) s += static_cast<double>(__uint_as_float(x[e]));
-    }
-    return s + __shfl_xor_sync(kFullMask, s, 16);
-}
-__device__ __forceinline__ float sum_ge_f32(const unsigned char* wrow, int sw, int half, unsigned lo)
-{
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-        if (v.x >= lo) s[0] += __uint_as_float(v.x);
-        if (v.y >= lo) s[1] += __uint_as_float(v.y);
-        if (v.z >= lo) s[2] += __uint_as_float(v.z);
-        if (v.w >= lo) s[3] += __uint_as_float(v.w);
-    }
-    const float t = (s[0] + s[1]) + (s[2] + s[3]);
-    return t + __shfl_xor_sync(kFullMask, t, 16);
-}
-
-// Mask words of one token by the rank sort that the append kernels use (called by the whole warp; a page rarely needs it, so
-// it stays out of line and costs the loop above no registers).
-__device__ __noinline__ uint4 rank_mask(const unsigned char* wrow, int sw, int lane, float top_p, int cap)
-{
-    const uint4 v = *reinterpret_cast<const uint4*>(wrow + ((lane ^ sw) << 4));
-    const unsigned key[4] = {v.x, v.y, v.z, v.w};
-    SelectArgs sel;
-    sel.select = SPARK_SELECT_TOP_P; sel.top_p = top_p; sel.recovery = SPARK_RECOVER_DEGENERATE;
-    sel.rank_keep[0] = sel.rank_keep[1] = sel.rank_keep[2] = sel.rank_keep[3] = 0u;
-    bool kept[4];
-    select_by_rank(key, lane, sel, cap, kept);
-    return mask_words(kept, lane);
-}
-
-// The first look, ten octaves below the largest key.  us per prefill of 8192 tokens with a first look 5, 7, 10, 14, 20 octaves
-// below: p = 0.5 39.1, 39.7, 40.7, 41.9, 43.3; 0.9 45.4, 42.5, 45.0, 46.9, 44.9; 0.95 50.1, 42.5, 44.4, 47.9, 46.0; 0.99 55.5,
-// 49.6, 43.8, 47.9, 48.9.
-constexpr int kFirstLook = 0x500;
-
-__device__ __forceinline__ int select_section_topp(const unsigned char* tile, unsigned char* wsm, unsigned char* image, int vals_off,
-                                                   int mask_off, int mu_off, int T, float top_p, int n, int lane, const float* a_all)
-{
-    const int p = lane & 15, half = lane >> 4, sw = p & 7;
-    const bool live = p < n;
-    const unsigned char* row = tile + p * (kHeadDim * 2);
-    unsigned char* wrow = wsm + p * (kHeadDim * 4);
-    const float* a = a_all + 64 * half;
-    float top_w = 0.f;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + c) ^ sw) << 4));
-        const unsigned x[4] = {v.x, v.y, v.z, v.w};
-        const float4 f0 = *reinterpret_cast<const float4*>(a + 8 * c), f1 = *reinterpret_cast<const float4*>(a + 8 * c + 4);
-        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-        float w[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            w[2 * j] = __fmul_rn(f[2 * j], fabsf(__uint_as_float(x[j] << 16)));
-            w[2 * j + 1] = __fmul_rn(f[2 * j + 1], fabsf(__uint_as_float(x[j] & 0xffff0000u)));
-            top_w = fmaxf(top_w, fmaxf(w[2 * j], w[2 * j + 1]));
-        }
-        *reinterpret_cast<float4*>(wrow + (((16 * half + 2 * c) ^ sw) << 4)) = make_float4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<float4*>(wrow + (((16 * half + 2 * c + 1) ^ sw) << 4)) = make_float4(w[4], w[5], w[6], w[7]);
-    }
-    top_w = fmaxf(top_w, __shfl_xor_sync(kFullMask, top_w, 16));
-    // (a lane reads only what it wrote)
-    const double total = sum_ge(wrow, sw, half, 0u);
-    const double goal = static_cast<double>(top_p) * total;
-    const float goal_f = static_cast<float>(goal);
-    const bool finite = total < static_cast<double>(INFINITY);                  // (false for NaN)
-    const bool search = live && finite;
-    // full-key bounds: the sum of keys >= lo reaches the goal, that of keys >= hi does not
-    unsigned lo = 0u, hi = 0u;
-    double above = 0.0;                                        // sum of the keys >= hi, in double
-    bool exact = false;
-    for (;;) {
-        int l16 = 0, h16 = static_cast<int>(__float_as_uint(top_w) >> 16) + 1;
-        double f_lo = total, f_hi = 0.0;                       // (in the first search fp32 values)
-        bool done = !search, lo_moved = true;
-        for (int it = 0; !__all_sync(kFullMask, done); ++it) {
-            const int span = h16 - l16;
-            const float vl = __uint_as_float(static_cast<unsigned>(l16) << 16);
-            // every key between the ends is at least vl: fewer than four of them
-            if (span <= 1 || (!exact && vl > 0.f && static_cast<float>(f_lo - f_hi) < 3.9f * vl)) done = true;
-            // interpolate; then look a quarter of the span inside the end that moved (the crossing is near it, and the
-            // other end has to follow); now and then bisect
-            int step = span >> 1;
-            if (it == 0 && span > kFirstLook) step = span - kFirstLook;
-            else if (it % 6 == 5) step = span >> 1;
-            else if (it & 1) step = static_cast<int>(static_cast<float>(span) * __fdividef(static_cast<float>(f_lo - goal), static_cast<float>(f_lo - f_hi)));
-            else step = lo_moved ? (span >> 2) + 1 : span - (span >> 2) - 1;
-            step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
-            const int t = l16 + (span > 1 ? step : 0);
-            const unsigned tk = static_cast<unsigned>(t) << 16;
-            const double f = exact ? sum_ge(wrow, sw, half, tk) : static_cast<double>(sum_ge_f32(wrow, sw, half, tk));
-            if (!done) {
-                lo_moved = exact ? f >= goal : static_cast<float>(f) >= goal_f;
-                if (lo_moved) { l16 = t; f_lo = f; } else { h16 = t; f_hi = f; }
-            }
-        }
-        lo = static_cast<unsigned>(l16) << 16;
-        hi = static_cast<unsigned>(h16) << 16;
-        above = sum_ge(wrow, sw, half, hi);
-        const bool bad = search && !exact && above >= goal && goal > 0.0;      // fp32 had put the upper end too low
-        if (!__any_sync(kFullMask, bad)) break;
-        exact = true;                                          // rare: all tokens of the warp again, in double
-    }
-    // kept so far: keys >= hi; candidates: keys in [lo, hi) and, should they not suffice, the ones below
-    unsigned got2[2] = {0u, 0u}, cand2[2] = {0u, 0u};
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-        const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const unsigned bit = 1u << ((4 * c + e) & 31);
-            if (x[e] >= hi) got2[c >> 3] |= bit;
-            if (x[e] >= lo) cand2[c >> 3] |= bit;
-        }
-    }
-    unsigned long long got = (static_cast<unsigned long long>(got2[1]) << 32) | got2[0];
-    unsigned long long cand = ((static_cast<unsigned long long>(cand2[1]) << 32) | cand2[0]) & ~got;
-    if (!search) got = cand = 0ull;
-    int count = __popcll(got);
-    count += __shfl_xor_sync(kFullMask, count, 16);
-    double sum = above, before = -1.0;                         // before the last key admitted here
-    while (__any_sync(kFullMask, search && count < kHeadDim && (sum < goal || count == 0))) {
-        const bool more = search && count < kHeadDim && (sum < goal || count == 0);
-        unsigned best = 0u;
-        unsigned long long eq = 0ull;
-        const int none = cand == 0ull, both = none & __shfl_xor_sync(kFullMask, none, 16);
-        if (both) cand = ~got;                                  // the candidates did not suffice: every key left
-        for (unsigned long long m = more ? cand : 0ull; m; m &= m - 1) {
-            const int ch = __ffsll(static_cast<long long>(m)) - 1;
-            const unsigned k = *reinterpret_cast<const unsigned*>(wrow + (((16 * half + (ch >> 2)) ^ sw) << 4) + (ch & 3) * 4);
-            if (k > best) { best = k; eq = 0ull; }
-            if (k == best) eq |= 1ull << ch;
-        }
-        const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
-        if (other > best) { best = other; eq = 0ull; }
-        const int mine = __popcll(eq), theirs = __shfl_xor_sync(kFullMask, mine, 16);
-        if (more) {
-            const double w = static_cast<double>(__uint_as_float(best));
-            int take = 0;                                      // equal keys: lower channels first, no more than the goal asks for
-            while (take < mine + theirs && (sum < goal || count + take == 0)) { before = sum; sum += w; ++take; }
-            int own = half ? take - theirs : take;
-            own = own < 0 ? 0 : (own > mine ? mine : own);
-            unsigned long long rest = eq;
-            for (int k = 0; k < own; ++k) rest &= rest - 1;
-            got |= eq & ~rest;
-            cand &= ~eq;
-            count += take;
-            if (mine + theirs == 0) count = kHeadDim;          // (nothing left)
-        }
-    }
-    const double slack = total * 0x1p-44;                      // more than 128 roundings
-    const bool close = live && (!finite || fabs(sum - goal) <= slack || fabs(before - goal) <= slack);
-    if (__any_sync(kFullMask, close)) {
-        // 128 terms add up exactly in double, in any order, when their exponents span at most 22
-        unsigned least = 0x7f800000u;
-#pragma unroll 1
-        for (int c = 0; c < 16; ++c) {
-            const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-            const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) least = x[e] ? min(least, x[e]) : least;
-        }
-        least = min(least, __shfl_xor_sync(kFullMask, least, 16));
-        const bool rank = close && (!finite || static_cast<int>(__float_as_uint(top_w) >> 23) - static_cast<int>(least >> 23) > 22);
-        for (unsigned todo = __ballot_sync(kFullMask, rank) & 0xffffu; todo; todo &= todo - 1) {
-            const int tok = __ffs(todo) - 1;
-            const uint4 m = rank_mask(wsm + tok * (kHeadDim * 4), tok & 7, lane, top_p, T);
-            if (p == tok) got = half ? (static_cast<unsigned long long>(m.w) << 32) | m.z : (static_cast<unsigned long long>(m.y) << 32) | m.x;
-        }
-    }
-    count = __popcll(got);
-    count += __shfl_xor_sync(kFullMask, count, 16);
-    if (count > T) {                                           // the page's capacity: the T most salient of them
-        // drop the least salient, higher channels first, until T are left (both lanes of the token take part)
-        for (int drop = count - T; drop > 0; --drop) {
-            unsigned low = 0xffffffffu;
-            int at = -1;
-            for (unsigned long long m = got; m; m &= m - 1) {
-                const int ch = __ffsll(static_cast<long long>(m)) - 1;
-                const unsigned k = *reinterpret_cast<const unsigned*>(wrow + (((16 * half + (ch >> 2)) ^ sw) << 4) + (ch & 3) * 4);
-                if (k <= low) { low = k; at = ch; }
-            }
-            const unsigned pair_mask = 0x00010001u << p;
-            const unsigned other = __shfl_xor_sync(pair_mask, low, 16);
-            const bool mine = half ? low <= other : low < other;
-            if (mine && at >= 0) got &= ~(1ull << at);
-        }
-        count = T;
-    }
-    __syncwarp();
-    double pruned = 0.0;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(wrow + (((16 * half + c) ^ sw) << 4));
-        const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (!((got >> (4 * c + e)) & 1ull)) pruned += static_cast<double>(__uint_as_float(x[e]));
-    }
-    pruned += __shfl_xor_sync(kFullMask, pruned, 16);
-    __syncwarp();                                              // every row of `wsm` has been read: the image may go over it
-    for (int i = lane; i < T * 2; i += 32) reinterpret_cast<uint4*>(image + vals_off)[i] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-    const unsigned kept[2] = {static_cast<unsigned>(got), static_cast<unsigned>(got >> 32)};
-    const int mine = __popcll(got);
-    const int theirs = __shfl_xor_sync(kFullMask, mine, 16);
-    unsigned char* dst = image + vals_off + val_offset(2, p, half ? theirs : 0);
-#pragma unroll
-    for (int g = 0; g < 2; ++g)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint4 v = *reinterpret_cast<const uint4*>(row + (((8 * half + 4 * g + c) ^ sw) << 4));
-            const unsigned x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if ((kept[g] >> (8 * c + i)) & 1u) {
-                    *reinterpret_cast<unsigned short*>(dst) = static_cast<unsigned short>((i & 1) ? x[i >> 1] >> 16 : x[i >> 1] & 0xffffu);
-                    dst += kPageTokens * 2;
-                }
-        }
-    *reinterpret_cast<uint2*>(image + mask_off + p * 16 + half * 8) = make_uint2(kept[0], kept[1]);
-    if (half == 0)
-        reinterpret_cast<float*>(image + mu_off)[p] =
-            live && count < kHeadDim ? static_cast<float>(pruned / static_cast<double>(kHeadDim - count)) : 0.f;
-    return live ? count : 0;
-}
-
-template <bool kPV, bool kTopP, int kWarps>
-__global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kTopP ? 4 : (kPV ? 5 : 6))) compress_pages_warp_kernel(CompressArgs A)
+template <bool kPV, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kPV ? 5 : 6)) compress_pages_warp_kernel(CompressArgs A)
 {
     extern __shared__ __align__(16) unsigned char page_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int blk = blockIdx.x * kWarps + warp, h = blockIdx.y, b = blockIdx.z;
     const PageLayout L = A.L;
-    // dense value rows go straight to the page; SparK-p pages carry the slot rows behind them, and in shared memory those
-    // (and the head of the page) come to lie over the saliencies
-    const int image_bytes = kPV ? L.page_bytes : L.v_off;
-    const int image_room = kTopP ? warp_topp_room(L) : image_bytes;
+    const int image_bytes = kPV ? L.page_bytes : L.v_off;      // (dense value rows go straight to the page)
     float* a_s = reinterpret_cast<float*>(page_smem);
-    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_room);
+    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_bytes);
     unsigned char* image = tile + kTileBytes;
 
     // Without eviction the kernel before this one is the window norm, and what it waited for is complete (see
@@ -1241,7 +982,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kTopP ? 4 : (k
         return;
     }
     unsigned char* page = A.pages + page_id * L.page_bytes;
-    if (!kTopP && n < kPageTokens)                             // slots past the end of the sequence are zero
+    if (n < kPageTokens)                                       // slots past the end of the sequence are zero
         for (int i = lane; i < image_bytes / 16; i += 32) reinterpret_cast<uint4*>(image)[i] = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -1263,19 +1004,353 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kTopP ? 4 : (k
         }
         __syncwarp();
     }
-    if (kTopP) {
-        const int n_kept = select_section_topp(tile, image, image, L.v_off, L.mask_off, L.mu_off, L.keep, A.sel.top_p, n, lane, a_s);
-        const int rows = __reduce_max_sync(kFullMask, n_kept);
-        __syncwarp();
-        for (int i = lane; i < L.keep * 2; i += 32)
-            reinterpret_cast<uint4*>(page + L.vals_off)[i] = reinterpret_cast<const uint4*>(image + L.v_off)[i];
-        if (lane == 0) reinterpret_cast<int*>(A.pages + rows_offset(A.n_pool_pages, L.page_bytes))[page_id] = rows;
-    } else {
-        select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
-    }
+    select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
     __syncwarp();
     for (int i = lane; i < image_bytes / 16; i += 32)
         reinterpret_cast<uint4*>(page)[i] = reinterpret_cast<const uint4*>(image)[i];
+}
+
+// ------------------------------------------------------------------------------------------------
+// SparK-p pages of bf16 storage with dense values: per token the fewest most salient channels whose saliencies (summed in
+// double) reach top_p of the token's total, at least one and at most T.  Half a page per warp: a token belongs to four
+// lanes (channels 32 q .. 32 q + 31 = mask word q), which hold its saliencies in registers.
+//   A threshold on the keys' upper halves is searched by the sum R of the keys BELOW it, in fp32, against what the rule
+//   leaves out (total - goal), until fewer than kFewBelow keys can lie between the ends.  log R is nearly linear in the key's
+//   bits (= log2 of the key), so a first look, a secant and one step past the crossing usually leave two or three looks
+//   more: 4.7 looks (the most of eight tokens) for p = 0.5 .. 0.99 on Gaussian keys, where bisections and interpolation of
+//   the sum above took 11.  The sum below the lower end is then taken in double, and the keys between are ranked against
+//   each other.
+//   The rank sort of the append kernels (rank_mask, 2100 instructions a token) still decides where this could decide
+//   otherwise: a total that is not finite, a sum within rounding of the goal whose terms do not add up exactly, ends that fp32
+//   had put wrong, many keys with one upper half.
+//   What bounds it: latency (fixed and of shared memory) more than issue slots, hence as many warps as 64 registers allow: us
+//   per prefill of 8192 tokens, p = 0.99, with 20, 24, 28, 32, 36, 40 warps a SM 49.8, 51.5, 52.0, 47.0, 47.0, 51.9.  Two
+//   lanes per token with the saliencies in shared memory and 16 warps a SM took 62.3 (8192 tokens), 102.5 (16000 tokens, now
+//   70.5), 28.3 (500 tokens, p = 0.95, now 22.2).
+// ------------------------------------------------------------------------------------------------
+constexpr int kToppWarps = 4;          // two pages a CTA; one (two warps) where no sequence has more
+constexpr int kFewBelow = 8;           // keys between the ends that are ranked against each other
+constexpr int kToppStride = 36;        // floats between the four lanes' window norms (32 + 4: different banks)
+// shared memory of a page: its keys | the candidates of its tokens | rows used of the two halves | mask | mu | slot rows
+constexpr int kToppImage = kTileBytes + kPageTokens * kFewBelow * 4 + 16;
+__host__ __device__ inline int topp_page_room(const PageLayout& L) { return kToppImage + L.v_off + L.keep * kPageTokens * 2; }
+
+__device__ __forceinline__ int topp_chunk(int c, int row) { return ((c ^ ((c >> 3) << 1)) ^ (row & 7)) << 4; }    // 16-byte chunk c of a row: conflict-free by rows and by lanes
+template <typename N> __device__ __forceinline__ N quad_sum(N v)
+{
+    v += __shfl_xor_sync(kFullMask, v, 1);
+    v += __shfl_xor_sync(kFullMask, v, 2);
+    return v;
+}
+__device__ __forceinline__ int quad_exclusive(int v, int q)                // sum over the lower lanes of the four
+{
+    int x = v, t = __shfl_up_sync(kFullMask, x, 1, 4);
+    if (q >= 1) x += t;
+    t = __shfl_up_sync(kFullMask, x, 2, 4);
+    if (q >= 2) x += t;
+    return x - v;
+}
+__device__ __forceinline__ void pair_sync(int pg)                          // the two warps of a page
+{
+    if (pg == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else asm volatile("bar.sync 2, 64;" ::: "memory");
+}
+
+// Mask words of one token by the rank sort that the append kernels use (whole warp; rarely needed, so out of line).
+__device__ __noinline__ uint4 rank_mask(const unsigned char* row, int tok, int lane, const float* a_s, float top_p, int cap)
+{
+    const uint2 v = *reinterpret_cast<const uint2*>(row + topp_chunk(lane >> 1, tok) + (lane & 1) * 8);
+    const float f[4] = {__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u)};
+    const float* a = a_s + (lane >> 3) * kToppStride + 4 * (lane & 7);
+    unsigned key[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) key[i] = __float_as_uint(__fmul_rn(a[i], fabsf(f[i])));
+    SelectArgs sel;
+    sel.select = SPARK_SELECT_TOP_P; sel.top_p = top_p; sel.recovery = SPARK_RECOVER_DEGENERATE;
+    sel.rank_keep[0] = sel.rank_keep[1] = sel.rank_keep[2] = sel.rank_keep[3] = 0u;
+    bool kept[4];
+    select_by_rank(key, lane, sel, cap, kept);
+    return mask_words(kept, lane);
+}
+
+// What the search leaves open (whole warp; rare, so out of line): tokens whose sums decide only if they add up exactly
+// (`near`), tokens for the rank sort, tokens over the page's capacity (by `drop`), and sums to be taken again.
+__device__ __noinline__ unsigned topp_settle(const unsigned char* tile, int T, float top_p, bool near, bool rank, int drop,
+                                             unsigned got, int lane, const float* a_s, double& pruned)
+{
+    const int p8 = lane >> 2, q = lane & 3;
+    const unsigned char* row = tile + p8 * (kHeadDim * 2);
+    const float* a = a_s + q * kToppStride;
+    auto sal = [&](int r) {
+        const unsigned short x = *reinterpret_cast<const unsigned short*>(row + topp_chunk(4 * q + (r >> 3), p8) + (r & 7) * 2);
+        return __fmul_rn(a[r], fabsf(bf16_bits_to_float(x)));
+    };
+    if (__any_sync(kFullMask, near)) {
+        // 128 terms add up exactly in double, in any order, when their exponents span at most 22
+        unsigned least = 0x7f800000u, most = 0u;
+#pragma unroll 4
+        for (int r = 0; r < 32; ++r) {
+            const unsigned x = __float_as_uint(sal(r));
+            least = x ? min(least, x) : least;
+            most = max(most, x);
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            least = min(least, __shfl_xor_sync(kFullMask, least, o));
+            most = max(most, __shfl_xor_sync(kFullMask, most, o));
+        }
+        rank = rank || (near && static_cast<int>(most >> 23) - static_cast<int>(least >> 23) > 22);
+    }
+    unsigned flags = __ballot_sync(kFullMask, rank);           // any lane of a token
+    flags |= flags >> 1; flags |= flags >> 2;
+    for (unsigned todo = flags & 0x11111111u; todo; todo &= todo - 1) {
+        const int tok = (__ffs(todo) - 1) >> 2;
+        const uint4 m = rank_mask(tile + tok * (kHeadDim * 2), tok, lane, a_s, top_p, T);
+        if (p8 == tok) { got = q & 2 ? (q & 1 ? m.w : m.z) : (q & 1 ? m.y : m.x); drop = 0; }
+    }
+    // drop the least salient, higher channels first, until T are left
+    for (; __any_sync(kFullMask, drop > 0); --drop) {
+        unsigned low = 0xffffffffu;
+        int at = -1;
+        for (unsigned m = drop > 0 ? got : 0u; m; m &= m - 1) {
+            const int r = __ffs(m) - 1;
+            const unsigned x = __float_as_uint(sal(r));
+            if (x <= low) { low = x; at = 32 * q + r; }
+        }
+        int best = at;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            const unsigned other = __shfl_xor_sync(kFullMask, low, o);
+            const int other_at = __shfl_xor_sync(kFullMask, best, o);
+            if (other < low || (other == low && other_at > best)) { low = other; best = other_at; }
+        }
+        if (drop > 0 && best == at && at >= 0) got &= ~(1u << (at & 31));
+    }
+    double s = 0.0;
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r)
+        if (!((got >> r) & 1u)) s += static_cast<double>(sal(r));
+    pruned = quad_sum(s);
+    return got;
+}
+
+// Kept channels of this lane (bit r: channel 32 q + r) of the eight tokens whose key rows lie in `tile`; `pruned` receives
+// the token's sum of the others.  `list`: room for the tokens' candidates.
+__device__ __forceinline__ unsigned select_topp(const unsigned char* tile, float* list, int T, float top_p, bool live, int lane,
+                                                const float* a_s, double& pruned)
+{
+    const int p8 = lane >> 2, q = lane & 3;
+    const unsigned char* row = tile + p8 * (kHeadDim * 2);
+    const float* a = a_s + q * kToppStride;
+    list += p8 * kFewBelow;
+    float w[32], top_w = 0.f;
+    double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(row + topp_chunk(4 * q + c, p8));
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+        const float4 f0 = *reinterpret_cast<const float4*>(a + 8 * c), f1 = *reinterpret_cast<const float4*>(a + 8 * c + 4);
+        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float x0 = __fmul_rn(f[2 * j], fabsf(__uint_as_float(x[j] << 16)));      // the one rounding that decides selection
+            const float x1 = __fmul_rn(f[2 * j + 1], fabsf(__uint_as_float(x[j] & 0xffff0000u)));
+            w[8 * c + 2 * j] = x0; w[8 * c + 2 * j + 1] = x1;
+            top_w = fmaxf(top_w, fmaxf(x0, x1));
+            t0 += static_cast<double>(x0);
+            t1 += static_cast<double>(x1);
+        }
+    }
+    top_w = fmaxf(top_w, __shfl_xor_sync(kFullMask, top_w, 1));
+    top_w = fmaxf(top_w, __shfl_xor_sync(kFullMask, top_w, 2));
+    const double total = quad_sum(t0 + t1), goal = static_cast<double>(top_p) * total, left = total - goal;
+    const bool finite = total < static_cast<double>(INFINITY);                  // (false for NaN)
+    const bool search = live && finite && top_w > 0.f;
+    const float left_f = static_cast<float>(left), log_left = __log2f(left_f);
+    // ends of the search (upper halves): the keys below l sum up to what may be left out, those below h to more
+    const int h0 = static_cast<int>(__float_as_uint(top_w) >> 16) + 1;
+    int l = 0, h = h0, t = 0, pad = 14, side = 0;
+    float r_l = 0.f, r_h = static_cast<float>(total), y = 0.f, y_l = -INFINITY, y_h = __log2f(r_h) - log_left;     // y: log2(R / left)
+    bool done = !search;
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+        const int span = h - l;
+        const float v_l = __uint_as_float(static_cast<unsigned>(l) << 16);
+        if (span <= 1 || (l > 0 && r_h - r_l < (kFewBelow - 0.1f) * v_l)) done = true;     // every key between the ends is at least v_l
+        if (__all_sync(kFullMask, done)) break;
+        if (it == 0) t = static_cast<int>(__float_as_uint(left_f * 0.05f) >> 16);            // some forty keys of half the threshold's size
+        else if (it % 5 == 4 || !(left_f > 0.f)) t = l + (span >> 1);
+        else if (l == 0 || h == h0) {                          // one end not found yet: along R ~ t^1.4, and past the crossing
+            t += static_cast<int>(fminf(fmaxf(-y, -3.f), 3.f) * 91.f) + (y <= 0.f ? pad : -pad);
+            pad = min(2 * pad, 4096);
+        } else if (!(y_l > -INFINITY)) t = h - static_cast<int>(y_h * 91.f) - 14;
+        else t = l + static_cast<int>(static_cast<float>(span) * __fdividef(-y_l, y_h - y_l));
+        t = max(l + 1, min(t, h - 1));
+        const float tf = __uint_as_float(static_cast<unsigned>(t) << 16);
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int r = 0; r < 32; ++r)
+            if (w[r] < tf) s[r & 3] += w[r];
+        const float below = quad_sum((s[0] + s[1]) + (s[2] + s[3]));
+        if (!done) {
+            y = below > 0.f ? __log2f(below) - log_left : -INFINITY;
+            if (below <= left_f) { l = t; r_l = below; y_l = y; if (side > 0) y_h *= 0.5f; side = 1; }
+            else { h = t; r_h = below; y_h = y; if (side < 0) y_l *= 0.5f; side = -1; }
+        }
+    }
+    const float lo = __uint_as_float(static_cast<unsigned>(l) << 16), hi = __uint_as_float(static_cast<unsigned>(h) << 16);
+    unsigned got = 0u, cand = 0u;                              // keys >= hi; keys in [lo, hi)
+    t0 = t1 = 0.0;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        const bool ge = w[r] >= lo;
+        got |= w[r] >= hi ? 1u << r : 0u;
+        cand |= ge ? 1u << r : 0u;
+        (r & 1 ? t1 : t0) += static_cast<double>(ge ? 0.f : w[r]);
+    }
+    cand &= ~got;
+    pruned = t0 + t1;
+    if (!search) { got = live && top_w == 0.f && q == 0 ? 1u : 0u; cand = 0u; }            // all saliencies zero: the first channel
+    // candidates in channel order
+    const int mine = __popc(cand), first = quad_exclusive(mine, q), nc = quad_sum(mine), na = quad_sum(__popc(got));
+    {
+        int i = first;
+        for (unsigned m = cand; m; m &= m - 1, ++i) {
+            const int r = __ffs(m) - 1;
+            const unsigned short x = *reinterpret_cast<const unsigned short*>(row + topp_chunk(4 * q + (r >> 3), p8) + (r & 7) * 2);
+            if (i < kFewBelow) list[i] = __fmul_rn(a[r], fabsf(bf16_bits_to_float(x)));
+        }
+    }
+    __syncwarp();
+    float k[kFewBelow];
+    {
+        const float4 k0 = *reinterpret_cast<const float4*>(list), k1 = *reinterpret_cast<const float4*>(list + 4);
+        k[0] = k0.x; k[1] = k0.y; k[2] = k0.z; k[3] = k0.w; k[4] = k1.x; k[5] = k1.y; k[6] = k1.z; k[7] = k1.w;
+    }
+    double between = 0.0;
+#pragma unroll
+    for (int i = 0; i < kFewBelow; ++i) if (i < nc) between += static_cast<double>(k[i]);
+    const double reach = total - quad_sum(pruned);             // the keys >= lo
+    const double above = na > 0 ? reach - between : 0.0;       // the keys >= hi
+    const double slack = total * 0x1p-44;                      // more than 128 roundings
+    bool near = fabs(reach - goal) <= slack || fabs(above - goal) <= slack;
+    unsigned admit = 0u;                                       // a lane decides on two candidates: admitted when the sum before falls short
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int i = 2 * q + e;
+        const float own = e ? (q & 2 ? (q & 1 ? k[7] : k[5]) : (q & 1 ? k[3] : k[1])) : (q & 2 ? (q & 1 ? k[6] : k[4]) : (q & 1 ? k[2] : k[0]));
+        double before = above;
+#pragma unroll
+        for (int j = 0; j < kFewBelow; ++j)
+            if (j < nc && (k[j] > own || (k[j] == own && j < i))) before += static_cast<double>(k[j]);      // equal keys: lower channels first
+        if (i < nc) {
+            near = near || fabs(before - goal) <= slack;
+            if (before < goal) admit |= 1u << i;
+        }
+    }
+    admit |= __shfl_xor_sync(kFullMask, admit, 1);
+    admit |= __shfl_xor_sync(kFullMask, admit, 2);
+    {
+        int i = first;
+        for (unsigned m = nc <= kFewBelow ? cand : 0u; m; m &= m - 1, ++i) {
+            if ((admit >> i) & 1u) got |= m & (0u - m);
+            else pruned += static_cast<double>(list[i]);
+        }
+    }
+    const bool rank = live && (!finite || (search && (nc > kFewBelow || (na > 0 && above >= goal) || reach < goal)));
+    const int drop = quad_sum(__popc(got)) - T;                // over the page's capacity
+    near = near && search;
+    if (__any_sync(kFullMask, (live && !search) || near || rank || drop > 0))
+        return topp_settle(tile, T, top_p, near, rank, drop, got, lane, a_s, pruned);
+    pruned = quad_sum(pruned);
+    return got;
+}
+
+template <int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, kWarps == 2 ? 1 : 8) compress_topp_kernel(CompressArgs A)
+{
+    extern __shared__ __align__(16) unsigned char topp_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pg = warp >> 1, hw = warp & 1;
+    const int blk = blockIdx.x * (kWarps / 2) + pg, h = blockIdx.y, b = blockIdx.z;
+    const PageLayout L = A.L;
+    float* a_s = reinterpret_cast<float*>(topp_smem);
+    unsigned char* own = topp_smem + 4 * kToppStride * 4 + pg * topp_page_room(L);
+    unsigned char* tile = own + hw * (kTileBytes / 2);
+    float* list = reinterpret_cast<float*>(own + kTileBytes) + hw * 8 * kFewBelow;
+    int* rows_used = reinterpret_cast<int*>(own + kTileBytes + kPageTokens * kFewBelow * 4);
+    unsigned char* image = own + kToppImage;
+
+    if (A.gather) { grid_wait(); grid_release(); }             // what may be read before: as in compress_pages_warp_kernel
+    int len = A.lens[b];
+    len = len > A.max_len ? A.max_len : len;
+    const int t0 = blk * kPageTokens;
+    const int n = len - t0 < kPageTokens ? len - t0 : kPageTokens;
+    const int c16 = lane & 15, r2 = lane >> 4;                 // a row per half warp, a 16-byte chunk per lane
+    int64_t src_row = t0 + 8 * hw + (lane & 7);
+    if (A.gather && 8 * hw + (lane & 7) < n) src_row = A.gather[(static_cast<int64_t>(b) * A.Hkv + h) * A.gather_stride + src_row];
+    const int64_t base = static_cast<int64_t>(b) * A.sb + static_cast<int64_t>(h) * A.sh + c16 * 8;
+    uint4 kr[4], vr[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t row = base + __shfl_sync(kFullMask, src_row, 2 * i + r2) * A.st;
+        kr[i] = vr[i] = make_uint4(0, 0, 0, 0);
+        if (8 * hw + 2 * i + r2 < n) {
+            kr[i] = *reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(A.k) + row);
+            vr[i] = *reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(A.v) + row);
+        }
+    }
+    const int64_t entry = (static_cast<int64_t>(b) * A.Hkv + h) * A.max_blocks + blk;
+    int64_t page_id = 0;
+    if (n > 0) page_id = A.block_table ? A.block_table[entry] : entry;        // no table: contiguous cache
+    const bool page_ok = page_id >= 0 && page_id < A.n_pool_pages;
+    for (int i = (hw << 5) + lane; i < L.keep * 2; i += 64) reinterpret_cast<uint4*>(image + L.v_off)[i] = make_uint4(0, 0, 0, 0);
+    if (!A.gather) { grid_wait(); grid_release(); }
+#pragma unroll
+    for (int j = threadIdx.x; j < kHeadDim; j += kWarps * 32)
+        a_s[(j >> 5) * kToppStride + (j & 31)] = A.qnorm[(static_cast<int64_t>(b) * A.Hkv + h) * kHeadDim + j];
+    __syncthreads();                                           // (the cleared slot rows too)
+    if (n <= 0) return;                                        // both warps of the page; no CTA barrier below
+    if (!page_ok) {
+        if (lane == 0) record_error(A.status, SPARK_ERR_DEVICE_BOUNDS);
+        return;
+    }
+    unsigned char* page = A.pages + page_id * L.page_bytes;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int row = 2 * i + r2;
+        *reinterpret_cast<uint4*>(page + L.v_off + v_chunk_offset(2, 8 * hw + row, c16)) = vr[i];
+        *reinterpret_cast<uint4*>(tile + row * (kHeadDim * 2) + topp_chunk(c16, row)) = kr[i];
+    }
+    __syncwarp();
+    const int p8 = lane >> 2, q = lane & 3, p = 8 * hw + p8;
+    const bool live = p < n;
+    double pruned;
+    const unsigned got = select_topp(tile, list, L.keep, A.sel.top_p, live, lane, a_s, pruned);
+    const int mine = __popc(got), count = quad_sum(mine);
+    unsigned char* dst = image + L.v_off + val_offset(2, p, quad_exclusive(mine, q));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4*>(tile + p8 * (kHeadDim * 2) + topp_chunk(4 * q + c, p8));
+        const unsigned x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if ((got >> (8 * c + i)) & 1u) {
+                *reinterpret_cast<unsigned short*>(dst) = static_cast<unsigned short>((i & 1) ? x[i >> 1] >> 16 : x[i >> 1] & 0xffffu);
+                dst += kPageTokens * 2;
+            }
+    }
+    reinterpret_cast<unsigned*>(image + L.mask_off)[p * kMaskWords + q] = got;
+    if (q == 0)
+        reinterpret_cast<float*>(image + L.mu_off)[p] =
+            live && count < kHeadDim ? static_cast<float>(pruned / static_cast<double>(kHeadDim - count)) : 0.f;
+    const int rows = __reduce_max_sync(kFullMask, count);
+    if (lane == 0) rows_used[hw] = rows;
+    pair_sync(pg);
+    for (int i = (hw << 5) + lane; i < L.v_off / 16 + L.keep * 2; i += 64) {
+        unsigned char* to = page + (i < L.v_off / 16 ? i * 16 : L.vals_off + (i - L.v_off / 16) * 16);
+        *reinterpret_cast<uint4*>(to) = reinterpret_cast<const uint4*>(image)[i];
+    }
+    if (hw == 0 && lane == 0) reinterpret_cast<int*>(A.pages + rows_offset(A.n_pool_pages, L.page_bytes))[page_id] = max(rows_used[0], rows_used[1]);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1801,17 +1876,23 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const bool pv = A.L.keep_v < kHeadDim, topp = p.select == SPARK_SELECT_TOP_P;
     if (p.dtype == SPARK_BF16 && p.recovery == SPARK_RECOVER_DEGENERATE && (p.select == SPARK_SELECT_FIXED || (topp && !pv))) {
         if (!evict) A.lens = seq_lens;                         // readable before the window norm has ended
-        const int warps = n_blocks == 1 ? 1 : kWarpPageWarps;
-        const size_t smem = kHeadDim * 4 + warps * (kTileBytes + static_cast<size_t>(topp ? warp_topp_room(A.L) : (pv ? A.L.page_bytes : A.L.v_off)));
-        auto pick = [&](auto w) {
-            constexpr int kWarps = decltype(w)::value;
-            return topp ? compress_pages_warp_kernel<false, true, kWarps> : (pv ? compress_pages_warp_kernel<true, false, kWarps> : compress_pages_warp_kernel<false, false, kWarps>);
-        };
-        auto kernel = warps == 1 ? pick(std::integral_constant<int, 1>()) : pick(std::integral_constant<int, kWarpPageWarps>());
-        static unsigned char smem_raised[3][kMaxDevices] = {};                // (a single warp needs less than the limit)
-        if (smem > 48 * 1024 && !allow_max_smem(kernel, smem_raised[topp ? 2 : (pv ? 1 : 0)])) return SPARK_ERR_CUDA;
-        const dim3 wgrid((n_blocks + warps - 1) / warps, p.n_kv_heads, p.batch);
-        const cudaError_t e = launch_kernel(kernel, wgrid, dim3(warps * 32), smem, stream, A);
+        const int per_cta = n_blocks == 1 ? 1 : (topp ? kToppWarps / 2 : kWarpPageWarps);         // pages
+        const dim3 wgrid((n_blocks + per_cta - 1) / per_cta, p.n_kv_heads, p.batch);
+        static unsigned char smem_raised[2][kMaxDevices] = {};                // (a single page needs less than the limit)
+        cudaError_t e;
+        if (topp) {                                            // (two pages: at most 19 KB)
+            auto kernel = per_cta == 1 ? compress_topp_kernel<2> : compress_topp_kernel<kToppWarps>;
+            e = launch_kernel(kernel, wgrid, dim3(per_cta * 64), 4 * kToppStride * 4 + per_cta * topp_page_room(A.L), stream, A);
+        } else {
+            const size_t smem = kHeadDim * 4 + per_cta * (kTileBytes + static_cast<size_t>(pv ? A.L.page_bytes : A.L.v_off));
+            auto pick = [&](auto w) {
+                constexpr int kWarps = decltype(w)::value;
+                return pv ? compress_pages_warp_kernel<true, kWarps> : compress_pages_warp_kernel<false, kWarps>;
+            };
+            auto kernel = per_cta == 1 ? pick(std::integral_constant<int, 1>()) : pick(std::integral_constant<int, kWarpPageWarps>());
+            if (smem > 48 * 1024 && !allow_max_smem(kernel, smem_raised[pv ? 1 : 0])) return SPARK_ERR_CUDA;
+            e = launch_kernel(kernel, wgrid, dim3(per_cta * 32), smem, stream, A);
+        }
         ++*launches;
         return e == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }

@@ -57,6 +57,34 @@ def test_top_p_selection_with_ties(kind, p, cap):
     assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("close", [1, 7, 8, 9, 60])
+@pytest.mark.parametrize("cap", [128, 30])
+def test_top_p_threshold_among_close_keys(close, cap):
+    """The threshold falls among `close` keys that share their upper 16 bits (up to eight are ranked against each other, more
+    go to the rank sort); lengths end in either half of a page.  Few exponents: every sum is exact, the sets are the oracle's."""
+    lens = [1, 7, 8, 9, 16, 24, 25, 33]
+    wl = make("bf16", len(lens), 8, 2, lens, 8, 64, seed=320, gap=False)
+    g = torch.Generator(device="cuda").manual_seed(320 + close)
+    wl.q_win = (1.0 + 2.0 ** -7 * torch.randint(0, 3, wl.q_win.shape, generator=g, device="cuda")).to(wl.q_win.dtype)
+    k = 2.0 ** torch.randint(-6, -2, wl.k.shape, generator=g, device="cuda").float()
+    order = torch.rand(wl.k.shape, generator=g, device="cuda").argsort(-1)
+    k.scatter_(-1, order[..., :close], 1.0)
+    k.scatter_(-1, order[..., close:close + 3], 4.0)
+    wl.k = k.to(wl.k.dtype)
+    # goal: the three large keys and half of the close ones
+    mid = float((12.0 + 0.5 * close) / k.sum(-1).mean())
+    wl_cpu = wl.to("cpu")
+    _, a = oracle.window_mean(wl_cpu.q_win, 2)
+    ref = oracle.select_variant(wl_cpu.k, wl_cpu.seq_lens, a, top_p=mid, cap=cap)
+    cache = SparkCache(batch=len(lens), n_q_heads=8, n_kv_heads=2, window=8, keep=cap, dtype="bf16", max_tokens=max(lens), top_p=mid,
+                       guard=True)
+    cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+    u = cache.unpack()
+    assert cache.status() == 0 and cache.broken_guards() == []
+    assert np.array_equal(u["mask"].cpu().numpy().view(np.uint32), ref["mask"])
+    assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
+
+
 @pytest.mark.parametrize("n_seq,longest", [(1, 8200), (2, 8200), (4, 9000), (8, 8500), (9, 8300), (20, 700)])
 def test_eviction_select_clusters(n_seq, longest):
     """Eight, four, two and one CTA per (sequence, KV head), by the number of units and the longest prefix."""
