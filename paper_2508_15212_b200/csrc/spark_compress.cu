@@ -682,17 +682,22 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 // selection serves sixteen tokens and needs one shuffle, and a warp owns its page from the loads to the stores
 // without a CTA barrier.
 //   Selection.  Any threshold t with exactly T keys >= t names the kept set, so the search need not descend bit by bit:
-//   it interpolates the count between its two ends (every sixth step bisects, which bounds it) over the keys' upper
-//   halves, two keys per compare, until T is hit or at most two keys lie between the ends; those (and any that share an
-//   upper half) are told apart by their full bits, in order of key and then of channel.
-//   What bounds it: issue slots.  183 instructions a token against 308 with eight lanes per token and a bitwise
-//   descent (compress_pages4_kernel, which fp32 storage and sampled recovery keep); 8 heads x 32768 tokens:
-//   104 -> 62 us; prefill of 32K tokens 132.4 -> 88 us (24 warps a SM; with 16 3 us more).
+//   it counts over the keys' upper halves, two keys per compare, until T is hit or at most kFewKeys keys lie between the
+//   ends; those are ranked against each other by their full bits, in order of key and then of channel.  The first look is at
+//   the mean of the token's key bits (the mean of the logarithms, near the median), moved by T's distance from the middle; then
+//   by the usual density and a step past the crossing until both ends are known, then false position: 3.8 looks (the most of
+//   sixteen tokens, T = 25 .. 89, Gaussian keys) where interpolation from the least and the largest key down to two keys took 8.3.
+//   What bounds it: issue slots (164 instructions a token, 71 % of the slots), then shared-memory wavefronts (55 %).
+//   8 heads x 32768 tokens: 104 us with eight lanes per token and a bitwise descent (compress_pages4_kernel, which fp32
+//   storage and sampled recovery keep), 60 with the 8.3 looks, 57 now; the same kernel without selection, slots and mean 43.
+//   Prefill of 32K tokens 89.1 -> 85.7 us with 24 warps a SM; 87.8, 95.0, 100.4 with 20, 28, 32.
 // ------------------------------------------------------------------------------------------------
 constexpr int kWarpPageWarps = 4;      // pages (warps) of a CTA; one where no sequence has more (1000 x 16 tokens: 84 us with four, 57 with one)
-constexpr int kFewKeys = 2;            // keys left between the ends that are told apart by their full bits
+constexpr int kFewKeys = 8;            // keys left between the ends that are ranked by their full bits
+constexpr int kBitsPerKey = 6;         // steps of the upper half from one key of a token to the next, about (a guess that only costs looks)
 constexpr int kAdmitPasses = 4;        // values of the boundary's upper half admitted one by one; more go to the bitwise descent
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
+constexpr int kWarpPageFixed = kTileBytes + kPageTokens * kFewKeys * 4;      // a page's rows and its tokens' candidates
 
 __device__ __forceinline__ unsigned bits_max2(unsigned a, unsigned b)          // bf16 pairs; a NaN wins
 {
@@ -759,11 +764,53 @@ __device__ __noinline__ uint4 descent_mask(const unsigned char* row, int sw, int
     return mask_words(kept, lane);
 }
 
+// The `need` largest of a token's candidates when more than kFewKeys share one upper half (whole warp, tokens without need
+// idle; rare, so out of line): value by value, equal keys in ascending channel order, many distinct ones by the descent.
+// Returns the lane's admitted channels (every key above the candidates may be among them).
+template <bool kValue>
+__device__ __noinline__ unsigned long long admit_many(const unsigned char* tile, unsigned long long cand, int need, int T, int lane, const float* a_all)
+{
+    const int p = lane & 15, half = lane >> 4, sw = p & 7;
+    const unsigned char* row = tile + p * (kHeadDim * 2);
+    const float* a = a_all + 64 * half;
+    unsigned long long got = 0ull;
+    for (int pass = 0; __any_sync(kFullMask, need > 0); ++pass) {
+        if (pass == kAdmitPasses || (pass == 1 && __any_sync(kFullMask, need > 0 && __popcll(cand) > 8))) {   // many distinct keys in one upper half
+            for (unsigned todo = __ballot_sync(kFullMask, need > 0) & 0xffffu; todo; todo &= todo - 1) {
+                const int tok = __ffs(todo) - 1;
+                const uint4 m = descent_mask<kValue>(tile + tok * (kHeadDim * 2), tok & 7, lane, T, a_all);
+                if (p == tok) got = half ? (static_cast<unsigned long long>(m.w) << 32) | m.z : (static_cast<unsigned long long>(m.y) << 32) | m.x;
+            }
+            break;
+        }
+        unsigned best = 0u;                                     // largest full key left (keys compare as their bits)
+        unsigned long long eq = 0ull;
+        for (unsigned long long m = need > 0 ? cand : 0ull; m; m &= m - 1) {
+            const int ch = __ffsll(static_cast<long long>(m)) - 1;
+            const unsigned k = full_key<kValue>(row, sw, half, ch, a);
+            if (k > best) { best = k; eq = 0ull; }
+            if (k == best) eq |= 1ull << ch;
+        }
+        const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
+        if (other > best) eq = 0ull;
+        const int mine = __popcll(eq), theirs = __shfl_xor_sync(kFullMask, mine, 16);
+        int take = half ? need - theirs : need;                 // equal keys: lower channels first
+        take = take < 0 ? 0 : (take > mine ? mine : take);
+        unsigned long long rest = eq;
+        for (int k = 0; k < take; ++k) rest &= rest - 1;
+        got |= eq & ~rest;
+        cand &= ~eq;
+        need -= mine + theirs;
+        if (mine + theirs == 0) need = 0;                       // (no candidate left)
+    }
+    return got;
+}
+
 // One section of a page from the rows in `tile` (16 rows of 256 bytes, 16-byte chunk c of row p at c ^ (p & 7)): kept
 // values in slot order, mask words, and for keys (kValue false) the mean of the pruned saliencies.
 template <bool kValue>
 __device__ __forceinline__ void select_section(const unsigned char* tile, unsigned char* image, int vals_off, int mask_off,
-                                               int mu_off, int T, int n, int lane, const float* a_all, double inv_pruned)
+                                               int mu_off, int T, int n, int lane, const float* a_all, double inv_pruned, unsigned* list)
 {
     const int p = lane & 15, half = lane >> 4, sw = p & 7;
     const bool live = p < n;
@@ -805,31 +852,34 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
 #pragma unroll
             for (int j = 0; j < 16; ++j) hk[16 * g + j] = w[j];
         }
-        unsigned mx = hk[0], mn = hk[0];
+        // mean of the keys' bits (= of their logarithms), and whether a NaN is among them
+        unsigned sum = 0u;
+        __nv_bfloat162 nan2 = *reinterpret_cast<const __nv_bfloat162*>(&hk[0]);
 #pragma unroll
-        for (int j = 1; j < 32; ++j) { mx = bits_max2(mx, hk[j]); mn = bits_min2(mn, hk[j]); }
-        mx = bits_max2(mx, mx >> 16 | mx << 16); mn = bits_min2(mn, mn >> 16 | mn << 16);
-        mx = bits_max2(mx, __shfl_xor_sync(kFullMask, mx, 16)) & 0xffffu;
-        mn = bits_min2(mn, __shfl_xor_sync(kFullMask, mn, 16)) & 0xffffu;
-        if (__any_sync(kFullMask, mx > 0x7f80u)) {             // NaN saliencies order above infinity, by their bits
+        for (int j = 0; j < 32; ++j) sum = __dp2a_lo(hk[j], 0x0101u, sum);
+#pragma unroll
+        for (int j = 1; j < 32; ++j) nan2 = __hadd2(nan2, *reinterpret_cast<const __nv_bfloat162*>(&hk[j]));      // non-negative numbers: NaN only from NaN
+        sum += __shfl_xor_sync(kFullMask, sum, 16);
+        if (__any_sync(kFullMask, __hisnan(nan2.x) || __hisnan(nan2.y))) {      // NaN saliencies order above infinity, by their bits
 #pragma unroll
             for (int j = 0; j < 32; ++j) hk[j] = bits_min2(hk[j], 0x7f807f80u);
-            mx = mx > 0x7f80u ? 0x7f80u : mx;
-            mn = mn > 0x7f80u ? 0x7f80u : mn;
         }
-        int lo = static_cast<int>(mn), hi = static_cast<int>(mx) + 1, c_lo = kHeadDim, c_hi = 0;   // counts at lo (>= T) and hi (< T)
+        int lo = 0, hi = 0x7f81, c_lo = kHeadDim, c_hi = 0;    // counts at lo (>= T) and hi (< T)
+        int t = static_cast<int>(sum >> 7) + (kHeadDim / 2 - T) * kBitsPerKey, c = T, pad = kBitsPerKey, side = 0;
         // weights of the two ends (distances of their counts from T; an end that stays while the other moves twice counts half:
         // the "Illinois" false position), every sixth step bisects
         float w_lo = static_cast<float>(kHeadDim - T) + 0.5f, w_hi = static_cast<float>(T) - 0.5f;
-        int side = 0;
-        bool done = !live || hi - lo == 1;
+        bool done = !live;
+#pragma unroll 1
         for (int it = 0; !__all_sync(kFullMask, done); ++it) {
             const int span = hi - lo;
-            int step = span >> 1;
-            if (it % 6 != 5) step = static_cast<int>(static_cast<float>(span) * __fdividef(w_lo, w_lo + w_hi));
-            step = step < 1 ? 1 : (step > span - 1 ? span - 1 : step);
-            const int t = lo + step;
-            int c = count_ge(hk, static_cast<unsigned>(t) * 0x00010001u);
+            if (it % 6 == 5) t = lo + (span >> 1);
+            else if (it > 0 && (lo == 0 || hi == 0x7f81)) {    // one end not found yet: by the usual density, and past the crossing
+                t += (c - T) * kBitsPerKey + (c > T ? pad : -pad);
+                pad = min(2 * pad, 0x4000);
+            } else if (it > 0) t = lo + static_cast<int>(static_cast<float>(span) * __fdividef(w_lo, w_lo + w_hi));
+            t = max(lo + 1, min(t, hi - 1));
+            c = count_ge(hk, static_cast<unsigned>(t) * 0x00010001u);
             c += __shfl_xor_sync(kFullMask, c, 16);
             if (!done) {
                 if (c >= T) {
@@ -851,7 +901,7 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
         unsigned ge[2] = {0u, 0u};
 #pragma unroll
         for (int j = 0; j < 32; ++j) ge[j >> 4] |= ge_mask_bf16x2(hk[j], t2) & (0x00010001u << (j & 15));
-        int need = live && c_lo != T ? T - c_hi : 0;           // keys between the ends to admit
+        const int need = live && c_lo != T ? T - c_hi : 0;     // keys between the ends to admit
         kept[0] &= ge[0]; kept[1] &= ge[1];
         if (__any_sync(kFullMask, need > 0)) {
             const unsigned u2 = static_cast<unsigned>(hi) * 0x00010001u;
@@ -860,41 +910,44 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
 #pragma unroll
                 for (int j = 0; j < 32; ++j) gt[j >> 4] |= ge_mask_bf16x2(hk[j], u2) & (0x00010001u << (j & 15));
             }
-            unsigned long long cand = 0ull, got = 0ull;
-            if (need > 0) {
-                cand = (static_cast<unsigned long long>(ge[1] & ~gt[1]) << 32) | (ge[0] & ~gt[0]);
-                got = (static_cast<unsigned long long>(gt[1]) << 32) | gt[0];
+            unsigned long long cand = 0ull;
+            if (need > 0) cand = (static_cast<unsigned long long>(ge[1] & ~gt[1]) << 32) | (ge[0] & ~gt[0]);
+            const bool many = c_lo - c_hi > kFewKeys;
+            // up to kFewKeys candidates in channel order, ranked against each other by their full bits
+            unsigned* mylist = list + p * kFewKeys;
+            *reinterpret_cast<uint4*>(mylist + 4 * half) = make_uint4(0u, 0u, 0u, 0u);
+            const int mine = __popcll(cand), theirs = __shfl_xor_sync(kFullMask, mine, 16), first = half ? theirs : 0;
+            __syncwarp();
+            {
+                int i = first;
+                for (unsigned long long m = many ? 0ull : cand; m; m &= m - 1, ++i)
+                    mylist[i] = full_key<kValue>(row, sw, half, __ffsll(static_cast<long long>(m)) - 1, a);
             }
-            for (int pass = 0; __any_sync(kFullMask, need > 0); ++pass) {
-                if (pass == kAdmitPasses || (pass == 1 && __any_sync(kFullMask, need > 0 && __popcll(cand) > 8))) {   // many distinct keys in one upper half
-                    for (unsigned todo = __ballot_sync(kFullMask, need > 0) & 0xffffu; todo; todo &= todo - 1) {
-                        const int tok = __ffs(todo) - 1;
-                        const uint4 m = descent_mask<kValue>(tile + tok * (kHeadDim * 2), tok & 7, lane, T, a_all);
-                        if (p == tok) got = half ? (static_cast<unsigned long long>(m.w) << 32) | m.z : (static_cast<unsigned long long>(m.y) << 32) | m.x;
-                    }
-                    break;
-                }
-                unsigned best = 0u;                             // largest full key left (keys compare as their bits)
-                unsigned long long eq = 0ull;
-                for (unsigned long long m = need > 0 ? cand : 0ull; m; m &= m - 1) {
-                    const int ch = __ffsll(static_cast<long long>(m)) - 1;
-                    const unsigned k = full_key<kValue>(row, sw, half, ch, a);
-                    if (k > best) { best = k; eq = 0ull; }
-                    if (k == best) eq |= 1ull << ch;
-                }
-                const unsigned other = __shfl_xor_sync(kFullMask, best, 16);
-                if (other > best) eq = 0ull;
-                const int mine = __popcll(eq), theirs = __shfl_xor_sync(kFullMask, mine, 16);
-                int take = half ? need - theirs : need;         // equal keys: lower channels first
-                take = take < 0 ? 0 : (take > mine ? mine : take);
-                unsigned long long rest = eq;
-                for (int k = 0; k < take; ++k) rest &= rest - 1;
-                got |= eq & ~rest;
-                cand &= ~eq;
-                need -= mine + theirs;
-                if (mine + theirs == 0) need = 0;               // (no candidate left)
+            __syncwarp();
+            const uint4 k0 = *reinterpret_cast<const uint4*>(mylist), k1 = *reinterpret_cast<const uint4*>(mylist + 4);
+            const unsigned k[kFewKeys] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+            unsigned admit = 0u;                                // a lane ranks four of them
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const unsigned own = half ? k[4 + e] : k[e], between = half ? own : own + 1u;
+                int above = 0;                                  // equal keys: lower channels first
+#pragma unroll
+                for (int j = 0; j < kFewKeys; ++j) above += k[j] >= (j < e ? own : (j >= 4 + e ? own + 1u : between)) ? 1 : 0;
+                admit |= above < need ? 1u << e : 0u;
             }
-            if (live && c_lo != T) { kept[0] = static_cast<unsigned>(got); kept[1] = static_cast<unsigned>(got >> 32); }
+            admit <<= 4 * half;
+            admit |= __shfl_xor_sync(kFullMask, admit, 16);
+            unsigned long long out = 0ull;
+            {
+                int i = first;
+                for (unsigned long long m = many ? 0ull : cand; m; m &= m - 1, ++i)
+                    if (!((admit >> i) & 1u)) out |= m & (0ull - m);
+            }
+            if (__any_sync(kFullMask, need > 0 && many)) {
+                const unsigned long long got = admit_many<kValue>(tile, cand, need > 0 && many ? need : 0, T, lane, a_all);
+                if (need > 0 && many) out = cand & ~got;
+            }
+            kept[0] &= ~static_cast<unsigned>(out); kept[1] &= ~static_cast<unsigned>(out >> 32);
         }
     }
     const int mine = __popc(kept[0]) + __popc(kept[1]);
@@ -917,12 +970,12 @@ __device__ __forceinline__ void select_section(const unsigned char* tile, unsign
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const unsigned h = (i & 1) ? x[i >> 1] >> 16 : x[i >> 1] & 0xffffu;
-                if ((kb >> (8 * c + i)) & 1u) {
+                const bool keep = (kb >> (8 * c + i)) & 1u;
+                if (keep) {
                     *reinterpret_cast<unsigned short*>(dst) = static_cast<unsigned short>(h);
                     dst += kPageTokens * 2;
-                } else if (!kValue) {
-                    pruned += static_cast<double>(__fmul_rn(f[i], fabsf(__uint_as_float(h << 16))));
                 }
+                if (!kValue) pruned += static_cast<double>(keep ? 0.f : __fmul_rn(f[i], fabsf(__uint_as_float(h << 16))));
             }
         }
     }
@@ -942,8 +995,9 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kPV ? 5 : 6)) 
     const PageLayout L = A.L;
     const int image_bytes = kPV ? L.page_bytes : L.v_off;      // (dense value rows go straight to the page)
     float* a_s = reinterpret_cast<float*>(page_smem);
-    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kTileBytes + image_bytes);
-    unsigned char* image = tile + kTileBytes;
+    unsigned char* tile = page_smem + kHeadDim * 4 + warp * (kWarpPageFixed + image_bytes);
+    unsigned* list = reinterpret_cast<unsigned*>(tile + kTileBytes);
+    unsigned char* image = tile + kWarpPageFixed;
 
     // Without eviction the kernel before this one is the window norm, and what it waited for is complete (see
     // grid_release): keys, values and lengths may be read before it ends.
@@ -995,7 +1049,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kPV ? 5 : 6)) 
     }
     __syncwarp();
     if (kPV) {                                                 // value-channel pruning: the same selection on |V|
-        select_section<true>(tile, image, L.v_off, L.vmask_off, 0, L.keep_v, n, lane, a_s, 0.0);
+        select_section<true>(tile, image, L.v_off, L.vmask_off, 0, L.keep_v, n, lane, a_s, 0.0, list);
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -1004,7 +1058,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == 1 ? 1 : (kPV ? 5 : 6)) 
         }
         __syncwarp();
     }
-    select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned);
+    select_section<false>(tile, image, L.vals_off, L.mask_off, L.mu_off, L.keep, n, lane, a_s, A.inv_pruned, list);
     __syncwarp();
     for (int i = lane; i < image_bytes / 16; i += 32)
         reinterpret_cast<uint4*>(page)[i] = reinterpret_cast<const uint4*>(image)[i];
@@ -1884,7 +1938,7 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
             auto kernel = per_cta == 1 ? compress_topp_kernel<2> : compress_topp_kernel<kToppWarps>;
             e = launch_kernel(kernel, wgrid, dim3(per_cta * 64), 4 * kToppStride * 4 + per_cta * topp_page_room(A.L), stream, A);
         } else {
-            const size_t smem = kHeadDim * 4 + per_cta * (kTileBytes + static_cast<size_t>(pv ? A.L.page_bytes : A.L.v_off));
+            const size_t smem = kHeadDim * 4 + per_cta * (kWarpPageFixed + static_cast<size_t>(pv ? A.L.page_bytes : A.L.v_off));
             auto pick = [&](auto w) {
                 constexpr int kWarps = decltype(w)::value;
                 return pv ? compress_pages_warp_kernel<true, kWarps> : compress_pages_warp_kernel<false, kWarps>;

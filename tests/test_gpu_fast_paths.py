@@ -57,6 +57,25 @@ def test_top_p_selection_with_ties(kind, p, cap):
     assert np.allclose(u["mu"].cpu().numpy(), ref["mu"], rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("close", [1, 2, 7, 8, 9, 16, 128])
+@pytest.mark.parametrize("keep,keep_v", [(1, 0), (30, 4), (64, 0), (126, 127)])
+def test_fixed_threshold_among_close_keys(close, keep, keep_v):
+    """The T-th key lies among `close` keys (and values) that share their upper 16 bits: up to eight are ranked against each
+    other, more are admitted value by value or by the descent."""
+    lens = [1, 15, 16, 17, 33]
+    wl = make("bf16", len(lens), 8, 2, lens, 8, 64, seed=330, gap=False)
+    g = torch.Generator(device="cuda").manual_seed(330 + close)
+    wl.q_win = (1.0 + 2.0 ** -7 * torch.randint(0, 3, wl.q_win.shape, generator=g, device="cuda")).to(wl.q_win.dtype)
+    # octaves by rank, the close keys around rank T; at most 4, so that scores stay below some 50 and the bar of 1e-3 on the
+    # log-sum-exp is 300 roundings of them (50 * 2^-24 each)
+    for x in (wl.k, wl.v):
+        order = torch.rand(x.shape, generator=g, device="cuda").argsort(-1)
+        rank = order.argsort(-1).float()
+        first = max(0, min(128 - close, keep - close // 2))
+        x.copy_(torch.where((rank >= first) & (rank < first + close), 1.0, 2.0 ** ((first - rank) / 8).clamp(-12, 2).round()))
+    check_case(wl, keep, keep_v=keep_v)
+
+
 @pytest.mark.parametrize("close", [1, 7, 8, 9, 60])
 @pytest.mark.parametrize("cap", [128, 30])
 def test_top_p_threshold_among_close_keys(close, cap):
