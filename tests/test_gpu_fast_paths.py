@@ -111,6 +111,39 @@ def test_eviction_select_clusters(n_seq, longest):
     check_eviction_case("bf16", lens, 4, 300, 1, Hkv=8, pool=7, seed=501)
 
 
+@pytest.mark.parametrize("G,W", [(1, 16), (2, 24), (4, 32), (5, 32), (7, 32), (8, 32)])
+def test_eviction_votes_at_tile_edges(G, W):
+    """One and two blocks of 128 query rows, rows that end inside a block; sequences that end on, before and behind a tile of
+    128 keys, in their CTA's first tile or a later one."""
+    check_eviction_case("bf16", [127, 128, 129, 255, 256, 257, 1152, 1281, 40], W, 60, G, Hkv=2, pool=3, seed=510 + G)
+
+
+@pytest.mark.parametrize("layout", ["token-major", "keys shared by the heads", "keys shared by the sequences", "no more rows than tokens"])
+def test_eviction_key_layouts(layout):
+    """Every order and stride of the keys that the call takes gives what the same keys in a plain tensor give.  The cache may
+    be made for longer prompts than it is given: no row past the prompt's own tensor may be read."""
+    lens = [1000, 1000, 1000] if layout == "no more rows than tokens" else [1000, 130, 640]
+    wl = make("bf16", 3, 8, 2, lens, 32, 64, seed=521, gap=False)
+    k, v = wl.k, wl.v
+    if layout == "token-major":
+        k2, v2 = (x.transpose(1, 2).contiguous().transpose(1, 2) for x in (k, v))
+    elif layout == "keys shared by the heads":
+        k2, v2 = (x[:, :1].expand(-1, 2, -1, -1) for x in (k, v))
+    elif layout == "keys shared by the sequences":
+        k2, v2 = (x[:1].expand(3, -1, -1, -1) for x in (k, v))
+    else:
+        k2, v2 = k[:, :, :1000].contiguous(), v[:, :, :1000].contiguous()
+    got = []
+    for kk, vv, room in ((k2.contiguous(), v2.contiguous(), max(lens)), (k2, v2, 5000)):
+        cache = SparkCache(batch=3, n_q_heads=8, n_kv_heads=2, window=32, keep=64, dtype="bf16", max_tokens=room, token_budget=100, guard=True)
+        cache.compress(wl.q_win, kk, vv, wl.seq_lens)
+        u = cache.unpack()
+        assert cache.status() == 0 and cache.broken_guards() == []
+        got.append((cache.kept_tokens.clone(), u["mask"][:, :, :100].clone(), u["v"][:, :, :100].clone()))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("p,cap", [(0.5, 128), (0.95, 128), (1.0, 128), (1.0, 40), (0.95, 40)])
 def test_top_p_of_odd_values_equals_appending_them(p, cap):
     """Infinities, NaN, all-zero rows, saliencies over more than 22 octaves (their sums round, and p = 1 asks for all of
