@@ -72,6 +72,7 @@ struct DecodeArgs {
     int per_unit, extra;                     // aligned mode (see Plan): CTAs per unit; units with one more
     FastDiv by_q, by_q1;                     // per_unit and per_unit + 1
     EpochCaps caps;                          // units per epoch, chosen with the plan
+    int slack, ragged_slack;                 // steps that the longest share may be above the even one (see Plan)
     int whole_steps;                         // a step per consumer warp; units up to this are not split (see Plan)
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix); records and tables follow it
@@ -284,19 +285,25 @@ struct EpochUnit {
 // How the step line is divided among the CTAs.
 //   stream mode : CTA c owns steps [c*chunk, (c+1)*chunk) of the whole line; a CTA may cross unit
 //                 boundaries (exact balance; used when sequences differ in length or units are many).
-//   aligned mode: all units have the same number of steps and there are several CTAs per unit; unit u
-//                 gets q or q+1 whole CTAs (the first `rem` units get q+1) and is split evenly among
-//                 them, so no CTA crosses a unit boundary and every CTA publishes exactly once.
+//   aligned mode: every unit gets whole CTAs and is split evenly among them, so no CTA crosses a unit boundary and every CTA
+//                 publishes exactly once.  Equally long units: q or q+1 CTAs each.  Unequal ones: as many as keep every share at
+//                 or below the smallest bound for which the grid suffices.  Taken where the longest share is at most 4 % (and,
+//                 up to kShortShare steps, kSplitSlack or kRaggedSlack steps) above the even one: a boundary inside a CTA's run
+//                 costs it a second table, merge and publication (up to 4 us), and all wait for it.  us, stream mode -> aligned:
+//                 1 x 2048 tokens 14.0 -> 9.6, 1 x 4096 15.0 -> 11.0, 2 x 2048 12.6 -> 10.9, 8 x 700 13.9 -> 12.1; unequal ones:
+//                 2 x 3000..7000 15.9 -> 14.9, 8 x 150..4000 20.7 -> 19.3 (a slack of 10 does not reach it), 4 x 800..4000 with
+//                 28 / 4 heads 16.0 -> 14.1.  With the slack at any share 4 x 10000 29.2 -> 29.7, 4 x 4000..20000 33.4 -> 34.3.
 //   whole units : CTA u owns unit u.  For units of at most a step per warp, where a split saves nothing and adds a
 //                 partial, a ticket and the last arriver's merge (240 tokens: 8.4 us against 9.1; with two steps per warp
 //                 9.7 against 9.2), and for units of up to three steps per warp where they fill most of the grid anyway
 //                 (16 sequences of 60..700 tokens, 128 units: 12.7 us against 18.7).
+constexpr int kSplitSlack = 10, kRaggedSlack = 20, kShortShare = 100;
 struct Plan {
     int total;        // steps on the line
     int chunk;        // stream mode: steps per CTA
     int aligned;      // 0: stream, 1: aligned mode, 2: whole units
-    int unit_steps;   // aligned: steps of every unit
-    int q, rem;       // aligned: CTAs per unit
+    int first_cta;    // aligned: first CTA of this CTA's unit
+    int share;        // aligned: steps per CTA of the unit
     int cap, nslots;  // units per epoch and the ring slots that they leave
     int merge_off, tab_off;      // shared-memory offsets of the records and of the operand tables (behind the ring)
 };
@@ -381,6 +388,65 @@ __device__ __forceinline__ int choose_cap(const EpochCaps& E, const Plan& pl, in
     return min(meets, pl.chunk <= kRunShort ? E.shortest : (pl.chunk <= kRunMiddle ? E.middle : (pl.chunk <= kRunLong ? E.even : E.longest)));
 }
 
+// ceil(x / c) for 0 <= x < 2^22 and a quotient below 2^21; rc = 1 / c
+__device__ __forceinline__ int ceil_div(int x, int c, float rc)
+{
+    int q = static_cast<int>(static_cast<float>(x + c - 1) * rc);
+    const int r = x + c - 1 - q * c;
+    q += r >= c ? 1 : (r < 0 ? -1 : 0);
+    return q;
+}
+__device__ __forceinline__ int ceil_div(int x, int c) { return ceil_div(x, c, __fdividef(1.f, static_cast<float>(c))); }
+
+// Unequal units, whole CTAs: the smallest of 32 bounds on a CTA's share, between the even share and the longest one that is
+// worth it, for which the grid suffices, and this CTA's unit and its share of it under that bound; false: none.  The producer
+// warp: a lane holds a sequence to see whether any bound does, then tries one, then holds a sequence again to find the CTA's.
+// (Out of line: the start of a step runs cold, and most divisions do without.  The result is left in the control block.)
+static __device__ __noinline__ bool ragged_run(const int* prefix, int B, int Hkv, int even, int extra, int cta, int nct, int lane, CtaRun* run, Plan* pl)
+{
+    int ctas = 0;
+#pragma unroll 1
+    for (int b = lane; b < B; b += 32) ctas += ceil_div(prefix[b + 1] - prefix[b], even + extra);
+    if (__reduce_add_sync(kFull, ctas) * Hkv > nct) return false;
+    const int tried = even + (extra * lane + 30) / 31;
+    const float rc = __fdividef(1.f, static_cast<float>(tried));
+    ctas = 0;
+#pragma unroll 4
+    for (int b = 0; b < B; ++b) ctas += ceil_div(prefix[b + 1] - prefix[b], tried, rc);
+    const int bound = __shfl_sync(kFull, tried, __ffs(__ballot_sync(kFull, ctas * Hkv <= nct)) - 1);
+    CtaRun r;
+    r.c0 = r.c1 = r.first.b = r.first.h = r.first.start = r.first.steps = 0;       // (a CTA too many has nothing to do)
+    int first_cta = 0, share = 1;
+    int before = 0;                                        // CTAs of the sequences before
+#pragma unroll 1
+    for (int b0 = 0; b0 < B; b0 += 32) {
+        const int b = b0 + lane, st = b < B ? prefix[b + 1] - prefix[b] : 0, n = ceil_div(st, bound), x = n * Hkv;
+        int inc = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += up;
+        }
+        const unsigned past = __ballot_sync(kFull, before + inc > cta);
+        if (past) {
+            const int src = __ffs(past) - 1, n_u = __shfl_sync(kFull, n, src), steps = __shfl_sync(kFull, st, src);
+            const int place = cta - before - __shfl_sync(kFull, inc - x, src);
+            const int h = ceil_div(place + 1, n_u) - 1, k = place - h * n_u;
+            share = ceil_div(steps, n_u);
+            first_cta = cta - k;
+            r.first.b = b0 + src; r.first.h = h; r.first.steps = steps;
+            r.first.start = Hkv * prefix[b0 + src] + h * steps;
+            r.c0 = r.first.start + min(steps, k * share);
+            r.c1 = r.first.start + min(steps, (k + 1) * share);
+            break;
+        }
+        before += __shfl_sync(kFull, inc, 31);
+    }
+    if (lane == 0) { *run = r; pl->first_cta = first_cta; pl->share = share; }
+    __syncwarp();
+    return true;
+}
+
 __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const Ctrl& C, int lane, int n_threads, Plan& pl)
 {
     const int max_tokens = A.max_blocks * kPageTokens;
@@ -433,7 +499,9 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
     __syncwarp();                                          // the prefix is written
     pl.total = A.Hkv * running;
     pl.chunk = A.by_grid.div(pl.total + nct - 1);
-    pl.aligned = 0; pl.unit_steps = smax; pl.q = A.per_unit; pl.rem = A.extra;
+    pl.aligned = 0; pl.first_cta = 0; pl.share = 1;
+    // ragged units in whole CTAs: a unit wastes half a share on average, so where a third each would not fit it is not tried
+    const int extra = pl.chunk / 25 + (pl.chunk <= kShortShare ? A.ragged_slack : 0);
     CtaRun run;
     run.first.b = run.first.h = run.first.start = run.first.steps = 0;
     if (units <= nct && (smax <= A.whole_steps || (2 * units > nct && smax <= 3 * A.whole_steps))) {
@@ -443,12 +511,19 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
         run.first.start = wb < A.B ? A.Hkv * C.prefix[wb] + wh * run.first.steps : 0;
         run.c0 = run.first.start;
         run.c1 = run.c0 + run.first.steps;
-    } else if (smin == smax && smax > 0 && A.per_unit >= 2 && A.by_q.div(smax + A.per_unit - 1) * 25 <= pl.chunk * 26) {
-        pl.aligned = 1;                                    // the longest share is within 4 % of the even split
+    } else if (smin == smax && smax > 0 && A.per_unit >= 1 && A.by_q.div(smax + A.per_unit - 1) * 25 <= pl.chunk * 26 + (pl.chunk <= kShortShare ? A.slack * 25 : 0)) {
+        pl.aligned = 1;
         const int per = (n == A.per_unit ? A.by_q : A.by_q1).div(smax + n - 1);
         run.first.b = ub; run.first.h = u - ub * A.Hkv; run.first.steps = smax; run.first.start = u * smax;
         run.c0 = run.first.start + min(smax, k * per);
         run.c1 = run.first.start + min(smax, (k + 1) * per);
+        pl.first_cta = cta - k; pl.share = per;
+    } else if (units <= nct && smin != smax && smax < (1 << 22) && 3.f * static_cast<float>(pl.total) <= (3 * nct - units) * static_cast<float>(pl.chunk + extra) &&
+               ragged_run(C.prefix, A.B, A.Hkv, pl.chunk, extra, cta, nct, lane, C.run, C.plan)) {
+        pl.aligned = 1;
+        pl.first_cta = C.plan->first_cta; pl.share = C.plan->share;
+        run = *C.run;
+        __syncwarp();
     } else {
         run.c0 = min(pl.total, cta * pl.chunk);
         run.c1 = min(pl.total, run.c0 + pl.chunk);
@@ -489,11 +564,8 @@ __device__ __forceinline__ void unit_parts(const Plan& pl, int unit_start, int u
         n_parts = (unit_start + unit_steps - 1) / pl.chunk - first_cta + 1;
         return;
     }
-    const int u = unit_start / pl.unit_steps;
-    const int n = pl.q + (u < pl.rem ? 1 : 0);
-    first_cta = u * pl.q + min(u, pl.rem);
-    const int per = (pl.unit_steps + n - 1) / n;
-    n_parts = (pl.unit_steps + per - 1) / per;             // trailing CTAs of the unit may be empty
+    first_cta = pl.first_cta;
+    n_parts = (unit_steps + pl.share - 1) / pl.share;      // (trailing CTAs of the unit may be empty)
 }
 
 // The producer warp.  Lane i owns ring slot i: it handles this CTA's ring steps i, i + nslots, i + 2 nslots,

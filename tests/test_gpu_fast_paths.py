@@ -188,6 +188,12 @@ def test_top_p_of_odd_values_equals_appending_them(p, cap):
     ("short ragged units, several per CTA", 8, 4, [4000, 150, 700, 1300, 16, 0, 2900, 333]),
     ("more tiny units than an epoch holds", 16, 8, [1 + (7 * i) % 40 for i in range(60)]),
     ("seven heads per group", 28, 4, [100 + 97 * i for i in range(20)]),
+    ("equal units, a share of one step more than even", 16, 8, [4096]),
+    ("equal units, some with two CTAs", 8, 4, [800] * 32),
+    ("unequal units in whole CTAs", 16, 8, [150 + 550 * i for i in range(8)]),
+    ("unequal units in whole CTAs, empty sequences, CTAs to spare", 4, 4, [0, 3000, 0, 17, 1200, 0]),
+    ("more sequences than lanes, whole CTAs", 4, 2, [30 * (i % 3) for i in range(39)] + [2500]),
+    ("as many units as CTAs", 2, 1, [900 + i for i in range(148)]),
 ])
 def test_division_of_the_step(name, Hq, Hkv, lens):
     check_case(make("bf16", len(lens), Hq, Hkv, lens, 8, 64, seed=400 + len(lens), gap=False), 64, check_vals=False)
