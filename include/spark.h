@@ -339,7 +339,7 @@ spark_status spark_decode_attn_host(const spark_params *p, const void *q_host, v
  * was divided up once at start-up, a plug-in inside another runtime, a framework section in which
  * cudaMalloc is forbidden.  Such a caller can supply inputs and outputs but not the scratch that split
  * decoding needs, so this variant uses a fixed scratch array that lives in the library's own device
- * image (about 1.3 MB per GPU that loads the library, held until the process exits).  It calls no
+ * image (about 1.4 MB per GPU that loads the library, held until the process exits).  It calls no
  * cudaMalloc, cudaFree or allocating library routine.
  *
  *   - Limit: batch * n_kv_heads <= 64 (any group size up to 8).  Larger problems are refused with

@@ -80,8 +80,7 @@ template <int G> struct SmemF32 {
     static constexpr int kTabBytes = kHeadDim * GPD * 8; // sized for the double table (>= the float one)
     static constexpr int kQsum = kCtrlBytes;             // [kMaxCap][8] double
     static constexpr int kPscr = kQsum + kMaxCap * 64;
-    static constexpr int kMl = kPscr + kConsumerWarps * 32 * GPP * 4;        // [kMaxCap][G] (M, L) of the epoch's units
-    static constexpr int kEnd = (kMl + kMaxCap * G * 8 + 127) / 128 * 128;   // then prefix, ring, records, tables
+    static constexpr int kEnd = (kPscr + kConsumerWarps * 32 * GPP * 4 + 127) / 128 * 128;   // then prefix, ring, records, tables
 };
 
 template <int G, typename E, int R>
@@ -98,7 +97,6 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
     const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
     double* qsum_all = reinterpret_cast<double*>(smem + S::kQsum);
     float* pscr_all = reinterpret_cast<float*>(smem + S::kPscr);
-    float* unit_ml = reinterpret_cast<float*>(smem + S::kMl);
     unsigned char* ring = smem + A.ring_off;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -357,8 +355,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
             if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kConsumerThreads>();
-        merge_and_publish<G, kConsumerWarps>(A, C, merge, unit_ml, C.epoch[1], tid);
+        merge_and_publish<G, kConsumerWarps>(A, C, merge, cap, warp, lane);
         g = C.epoch[0];
+        if (g < c1) consumer_sync<kConsumerThreads>();         // the records and the epoch's description are free
     }
     if (A.late_wait) {
         grid_wait();
@@ -391,8 +390,8 @@ size_t decode_workspace_bytes(const spark_params& p)
     const int G = p.n_q_heads / p.n_kv_heads;
     const size_t units = static_cast<size_t>(p.batch) * p.n_kv_heads;
     size_t bytes = kWorkspaceHeader;
-    bytes += align_up(units * sizeof(int), 256);
-    bytes += (kMaxCtas + units) * G * kRec * sizeof(float);
+    bytes += align_up(units * kTickets * sizeof(int), 256);
+    bytes += (kMaxCtas + units) * G * kPart * sizeof(float);
     return align_up(bytes, 256);
 }
 
@@ -490,7 +489,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     A.status = reinterpret_cast<int*>(ws);
     A.tickets = reinterpret_cast<int*>(ws + kWorkspaceHeader);
-    A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(units * sizeof(int), 256));
+    A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(units * kTickets * sizeof(int), 256));
     A.slot_stride = 0; A.pps = 1; A.caps = EpochCaps{}; A.prefix_off = 0; A.ring_off = 0;
     A.overlap = (p.flags & SPARK_FLAG_OVERLAP_PREVIOUS) ? 1 : 0;
     A.seed = p.seed;

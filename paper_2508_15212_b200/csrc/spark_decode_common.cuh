@@ -93,14 +93,9 @@ constexpr int kCtrlBytes = 1024;                                 // full[32], em
 // are as large as the batch needs, so small batches leave their room to the ring
 inline int prefix_bytes(int batch) { return ((2 * batch + 1) * 4 + 127) / 128 * 128; }
 
-// Shared merge area: `nw + cap - 1` states of `g` heads ([record][head][kRec] floats: 128 outputs, m, l, and a spare
-// word for the record's weight), reused by the final combine for the weights of up to kMaxCtas parts, the heads'
-// (M, L) and one float4 per consumer thread.
+// Shared merge area: `nw + cap - 1` states of `g` heads ([record][head][kRec] floats: 128 outputs, m, l).
 __host__ __device__ constexpr int merge_step(int g) { return (g * kRec * 4 + 127) / 128 * 128; }
-__host__ __device__ constexpr int merge_base(int nw, int g)
-{
-    return ((nw * g * kRec > kMaxCtas * g * 2 + nw * 32 * 4 ? nw * g * kRec : kMaxCtas * g * 2 + nw * 32 * 4) * 4 + 127) / 128 * 128;
-}
+__host__ __device__ constexpr int merge_base(int nw, int g) { return (nw * g * kRec * 4 + 127) / 128 * 128; }
 
 // ---- PTX helpers ----------------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void* p)
@@ -319,7 +314,6 @@ struct Ctrl {
     uint64_t* empty;
     volatile int* abort_flag;
     volatile int* seq;        // [32] revolution + 1 for which each slot was last armed
-    volatile int* last_flag;  // [kMaxCap] this CTA is the last arriver of the epoch's unit
     Plan* plan;
     volatile int* epoch;      // [2] the epoch's end and its number of units
     EpochUnit* units;         // [kMaxCap]
@@ -335,9 +329,8 @@ __device__ __forceinline__ Ctrl make_ctrl(unsigned char* smem, int prefix_off, i
     c.empty = c.full + kMaxSlots;
     c.abort_flag = reinterpret_cast<volatile int*>(smem + 512);
     c.plan = reinterpret_cast<Plan*>(smem + 528);
-    c.last_flag = reinterpret_cast<volatile int*>(smem + 576);
     c.epoch = reinterpret_cast<volatile int*>(smem + 608);
-    static_assert(528 + sizeof(Plan) <= 576 && 576 + kMaxCap * 4 <= 608, "control block");
+    static_assert(528 + sizeof(Plan) <= 608, "control block");
     c.seq = reinterpret_cast<volatile int*>(smem + 640);
     c.units = reinterpret_cast<EpochUnit*>(smem + 768);
     c.run = reinterpret_cast<CtaRun*>(smem + 960);
@@ -745,30 +738,73 @@ __device__ __forceinline__ PublishWeights publish_weights(const DecodeArgs& A, i
     return w;
 }
 
-// Merge the records of an epoch ([record][G][kRec]: 128 unnormalised outputs, m, l) unit by unit and publish
-// the units' results: directly where this CTA holds the whole unit, else as a partial followed by the
-// last-arriver merge (only the first and the last unit of a CTA's run can be split).  Called by all consumer
-// threads after a consumer_sync(); ends with a consumer_sync().
+// Merge the records of an epoch ([record][G][kRec]: 128 unnormalised outputs, m, l) unit by unit and publish the units'
+// results: directly where this CTA holds the whole unit, else as a partial followed by the last-arriver merge (only the first
+// and the last unit of a CTA's run can be split).  Called by all consumer threads after a consumer_sync().
 //
-// Both merges are laid out so that no thread walks a chain of dependent shared-memory loads: the
-// log-sum-exp weights of the parts are computed once, by one warp per head with warp reductions, and the
-// weighted sums then read independent operands.
-template <int G, int NW>
-__device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge, float* unit_ml,
-                                                  int n_units, int tid)
+// A warp serves a slice (all, half or a quarter of the 128 channels) of one head of one unit from the records to the result:
+// it takes the log-sum-exp weights of the records itself (lane = record), adds up its channels, and where the unit is split
+// leaves its slice, takes a ticket of the slice's own and, arriving last, merges the slice of all parts.  So no barrier of the
+// CTA stands between the records and the result, and the slices of a unit are merged by several warps at once, of whatever
+// CTAs come last.  A ticket per unit and one CTA merging all of it behind four barriers took 3.6 us from the last record to
+// the result of a 32768-token step.  us before -> after: 1 x 500 tokens 9.1 -> 8.7, 32 x 2048 41.4 -> 39.5, 8 x 5000 29.7 ->
+// 28.2, 8 x 2000..16000 44.1 -> 42.1, 1 x 4096 with 64 / 8 heads 13.7 -> 12.7, fp32 1 x 1024 13.05 -> 12.8.
+__host__ __device__ constexpr int slices_of(int g, int nw) { return 4 * g <= nw ? 4 : (2 * g <= nw ? 2 : 1); }
+constexpr int kTickets = 16;                                  // per unit; at most 14 are used (seven heads in halves)
+constexpr int kPart = kHeadDim + 8;                           // floats of a head's partial: 128 outputs and (m, l) once per slice
+
+template <int N> __device__ __forceinline__ void load_floats(float (&x)[N], const float* p)
 {
-    constexpr int NT = NW * 32;
-    static_assert(NW <= 32, "one warp computes the weights of up to 32 records");
-    const int warp = tid >> 5, lane = tid & 31;
-    constexpr int kWt = kHeadDim + 2;                         // spare word of a record: its weight
-    // ---- weights of the records: a warp serves one head of one unit, lane k holds the unit's record k ----
+    if constexpr (N == 4) { const float4 v = *reinterpret_cast<const float4*>(p); x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
+    else if constexpr (N == 2) { const float2 v = *reinterpret_cast<const float2*>(p); x[0] = v.x; x[1] = v.y; }
+    else x[0] = *p;
+}
+template <int N> __device__ __forceinline__ void store_floats(float* p, const float (&x)[N])
+{
+    if constexpr (N == 4) *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+    else if constexpr (N == 2) *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+    else *p = x[0];
+}
+// N channels of a row of the result from its unnormalised sum
+template <int N>
+__device__ __forceinline__ void publish(const DecodeArgs& A, int64_t row, int ch, float (&O)[N], float M, float Ls, bool lse)
+{
+    const PublishWeights w = publish_weights(A, row, M, Ls);
+#pragma unroll
+    for (int j = 0; j < N; ++j) O[j] *= w.own;
+    if (A.other_out) {
+        float x[N];
+        load_floats<N>(x, A.other_out + row * kHeadDim + ch);
+#pragma unroll
+        for (int j = 0; j < N; ++j) O[j] = fmaf(w.other, x[j], O[j]);
+    }
+    store_floats<N>(A.out + row * kHeadDim + ch, O);
+    if (lse && A.lse) A.lse[row] = w.lse;
+}
+
+template <int G, int NW, int NS>
+__device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUnit* units, float* merge, int n_units, int warp, int lane)
+{
+    constexpr int kItems = G * NS;                                // slices of a unit
+    constexpr int kCh = kHeadDim / NS, VE = kCh / 32;             // channels of a slice; per lane
+    static_assert(NW <= 32 && kItems <= kTickets, "a lane per record; a ticket per slice");
+    bool split = false;
+    // ---- a slice of the unit's sum over this CTA's records ----
 #pragma unroll 1
-    for (int pr = warp; pr < n_units * G; pr += NW) {
-        const int e = pr / G, gg = pr - e * G;
-        const int rec0 = C.units[e].rec0, n_rec = C.units[e].n_rec;
-        float* rec = merge + ((rec0 + lane) * G + gg) * kRec;
-        const float m = lane < n_rec ? rec[kHeadDim] : -INFINITY;
-        const float l = lane < n_rec ? rec[kHeadDim + 1] : 0.f;
+    for (int it = warp; it < n_units * kItems; it += NW) {
+        const int e = it / kItems, gg = (it - e * kItems) / NS, s = (it - e * kItems) % NS;
+        const EpochUnit d = units[e];
+        const float* rec = merge + (d.rec0 * G + gg) * kRec;
+        const float m = lane < d.n_rec ? rec[lane * (G * kRec) + kHeadDim] : -INFINITY;
+        const float l = lane < d.n_rec ? rec[lane * (G * kRec) + kHeadDim + 1] : 0.f;
+        const int ch = s * kCh + lane * VE;
+        float v[NW][VE];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {                            // every load before the first use
+#pragma unroll
+            for (int j = 0; j < VE; ++j) v[k][j] = 0.f;
+            if (k < d.n_rec) load_floats<VE>(v[k], rec + k * (G * kRec) + ch);
+        }
         float M = m;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
@@ -776,169 +812,107 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
         float Ls = l * wt;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(kFull, Ls, o);
-        if (lane < n_rec) rec[kWt] = wt;
-        if (lane == 0) { unit_ml[2 * pr] = M; unit_ml[2 * pr + 1] = Ls; }
-    }
-    consumer_sync<NT>();
-    // ---- weighted sums: a thread owns two channels of one head of one unit ----
-#pragma unroll 1
-    for (int idx = tid; idx < n_units * G * (kHeadDim / 2); idx += NT) {
-        const int pr = idx / (kHeadDim / 2), c2 = idx - pr * (kHeadDim / 2);
-        const int e = pr / G, gg = pr - e * G;
-        const EpochUnit d = C.units[e];
-        const float* rec = merge + (d.rec0 * G + gg) * kRec;
-        float2 v[NW];
-        float f[NW];
+        float O[VE];
 #pragma unroll
-        for (int k = 0; k < NW; ++k) {                        // every load before the first use
-            v[k] = make_float2(0.f, 0.f);
-            f[k] = 0.f;
-            if (k < d.n_rec) {
-                v[k] = *reinterpret_cast<const float2*>(rec + k * (G * kRec) + 2 * c2);
-                f[k] = rec[k * (G * kRec) + kWt];
-            }
-        }
-        float2 O = make_float2(0.f, 0.f);
+        for (int j = 0; j < VE; ++j) O[j] = 0.f;
 #pragma unroll
         for (int k = 0; k < NW; ++k) {
-            O.x = fmaf(v[k].x, f[k], O.x);
-            O.y = fmaf(v[k].y, f[k], O.y);
+            const float f = __shfl_sync(kFull, wt, k);
+#pragma unroll
+            for (int j = 0; j < VE; ++j) O[j] = fmaf(v[k][j], f, O[j]);
         }
-        const float M = unit_ml[2 * pr], Ls = unit_ml[2 * pr + 1];
-        const int64_t row = static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg;
         if (d.n_parts == 1) {
             if (A.late_wait) grid_wait();
-            const PublishWeights pw = publish_weights(A, row, M, Ls);
-            O.x *= pw.own; O.y *= pw.own;
-            if (A.other_out) {
-                const float2 x = *reinterpret_cast<const float2*>(A.other_out + row * kHeadDim + 2 * c2);
-                O.x = fmaf(pw.other, x.x, O.x); O.y = fmaf(pw.other, x.y, O.y);
-            }
-            *reinterpret_cast<float2*>(A.out + row * kHeadDim + 2 * c2) = O;
-            if (c2 == 0 && A.lse) A.lse[row] = pw.lse;
+            publish<VE>(A, static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg, ch, O, M, Ls, s == 0 && lane == 0);
         } else {
-            float* part_out = A.partials + static_cast<int64_t>(blockIdx.x + d.b * A.Hkv + d.h) * G * kRec;
-            *reinterpret_cast<float2*>(part_out + gg * kRec + 2 * c2) = O;
-            if (c2 == 0) *reinterpret_cast<float2*>(part_out + gg * kRec + kHeadDim) = make_float2(M, Ls);
+            split = true;
+            float* part = A.partials + (static_cast<int64_t>(blockIdx.x + d.b * A.Hkv + d.h) * G + gg) * kPart;
+            store_floats<VE>(part + ch, O);
+            if (lane == 0) *reinterpret_cast<float2*>(part + kHeadDim + 2 * s) = make_float2(M, Ls);
         }
     }
-    bool split = false;
+    // ---- the slices of split units: the last warp to arrive merges the parts ----
 #pragma unroll 1
-    for (int e = 0; e < n_units; ++e) split = split || C.units[e].n_parts > 1;         // the same in every thread
-    if (split) {
-        // The barrier orders every consumer thread's partial stores before the tickets' gpu-scope
-        // release; the last arriver's acquire (same atomic) plus the next barrier orders its reads
-        // after all partials.
-        consumer_sync<NT>();
-        if (tid < n_units) {
-            int last = 0;
-            if (C.units[tid].n_parts > 1) {
-                int old;
-                asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;"
-                             : "=r"(old) : "l"(A.tickets + C.units[tid].b * A.Hkv + C.units[tid].h) : "memory");
-                last = (old == C.units[tid].n_parts - 1) ? 1 : 0;
-            }
-            C.last_flag[tid] = last;
+    for (int it = split ? warp : n_units * kItems; it < n_units * kItems; it += NW) {
+        const int e = it / kItems, gg = (it - e * kItems) / NS, s = (it - e * kItems) % NS;
+        const EpochUnit d = units[e];
+        if (d.n_parts == 1) continue;
+        const int unit = d.b * A.Hkv + d.h, n_parts = d.n_parts;
+        int* ticket = A.tickets + unit * kTickets + gg * NS + s;
+        // The warp barrier orders every lane's stores before lane 0's gpu-scope release; its acquire (same atomic) and the
+        // barrier behind it order every lane's reads after the other parts' stores.
+        __syncwarp();
+        int old = 0;
+        if (lane == 0) asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(ticket) : "memory");
+        __syncwarp();
+        if (__shfl_sync(kFull, old, 0) != n_parts - 1) continue;
+        constexpr int kLanes = kCh / 4, PP = 32 / kLanes;         // lanes of a part (four channels each); parts at a time
+        constexpr int kSteps = 32 / PP, kBatch = 8;               // steps of 32 parts; loads in flight of one group of parts
+        constexpr int kTwo = kSteps == kBatch ? 2 : 1;            // groups taken at once (one unit on the whole grid: 148 parts)
+        constexpr int kGroups = kMaxCtas / 32;                    // (m, l) pairs a lane may hold
+        constexpr int64_t kStride = static_cast<int64_t>(G) * kPart;
+        const float* base = A.partials + (static_cast<int64_t>(d.first_cta + unit) * G + gg) * kPart;
+        const int sub = lane / kLanes, c4 = lane % kLanes;
+        float2 ml[kGroups];
+#pragma unroll
+        for (int k = 0; k < kGroups; ++k) {
+            const int p = k * 32 + lane;
+            ml[k] = p < n_parts ? *reinterpret_cast<const float2*>(base + p * kStride + kHeadDim + 2 * s) : make_float2(-INFINITY, 0.f);
         }
-        consumer_sync<NT>();
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float M = -INFINITY, Ls = 0.f;
+#pragma unroll
+        for (int k = 0; k < kGroups; k += kTwo) {
+            if (k * 32 >= n_parts) break;
 #pragma unroll 1
-        for (int e = 0; e < n_units; ++e) {
-            if (!C.last_flag[e]) continue;
-            // Last CTA of this unit: merge all partials.  Every load is issued before the first use:
-            // thread (ph, g, c4) fetches channels 4*c4..4*c4+3 of head g for parts ph, ph+PH, ...;
-            // meanwhile warp g turns the (m, l) pairs of head g into weights (lane = part) and the
-            // head's (M, L).  After one barrier the weights are known, and the weighted sums are
-            // reduced over ph through shared memory.
-            constexpr int TPG = G * 32;                  // threads per part group
-            constexpr int PH = NT / TPG;                 // part groups
-            static_assert(PH >= 1, "a warp per head");
-            constexpr int kBatch = 8;
-            constexpr int kMlRegs = kMaxCtas / 32;       // (m, l) pairs a lane may hold
-            constexpr int64_t kStride = static_cast<int64_t>(G) * kRec;
-            const int b = C.units[e].b, h = C.units[e].h, n_parts = C.units[e].n_parts, unit = b * A.Hkv + h;
-            float* pw = merge;                           // [n_parts][G] weights, n_parts <= kMaxCtas
-            float* pML = merge + kMaxCtas * G;           // [G][2]
-            float4* red = reinterpret_cast<float4*>(merge + kMaxCtas * G * 2);
-            const float* base = A.partials + static_cast<int64_t>(C.units[e].first_cta + unit) * G * kRec;
-            const int ph = tid / TPG, rem = tid - ph * TPG, gg = rem >> 5, c4 = rem & 31;
-            const bool worker = ph < PH;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-            for (int p0 = 0; p0 < n_parts; p0 += kBatch * PH) {
-                float4 o4[kBatch];
+            for (int i0 = 0; i0 < kSteps && k * 32 + i0 * PP < n_parts; i0 += kBatch) {
+                float4 o4[kBatch * kTwo];
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int p = p0 + k * PH + ph;
-                    o4[k] = (worker && p < n_parts)
-                                ? *reinterpret_cast<const float4*>(base + p * kStride + gg * kRec + 4 * c4)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = 0; i < kBatch * kTwo; ++i) {
+                    const int p = k * 32 + (i0 + i) * PP + sub;
+                    o4[i] = p < n_parts ? *reinterpret_cast<const float4*>(base + p * kStride + s * kCh + 4 * c4) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-                if (p0 == 0) {
-                    if (warp < G) {
-                        float2 ml[kMlRegs];
+                if (k == 0 && i0 == 0) {                          // the weights, under the first loads
 #pragma unroll
-                        for (int k = 0; k < kMlRegs; ++k) {
-                            const int p = k * 32 + lane;
-                            ml[k] = p < n_parts ? *reinterpret_cast<const float2*>(base + p * kStride + warp * kRec + kHeadDim)
-                                                : make_float2(-INFINITY, 0.f);
-                        }
-                        float M = -INFINITY;
+                    for (int x = 0; x < kGroups; ++x) M = fmaxf(M, ml[x].x);
 #pragma unroll
-                        for (int k = 0; k < kMlRegs; ++k) M = fmaxf(M, ml[k].x);
+                    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
 #pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
-                        float Ls = 0.f;
-#pragma unroll
-                        for (int k = 0; k < kMlRegs; ++k) {
-                            const int p = k * 32 + lane;
-                            const float wt = (ml[k].x == -INFINITY) ? 0.f : exp2f(ml[k].x - M);
-                            Ls = fmaf(ml[k].y, wt, Ls);
-                            if (p < n_parts) pw[p * G + warp] = wt;
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(kFull, Ls, o);
-                        if (lane == 0) { pML[2 * warp] = M; pML[2 * warp + 1] = Ls; }
+                    for (int x = 0; x < kGroups; ++x) {
+                        ml[x].x = ml[x].x == -INFINITY ? 0.f : exp2f(ml[x].x - M);
+                        Ls = fmaf(ml[x].y, ml[x].x, Ls);
                     }
-                    consumer_sync<NT>();
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(kFull, Ls, o);
                 }
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int p = p0 + k * PH + ph;
-                    if (worker && p < n_parts) {
-                        const float f = pw[p * G + gg];
-                        acc.x = fmaf(o4[k].x, f, acc.x); acc.y = fmaf(o4[k].y, f, acc.y);
-                        acc.z = fmaf(o4[k].z, f, acc.z); acc.w = fmaf(o4[k].w, f, acc.w);
-                    }
+                for (int i = 0; i < kBatch * kTwo; ++i) {
+                    const float f = __shfl_sync(kFull, ml[k + i / kBatch].x, ((i0 + i) * PP + sub) & 31);
+                    acc.x = fmaf(o4[i].x, f, acc.x); acc.y = fmaf(o4[i].y, f, acc.y);
+                    acc.z = fmaf(o4[i].z, f, acc.z); acc.w = fmaf(o4[i].w, f, acc.w);
                 }
             }
-            if (PH > 1) {
-                if (worker && ph > 0) red[tid] = acc;
-                consumer_sync<NT>();
-                if (ph == 0)
-#pragma unroll
-                    for (int k = 1; k < PH; ++k) {
-                        const float4 v = red[k * TPG + tid];
-                        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-                    }
-            }
-            if (ph == 0) {
-                if (A.late_wait) grid_wait();
-                const int64_t row = static_cast<int64_t>(b) * A.Hq + h * G + gg;
-                const PublishWeights w = publish_weights(A, row, pML[2 * gg], pML[2 * gg + 1]);
-                acc.x *= w.own; acc.y *= w.own; acc.z *= w.own; acc.w *= w.own;
-                if (A.other_out) {
-                    const float4 x = *reinterpret_cast<const float4*>(A.other_out + row * kHeadDim + 4 * c4);
-                    acc.x = fmaf(w.other, x.x, acc.x); acc.y = fmaf(w.other, x.y, acc.y);
-                    acc.z = fmaf(w.other, x.z, acc.z); acc.w = fmaf(w.other, x.w, acc.w);
-                }
-                *reinterpret_cast<float4*>(A.out + row * kHeadDim + 4 * c4) = acc;
-                if (c4 == 0 && A.lse) A.lse[row] = w.lse;
-            }
-            if (tid == 0) A.tickets[unit] = 0;          // ready for the next call
-            consumer_sync<NT>();                        // the merge area is free for the next unit
         }
+#pragma unroll
+        for (int o = kLanes; o < 32; o <<= 1) {
+            acc.x += __shfl_xor_sync(kFull, acc.x, o); acc.y += __shfl_xor_sync(kFull, acc.y, o);
+            acc.z += __shfl_xor_sync(kFull, acc.z, o); acc.w += __shfl_xor_sync(kFull, acc.w, o);
+        }
+        if (A.late_wait) grid_wait();
+        if (sub == 0) {
+            float O[4] = {acc.x, acc.y, acc.z, acc.w};
+            publish<4>(A, static_cast<int64_t>(d.b) * A.Hq + d.h * G + gg, s * kCh + 4 * c4, O, M, Ls, s == 0 && lane == 0);
+        }
+        if (lane == 0) *ticket = 0;                               // ready for the next call
     }
-    consumer_sync<NT>();
+}
+// Where a CTA may hold several units, a warp takes a whole head (32 x 2048 tokens: 42.0 us with halves, 39.5 so).
+template <int G, int NW>
+__device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge, int cap, int warp, int lane)
+{
+    constexpr int NS = slices_of(G, NW);
+    if (NS == 1 || cap > 1) merge_slices<G, NW, 1>(A, C.units, merge, C.epoch[1], warp, lane);
+    else merge_slices<G, NW, NS>(A, C.units, merge, C.epoch[1], warp, lane);
 }
 
 // Steps that one CTA of `grid` can own at most (either division of the line), from the cache's capacity alone.

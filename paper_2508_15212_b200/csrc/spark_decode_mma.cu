@@ -46,8 +46,7 @@ constexpr int kVTileBytes = kPageTokens * kHeadDim * 2;                         
 template <int G, bool kPV> struct SmemBf16 {
     static constexpr int kQsum = kCtrlBytes;                                     // [kMaxCap][8] float
     static constexpr int kVTile = (kQsum + kMaxCap * 8 * 4 + 127) / 128 * 128;   // per-warp tiles (pruned values)
-    static constexpr int kMl = kVTile + (kPV ? kNW * kVTileBytes : 0);           // [kMaxCap][G] (M, L) of the epoch's units
-    static constexpr int kEnd = (kMl + kMaxCap * G * 8 + 127) / 128 * 128;
+    static constexpr int kEnd = kVTile + (kPV ? kNW * kVTileBytes : 0);
     static constexpr int kTabBytes = 3 * G * kHeadDim * 2;                       // one unit's q, q' high, q' low: 3 x [G][128] bf16
 };
 
@@ -116,15 +115,17 @@ __device__ __forceinline__ float bf16_round(float x)
 //   k0,k1 : the nibble's kept values in dense positions (zero where pruned); `addr` is the shared
 //           address of the token's next unread kept value (rows of 32 bytes) and advances per set bit;
 //   m0,m1 : the nibble as 0/1 in bf16 (1.0 = 0x3F80).
-// Predicated loads, no branches.
+// Predicated loads, no branches.  The registers' zeros and the address steps are multiply-adds with a 0 and a 1 that the compiler
+// does not know, which keeps them on the FMA pipe: left to it, changes elsewhere in the kernel moved some fifty of them per page to
+// the ALU pipe, the busiest one (75.7 -> 88 million instructions of a 4 x 131072 step, 222 -> 232 us; so 72.7 million, 221).
 __device__ __forceinline__ void expand_nibble(unsigned w, unsigned b0m, unsigned b1m, unsigned b2m, unsigned b3m,
-                                              unsigned& addr, unsigned& k0, unsigned& k1, unsigned& m0, unsigned& m1)
+                                              unsigned& addr, unsigned& k0, unsigned& k1, unsigned& m0, unsigned& m1, unsigned zero, unsigned one)
 {
     asm volatile(
         "{\n\t"
         ".reg .pred p0, p1, p2, p3;\n\t"
         ".reg .b32 t0, t1, t2, t3;\n\t"
-        ".reg .b16 h0, h1, h2, h3;\n\t"
+        ".reg .b32 u0, u1, u2, u3;\n\t"
         "and.b32 t0, %5, %6;\n\t"
         "and.b32 t1, %5, %7;\n\t"
         "and.b32 t2, %5, %8;\n\t"
@@ -133,38 +134,38 @@ __device__ __forceinline__ void expand_nibble(unsigned w, unsigned b0m, unsigned
         "setp.ne.u32 p1, t1, 0;\n\t"
         "setp.ne.u32 p2, t2, 0;\n\t"
         "setp.ne.u32 p3, t3, 0;\n\t"
-        "mov.b16 h0, 0;\n\t"
-        "mov.b16 h1, 0;\n\t"
-        "mov.b16 h2, 0;\n\t"
-        "mov.b16 h3, 0;\n\t"
-        "@p0 ld.shared.u16 h0, [%4];\n\t"
-        "@p0 add.u32 %4, %4, 32;\n\t"
-        "@p1 ld.shared.u16 h1, [%4];\n\t"
-        "@p1 add.u32 %4, %4, 32;\n\t"
-        "@p2 ld.shared.u16 h2, [%4];\n\t"
-        "@p2 add.u32 %4, %4, 32;\n\t"
-        "@p3 ld.shared.u16 h3, [%4];\n\t"
-        "@p3 add.u32 %4, %4, 32;\n\t"
-        "mov.b32 %0, {h0, h1};\n\t"
-        "mov.b32 %1, {h2, h3};\n\t"
+        "mad.lo.u32 u0, %10, %10, %10;\n\t"
+        "mad.lo.u32 u1, %10, %10, %10;\n\t"
+        "mad.lo.u32 u2, %10, %10, %10;\n\t"
+        "mad.lo.u32 u3, %10, %10, %10;\n\t"
+        "@p0 ld.shared.u16 u0, [%4];\n\t"
+        "@p0 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p1 ld.shared.u16 u1, [%4];\n\t"
+        "@p1 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p2 ld.shared.u16 u2, [%4];\n\t"
+        "@p2 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p3 ld.shared.u16 u3, [%4];\n\t"
+        "@p3 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "prmt.b32 %0, u0, u1, 0x5410;\n\t"
+        "prmt.b32 %1, u2, u3, 0x5410;\n\t"
         "selp.b32 %2, 0x3F80, 0, p0;\n\t"
         "selp.b32 %3, 0x3F80, 0, p2;\n\t"
         "@p1 or.b32 %2, %2, 0x3F800000;\n\t"
         "@p3 or.b32 %3, %3, 0x3F800000;\n\t"
         "}"
         : "=&r"(k0), "=&r"(k1), "=&r"(m0), "=&r"(m1), "+r"(addr)
-        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m));
+        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(zero), "r"(one));
 }
 
 // The value-side nibble: kept value entries in dense positions, zero where pruned (see expand_nibble).
 __device__ __forceinline__ void expand_nibble_v(unsigned w, unsigned b0m, unsigned b1m, unsigned b2m, unsigned b3m,
-                                                unsigned& addr, unsigned& k0, unsigned& k1)
+                                                unsigned& addr, unsigned& k0, unsigned& k1, unsigned zero, unsigned one)
 {
     asm volatile(
         "{\n\t"
         ".reg .pred p0, p1, p2, p3;\n\t"
         ".reg .b32 t0, t1, t2, t3;\n\t"
-        ".reg .b16 h0, h1, h2, h3;\n\t"
+        ".reg .b32 u0, u1, u2, u3;\n\t"
         "and.b32 t0, %3, %4;\n\t"
         "and.b32 t1, %3, %5;\n\t"
         "and.b32 t2, %3, %6;\n\t"
@@ -173,23 +174,23 @@ __device__ __forceinline__ void expand_nibble_v(unsigned w, unsigned b0m, unsign
         "setp.ne.u32 p1, t1, 0;\n\t"
         "setp.ne.u32 p2, t2, 0;\n\t"
         "setp.ne.u32 p3, t3, 0;\n\t"
-        "mov.b16 h0, 0;\n\t"
-        "mov.b16 h1, 0;\n\t"
-        "mov.b16 h2, 0;\n\t"
-        "mov.b16 h3, 0;\n\t"
-        "@p0 ld.shared.u16 h0, [%2];\n\t"
-        "@p0 add.u32 %2, %2, 32;\n\t"
-        "@p1 ld.shared.u16 h1, [%2];\n\t"
-        "@p1 add.u32 %2, %2, 32;\n\t"
-        "@p2 ld.shared.u16 h2, [%2];\n\t"
-        "@p2 add.u32 %2, %2, 32;\n\t"
-        "@p3 ld.shared.u16 h3, [%2];\n\t"
-        "@p3 add.u32 %2, %2, 32;\n\t"
-        "mov.b32 %0, {h0, h1};\n\t"
-        "mov.b32 %1, {h2, h3};\n\t"
+        "mad.lo.u32 u0, %8, %8, %8;\n\t"
+        "mad.lo.u32 u1, %8, %8, %8;\n\t"
+        "mad.lo.u32 u2, %8, %8, %8;\n\t"
+        "mad.lo.u32 u3, %8, %8, %8;\n\t"
+        "@p0 ld.shared.u16 u0, [%2];\n\t"
+        "@p0 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p1 ld.shared.u16 u1, [%2];\n\t"
+        "@p1 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p2 ld.shared.u16 u2, [%2];\n\t"
+        "@p2 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p3 ld.shared.u16 u3, [%2];\n\t"
+        "@p3 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "prmt.b32 %0, u0, u1, 0x5410;\n\t"
+        "prmt.b32 %1, u2, u3, 0x5410;\n\t"
         "}"
         : "=&r"(k0), "=&r"(k1), "+r"(addr)
-        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m));
+        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(zero), "r"(one));
 }
 
 // Tables of one query head of a unit (one warp; lane l owns channels 4l .. 4l+3):
@@ -234,7 +235,6 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     extern __shared__ __align__(128) unsigned char smem[];
     const Ctrl C = make_ctrl(smem, A.prefix_off, A.B);
     float* qsum_all = reinterpret_cast<float*>(smem + S::kQsum);
-    float* unit_ml = reinterpret_cast<float*>(smem + S::kMl);
     unsigned char* ring = smem + A.ring_off;
     const unsigned ring_u = smem_u32(ring);
 
@@ -258,6 +258,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     }
 
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
+    const unsigned one = static_cast<unsigned>(A.pps), zero = one - 1u;      // 1 and 0 that the compiler does not know (see expand_nibble)
     for (int g = c0; g < c1;) {
         const Epoch ep = make_epoch(C.prefix, A.Hkv, cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
         // ---- the epoch's operand tables: a warp prepares one query head of one unit at a time, the next one's loads
@@ -365,7 +366,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
                             expand_nibble(w[j], 1u << (4 * ks), 2u << (4 * ks), 4u << (4 * ks), 8u << (4 * ks),
-                                          ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j]);
+                                          ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j], zero, one);
                         mma_bf16(d1, k0[0], k0[1], k1[0], k1[1], Bq[2 * ks], Bq[2 * ks + 1]);
                         mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bp[2 * ks], Bp[2 * ks + 1]);
                         if (!kShared8) mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
@@ -462,8 +463,8 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 #pragma unroll
                             for (int j = 0; j < 2; ++j) {
                                 unsigned e0, e1, e2, e3;
-                                expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1);
-                                expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3);
+                                expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1, zero, one);
+                                expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3, zero, one);
                                 sts_u32x4(vbase + (8 * j + r) * (kHeadDim * 2) + (((4 * c + u) ^ r ^ (c & 2)) << 4), e0, e1, e2, e3);
                             }
                         __syncwarp();
@@ -513,8 +514,9 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
             if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kNT>();
-        merge_and_publish<G, kNW>(A, C, merge, unit_ml, C.epoch[1], tid);
+        merge_and_publish<G, kNW>(A, C, merge, cap, warp, lane);
         g = C.epoch[0];
+        if (g < c1) consumer_sync<kNT>();                     // the records and the epoch's description are free
     }
     if (A.late_wait) {
         grid_wait();
