@@ -139,6 +139,7 @@ constexpr int kTailMax = 128;         // tokens of a dense tail that tail_attn_k
 // cannot write:
 //   - compress_pages_warp_kernel and compress_topp_kernel without eviction: keys, values, lengths and block table; behind the window norm;
 //   - evict_scores_tc_kernel<2>: queries, keys and lengths; behind pass 1 of the same call;
+//   - evict_select_kernel behind the second vote pass: window queries, and it writes the window norm, which that pass does not read;
 //   - a decode step with SPARK_FLAG_OVERLAP_PREVIOUS: lengths, block table and pages; the caller vouches for the
 //     predecessor.  Its consumers wait and release, not its producer (consumer_wait_previous);
 //   - a decode step merged with a dense tail (late_wait): everything but the tail's result; behind tail_attn_kernel, which
@@ -146,6 +147,54 @@ constexpr int kTailMax = 128;         // tokens of a dense tail that tail_attn_k
 //     before the tail kernel, and not on the tail's result, which only this step reads.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// a[b][h][j] = max(|mean over the G*W window queries of the group|, eps) by the first kThreads threads of a CTA (the others
+// only meet the barriers; `between` runs between the two): a thread sums 16 bytes' worth of channels over every 32nd (fp32: 16th)
+// row of 512 threads in double, the row groups are then added in a fixed order.  (The sum is exact in double for any order unless its
+// terms differ by more than 2^21.)  `part`: half as many rows of sums as there are row groups.
+template <typename E, int kThreads, typename F>
+__device__ __forceinline__ void window_norm(const void* __restrict__ q_win, int Hq, int Hkv, int W, float eps, float* __restrict__ qnorm,
+                                            int h, int b, int tid, double (*part)[kHeadDim], F between)
+{
+    constexpr int kVec = 16 / sizeof(E);                       // channels per 16-byte load
+    constexpr int kChunks = kHeadDim / kVec, kGroups = kThreads / kChunks;
+    const int G = Hq / Hkv, rows = G * W;
+    const int c = tid % kChunks, grp = tid / kChunks;
+    const bool on = tid < kThreads;
+    // the group's G*W window rows are consecutive in memory, (g outer, w inner)
+    const E* src = static_cast<const E*>(q_win) + (static_cast<int64_t>(b) * Hq + h * G) * W * kHeadDim + c * kVec;
+    double acc[kVec];
+#pragma unroll
+    for (int i = 0; i < kVec; ++i) acc[i] = 0.0;
+    const bool aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;
+#pragma unroll 4
+    for (int r = on ? grp : rows; r < rows; r += kGroups) {
+        alignas(16) E x[kVec];
+        const E* row = src + static_cast<int64_t>(r) * kHeadDim;
+        if (aligned) *reinterpret_cast<uint4*>(x) = *reinterpret_cast<const uint4*>(row);
+        else
+            for (int i = 0; i < kVec; ++i) x[i] = row[i];
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) acc[i] += static_cast<double>(static_cast<float>(x[i]));
+    }
+    if (on && grp >= kGroups / 2)
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) part[grp - kGroups / 2][c * kVec + i] = acc[i];
+    __syncthreads();
+    if (grp < kGroups / 2)
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) part[grp][c * kVec + i] += acc[i];
+    between();
+    __syncthreads();
+    if (tid < kHeadDim) {
+        double sum = 0.0;
+#pragma unroll
+        for (int g = 0; g < kGroups / 2; ++g) sum += part[g][tid];
+        const float m = static_cast<float>(sum / static_cast<double>(rows));
+        qnorm[(static_cast<int64_t>(b) * Hkv + h) * kHeadDim + tid] = fmaxf(fabsf(m), eps);
+    }
+}
+inline float norm_floor(const spark_params& p) { return p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f; }
 
 // Launch as a programmatic dependent, in clusters of `cluster` CTAs along x.
 template <typename... Params, typename... Args>
@@ -247,7 +296,7 @@ spark_status launch_merge_attn(int rows, const float* out_a, const float* lse_a,
 size_t decode_workspace_bytes(const spark_params& p);
 size_t evict_workspace_bytes(const spark_params& p, int64_t max_seq_tokens);
 spark_status launch_evict(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
-                          int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, int32_t* packed_lens,
+                          int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* qnorm, int32_t* packed_lens,
                           int32_t* kept_tokens, void* workspace, cudaStream_t stream, int* launches);
 size_t compress_workspace_bytes(const spark_params& p, int64_t max_seq_tokens);
 

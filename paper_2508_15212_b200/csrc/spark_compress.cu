@@ -16,12 +16,10 @@ namespace spark {
 constexpr unsigned kFullMask = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------------
-// a[b][h][j] = max(|mean over the G*W window queries of the group|, eps).
-// 128 to 512 threads (qnorm_threads): a thread sums 16 bytes' worth of channels over every 32nd (fp32: 16th) row of 512
-// threads in double, the row groups are then added in a fixed order.  (The sum is exact in double for any order unless its terms differ by more than
-// 2^21.)  The chain that bounds the kernel is a load and a few adds: one thread per channel walking all rows took
-// 8.3 us for 128 rows, this 7.1 (both cold), and the page kernel's first loads now run under it.
-// Thread 0 of the first head also publishes packed_lens when there is no eviction step.
+// The window norm (window_norm) as a launch of its own; with eviction the select kernel does it.  128 to 512 threads
+// (qnorm_threads).  The chain that bounds it is a load and a few adds: one thread per channel walking all rows took 8.3 us for
+// 128 rows, this 7.1 (both cold), and the page kernel's first loads run under it.
+// Thread 0 of the first head also publishes packed_lens.
 // ------------------------------------------------------------------------------------------------
 template <typename E, int kThreads, bool kReleaseEarly>
 __global__ void __launch_bounds__(kThreads)
@@ -29,47 +27,13 @@ window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, floa
                     float* __restrict__ qnorm, const int32_t* __restrict__ seq_lens,
                     int32_t* __restrict__ packed_lens, int max_seq_tokens, int* status)
 {
-    constexpr int kVec = 16 / sizeof(E);                       // channels per 16-byte load
-    constexpr int kChunks = kHeadDim / kVec, kGroups = kThreads / kChunks;
+    constexpr int kGroups = kThreads / (kHeadDim / (16 / static_cast<int>(sizeof(E))));
     __shared__ double part[kGroups / 2][kHeadDim];
     grid_wait();
     if (kReleaseEarly) grid_release();
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    const int G = Hq / Hkv, rows = G * W;
-    const int c = tid % kChunks, grp = tid / kChunks;
-    // the group's G*W window rows are consecutive in memory, (g outer, w inner)
-    const E* src = static_cast<const E*>(q_win) + (static_cast<int64_t>(b) * Hq + h * G) * W * kHeadDim + c * kVec;
-    double acc[kVec];
-#pragma unroll
-    for (int i = 0; i < kVec; ++i) acc[i] = 0.0;
-    const bool aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;
-#pragma unroll 4
-    for (int r = grp; r < rows; r += kGroups) {
-        alignas(16) E x[kVec];
-        const E* row = src + static_cast<int64_t>(r) * kHeadDim;
-        if (aligned) *reinterpret_cast<uint4*>(x) = *reinterpret_cast<const uint4*>(row);
-        else
-            for (int i = 0; i < kVec; ++i) x[i] = row[i];
-#pragma unroll
-        for (int i = 0; i < kVec; ++i) acc[i] += static_cast<double>(static_cast<float>(x[i]));
-    }
-    if (grp >= kGroups / 2)
-#pragma unroll
-        for (int i = 0; i < kVec; ++i) part[grp - kGroups / 2][c * kVec + i] = acc[i];
-    __syncthreads();
-    if (grp < kGroups / 2)
-#pragma unroll
-        for (int i = 0; i < kVec; ++i) part[grp][c * kVec + i] += acc[i];
-    if (!kReleaseEarly) grid_release();
-    __syncthreads();
-    if (tid < kHeadDim) {
-        double sum = 0.0;
-#pragma unroll
-        for (int g = 0; g < kGroups / 2; ++g) sum += part[g][tid];
-        const float m = static_cast<float>(sum / static_cast<double>(rows));
-        qnorm[(static_cast<int64_t>(b) * Hkv + h) * kHeadDim + tid] = fmaxf(fabsf(m), eps);
-    }
-    if (packed_lens && h == 0 && tid == 0) {
+    window_norm<E, kThreads>(q_win, Hq, Hkv, W, eps, qnorm, h, b, tid, part, [] { if (!kReleaseEarly) grid_release(); });
+    if (h == 0 && tid == 0) {
         int len = seq_lens[b];
         if (len < 0 || len > max_seq_tokens) {
             record_error(status, SPARK_ERR_DEVICE_BOUNDS);
@@ -1887,21 +1851,21 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     (void)workspace_bytes;
     int* status = static_cast<int*>(workspace);
     const bool evict = p.token_budget > 0;
-    if (evict) {            // writes kept_tokens and packed_lens
-        const spark_status st_e = launch_evict(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, packed_lens,
+    if (evict) {            // writes kept_tokens, packed_lens and qnorm
+        const spark_status st_e = launch_evict(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, qnorm, packed_lens,
                                                kept_tokens, workspace, stream, launches);
         if (st_e != SPARK_OK) return st_e;
     }
     const int max_packed = (evict && p.token_budget < max_seq_tokens) ? p.token_budget : max_seq_tokens;
     const int n_blocks = (max_packed + kPageTokens - 1) / kPageTokens;
-    const float eps = p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f;
+    const float eps = norm_floor(p);
     const dim3 qgrid(p.n_kv_heads, p.batch);
     const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
     const int rows = p.n_q_heads / p.n_kv_heads * p.window;
     auto window_norm = [&](auto elem, auto threads, auto early) {
         constexpr int kThreads = decltype(threads)::value;
         launch_kernel(window_qnorm_kernel<decltype(elem), kThreads, decltype(early)::value>, qgrid, dim3(kThreads), 0, stream, q_win, p.n_q_heads,
-                      p.n_kv_heads, p.window, eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
+                      p.n_kv_heads, p.window, eps, qnorm, seq_lens, packed_lens, max_seq_tokens, status);
     };
     auto by_threads = [&](auto elem, auto early) {
         const int n = qnorm_threads(units, rows, p.dtype == SPARK_BF16);
@@ -1913,10 +1877,12 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
         if (qnorm_release_early(units, rows, n_blocks)) by_threads(elem, std::true_type());
         else by_threads(elem, std::false_type());
     };
-    if (p.dtype == SPARK_BF16) by_release(__nv_bfloat16());
-    else by_release(0.f);
-    ++*launches;
-    if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
+    if (!evict) {                                              // (the eviction's last kernel has done it)
+        if (p.dtype == SPARK_BF16) by_release(__nv_bfloat16());
+        else by_release(0.f);
+        ++*launches;
+        if (cudaGetLastError() != cudaSuccess) return SPARK_ERR_CUDA;
+    }
     if (n_blocks == 0) return SPARK_OK;
     CompressArgs A;
     A.k = k; A.v = v; A.sb = sb; A.sh = sh; A.st = st;

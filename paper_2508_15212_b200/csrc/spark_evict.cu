@@ -43,6 +43,10 @@ struct EvictArgs {
     int32_t* kept;       // [units][budget]
     int32_t* packed_lens;
     int* status;
+    float* qnorm;        // [units][128], written by the select kernel
+    float eps;
+    int bf16;            // the window queries' type
+    int scored;          // the kernel before the select is the second vote pass of this call
 };
 
 template <typename E, int PASS>
@@ -249,7 +253,16 @@ __global__ void __launch_bounds__(kSelThreads) evict_select_kernel(EvictArgs A)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float* raw = reinterpret_cast<float*>(key_smem + A.key_cap);              // [kVoteTile + 2 * kVoteHalo]
     for (int i = tid; i < 4096; i += kSelThreads) hist[i] = sums[i] = 0;
-    grid_wait();
+    // The window norm of the unit, by the last CTA of its cluster: under the vote pass's last CTAs (see grid_release) where there
+    // was one.  (As a launch of its own behind this kernel it cost 3 us of a prefill.)
+    if (!A.scored) grid_wait();
+    if (rank == ctas - 1) {
+        double (*part)[kHeadDim] = reinterpret_cast<double (*)[kHeadDim]>(key_smem);      // (at most 16 KB; the staging tile alone has 18)
+        if (A.bf16) window_norm<__nv_bfloat16, 512>(A.q_win, A.Hq, A.Hkv, A.W, A.eps, A.qnorm, h, b, tid, part, [] {});
+        else window_norm<float, 512>(A.q_win, A.Hq, A.Hkv, A.W, A.eps, A.qnorm, h, b, tid, part, [] {});
+        __syncthreads();                                       // the keys go there next
+    }
+    if (A.scored) grid_wait();
     grid_release();
     int S = A.seq_lens[b];
     if (S < 0 || S > A.S_max) {
@@ -469,7 +482,7 @@ size_t evict_workspace_bytes(const spark_params& p, int64_t max_seq_tokens)
 }
 
 spark_status launch_evict(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
-                          int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, int32_t* packed_lens,
+                          int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* qnorm, int32_t* packed_lens,
                           int32_t* kept_tokens, void* workspace, cudaStream_t stream, int* launches)
 {
     const size_t units = static_cast<size_t>(p.batch) * p.n_kv_heads;
@@ -488,11 +501,13 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     const size_t smem = (static_cast<size_t>(kEvTile + kEvRows) * kEvStride + kEvTile) * sizeof(float);
     const dim3 grid(A.n_tiles, p.n_kv_heads, p.batch), ugrid(p.n_kv_heads, p.batch);
     const bool bf16 = p.dtype == SPARK_BF16;
-    if (A.n_tiles > 0 && max_seq_tokens > p.token_budget && evict_tc_supported(p)) {
+    A.qnorm = qnorm; A.eps = norm_floor(p); A.bf16 = bf16;
+    A.scored = A.n_tiles > 0 && max_seq_tokens > p.token_budget;
+    if (A.scored && evict_tc_supported(p)) {
         const spark_status st_tc = launch_evict_votes_tc(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, A.partial,
                                                          A.votes, A.status, stream, launches);
         if (st_tc != SPARK_OK) return st_tc;
-    } else if (A.n_tiles > 0 && max_seq_tokens > p.token_budget) {
+    } else if (A.scored) {
         static unsigned char smem_raised[4][kMaxDevices] = {};
         if (!(bf16 ? allow_max_smem(evict_scores_kernel<__nv_bfloat16, 1>, smem_raised[0]) && allow_max_smem(evict_scores_kernel<__nv_bfloat16, 2>, smem_raised[1])
                    : allow_max_smem(evict_scores_kernel<float, 1>, smem_raised[2]) && allow_max_smem(evict_scores_kernel<float, 2>, smem_raised[3])))
