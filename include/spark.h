@@ -159,7 +159,7 @@ spark_status spark_workspace_bytes(const spark_params *p, int64_t max_seq_tokens
                                    size_t *compress_bytes, size_t *decode_bytes);
 
 /* Zero a workspace.  Must be enqueued once before the first call that uses the
- * workspace; the calls leave it ready for the next one. */
+ * workspace; the calls leave it ready for the next one, also where that one has other sizes (and fits it). */
 spark_status spark_workspace_init(void *workspace, size_t workspace_bytes, spark_stream_t stream);
 
 /*

@@ -389,8 +389,7 @@ size_t decode_workspace_bytes(const spark_params& p)
 {
     const int G = p.n_q_heads / p.n_kv_heads;
     const size_t units = static_cast<size_t>(p.batch) * p.n_kv_heads;
-    size_t bytes = kWorkspaceHeader;
-    bytes += align_up(units * kTickets * sizeof(int), 256);
+    size_t bytes = kWorkspaceHeader + kTicketBytes;
     bytes += (kMaxCtas + units) * G * kPart * sizeof(float);
     return align_up(bytes, 256);
 }
@@ -476,7 +475,6 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     DeviceInfo info;
     if (!device_info(&dev, &info)) return SPARK_ERR_CUDA;
     const int G = p.n_q_heads / p.n_kv_heads;
-    const size_t units = static_cast<size_t>(p.batch) * p.n_kv_heads;
     DecodeArgs A;
     A.q = q; A.pages = static_cast<const unsigned char*>(pages); A.block_table = block_table;
     A.max_blocks = max_blocks; A.lens = packed_lens; A.qnorm = qnorm; A.out = out; A.lse = lse;
@@ -489,7 +487,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     A.status = reinterpret_cast<int*>(ws);
     A.tickets = reinterpret_cast<int*>(ws + kWorkspaceHeader);
-    A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(units * kTickets * sizeof(int), 256));
+    A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + kTicketBytes);
     A.slot_stride = 0; A.pps = 1; A.caps = EpochCaps{}; A.prefix_off = 0; A.ring_off = 0;
     A.overlap = (p.flags & SPARK_FLAG_OVERLAP_PREVIOUS) ? 1 : 0;
     A.seed = p.seed;

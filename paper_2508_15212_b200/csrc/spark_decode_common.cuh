@@ -750,7 +750,11 @@ __device__ __forceinline__ PublishWeights publish_weights(const DecodeArgs& A, i
 // the result of a 32768-token step.  us before -> after: 1 x 500 tokens 9.1 -> 8.7, 32 x 2048 41.4 -> 39.5, 8 x 5000 29.7 ->
 // 28.2, 8 x 2000..16000 44.1 -> 42.1, 1 x 4096 with 64 / 8 heads 13.7 -> 12.7, fp32 1 x 1024 13.05 -> 12.8.
 __host__ __device__ constexpr int slices_of(int g, int nw) { return 4 * g <= nw ? 4 : (2 * g <= nw ? 2 : 1); }
-constexpr int kTickets = 16;                                  // per unit; at most 14 are used (seven heads in halves)
+// Tickets of a split unit: a slice's each, at the unit's first CTA.  (No two split units have the same one: the first ends in a
+// later CTA than it starts in.)  So where tickets and partials lie does not depend on the problem, and calls of any shapes may
+// take turns on one workspace.
+constexpr int kTickets = 16;
+constexpr size_t kTicketBytes = kMaxCtas * kTickets * sizeof(int);
 constexpr int kPart = kHeadDim + 8;                           // floats of a head's partial: 128 outputs and (m, l) once per slice
 
 template <int N> __device__ __forceinline__ void load_floats(float (&x)[N], const float* p)
@@ -838,7 +842,7 @@ __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUni
         const EpochUnit d = units[e];
         if (d.n_parts == 1) continue;
         const int unit = d.b * A.Hkv + d.h, n_parts = d.n_parts;
-        int* ticket = A.tickets + unit * kTickets + gg * NS + s;
+        int* ticket = A.tickets + d.first_cta * kTickets + gg * NS + s;
         // The warp barrier orders every lane's stores before lane 0's gpu-scope release; its acquire (same atomic) and the
         // barrier behind it order every lane's reads after the other parts' stores.
         __syncwarp();

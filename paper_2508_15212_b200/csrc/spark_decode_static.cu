@@ -17,9 +17,8 @@ namespace spark {
 
 // Largest problem the built-in scratch serves: batch * n_kv_heads <= 64 (any G <= 8).
 constexpr int kNoAllocMaxUnits = 64;
-constexpr size_t kNoAllocTicketBytes = kNoAllocMaxUnits * kTickets * sizeof(int);
 constexpr size_t kNoAllocScratchBytes =
-    kWorkspaceHeader + kNoAllocTicketBytes +
+    kWorkspaceHeader + kTicketBytes +
     static_cast<size_t>(kMaxCtas + kNoAllocMaxUnits) * kMaxGroup * kPart * sizeof(float);            // ~1.4 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -70,7 +69,7 @@ extern "C" spark_status spark_decode_attn_noalloc(const spark_params* p, const v
     if (st != SPARK_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // status word and tickets must start at zero; the array keeps whatever the last call left
-    if (cudaMemsetAsync(scratch, 0, kWorkspaceHeader + kNoAllocTicketBytes, s) != cudaSuccess) return SPARK_ERR_CUDA;
+    if (cudaMemsetAsync(scratch, 0, kWorkspaceHeader + kTicketBytes, s) != cudaSuccess) return SPARK_ERR_CUDA;
     int launches = 0;
     return launch_decode(*p, q, pages, block_table, max_blocks, packed_lens, qnorm, out, lse, scratch,
                          kNoAllocScratchBytes, s, &launches);

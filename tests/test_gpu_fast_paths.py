@@ -259,3 +259,22 @@ def test_threads_with_different_shared_memory_needs():
     torch.cuda.synchronize()
     assert refused == [0] * len(made)
     assert all(cache.status() == 0 for _, cache, _ in made)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_steps_of_several_shapes_take_turns_on_one_workspace(dtype):
+    """A batch that grows and shrinks between steps, units split over CTAs in each: the workspace of the largest serves all."""
+    made = []
+    for Hq, Hkv, lens in ((16, 8, [3000] * 8), (8, 4, [5000]), (4, 4, [900, 2500, 40]), (7, 1, [4000, 4000])):
+        wl = make(dtype, len(lens), Hq, Hkv, lens, 8, 64, seed=470 + len(lens), sigma=1.0 if dtype == "bf16" else 0.5, gap=False)
+        cache = SparkCache(batch=len(lens), n_q_heads=Hq, n_kv_heads=Hkv, window=8, keep=64, dtype=dtype, max_tokens=max(lens))
+        cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+        made.append((cache, wl.q, cache.decode(wl.q).clone()))
+        assert cache.status() == 0
+    shared = torch.empty(max(c.ws_decode.numel() for c, _, _ in made), dtype=torch.uint8, device="cuda")
+    B.spark_workspace_init(shared)
+    for i in (0, 1, 0, 2, 3, 0, 3, 1, 2, 0):
+        cache, q, want = made[i]
+        cache.ws_decode = shared
+        assert torch.equal(cache.decode(q, out=torch.full_like(want, float("nan"))), want)
+        assert cache.status() == 0
