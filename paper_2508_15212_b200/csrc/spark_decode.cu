@@ -488,7 +488,7 @@ spark_status launch_decode(const spark_params& p, const void* q, const void* pag
     A.status = reinterpret_cast<int*>(ws);
     A.tickets = reinterpret_cast<int*>(ws + kWorkspaceHeader);
     A.partials = reinterpret_cast<float*>(ws + kWorkspaceHeader + kTicketBytes);
-    A.slot_stride = 0; A.pps = 1; A.caps = EpochCaps{}; A.prefix_off = 0; A.ring_off = 0;
+    A.slot_stride = 0; A.pps = 1; A.one = 1; A.caps = EpochCaps{}; A.prefix_off = 0; A.ring_off = 0;
     A.overlap = (p.flags & SPARK_FLAG_OVERLAP_PREVIOUS) ? 1 : 0;
     A.seed = p.seed;
     A.q_by_value = q_by_value ? 1 : 0;

@@ -68,6 +68,7 @@ struct DecodeArgs {
     float* partials;
     int slot_stride;
     int pps;                                 // pages per step (= per ring slot): 1 or 2
+    unsigned one;                            // 1, which the compiler does not know (see expand_nibble)
     FastDiv by_grid, by_hkv;                 // CTAs of the grid; KV heads
     int per_unit, extra;                     // aligned mode (see Plan): CTAs per unit; units with one more
     FastDiv by_q, by_q1;                     // per_unit and per_unit + 1

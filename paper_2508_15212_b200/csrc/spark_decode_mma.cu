@@ -115,11 +115,12 @@ __device__ __forceinline__ float bf16_round(float x)
 //   k0,k1 : the nibble's kept values in dense positions (zero where pruned); `addr` is the shared
 //           address of the token's next unread kept value (rows of 32 bytes) and advances per set bit;
 //   m0,m1 : the nibble as 0/1 in bf16 (1.0 = 0x3F80).
-// Predicated loads, no branches.  The registers' zeros and the address steps are multiply-adds with a 0 and a 1 that the compiler
-// does not know, which keeps them on the FMA pipe: left to it, changes elsewhere in the kernel moved some fifty of them per page to
-// the ALU pipe, the busiest one (75.7 -> 88 million instructions of a 4 x 131072 step, 222 -> 232 us; so 72.7 million, 221).
+// Predicated loads, no branches.  An address step is a multiply-add with a 1 that the compiler does not know, which keeps it on the
+// FMA pipe: the ALU pipe is the busiest one.  (us with address steps and zeros as the compiler places them / both forced onto the FMA
+// pipe / address steps only, as here: 16 x 8192..131072 tokens, 28 / 4 heads 347 / 344 / 336; 4 x 65536, T = 25, with pruned values
+// 8 / 8 heads 194 / 185 / 180, 16 / 8 195 / 187 / 182, 32 / 8 191 / 182 / 182, 48 / 8 206 / 201 / 195; with dense ones 48 / 8 151 / 144 / 143.)
 __device__ __forceinline__ void expand_nibble(unsigned w, unsigned b0m, unsigned b1m, unsigned b2m, unsigned b3m,
-                                              unsigned& addr, unsigned& k0, unsigned& k1, unsigned& m0, unsigned& m1, unsigned zero, unsigned one)
+                                              unsigned& addr, unsigned& k0, unsigned& k1, unsigned& m0, unsigned& m1, unsigned one)
 {
     asm volatile(
         "{\n\t"
@@ -134,18 +135,18 @@ __device__ __forceinline__ void expand_nibble(unsigned w, unsigned b0m, unsigned
         "setp.ne.u32 p1, t1, 0;\n\t"
         "setp.ne.u32 p2, t2, 0;\n\t"
         "setp.ne.u32 p3, t3, 0;\n\t"
-        "mad.lo.u32 u0, %10, %10, %10;\n\t"
-        "mad.lo.u32 u1, %10, %10, %10;\n\t"
-        "mad.lo.u32 u2, %10, %10, %10;\n\t"
-        "mad.lo.u32 u3, %10, %10, %10;\n\t"
+        "mov.b32 u0, 0;\n\t"
+        "mov.b32 u1, 0;\n\t"
+        "mov.b32 u2, 0;\n\t"
+        "mov.b32 u3, 0;\n\t"
         "@p0 ld.shared.u16 u0, [%4];\n\t"
-        "@p0 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p0 mad.lo.u32 %4, %10, 32, %4;\n\t"
         "@p1 ld.shared.u16 u1, [%4];\n\t"
-        "@p1 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p1 mad.lo.u32 %4, %10, 32, %4;\n\t"
         "@p2 ld.shared.u16 u2, [%4];\n\t"
-        "@p2 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p2 mad.lo.u32 %4, %10, 32, %4;\n\t"
         "@p3 ld.shared.u16 u3, [%4];\n\t"
-        "@p3 mad.lo.u32 %4, %11, 32, %4;\n\t"
+        "@p3 mad.lo.u32 %4, %10, 32, %4;\n\t"
         "prmt.b32 %0, u0, u1, 0x5410;\n\t"
         "prmt.b32 %1, u2, u3, 0x5410;\n\t"
         "selp.b32 %2, 0x3F80, 0, p0;\n\t"
@@ -154,12 +155,12 @@ __device__ __forceinline__ void expand_nibble(unsigned w, unsigned b0m, unsigned
         "@p3 or.b32 %3, %3, 0x3F800000;\n\t"
         "}"
         : "=&r"(k0), "=&r"(k1), "=&r"(m0), "=&r"(m1), "+r"(addr)
-        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(zero), "r"(one));
+        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(one));
 }
 
 // The value-side nibble: kept value entries in dense positions, zero where pruned (see expand_nibble).
 __device__ __forceinline__ void expand_nibble_v(unsigned w, unsigned b0m, unsigned b1m, unsigned b2m, unsigned b3m,
-                                                unsigned& addr, unsigned& k0, unsigned& k1, unsigned zero, unsigned one)
+                                                unsigned& addr, unsigned& k0, unsigned& k1, unsigned one)
 {
     asm volatile(
         "{\n\t"
@@ -174,23 +175,23 @@ __device__ __forceinline__ void expand_nibble_v(unsigned w, unsigned b0m, unsign
         "setp.ne.u32 p1, t1, 0;\n\t"
         "setp.ne.u32 p2, t2, 0;\n\t"
         "setp.ne.u32 p3, t3, 0;\n\t"
-        "mad.lo.u32 u0, %8, %8, %8;\n\t"
-        "mad.lo.u32 u1, %8, %8, %8;\n\t"
-        "mad.lo.u32 u2, %8, %8, %8;\n\t"
-        "mad.lo.u32 u3, %8, %8, %8;\n\t"
+        "mov.b32 u0, 0;\n\t"
+        "mov.b32 u1, 0;\n\t"
+        "mov.b32 u2, 0;\n\t"
+        "mov.b32 u3, 0;\n\t"
         "@p0 ld.shared.u16 u0, [%2];\n\t"
-        "@p0 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p0 mad.lo.u32 %2, %8, 32, %2;\n\t"
         "@p1 ld.shared.u16 u1, [%2];\n\t"
-        "@p1 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p1 mad.lo.u32 %2, %8, 32, %2;\n\t"
         "@p2 ld.shared.u16 u2, [%2];\n\t"
-        "@p2 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p2 mad.lo.u32 %2, %8, 32, %2;\n\t"
         "@p3 ld.shared.u16 u3, [%2];\n\t"
-        "@p3 mad.lo.u32 %2, %9, 32, %2;\n\t"
+        "@p3 mad.lo.u32 %2, %8, 32, %2;\n\t"
         "prmt.b32 %0, u0, u1, 0x5410;\n\t"
         "prmt.b32 %1, u2, u3, 0x5410;\n\t"
         "}"
         : "=&r"(k0), "=&r"(k1), "+r"(addr)
-        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(zero), "r"(one));
+        : "r"(w), "r"(b0m), "r"(b1m), "r"(b2m), "r"(b3m), "r"(one));
 }
 
 // Tables of one query head of a unit (one warp; lane l owns channels 4l .. 4l+3):
@@ -250,16 +251,23 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
     }
     consumer_wait_plan(kThreads);
     const int c0 = C.run->c0, c1 = C.run->c1, NS = C.plan->nslots, cap = C.plan->cap;
-    float* merge = reinterpret_cast<float*>(smem + C.plan->merge_off);
-    unsigned char* tab_all = smem + C.plan->tab_off;
+    // One or two heads a group and pruned values: what the merge needs is read again there, so that none of it holds a register
+    // through the page loop.  (us with the values from here -> read again: 4 x 65536, T = 25, 8 / 8 heads 184 -> 180, 16 / 8 186 -> 182;
+    // but 24 / 8 181.6 -> 182.6, 48 / 8 194.4 -> 195.6, and one step of 32768 with 32 / 8 33.4 -> 33.6.)
+    constexpr bool kAgain = kPV && G <= 2;
+    auto merge_area = [&]() { return reinterpret_cast<float*>(smem + C.plan->merge_off); };
+    auto tables = [&]() { return smem + C.plan->tab_off; };
+    float* const merge0 = merge_area();
+    unsigned char* const tab0 = tables();
     if (!A.late_wait) {
         consumer_wait_previous(A);                         // q, qnorm, out and the workspace from here on
         write_empty_sequences<kNT>(A, C.prefix, tid);
     }
 
+    const unsigned one = A.one;
     const int c = lane & 3, r = lane >> 2;                 // quad lane / fragment row
-    const unsigned one = static_cast<unsigned>(A.pps), zero = one - 1u;      // 1 and 0 that the compiler does not know (see expand_nibble)
     for (int g = c0; g < c1;) {
+        unsigned char* tab_all = kAgain ? tables() : tab0;
         const Epoch ep = make_epoch(C.prefix, A.Hkv, cap, g == c0 ? C.run->first : locate_unit(C.prefix, A.B, A.Hkv, g), g, c1);
         // ---- the epoch's operand tables: a warp prepares one query head of one unit at a time, the next one's loads
         //      in flight meanwhile (first pass: only loads) ----
@@ -366,7 +374,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
                             expand_nibble(w[j], 1u << (4 * ks), 2u << (4 * ks), 4u << (4 * ks), 8u << (4 * ks),
-                                          ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j], zero, one);
+                                          ks < 4 ? vaddr[j] : vaddr_hi[j], k0[j], k1[j], m0[j], m1[j], one);
                         mma_bf16(d1, k0[0], k0[1], k1[0], k1[1], Bq[2 * ks], Bq[2 * ks + 1]);
                         mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bp[2 * ks], Bp[2 * ks + 1]);
                         if (!kShared8) mma_bf16(d2, m0[0], m0[1], m1[0], m1[1], Bpl[2 * ks], Bpl[2 * ks + 1]);
@@ -463,8 +471,8 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 #pragma unroll
                             for (int j = 0; j < 2; ++j) {
                                 unsigned e0, e1, e2, e3;
-                                expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1, zero, one);
-                                expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3, zero, one);
+                                expand_nibble_v(vw[j], 1u << (8 * u), 2u << (8 * u), 4u << (8 * u), 8u << (8 * u), va[j], e0, e1, one);
+                                expand_nibble_v(vw[j], 16u << (8 * u), 32u << (8 * u), 64u << (8 * u), 128u << (8 * u), va[j], e2, e3, one);
                                 sts_u32x4(vbase + (8 * j + r) * (kHeadDim * 2) + (((4 * c + u) ^ r ^ (c & 2)) << 4), e0, e1, e2, e3);
                             }
                         __syncwarp();
@@ -485,7 +493,7 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
 
             // ---------------- the state goes to the merge as record warp + eu ----------------
             {
-                float* rec = merge + (warp + eu) * G * kRec;
+                float* rec = (kAgain ? merge_area() : merge0) + (warp + eu) * G * kRec;
                 float lsum[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
@@ -514,7 +522,13 @@ __device__ __forceinline__ void decode_bf16_body(const DecodeArgs& A, const void
             if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kNT>();
-        merge_and_publish<G, kNW>(A, C, merge, cap, warp, lane);
+        if constexpr (kAgain) {
+            unsigned t;
+            asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+            merge_and_publish<G, kNW>(A, C, merge_area(), C.plan->cap, t >> 5, t & 31);
+        } else {
+            merge_and_publish<G, kNW>(A, C, merge0, cap, warp, lane);
+        }
         g = C.epoch[0];
         if (g < c1) consumer_sync<kNT>();                     // the records and the epoch's description are free
     }
