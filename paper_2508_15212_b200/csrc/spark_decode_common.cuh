@@ -853,7 +853,10 @@ __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUni
         if (__shfl_sync(kFull, old, 0) != n_parts - 1) continue;
         constexpr int kLanes = kCh / 4, PP = 32 / kLanes;         // lanes of a part (four channels each); parts at a time
         constexpr int kSteps = 32 / PP, kBatch = 8;               // steps of 32 parts; loads in flight of one group of parts
-        constexpr int kTwo = kSteps == kBatch ? 2 : 1;            // groups taken at once (one unit on the whole grid: 148 parts)
+        // Groups taken at once: two for a quarter of one head (one unit on the whole grid has 148 parts; bf16, 1 x 32768 tokens, one
+        // head 11.7 -> 11.2 us).  In the kernel of 8 warps the second one spills 36 to 44 bytes and gains nothing (fp32, 1 x 1024, one
+        // head 13.0 us with two, 12.6 with one; 4 x 200..3000 with 4 / 4 heads 15.2, 14.6).
+        constexpr int kTwo = kSteps == kBatch && NW > 8 ? 2 : 1;
         constexpr int kGroups = kMaxCtas / 32;                    // (m, l) pairs a lane may hold
         constexpr int64_t kStride = static_cast<int64_t>(G) * kPart;
         const float* base = A.partials + (static_cast<int64_t>(d.first_cta + unit) * G + gg) * kPart;
