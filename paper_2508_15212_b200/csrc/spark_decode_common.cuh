@@ -750,7 +750,9 @@ __device__ __forceinline__ PublishWeights publish_weights(const DecodeArgs& A, i
 // CTAs come last.  A ticket per unit and one CTA merging all of it behind four barriers took 3.6 us from the last record to
 // the result of a 32768-token step.  us before -> after: 1 x 500 tokens 9.1 -> 8.7, 32 x 2048 41.4 -> 39.5, 8 x 5000 29.7 ->
 // 28.2, 8 x 2000..16000 44.1 -> 42.1, 1 x 4096 with 64 / 8 heads 13.7 -> 12.7, fp32 1 x 1024 13.05 -> 12.8.
-__host__ __device__ constexpr int slices_of(int g, int nw) { return 4 * g <= nw ? 4 : (2 * g <= nw ? 2 : 1); }
+// (Three heads a group in halves: in quarters, us, 1 x 1000 tokens with 12 / 4 heads 9.2, in halves 8.9, whole 9.5; 1 x 16000 13.2, 13.0,
+// 13.7; 1 x 32768 with 6 / 2 heads 14.9, 14.5, 16.4.)
+__host__ __device__ constexpr int slices_of(int g, int nw) { return 4 * g <= 8 ? 4 : (2 * g <= nw ? 2 : 1); }
 // Tickets of a split unit: a slice's each, at the unit's first CTA.  (No two split units have the same one: the first ends in a
 // later CTA than it starts in.)  So where tickets and partials lie does not depend on the problem, and calls of any shapes may
 // take turns on one workspace.
