@@ -406,7 +406,8 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     const int64_t units = static_cast<int64_t>(A.B) * A.Hkv;
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     set_divisors(A, units, grid);
-    A.slack = A.ragged_slack = 4;                          // (4 x 200..3000 tokens, 4 KV heads: 19.1 -> 17.3 us)
+    A.slack = 4; A.ragged_slack = 0;
+    A.ragged_from = INFINITY;                              // (2 x 300..1000 tokens, 2 / 2 heads 13.6 us in whole CTAs, 13.0 in even runs; 4 x 200..3000, 4 / 4 heads 14.7 and 14.8)
     A.whole_steps = 0;                                     // (a step is 32 tokens of double sums: splitting pays)
     A.prefix_off = S::kEnd;
     A.ring_off = A.prefix_off + prefix_bytes(A.B);

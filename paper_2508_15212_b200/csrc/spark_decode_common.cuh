@@ -74,6 +74,7 @@ struct DecodeArgs {
     FastDiv by_q, by_q1;                     // per_unit and per_unit + 1
     EpochCaps caps;                          // units per epoch, chosen with the plan
     int slack, ragged_slack;                 // steps that the longest share may be above the even one (see Plan)
+    float ragged_from;                       // unequal units in whole CTAs from this many shortest units per even share
     int whole_steps;                         // a step per consumer warp; units up to this are not split (see Plan)
     int prefix_off;                          // shared-memory offset of the steps-per-sequence prefix and the lengths
     int ring_off;                            // shared-memory offset of the ring (behind the prefix); records and tables follow it
@@ -512,7 +513,7 @@ __device__ __forceinline__ CtaRun producer_prologue(const DecodeArgs& A, const C
         run.c0 = run.first.start + min(smax, k * per);
         run.c1 = run.first.start + min(smax, (k + 1) * per);
         pl.first_cta = cta - k; pl.share = per;
-    } else if (units <= nct && smin != smax && smax < (1 << 22) && 3.f * static_cast<float>(pl.total) <= (3 * nct - units) * static_cast<float>(pl.chunk + extra) &&
+    } else if (units <= nct && smin != smax && smax < (1 << 22) && static_cast<float>(pl.chunk) >= A.ragged_from * static_cast<float>(least) && 3.f * static_cast<float>(pl.total) <= (3 * nct - units) * static_cast<float>(pl.chunk + extra) &&
                ragged_run(C.prefix, A.B, A.Hkv, pl.chunk, extra, cta, nct, lane, C.run, C.plan)) {
         pl.aligned = 1;
         pl.first_cta = C.plan->first_cta; pl.share = C.plan->share;
@@ -916,12 +917,16 @@ __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUni
         if (lane == 0) *ticket = 0;                               // ready for the next call
     }
 }
-// Where a CTA may hold several units, a warp takes a whole head (32 x 2048 tokens: 42.0 us with halves, 39.5 so).
+// Fifteen warps: where a CTA may hold several units, a warp takes a whole head (32 x 2048 tokens, 32 / 8 heads: 42.0 us with halves,
+// 39.5 so; 2 x 3000..7000 16.1 and 14.2).  Eight warps, whose one or two heads would leave most of them idle: only with more than half
+// as many units as CTAs (fp32, 2 x 300..1000 tokens, 2 / 2 heads: whole 14.1, quarters 13.0; 4 x 200..1000, 2 / 1 heads 15.7 and 14.8;
+// but 16 x 100..2000, 8 / 8 heads 49.6 and 51.5).
 template <int G, int NW>
 __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge, int cap, int warp, int lane)
 {
     constexpr int NS = slices_of(G, NW);
-    if (NS == 1 || cap > 1) merge_slices<G, NW, 1>(A, C.units, merge, C.epoch[1], warp, lane);
+    const bool whole = NW > 8 ? cap > 1 : 2 * A.B * A.Hkv > static_cast<int>(gridDim.x);       // (the same in every CTA)
+    if (NS == 1 || whole) merge_slices<G, NW, 1>(A, C.units, merge, C.epoch[1], warp, lane);
     else merge_slices<G, NW, NS>(A, C.units, merge, C.epoch[1], warp, lane);
 }
 

@@ -205,6 +205,8 @@ def test_division_of_the_step(name, Hq, Hkv, lens):
     (8, 8, [1000] * 20),
     (28, 4, [100 + 97 * i for i in range(20)]),
     (16, 2, [5000, 1, 5000, 40, 3000, 900]),
+    (4, 4, [900, 2500, 40]),
+    (8, 1, [330, 20, 1000]),
 ])
 def test_division_of_the_step_with_head_room(dtype, Hq, Hkv, lens):
     """Units per epoch and ring slots follow the lengths: a cache with room for sixteen times the longest sequence gives what
