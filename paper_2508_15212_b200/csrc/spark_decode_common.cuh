@@ -283,13 +283,18 @@ struct EpochUnit {
 //   stream mode : CTA c owns steps [c*chunk, (c+1)*chunk) of the whole line; a CTA may cross unit
 //                 boundaries (exact balance; used when sequences differ in length or units are many).
 //   aligned mode: every unit gets whole CTAs and is split evenly among them, so no CTA crosses a unit boundary and every CTA
-//                 publishes exactly once.  Equally long units: q or q+1 CTAs each.  Unequal ones: as many as keep every share at
-//                 or below the smallest bound for which the grid suffices.  Taken where the longest share is at most 4 % (and,
-//                 up to kShortShare steps, kSplitSlack or kRaggedSlack steps) above the even one: a boundary inside a CTA's run
-//                 costs it a second table, merge and publication (up to 4 us), and all wait for it.  us, stream mode -> aligned:
-//                 1 x 2048 tokens 14.0 -> 9.6, 1 x 4096 15.0 -> 11.0, 2 x 2048 12.6 -> 10.9, 8 x 700 13.9 -> 12.1; unequal ones:
-//                 2 x 3000..7000 15.9 -> 14.9, 8 x 150..4000 20.7 -> 19.3 (a slack of 10 does not reach it), 4 x 800..4000 with
-//                 28 / 4 heads 16.0 -> 14.1.  With the slack at any share 4 x 10000 29.2 -> 29.7, 4 x 4000..20000 33.4 -> 34.3.
+//                 publishes exactly once: a boundary inside a CTA's run costs it a second table and merge, and all wait for it.
+//                 Equally long units: q or q+1 CTAs each.  Unequal ones: as many as keep every share at or below the smallest bound for
+//                 which the grid suffices.  Taken where the longest share is at most 4 % (and, up to kShortShare steps, kSplitSlack or
+//                 kRaggedSlack steps) above the even one.  us, stream mode -> aligned: 1 x 2048 tokens 14.0 -> 9.6, 1 x 4096 15.0 -> 11.0,
+//                 2 x 2048 12.6 -> 10.9, 8 x 700 13.9 -> 12.1.  With the slack at any share 4 x 10000 29.2 -> 29.7, 4 x 4000..20000 33.4 -> 34.3.
+//                 Unequal units (ragged_from): with up to six heads a group from two shortest units per even share, where runs of the
+//                 line would meet several units; with seven or eight, whose tables and merges take longest, always; with one or two
+//                 never.  8 / 8 and 16 / 8 heads: 8 x 150..4000 17.1 -> 18.6 and 17.4 -> 18.9, 4 x 100..6000 15.1 -> 15.7 and 15.1 -> 15.8;
+//                 32 / 8: 8 x 150..4000 19.3 -> 18.7, 6 x 60..4000 23.3 -> 16.3, 6 x 300..6000 20.1 -> 19.4, but below two 5 x 700..6000 17.1 ->
+//                 18.0, 4 x 2000..9000 19.6 -> 20.3; 40 / 8: 8 x 500..2500 16.2 -> 17.3; 28 / 4: 2 x 600..6000 14.0 -> 13.1, 12 x 300..3000 18.6 -> 16.1;
+//                 64 / 8: 2 x 600..6000 18.6 -> 14.6.  A slack of 10 or 30 steps in place of 20 gives the same within 0.1 in 26 sizes of shares
+//                 of 5 to 110 steps, but for 8 x 150..4000 with 32 / 8 heads, where one of 10 does not find a division (19.8).
 //   whole units : CTA u owns unit u.  For units of at most a step per warp, where a split saves nothing and adds a
 //                 partial, a ticket and the last arriver's merge (240 tokens: 8.4 us against 9.1; with two steps per warp
 //                 9.7 against 9.2), and for units of up to three steps per warp where they fill most of the grid anyway

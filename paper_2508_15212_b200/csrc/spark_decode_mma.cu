@@ -582,7 +582,7 @@ static spark_status launch_bf16(const DecodeArgs& A0, int dev, const DeviceInfo&
     const int grid = decode_grid(n_sms, units, A.max_blocks, A.pps);
     set_divisors(A, units, grid);
     A.whole_steps = kNW;
-    A.slack = kSplitSlack; A.ragged_slack = kRaggedSlack; A.ragged_from = 0.f;
+    A.slack = kSplitSlack; A.ragged_slack = kRaggedSlack; A.ragged_from = G <= 2 ? INFINITY : (G <= 6 ? 2.f : 0.f);
     A.prefix_off = S::kEnd;
     A.ring_off = A.prefix_off + prefix_bytes(A.B);
     const EpochRoom room = epoch_room(A, kNW, G, S::kTabBytes, smem_optin, kMaxSlots);

@@ -190,10 +190,16 @@ def test_top_p_of_odd_values_equals_appending_them(p, cap):
     ("seven heads per group", 28, 4, [100 + 97 * i for i in range(20)]),
     ("equal units, a share of one step more than even", 16, 8, [4096]),
     ("equal units, some with two CTAs", 8, 4, [800] * 32),
-    ("unequal units in whole CTAs", 16, 8, [150 + 550 * i for i in range(8)]),
-    ("unequal units in whole CTAs, empty sequences, CTAs to spare", 4, 4, [0, 3000, 0, 17, 1200, 0]),
-    ("more sequences than lanes, whole CTAs", 4, 2, [30 * (i % 3) for i in range(39)] + [2500]),
-    ("as many units as CTAs", 2, 1, [900 + i for i in range(148)]),
+    ("unequal units, two heads a group", 16, 8, [150 + 550 * i for i in range(8)]),
+    ("unequal units, one head a group, empty sequences", 4, 4, [0, 3000, 0, 17, 1200, 0]),
+    ("more sequences than lanes, two heads a group", 4, 2, [30 * (i % 3) for i in range(39)] + [2500]),
+    ("as many units as CTAs, two heads a group", 2, 1, [900 + i for i in range(148)]),
+    ("unequal units in whole CTAs", 32, 8, [150 + 550 * i for i in range(8)]),
+    ("unequal units in whole CTAs, eight heads a group", 16, 2, [150 + 550 * i for i in range(8)]),
+    ("unequal units in whole CTAs, empty sequences, CTAs to spare", 16, 4, [0, 3000, 0, 17, 1200, 0]),
+    ("more sequences than lanes, whole CTAs", 8, 2, [30 * (i % 3) for i in range(39)] + [2500]),
+    ("as many units as CTAs", 8, 1, [900 + i for i in range(148)]),
+    ("shares of less than two of the shortest unit", 16, 4, [700, 2500, 900, 1700]),
 ])
 def test_division_of_the_step(name, Hq, Hkv, lens):
     check_case(make("bf16", len(lens), Hq, Hkv, lens, 8, 64, seed=400 + len(lens), gap=False), 64, check_vals=False)
