@@ -123,21 +123,14 @@ __device__ __forceinline__ void tc_ld64(unsigned taddr, float (&v)[64])
 }
 
 // Copy `rows` rows of 128 bf16 channels (row i at src + i*stride elements; rows >= valid are zero) into
-// the two 64-channel swizzled blocks at dst (block 0 at dst, block 1 at dst + rows_alloc*128 bytes).  kAligned: the rows start
-// on 16-byte boundaries (keys always do; window queries need not).
-template <bool kAligned>
+// the two 64-channel swizzled blocks at dst (block 0 at dst, block 1 at dst + rows_alloc*128 bytes).
 __device__ __forceinline__ void tc_stage_rows(unsigned char* dst, int rows_alloc, const unsigned short* src, int64_t stride,
                                               int valid, int tid, int threads)
 {
     for (int i = tid; i < rows_alloc * 16; i += threads) {
         const int r = i >> 4, ch16 = i & 15;
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (r < valid) {
-            const unsigned short* s = src + static_cast<int64_t>(r) * stride + ch16 * 8;
-            if (kAligned) v = *reinterpret_cast<const uint4*>(s);
-            else v = make_uint4(s[0] | static_cast<unsigned>(s[1]) << 16, s[2] | static_cast<unsigned>(s[3]) << 16,
-                                s[4] | static_cast<unsigned>(s[5]) << 16, s[6] | static_cast<unsigned>(s[7]) << 16);
-        }
+        if (r < valid) v = *reinterpret_cast<const uint4*>(src + static_cast<int64_t>(r) * stride + ch16 * 8);
         const int kb = ch16 >> 3, c8 = ch16 & 7;
         *reinterpret_cast<uint4*>(dst + static_cast<size_t>(kb) * rows_alloc * 128 + r * 128 + ((c8 ^ (r & 7)) << 4)) = v;
     }
@@ -289,11 +282,10 @@ __global__ void __launch_bounds__(tc_threads(kBlocks), kBlocks == 1 ? 2 : 1) evi
         for (int i = ragged ? 1 : 0; i < min(kBufs, n_tiles); ++i) load_tile(i);
     }
     // query rows of the group: row = g*W + w  ->  q_win[b][h*G+g][w][:]  (contiguous over (g, w))
-    const unsigned short* q_unit = static_cast<const unsigned short*>(A.q_win) + (static_cast<int64_t>(b) * A.Hq + h * G) * A.W * kHeadDim;
-    if ((reinterpret_cast<uintptr_t>(q_unit) & 15) == 0) tc_stage_rows<true>(q_s, kRows, q_unit, kHeadDim, R, tid, kThreads);
-    else tc_stage_rows<false>(q_s, kRows, q_unit, kHeadDim, R, tid, kThreads);
+    tc_stage_rows(q_s, kRows, static_cast<const unsigned short*>(A.q_win) + (static_cast<int64_t>(b) * A.Hq + h * G) * A.W * kHeadDim,
+                  kHeadDim, R, tid, kThreads);
     if (ragged)
-        tc_stage_rows<true>(k_s, kTcTile, static_cast<const unsigned short*>(A.k) + static_cast<int64_t>(b) * A.sb + static_cast<int64_t>(h) * A.sh +
+        tc_stage_rows(k_s, kTcTile, static_cast<const unsigned short*>(A.k) + static_cast<int64_t>(b) * A.sb + static_cast<int64_t>(h) * A.sh +
                       static_cast<int64_t>(tile1 - 1) * kTcTile * A.st, A.st, S - (tile1 - 1) * kTcTile, tid, kThreads);
     if (PASS == 2) {                                       // p = 2^(s - c), c = row max + log2(row sum); padding rows give 0
         grid_wait();
