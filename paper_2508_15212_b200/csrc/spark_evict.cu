@@ -503,8 +503,7 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     const bool bf16 = p.dtype == SPARK_BF16;
     A.qnorm = qnorm; A.eps = norm_floor(p); A.bf16 = bf16;
     A.scored = A.n_tiles > 0 && max_seq_tokens > p.token_budget;
-    // (The tensor-core kernels read the window queries 16 bytes at a time, which the call does not ask their alignment for.  A second way of
-    // reading in those kernels made every prefill pay: 1 x 131072 tokens 146 -> 149 us.)
+    // (the tensor-core kernels read the window queries 16 bytes at a time; the call does not ask for that alignment)
     const bool q_aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;
     if (A.scored && q_aligned && evict_tc_supported(p)) {
         const spark_status st_tc = launch_evict_votes_tc(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, A.partial,
