@@ -194,6 +194,12 @@ __device__ __forceinline__ void window_norm(const void* __restrict__ q_win, int 
         qnorm[(static_cast<int64_t>(b) * Hkv + h) * kHeadDim + tid] = fmaxf(fabsf(m), eps);
     }
 }
+// With eviction the window norm is done by the select kernel, under the vote pass's last CTAs, where all its CTAs (1024 threads each, two
+// to an SM) are resident at once; with more units only the first of several rounds would hide it, and a launch of its own is
+// better.  us per evicting prefill with a launch / in the select kernel: 1 x 131072 with 8 KV heads 154.2 / 153.3, 1 x 100000 with 4
+// 122.6 / 119.1, 4 x 4000 64.1 / 61.5, 32 x 3000 (256 units) 199.8 / 198.0; 64 x 1000 (512) 166.7 / 175.6, 64 x 1500 294.6 / 300.3,
+// 128 x 1500 (1024) 416 / 424.
+inline bool norm_in_select(int64_t units) { return units <= 256; }
 inline float norm_floor(const spark_params& p) { return p.qnorm_eps > 0.f ? p.qnorm_eps : 1e-12f; }
 
 // Launch as a programmatic dependent, in clusters of `cluster` CTAs along x.

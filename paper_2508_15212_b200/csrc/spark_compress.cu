@@ -16,10 +16,10 @@ namespace spark {
 constexpr unsigned kFullMask = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------------
-// The window norm (window_norm) as a launch of its own; with eviction the select kernel does it.  128 to 512 threads
+// The window norm (window_norm) as a launch of its own; with eviction and few units the select kernel does it (norm_in_select).  128 to 512 threads
 // (qnorm_threads).  The chain that bounds it is a load and a few adds: one thread per channel walking all rows took 8.3 us for
 // 128 rows, this 7.1 (both cold), and the page kernel's first loads run under it.
-// Thread 0 of the first head also publishes packed_lens.
+// Thread 0 of the first head also publishes packed_lens (where there is no eviction).
 // ------------------------------------------------------------------------------------------------
 template <typename E, int kThreads, bool kReleaseEarly>
 __global__ void __launch_bounds__(kThreads)
@@ -33,7 +33,7 @@ window_qnorm_kernel(const void* __restrict__ q_win, int Hq, int Hkv, int W, floa
     if (kReleaseEarly) grid_release();
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     window_norm<E, kThreads>(q_win, Hq, Hkv, W, eps, qnorm, h, b, tid, part, [] { if (!kReleaseEarly) grid_release(); });
-    if (h == 0 && tid == 0) {
+    if (packed_lens && h == 0 && tid == 0) {
         int len = seq_lens[b];
         if (len < 0 || len > max_seq_tokens) {
             record_error(status, SPARK_ERR_DEVICE_BOUNDS);
@@ -1851,7 +1851,8 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     (void)workspace_bytes;
     int* status = static_cast<int*>(workspace);
     const bool evict = p.token_budget > 0;
-    if (evict) {            // writes kept_tokens, packed_lens and qnorm
+    const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
+    if (evict) {            // writes kept_tokens, packed_lens and, where norm_in_select, qnorm
         const spark_status st_e = launch_evict(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, qnorm, packed_lens,
                                                kept_tokens, workspace, stream, launches);
         if (st_e != SPARK_OK) return st_e;
@@ -1860,12 +1861,11 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
     const int n_blocks = (max_packed + kPageTokens - 1) / kPageTokens;
     const float eps = norm_floor(p);
     const dim3 qgrid(p.n_kv_heads, p.batch);
-    const int64_t units = static_cast<int64_t>(p.batch) * p.n_kv_heads;
     const int rows = p.n_q_heads / p.n_kv_heads * p.window;
     auto window_norm = [&](auto elem, auto threads, auto early) {
         constexpr int kThreads = decltype(threads)::value;
         launch_kernel(window_qnorm_kernel<decltype(elem), kThreads, decltype(early)::value>, qgrid, dim3(kThreads), 0, stream, q_win, p.n_q_heads,
-                      p.n_kv_heads, p.window, eps, qnorm, seq_lens, packed_lens, max_seq_tokens, status);
+                      p.n_kv_heads, p.window, eps, qnorm, seq_lens, evict ? nullptr : packed_lens, max_seq_tokens, status);
     };
     auto by_threads = [&](auto elem, auto early) {
         const int n = qnorm_threads(units, rows, p.dtype == SPARK_BF16);
@@ -1877,7 +1877,7 @@ spark_status launch_compress(const spark_params& p, const void* q_win, const voi
         if (qnorm_release_early(units, rows, n_blocks)) by_threads(elem, std::true_type());
         else by_threads(elem, std::false_type());
     };
-    if (!evict) {                                              // (the eviction's last kernel has done it)
+    if (!evict || !norm_in_select(units)) {
         if (p.dtype == SPARK_BF16) by_release(__nv_bfloat16());
         else by_release(0.f);
         ++*launches;

@@ -13,7 +13,8 @@
 //   evict_rowstats_kernel        merge the tile partials into the row's softmax normaliser
 //   evict_scores_kernel<pass 2>  recompute the tile's scores, accumulate the column sums = votes
 //   evict_select_kernel          pooled max of the votes, exact radix select of the k-th largest, ordered compaction
-//                                of the kept positions into kept_tokens: one launch, a cluster per unit
+//                                of the kept positions into kept_tokens: one launch, a cluster per unit; with up to 256 units
+//                                (norm_in_select) also the window norm
 // Column sums are accumulated inside one CTA in a fixed order, so the votes are reproducible.
 #include <cooperative_groups.h>
 
@@ -47,6 +48,7 @@ struct EvictArgs {
     float eps;
     int bf16;            // the window queries' type
     int scored;          // the kernel before the select is the second vote pass of this call
+    int norm;            // the select kernel does the window norm too
 };
 
 template <typename E, int PASS>
@@ -253,10 +255,10 @@ __global__ void __launch_bounds__(kSelThreads) evict_select_kernel(EvictArgs A)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float* raw = reinterpret_cast<float*>(key_smem + A.key_cap);              // [kVoteTile + 2 * kVoteHalo]
     for (int i = tid; i < 4096; i += kSelThreads) hist[i] = sums[i] = 0;
-    // The window norm of the unit, by the last CTA of its cluster: under the vote pass's last CTAs (see grid_release) where there
-    // was one.  (As a launch of its own behind this kernel it cost 3 us of a prefill.)
+    // The window norm of the unit, by the last CTA of its cluster (see norm_in_select): before the wait where the vote pass ran
+    // (see grid_release).
     if (!A.scored) grid_wait();
-    if (rank == ctas - 1) {
+    if (A.norm && rank == ctas - 1) {
         double (*part)[kHeadDim] = reinterpret_cast<double (*)[kHeadDim]>(key_smem);      // (at most 16 KB; the staging tile alone has 18)
         if (A.bf16) window_norm<__nv_bfloat16, 512>(A.q_win, A.Hq, A.Hkv, A.W, A.eps, A.qnorm, h, b, tid, part, [] {});
         else window_norm<float, 512>(A.q_win, A.Hq, A.Hkv, A.W, A.eps, A.qnorm, h, b, tid, part, [] {});
@@ -501,7 +503,7 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     const size_t smem = (static_cast<size_t>(kEvTile + kEvRows) * kEvStride + kEvTile) * sizeof(float);
     const dim3 grid(A.n_tiles, p.n_kv_heads, p.batch), ugrid(p.n_kv_heads, p.batch);
     const bool bf16 = p.dtype == SPARK_BF16;
-    A.qnorm = qnorm; A.eps = norm_floor(p); A.bf16 = bf16;
+    A.qnorm = qnorm; A.eps = norm_floor(p); A.bf16 = bf16; A.norm = norm_in_select(static_cast<int64_t>(units));
     A.scored = A.n_tiles > 0 && max_seq_tokens > p.token_budget;
     // (the tensor-core kernels read the window queries 16 bytes at a time; the call does not ask for that alignment)
     const bool q_aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;

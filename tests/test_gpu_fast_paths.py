@@ -164,6 +164,22 @@ def test_eviction_with_window_queries_off_a_16_byte_boundary(dtype, G, W):
         assert y == sorted(y) and len(set(x) & set(y)) >= 99
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("n_seq,Hkv,longest,budget", [(2, 2, 700, 100), (3, 2, 90, 100), (32, 8, 80, 40), (33, 8, 80, 40), (33, 8, 30, 40)])
+def test_eviction_window_norm(dtype, n_seq, Hkv, longest, budget):
+    """The select kernel's window norm (up to 256 units), and the one of its own launch, with prompts that are evicted and
+    batches that are kept whole: bit for bit what a call without eviction writes."""
+    lens = [longest - 7 * (i % 3) for i in range(n_seq)]
+    wl = make(dtype, n_seq, 4 * Hkv, Hkv, lens, 16, 64, seed=540 + n_seq, gap=False)
+    norms = []
+    for b in (0, budget):
+        cache = SparkCache(batch=n_seq, n_q_heads=4 * Hkv, n_kv_heads=Hkv, window=16, keep=64, dtype=dtype, max_tokens=longest, token_budget=b, guard=True)
+        cache.compress(wl.q_win, wl.k, wl.v, wl.seq_lens)
+        assert cache.status() == 0 and cache.broken_guards() == []
+        norms.append(cache.qnorm)
+    assert torch.equal(*norms)
+
+
 @pytest.mark.parametrize("p,cap", [(0.5, 128), (0.95, 128), (1.0, 128), (1.0, 40), (0.95, 40)])
 def test_top_p_of_odd_values_equals_appending_them(p, cap):
     """Infinities, NaN, all-zero rows, saliencies over more than 22 octaves (their sums round, and p = 1 asks for all of
