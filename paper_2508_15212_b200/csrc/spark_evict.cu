@@ -469,7 +469,7 @@ inline int select_cluster(int64_t units, int prefix, int pool)
 bool evict_tc_supported(const spark_params& p);
 spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
                                    int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* partial,
-                                   float* votes, int* status, cudaStream_t stream, int* launches);
+                                   float* votes, int* status, cudaStream_t stream, int* launches, bool* done);
 
 size_t evict_workspace_bytes(const spark_params& p, int64_t max_seq_tokens)
 {
@@ -507,11 +507,13 @@ spark_status launch_evict(const spark_params& p, const void* q_win, const void* 
     A.scored = A.n_tiles > 0 && max_seq_tokens > p.token_budget;
     // (the tensor-core kernels read the window queries 16 bytes at a time; the call does not ask for that alignment)
     const bool q_aligned = (reinterpret_cast<uintptr_t>(q_win) & 15) == 0;
+    bool voted = !A.scored;
     if (A.scored && q_aligned && evict_tc_supported(p)) {
         const spark_status st_tc = launch_evict_votes_tc(p, q_win, k, sb, sh, st, seq_lens, max_seq_tokens, A.partial,
-                                                         A.votes, A.status, stream, launches);
+                                                         A.votes, A.status, stream, launches, &voted);
         if (st_tc != SPARK_OK) return st_tc;
-    } else if (A.scored) {
+    }
+    if (!voted) {
         static unsigned char smem_raised[4][kMaxDevices] = {};
         if (!(bf16 ? allow_max_smem(evict_scores_kernel<__nv_bfloat16, 1>, smem_raised[0]) && allow_max_smem(evict_scores_kernel<__nv_bfloat16, 2>, smem_raised[1])
                    : allow_max_smem(evict_scores_kernel<float, 1>, smem_raised[2]) && allow_max_smem(evict_scores_kernel<float, 2>, smem_raised[3])))

@@ -485,7 +485,8 @@ bool evict_tc_supported(const spark_params& p)
 }
 
 // Tensor map of the keys: (channel, token, head, sequence), copied in blocks of 64 channels x 128 tokens.  The kernels copy
-// only blocks whose rows all lie inside their sequence, so the token extent is only a bound.
+// only blocks whose rows all lie inside their sequence, so the token extent is only a bound.  False where the driver makes none: a
+// stride of 2^40 bytes or more, or a driver that wants ascending strides (the heads of token-major keys lie closer than the tokens).
 static bool key_tensor_map(CUtensorMap* map, EvictTcArgs& A, const spark_params& p, int dev)
 {
     using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -514,10 +515,11 @@ static bool key_tensor_map(CUtensorMap* map, EvictTcArgs& A, const spark_params&
     return make() || (cudaSetDevice(dev) == cudaSuccess && make());
 }
 
-// Tensor-core votes: the workspace regions `partial` and `votes` of the CUDA-core path (row statistics stay on chip).
+// Tensor-core votes: the workspace regions `partial` and `votes` of the CUDA-core path (row statistics stay on chip).  `done` says
+// whether they were enqueued: where the keys have no tensor map they are not, and nothing is.
 spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, const void* k, int64_t sb, int64_t sh,
                                    int64_t st, const int32_t* seq_lens, int32_t max_seq_tokens, float* partial,
-                                   float* votes, int* status, cudaStream_t stream, int* launches)
+                                   float* votes, int* status, cudaStream_t stream, int* launches, bool* done)
 {
     const int R = (p.n_q_heads / p.n_kv_heads) * p.window;
     const int Rpad = (R + 127) / 128 * 128;
@@ -542,7 +544,8 @@ spark_status launch_evict_votes_tc(const spark_params& p, const void* q_win, con
     A.parts = (n_tiles + A.tiles_per_cta - 1) / A.tiles_per_cta;
     A.partial = partial; A.votes = votes; A.status = status;
     CUtensorMap key_map;
-    if (!key_tensor_map(&key_map, A, p, dev)) return SPARK_ERR_CUDA;
+    *done = key_tensor_map(&key_map, A, p, dev);
+    if (!*done) return SPARK_OK;
     static unsigned char smem_raised[4][kMaxDevices] = {};
     auto both = [&](auto blocks) {
         constexpr int kBlocks = decltype(blocks)::value;

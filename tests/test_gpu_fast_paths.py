@@ -164,6 +164,23 @@ def test_eviction_with_window_queries_off_a_16_byte_boundary(dtype, G, W):
         assert y == sorted(y) and len(set(x) & set(y)) >= 99
 
 
+def test_eviction_of_keys_without_a_tensor_map():
+    """A stride that a tensor map cannot hold (2^40 bytes and more; to an empty sequence, so no row lies there): the CUDA-core
+    passes, with the kept sets of the tensor-core ones but for an exchange of two tokens with nearly equal votes."""
+    wl = make("bf16", 2, 8, 2, [1000, 0], 32, 64, seed=535, gap=False)
+    got = []
+    for stride_b in (wl.k.stride(0), 1 << 40):
+        c = SparkCache(batch=2, n_q_heads=8, n_kv_heads=2, window=32, keep=64, dtype="bf16", max_tokens=1000, token_budget=100, guard=True)
+        p = [ctypes.c_void_p(t.data_ptr()) for t in (wl.q_win, wl.k, wl.v, wl.seq_lens, c.pages, c.qnorm, c.packed_lens, c.kept_tokens, c.ws_compress)]
+        assert B.lib().spark_compress(ctypes.byref(c.params), p[0], p[1], p[2], stride_b, *wl.k.stride()[1:3], p[3], 1000, p[4], None, c.table_blocks,
+                                      *p[5:], c.ws_compress.numel(), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        assert c.status() == 0 and c.broken_guards() == [] and c.packed_lens.tolist() == [100, 0]
+        got.append(c.kept_tokens.cpu())
+    assert torch.equal(got[0][1], got[1][1])
+    for x, y in zip(got[0][0].tolist(), got[1][0].tolist()):
+        assert y == sorted(y) and len(set(x) & set(y)) >= 99
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("n_seq,Hkv,longest,budget", [(2, 2, 700, 100), (3, 2, 90, 100), (32, 8, 80, 40), (33, 8, 80, 40), (33, 8, 30, 40)])
 def test_eviction_window_norm(dtype, n_seq, Hkv, longest, budget):
