@@ -351,6 +351,7 @@ spark_status spark_unpack_pages(const spark_params* p, const void* pages, const 
     spark_status st = check_params(p);
     if (st != SPARK_OK) return st;
     if (!pages || !packed_lens) return SPARK_ERR_NULL;
+    if (misaligned(pages, 16)) return SPARK_ERR_BAD_SHAPE;
     if (contiguous_pool_too_small(p, block_table, max_blocks)) return SPARK_ERR_BAD_SHAPE;
     if (max_tokens < 0 || max_blocks < 0 || max_blocks > kMaxBlocksArg) return SPARK_ERR_BAD_SHAPE;
     if ((static_cast<int64_t>(max_tokens) + kPageTokens - 1) / kPageTokens > max_blocks)
@@ -367,6 +368,7 @@ spark_status spark_unpack_stats(const spark_params* p, const void* pages, const 
     if (st != SPARK_OK) return st;
     if (!pages || !packed_lens) return SPARK_ERR_NULL;
     if (p->recovery == SPARK_RECOVER_DEGENERATE) return SPARK_ERR_UNSUPPORTED;
+    if (misaligned(pages, 16)) return SPARK_ERR_BAD_SHAPE;
     if (contiguous_pool_too_small(p, block_table, max_blocks)) return SPARK_ERR_BAD_SHAPE;
     if (max_tokens < 0 || max_blocks < 0 || max_blocks > kMaxBlocksArg) return SPARK_ERR_BAD_SHAPE;
     if ((static_cast<int64_t>(max_tokens) + kPageTokens - 1) / kPageTokens > max_blocks)
@@ -382,6 +384,7 @@ spark_status spark_unpack_value_masks(const spark_params* p, const void* pages, 
     spark_status st = check_params(p);
     if (st != SPARK_OK) return st;
     if (!pages || !packed_lens || !vmask) return SPARK_ERR_NULL;
+    if (misaligned(pages, 16)) return SPARK_ERR_BAD_SHAPE;
     if (contiguous_pool_too_small(p, block_table, max_blocks)) return SPARK_ERR_BAD_SHAPE;
     if (max_tokens < 0 || max_blocks < 0) return SPARK_ERR_BAD_SHAPE;
     if ((static_cast<int64_t>(max_tokens) + kPageTokens - 1) / kPageTokens > max_blocks)

@@ -135,6 +135,15 @@ def test_misaligned_pointers_and_oversized_tables_are_refused_on_the_host(lib):
     assert rc == 2
 
 
+def test_unpacking_a_misaligned_pool_is_refused_on_the_host(lib):
+    """The pages are read 16 bytes at a time here too."""
+    p, sampled = params(), params(recovery=B.SPARK_RECOVER_GAUSSIAN)
+    null, one, off8 = ctypes.c_void_p(None), ctypes.c_void_p(4096), ctypes.c_void_p(4096 + 8)
+    assert lib.spark_unpack_pages(ctypes.byref(p), off8, one, 4, one, 64, one, null, null, null, null) == 2
+    assert lib.spark_unpack_value_masks(ctypes.byref(p), off8, one, 4, one, 64, one, null) == 2
+    assert lib.spark_unpack_stats(ctypes.byref(sampled), off8, one, 4, one, 64, one, one, null) == 2
+
+
 @pytest.mark.parametrize("gone", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
 def test_stream_handle_without_torchs_private_functions(monkeypatch, gone):
     """Every call looks the current stream up; a torch without the private functions takes the public one."""
