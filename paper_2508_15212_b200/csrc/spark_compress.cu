@@ -663,11 +663,6 @@ constexpr int kAdmitPasses = 4;        // values of the boundary's upper half ad
 constexpr int kTileBytes = kPageTokens * kHeadDim * 2;
 constexpr int kWarpPageFixed = kTileBytes + kPageTokens * kFewKeys * 4;      // a page's rows and its tokens' candidates
 
-__device__ __forceinline__ unsigned bits_max2(unsigned a, unsigned b)          // bf16 pairs; a NaN wins
-{
-    const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
-    return *reinterpret_cast<const unsigned*>(&r);
-}
 __device__ __forceinline__ unsigned bits_min2(unsigned a, unsigned b)          // bf16 pairs; a NaN loses
 {
     const __nv_bfloat162 r = __hmin2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));

@@ -438,7 +438,6 @@ __global__ void __launch_bounds__(tc_threads(kBlocks), kBlocks == 1 ? 2 : 1) evi
                         acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
                     }
                 }
-                if (n_rows <= 0) release();
                 if (kBlocks == 2) vote = sum_pairs(acc);
                 if (kBlocks == 2) {
                     // The second row block's warp leaves its share to the first's of the same lane quarter.  (Two slots in turn: it
