@@ -935,12 +935,12 @@ __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctr
     else merge_slices<G, NW, NS>(A, C.units, merge, C.epoch[1], warp, lane);
 }
 
-// Steps that one CTA of `grid` can own at most (either division of the line), from the cache's capacity alone.
-inline int64_t max_steps_per_cta(int64_t units, int max_blocks, int pps, int grid)
+// An even share of the line with the cache at its capacity, and 4 %.  Equal units in whole CTAs may exceed it by A.slack steps.
+inline int64_t even_steps_per_cta(int64_t units, int max_blocks, int pps, int grid)
 {
     const int64_t total = units * ((max_blocks + pps - 1) / pps);
     const int64_t chunk = (total + grid - 1) / grid;
-    return chunk + chunk / 25 + 1;                          // the aligned division may be 4 % above the even one
+    return chunk + chunk / 25 + 1;
 }
 // CTAs of the persistent grid: one per SM, fewer when the cache cannot hold a step for each.
 inline int decode_grid(int n_sms, int64_t units, int max_blocks, int pps)
