@@ -413,7 +413,7 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     A.ring_off = A.prefix_off + prefix_bytes(A.B);
     // No more slots than an even share has steps: a small call then leaves the SM room for the next kernel's CTA, whose
     // start-up runs under this one's end.  (A share with slack uses some of them twice.  With a slot for each of its steps too, us:
-    // 2 x 1000 tokens, 8 / 2 heads 16.4 -> 16.7, 2 x 200..2000, 4 / 1 18.1 -> 18.6, eleven other small batches within 0.1.)
+    // 2 x 1000 tokens, 8 / 2 heads 16.4 -> 16.7, 2 x 200..2000, 4 / 1 18.1 -> 18.6, eleven other small batches within 0.2.)
     const int64_t steps = even_steps_per_cta(units, A.max_blocks, A.pps, grid);
     const EpochRoom room = epoch_room(A, kConsumerWarps, G, S::kTabBytes, smem_optin, steps < 2 ? 2 : (steps > kMaxSlots ? kMaxSlots : static_cast<int>(steps)));
     const int one = room.ns[0];

@@ -118,10 +118,17 @@ def test_eviction_votes_at_tile_edges(G, W):
     check_eviction_case("bf16", [127, 128, 129, 255, 256, 257, 1152, 1281, 40], W, 60, G, Hkv=2, pool=3, seed=510 + G)
 
 
+@pytest.mark.parametrize("G", [4, 5])
+def test_eviction_votes_over_many_tiles(G):
+    """Up to twenty tiles a CTA with one and two blocks of query rows: every barrier comes back to its first parity and every key
+    buffer is used several times; lengths on, before and inside a tile."""
+    check_eviction_case("bf16", [5000, 4993, 5120, 5119, 4097, 3000, 5001, 2561], 32, 200, G, Hkv=8, pool=7, seed=525)
+
+
 @pytest.mark.parametrize("layout", ["token-major", "keys shared by the heads", "keys shared by the sequences", "no more rows than tokens"])
 def test_eviction_key_layouts(layout):
-    """Every order and stride of the keys that the call takes gives what the same keys in a plain tensor give.  The cache may
-    be made for longer prompts than it is given: no row past the prompt's own tensor may be read."""
+    """Every order and stride of the keys that the call takes gives what the same keys in a plain tensor give, also in a cache made
+    for longer prompts than it is given."""
     lens = [1000, 1000, 1000] if layout == "no more rows than tokens" else [1000, 130, 640]
     wl = make("bf16", 3, 8, 2, lens, 32, 64, seed=521, gap=False)
     k, v = wl.k, wl.v
