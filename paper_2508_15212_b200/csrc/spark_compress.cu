@@ -651,10 +651,11 @@ __global__ void __launch_bounds__(128, 8) compress_pages4_kernel(CompressArgs A)
 //   the mean of the token's key bits (the mean of the logarithms, near the median), moved by T's distance from the middle; then
 //   by the usual density and a step past the crossing until both ends are known, then false position: 3.8 looks (the most of
 //   sixteen tokens, T = 25 .. 89, Gaussian keys) where interpolation from the least and the largest key down to two keys took 8.3.
-//   What bounds it: issue slots (164 instructions a token, 71 % of the slots), then shared-memory wavefronts (55 %).
+//   What bounds it: issue slots (168 instructions a token, 71 % of the slots, ALU pipe 58 %), then shared memory (27 wavefronts a token,
+//   41 % of its rate).
 //   8 heads x 32768 tokens: 104 us with eight lanes per token and a bitwise descent (compress_pages4_kernel, which fp32
 //   storage and sampled recovery keep), 60 with the 8.3 looks, 57 now; the same kernel without selection, slots and mean 43.
-//   Prefill of 32K tokens 89.1 -> 85.7 us with 24 warps a SM; 87.8, 95.0, 100.4 with 20, 28, 32.
+//   Prefill of 32K tokens, builds in turn: 87.9 -> 86.6 us.  By warps a SM, in one other run: 87.8, 85.7, 95.0, 100.4 with 20, 24, 28, 32.
 // ------------------------------------------------------------------------------------------------
 constexpr int kWarpPageWarps = 4;      // pages (warps) of a CTA; one where no sequence has more (1000 x 16 tokens: 84 us with four, 57 with one)
 constexpr int kFewKeys = 8;            // keys left between the ends that are ranked by their full bits

@@ -755,7 +755,7 @@ __device__ __forceinline__ PublishWeights publish_weights(const DecodeArgs& A, i
 // CTA stands between the records and the result, and the slices of a unit are merged by several warps at once, of whatever
 // CTAs come last.  A ticket per unit and one CTA merging all of it behind four barriers took 3.6 us from the last record to
 // the result of a 32768-token step.  us before -> after: 1 x 500 tokens 9.1 -> 8.7, 32 x 2048 41.4 -> 39.5, 8 x 5000 29.7 ->
-// 28.2, 8 x 2000..16000 44.1 -> 42.1, 1 x 4096 with 64 / 8 heads 13.7 -> 12.7, fp32 1 x 1024 13.05 -> 12.8.
+// 28.2, 8 x 2000..16000 44.1 -> 42.1, 1 x 4096 with 64 / 8 heads 13.7 -> 12.7; fp32 1 x 1024, builds in turn, 13.0 -> 12.7.
 // (Three heads a group in halves: in quarters, us, 1 x 1000 tokens with 12 / 4 heads 9.2, in halves 8.9, whole 9.5; 1 x 16000 13.2, 13.0,
 // 13.7; 1 x 32768 with 6 / 2 heads 14.9, 14.5, 16.4.)
 __host__ __device__ constexpr int slices_of(int g, int nw) { return 4 * g <= 8 ? 4 : (2 * g <= nw ? 2 : 1); }

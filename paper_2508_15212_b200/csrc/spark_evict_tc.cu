@@ -14,11 +14,11 @@
 // multiplied into accumulator i & 1 as soon as its keys have landed and the accumulator has been read.  Two warpgroups per
 // block of 128 query rows take the accumulators in turn, each a whole tile, so no barrier of the CTA stands in the loop: all
 // hand-overs are mbarriers (the MMAs' through tcgen05.commit).  Every wait is bounded.
-// What bounds it: the keys' bytes (in the steady state 5.9 TB/s in pass 1), then the exponentials (1024 cycles of the SM's special function units
-// per 128 x 128 scores, 68 % busy), then a CTA's start.  With copies by all threads and a CTA barrier per tile the
-// passes over 8 x 131072 keys took 61 + 61 us, now 51 + 49: evicting prefill 170 -> 147 us; 1 x 100000 with 28 / 4 heads 155 ->
-// 122, 2 x 30000 112 -> 99.5, 4 x 4000 71 -> 66.  A quarter of the exponentials as a polynomial on the FMA pipe: 145 us
-// at 131072 and no faster elsewhere, not kept.
+// What bounds it: the exponentials (1024 cycles of the SM's special function units per 128 x 128 scores, 68 % busy in pass 1, 58 % in
+// pass 2), the keys' bytes (61 and 53 % of the DRAM's rate), then a CTA's start.  The passes over 8 x 131072 keys take 55 + 63 us one at a
+// time from a cold cache, 67 + 65 with copies by all threads and a CTA barrier per tile.  Evicting prefill then -> now (the window norm in
+// the select kernel too), builds in turn: 1 x 131072 174 -> 152 us, 1 x 100000 with 28 / 4 heads 154 -> 118, 2 x 30000 111 -> 98, 4 x 4000
+// 71 -> 61.  A quarter of the exponentials as a polynomial on the FMA pipe was no faster, but for 2 us at 131072: not kept.
 #include <cuda.h>
 
 #include <type_traits>
