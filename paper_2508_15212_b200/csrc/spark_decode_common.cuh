@@ -295,6 +295,9 @@ struct EpochUnit {
 //                 18.0, 4 x 2000..9000 19.6 -> 20.3; 40 / 8: 8 x 500..2500 16.2 -> 17.3; 28 / 4: 2 x 600..6000 14.0 -> 13.1, 12 x 300..3000 18.6 -> 16.1;
 //                 64 / 8: 2 x 600..6000 18.6 -> 14.6.  A slack of 10 or 30 steps in place of 20 gives the same within 0.1 in 26 sizes of shares
 //                 of 5 to 110 steps, but for 8 x 150..4000 with 32 / 8 heads, where one of 10 does not find a division (19.8).
+//                 kShortShare 50 / 100 / 200, 31 sizes with shares of 30 to 260 steps: 4 x 4000 16.7 / 17.2 / 17.1, 4 x 100..8000 21.4 / 17.9 / 17.8,
+//                 8 x 1000..12000 with 28 / 4 heads 26.4 / 24.0 / 24.0, 8 x 200..7000 27.5 / 27.4 / 27.8, 11 x 6000 with 16 / 4 24.7 / 24.7 / 25.3,
+//                 4 x 300..16000 27.7 / 27.0 / 25.6, 4 x 1000..14000 with 64 / 8 29.7 / 29.7 / 26.6; the others within 0.5.
 //   whole units : CTA u owns unit u.  For units of at most a step per warp, where a split saves nothing and adds a
 //                 partial, a ticket and the last arriver's merge (240 tokens: 8.4 us against 9.1; with two steps per warp
 //                 9.7 against 9.2), and for units of up to three steps per warp where they fill most of the grid anyway
