@@ -83,7 +83,12 @@ template <int G> struct SmemF32 {
     static constexpr int kEnd = (kPscr + kConsumerWarps * 32 * GPP * 4 + 127) / 128 * 128;   // then prefix, ring, records, tables
 };
 
-template <int G, typename E, int R>
+// Units of more parts than this are merged from two groups of 32 parts at a time (kWide), which takes 36 to 44 bytes of spilled registers
+// with one or two heads a group.  us with one group / two: one head, 1 x 1024 tokens (32 parts) 12.7 / 13.0, 1 x 2000 (63) 13.3 / 13.1,
+// 1 x 3685 (116) 14.5 / 13.9, 1 x 7500 (118) 14.3 / 13.8; two heads a group 14.4 / 14.7, 15.1 / 15.0, 16.5 / 16.0, 16.7 / 16.3; four KV heads,
+// 1 x 7500 (34) 14.8 / 14.7, 1 x 3685 (29) 13.0 / 13.3.
+constexpr int kFewParts = 40;
+template <int G, typename E, int R, bool kWide>
 __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const DecodeArgs A)
 {
     constexpr bool kBf16 = (sizeof(E) == 2);
@@ -355,7 +360,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_scalar_kernel(const 
             if (pos < pos_end) u = locate_unit(C.prefix, A.B, A.Hkv, pos);     // (found again: nothing of it stays in registers)
         }
         consumer_sync<kConsumerThreads>();
-        merge_and_publish<G, kConsumerWarps>(A, C, merge, cap, warp, lane);
+        merge_and_publish<G, kConsumerWarps, kWide>(A, C, merge, cap, warp, lane);
         g = C.epoch[0];
         if (g < c1) consumer_sync<kConsumerThreads>();         // the records and the epoch's description are free
     }
@@ -427,9 +432,16 @@ static spark_status launch_scalar(const DecodeArgs& A0, int dev, const DeviceInf
     }
     A.caps.middle = A.caps.longest = A.caps.even;
     const size_t smem = room.bytes(A.caps.shortest);
-    if (!allow_max_smem(decode_scalar_kernel<G, E, R>, dev, smem_optin, smem_raised)) return SPARK_ERR_CUDA;
-    return launch_kernel(decode_scalar_kernel<G, E, R>, dim3(grid), dim3(kDecodeThreads), smem, stream, A) == cudaSuccess
-               ? SPARK_OK : SPARK_ERR_CUDA;
+    auto launch = [&](auto kernel, unsigned char (&raised)[kMaxDevices]) {
+        return allow_max_smem(kernel, dev, smem_optin, raised) &&
+                       launch_kernel(kernel, dim3(grid), dim3(kDecodeThreads), smem, stream, A) == cudaSuccess
+                   ? SPARK_OK : SPARK_ERR_CUDA;
+    };
+    if constexpr (slices_of(G, kConsumerWarps) == 4) {
+        static unsigned char wide_raised[kMaxDevices] = {};
+        if (A.per_unit > kFewParts) return launch(decode_scalar_kernel<G, E, R, true>, wide_raised);
+    }
+    return launch(decode_scalar_kernel<G, E, R, false>, smem_raised);
 }
 
 template <typename E, int R>

@@ -798,7 +798,8 @@ __device__ __forceinline__ void publish(const DecodeArgs& A, int64_t row, int ch
     if (lse && A.lse) A.lse[row] = w.lse;
 }
 
-template <int G, int NW, int NS>
+// kWide: a quarter of a head is merged from two groups of 32 parts at a time.
+template <int G, int NW, int NS, bool kWide>
 __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUnit* units, float* merge, int n_units, int warp, int lane)
 {
     constexpr int kItems = G * NS;                                // slices of a unit
@@ -864,10 +865,8 @@ __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUni
         if (__shfl_sync(kFull, old, 0) != n_parts - 1) continue;
         constexpr int kLanes = kCh / 4, PP = 32 / kLanes;         // lanes of a part (four channels each); parts at a time
         constexpr int kSteps = 32 / PP, kBatch = 8;               // steps of 32 parts; loads in flight of one group of parts
-        // Groups taken at once: two for a quarter of one head (one unit on the whole grid has 148 parts; bf16, 1 x 32768 tokens, one
-        // head 11.7 -> 11.2 us).  In the kernel of 8 warps the second one spills 36 to 44 bytes and gains nothing (fp32, 1 x 1024, one
-        // head 13.0 us with two, 12.6 with one; 4 x 200..3000 with 4 / 4 heads 15.2, 14.6).
-        constexpr int kTwo = kSteps == kBatch && NW > 8 ? 2 : 1;
+        // groups taken at once (bf16, one unit on the whole grid, 148 parts: 1 x 32768 tokens 11.7 us with one, 11.2 with two)
+        constexpr int kTwo = kSteps == kBatch && kWide ? 2 : 1;
         constexpr int kGroups = kMaxCtas / 32;                    // (m, l) pairs a lane may hold
         constexpr int64_t kStride = static_cast<int64_t>(G) * kPart;
         const float* base = A.partials + (static_cast<int64_t>(d.first_cta + unit) * G + gg) * kPart;
@@ -929,13 +928,13 @@ __device__ __forceinline__ void merge_slices(const DecodeArgs& A, const EpochUni
 // 39.5 so; 2 x 3000..7000 16.1 and 14.2).  Eight warps, whose one or two heads would leave most of them idle: only with more than half
 // as many units as CTAs (fp32, 2 x 300..1000 tokens, 2 / 2 heads: whole 14.1, quarters 13.0; 4 x 200..1000, 2 / 1 heads 15.7 and 14.8;
 // but 16 x 100..2000, 8 / 8 heads 49.6 and 51.5).
-template <int G, int NW>
+template <int G, int NW, bool kWide = true>
 __device__ __forceinline__ void merge_and_publish(const DecodeArgs& A, const Ctrl& C, float* merge, int cap, int warp, int lane)
 {
     constexpr int NS = slices_of(G, NW);
     const bool whole = NW > 8 ? cap > 1 : 2 * A.B * A.Hkv > static_cast<int>(gridDim.x);       // (the same in every CTA)
-    if (NS == 1 || whole) merge_slices<G, NW, 1>(A, C.units, merge, C.epoch[1], warp, lane);
-    else merge_slices<G, NW, NS>(A, C.units, merge, C.epoch[1], warp, lane);
+    if (NS == 1 || whole) merge_slices<G, NW, 1, kWide>(A, C.units, merge, C.epoch[1], warp, lane);
+    else merge_slices<G, NW, NS, kWide>(A, C.units, merge, C.epoch[1], warp, lane);
 }
 
 // An even share of the line with the cache at its capacity, and 4 %.  Equal units in whole CTAs may exceed it by A.slack steps.

@@ -265,6 +265,12 @@ def test_division_of_the_step(name, Hq, Hkv, lens):
     check_case(make("bf16", len(lens), Hq, Hkv, lens, 8, 64, seed=400 + len(lens), gap=False), 64, check_vals=False)
 
 
+@pytest.mark.parametrize("Hq,Hkv,n", [(1, 1, 1280), (1, 1, 1312), (1, 1, 7500), (2, 1, 4736), (2, 1, 4737), (4, 2, 3000), (3, 3, 1600)])
+def test_fp32_units_of_many_parts(Hq, Hkv, n):
+    """One and two heads a group, a unit over up to 148 CTAs: one group of 32 parts at a time and two, whole and partly filled."""
+    check_case(make("f32", 1, Hq, Hkv, [n], 8, 64, seed=480 + Hq, sigma=0.5, gap=False), 64, check_vals=False)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("Hq,Hkv,lens", [
     (8, 4, [4000, 150, 700, 1300, 16, 0, 2900, 333]),
